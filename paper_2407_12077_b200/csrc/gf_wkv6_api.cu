@@ -81,9 +81,9 @@ gf_status_t run_exact(const IO* r, const IO* k, const IO* v, const IO* x, const 
 {
     const long long units = (long long)n_seq * H;
     if (units > 0x7fffffffLL) return GF_ERR_INVALID_ARG;
-    gf::wkv6_exact_kernel<IO><<<(unsigned)units, gf::EX_THREADS, 0, st>>>(r, k, v, x, u, state_in, state_out, y, cu, T, H);
+    const cudaError_t e = gf::launch_exact<IO>(units, gf::sm_count(), st, r, k, v, x, u, state_in, state_out, y, cu, T, H);
     g_launches.fetch_add(1, std::memory_order_relaxed);
-    return launch_result();
+    return e == cudaSuccess ? GF_OK : GF_ERR_CUDA;
 }
 
 template <typename IO>

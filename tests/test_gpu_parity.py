@@ -60,6 +60,14 @@ def test_exact_kernel_ragged_lengths(T, dtype):
     dense_case(2, T, 3, dtype, seed=100 + T, state_std=0.1, kernel="exact")
 
 
+@pytest.mark.parametrize("B,H", [(1, 18), (1, 19), (2, 37), (3, 25)])
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+def test_exact_kernel_column_slabs(B, H, dtype):
+    # units on both sides of the slab rule (eight, four or one CTA per unit on a GPU of 148 SMs); two tiles plus a token.
+    # Tolerance: the contract's.
+    dense_case(B, 33, H, dtype, seed=140 + B * H, state_std=0.1, kernel="exact")
+
+
 @pytest.mark.parametrize("T", [1, 2, 15, 16, 17, 63, 64, 65, 127, 128, 129, 200, 321, 1000])
 @pytest.mark.parametrize("state_std", [0.0, 0.1])
 def test_chunked_kernel_ragged_lengths(T, state_std):
