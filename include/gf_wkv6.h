@@ -219,7 +219,7 @@ GF_API size_t gf_wkv6_backward_varlen_workspace_bytes(int S, int total_T, int H,
 
 /* The training pair for packed sequences, as gf_wkv6_prefill_train / gf_wkv6_backward_saved for dense ones:
  * gf_wkv6_prefill_varlen_train / gf_wkv6_prefill_varlen_c2_train are gf_wkv6_prefill_varlen / gf_wkv6_prefill_varlen_c2
- * (same results; one CTA per sequence and head, never split and never persistent) that also leave the state before every
+ * (same results; never split, one or two kernels) that also leave the state before every
  * chunk of 64 tokens of every sequence, and after its last token, in `workspace`, the packed gradient's workspace
  * (gf_wkv6_backward_varlen_workspace_bytes(S,total_T,H,N) bytes); gf_wkv6_backward_varlen_saved /
  * gf_wkv6_backward_varlen_c2_saved are the packed gradient calls without their checkpoint launch.  The workspace must
@@ -299,7 +299,9 @@ GF_API size_t gf_wkv6_host_workspace_bytes(int B, int T, int H, int N);
  * (a unit's pipeline fill overlaps the drain of the one before); a packed call of that kind draws its units,
  * longest sequences first, from a counter in the workspace (a small kernel of the call itself, on `stream`,
  * zeroes the counter and ranks the sequences there) and falls back to one CTA per unit without a workspace; a
- * dense one needs none.  gf_wkv6_workspace_bytes returns what gf_wkv6_prefill(B,T,H,N) (packed: B = S,
+ * dense one needs none.  Where whole units would leave many SMs idle in the last round, a dense call with a state_out
+ * cuts units between neighbouring SMs and hands the state over in state_out[unit] and y while it runs (results as
+ * without the cut, bit for bit).  gf_wkv6_workspace_bytes returns what gf_wkv6_prefill(B,T,H,N) (packed: B = S,
  * T = max_seqlen) would use on the current device: the summaries and start-state copies of a split, 64 + 4*S
  * bytes (rounded up to 256) for more units than SMs, else 0.  gf_wkv6_set_workspace registers a caller-owned
  * DEVICE buffer (256-byte aligned; NULL unregisters) for all later calls of this process; the library

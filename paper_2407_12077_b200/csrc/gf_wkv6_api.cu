@@ -577,7 +577,7 @@ gf_status_t gf_wkv6_backward_varlen_c2_saved(const void* r, const void* k, const
 
 namespace {
 // forward pass of a training step over packed sequences: the packed prefill that also leaves its chunk-start states
-// (packed layout) in the packed gradient's workspace; one CTA per sequence and head, never split
+// (packed layout) in the packed gradient's workspace; never split
 gf_status_t prefill_varlen_train(const void* r, const void* k, const void* v, const void* x, const float* u,
                                  const void* u2, const float* state_in, float* state_out, void* y,
                                  const int32_t* cu_seqlens, int S, int total_T, int max_seqlen, int H, int N,
@@ -600,8 +600,10 @@ gf_status_t prefill_varlen_train(const void* r, const void* k, const void* v, co
     const size_t need = gf_wkv6_backward_varlen_workspace_bytes(S, total_T, H, N);
     if (need == 0) return GF_ERR_CUDA;
     if (!workspace || workspace_bytes < need) return GF_ERR_WORKSPACE;
+    size_t abytes = 0;
+    float* area = gf::backward_workspace_order_area(static_cast<float*>(workspace), S, total_T, H, gf::sm_count(), &abytes);
     const gf_status_t s = gf::chunked_prefill((const bf*)r, (const bf*)k, (const bf*)v, (const bf*)x, u, state_in, state_out,
-                                              (bf*)y, cu_seqlens, S, max_seqlen, total_T, H, st, &g_launches, nullptr, 0,
+                                              (bf*)y, cu_seqlens, S, max_seqlen, total_T, H, st, &g_launches, area, abytes,
                                               (const bf*)u2, c2 ? 1 : 0, static_cast<float*>(workspace));
     if (s != GF_OK) return s;
     return launch_result();

@@ -1082,6 +1082,16 @@ inline float* backward_workspace_forward_scratch(float* ws, long long units, int
     return ws + (size_t)units * nck * bc::CKPT_FLOATS + (size_t)units * nseg * 64 + (size_t)units * (nseg - 1) * bc::GSUM_FLOATS;
 }
 
+// The part of the packed gradient's workspace that its forward pass may use for the counter and the sequence order of a
+// persistent launch (the gradient call writes its own there).
+inline float* backward_workspace_order_area(float* ws, long long n_seq, long long total_rows, int H, int n_sm, size_t* bytes)
+{
+    const size_t slots = (size_t)(total_rows / ck::L + 2 * n_seq);
+    const size_t units = (size_t)n_seq * H, nmax = (size_t)packed_split_max((long long)units, n_sm);
+    *bytes = backward_order_floats(n_seq) * sizeof(float);
+    return ws + (size_t)H * slots * bc::CKPT_FLOATS + units * nmax * 64 + units * (nmax - 1) * bc::GSUM_FLOATS;
+}
+
 inline gf_status_t chunked_backward(const __nv_bfloat16* r, const __nv_bfloat16* k, const __nv_bfloat16* v,
                                     const __nv_bfloat16* x, const float* u, const float* state_in,
                                     const __nv_bfloat16* dy, const float* dstate_out, __nv_bfloat16* dr,

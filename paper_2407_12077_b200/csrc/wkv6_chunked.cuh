@@ -39,12 +39,14 @@
 // (the Finch-C2 form: keys times one minus their decay, no bonus, optional per-token vector added to
 // the output) and PERSIST (calls with more units than SMs: one CTA per SM walks a stream of units,
 // the producer leaving a descriptor per chunk and two end markers that every role hands on, so that
-// the pipeline is filled and drained once per CTA instead of once per unit).
+// the pipeline is filled and drained once per CTA instead of once per unit; PERSIST = 2 also cuts units
+// between neighbouring CTAs, so that every CTA gets the same number of chunks: see Params::bal_chunks).
 #pragma once
 #include <atomic>
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
+#include <random>
 #include <stdint.h>
 
 #include "device_info.cuh"
@@ -124,13 +126,16 @@ enum {
     BAR_SPRE = BAR_SSYNC + 1,            //   and before it is written,
     BAR_FB_READY = BAR_SPRE + 1,         //   fp32 state copy in place for the output warps,
     BAR_FB_DONE = BAR_FB_READY + 1,      //   and advanced by them over the chunk
-    BAR_U2 = BAR_FB_DONE + 1,            // Finch-C2 form: one per output warp, its second-value slab has landed
-    BAR_COUNT = BAR_U2 + N_GW
+    BAR_U2 = BAR_FB_DONE + 1,            // Finch-C2 form: per output warp and slab, its second-value rows have landed
+    BAR_COUNT = BAR_U2 + 2 * N_GW
 };
 // persistent launches: one descriptor per chunk of the CTA's chunk stream
 // {first row, valid tokens | flags | head << 16, unit, chunks left in the unit}
 constexpr int OFF_DESC = (OFF_BAR + BAR_COUNT * 8 + 15) & ~15;   // [NSIDE] int4
-constexpr int DESC_FIRST = 0x100, DESC_END = 0x200;              // flags beside the valid-token count (low byte)
+// flags beside the valid-token count (low byte): first chunk of a unit (or piece of one), no chunk, piece that continues
+// a unit another CTA began, last chunk of a piece
+constexpr int DESC_FIRST = 0x100, DESC_END = 0x200, DESC_CONT = 0x400, DESC_LAST = 0x800;
+constexpr int DESC_TAG = 0x1000;                                 // (balanced launches) parity of the ring's turn: (chunk / NSIDE) & 1
 constexpr int SMEM_BYTES = OFF_DESC + NSIDE * 16;
 constexpr int SMEM_ALLOC = SMEM_BYTES + 1024;              // slack for manual 1024-byte alignment
 static_assert(SMEM_ALLOC <= 232448, "shared memory budget of one sm_100 CTA");
@@ -231,6 +236,45 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, uint32_
 {
     if (mbar_try_wait(bar, parity)) return true;
     return mbar_wait_slow(bar, parity, abort_flag, poll_abort);
+}
+
+// Bounded wait for the tag of a chunk descriptor in shared memory; false as above.
+__device__ __noinline__ bool desc_wait(uint32_t meta_addr, uint32_t tag, uint32_t abort_flag)
+{
+    const unsigned long long t0 = globaltimer();
+    const unsigned long long limit_ns = 1000ull * lds32(abort_flag + 4);
+    for (;;) {
+        for (int it = 0; it < 64; ++it) {
+            uint32_t m;
+            asm volatile("ld.acquire.cta.shared::cta.u32 %0, [%1];" : "=r"(m) : "r"(meta_addr) : "memory");
+            if ((m & (uint32_t)DESC_TAG) == tag) return true;
+        }
+        if (lds32(abort_flag)) return false;
+        if (globaltimer() - t0 > limit_ns) break;
+        __nanosleep(64);
+    }
+    sts32(abort_flag, 1u);
+    atomicExch(&g_dev_status, 1);
+    return false;
+}
+// Bounded wait of one lane for a word another CTA writes (with release semantics); false as above.
+__device__ __noinline__ bool word_wait(const unsigned long long* w, unsigned long long value, uint32_t abort_flag)
+{
+    const unsigned long long t0 = globaltimer();
+    const unsigned long long limit_ns = 1000ull * lds32(abort_flag + 4);
+    for (;;) {
+        for (int it = 0; it < 64; ++it) {
+            unsigned long long v;
+            asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(w) : "memory");
+            if (v == value) return true;
+        }
+        if (lds32(abort_flag)) return false;
+        if (globaltimer() - t0 > limit_ns) break;
+        __nanosleep(64);
+    }
+    sts32(abort_flag, 1u);
+    atomicExch(&g_dev_status, 1);
+    return false;
 }
 
 // Warp-uniform form: every lane of a converged warp waits and all get the same answer, so the
@@ -486,6 +530,16 @@ struct Params {
     // ckpt_slots = total_T / 64 + 2 S.
     float* ckpt;
     long long ckpt_slots;
+    // Balanced persistent launches (PERSIST = 2; dense calls with more units than SMs, state_out given): bal_chunks =
+    // chunks per unit.  While at least two units per CTA are left they are handed out whole, unit b + k gridDim to CTA b;
+    // the chunks of the rest, in order, are cut into gridDim equal ranges of one to two units each, so a unit may
+    // begin in one CTA's range and end in the next one's.  A CTA takes the beginning of such a unit first of all and
+    // the end of one last, so the state at the cut is there long before it is wanted: it is handed over in
+    // state_out[unit] (which the unit's end overwrites with the final state), announced by four words equal to `nonce`
+    // (one per state warp; a number no earlier launch has used) in the first y row after the cut, which that chunk's
+    // output overwrites.  The launch is cooperative: every CTA a cut waits for is resident.
+    int bal_chunks;
+    unsigned long long nonce;
 };
 constexpr int SUMMARY_FLOATS = 64 + 64 * 64;
 
@@ -639,11 +693,12 @@ __device__ __forceinline__ void exact_chunk(float* scr, const Params& p, int h, 
 // the second MMA warp idle, the output warps only serve the token-by-token path) and writes the
 // segment's summary.
 // C2 = true: the Finch-C2 form (keys times one minus their decay, no bonus, optional second-value vector).
-// PERSIST = true: the CTA walks a stream of units (see Params::n_units); the producer warp leaves a descriptor per
-// chunk and two end markers, which every role passes down its own signalling path before it leaves.
-// CKPT = true (single-unit launches of the prefill proper, split or not): the state before every chunk and after the last
-// one is also left in Params::ckpt, for the gradient call that follows a training step's forward pass.
-template <bool SUMMARY, bool C2, bool PERSIST = false, bool CKPT = false>
+// PERSIST != 0: the CTA walks a stream of units (see Params::n_units); the producer warp leaves a descriptor per
+// chunk and two end markers, which every role passes down its own signalling path before it leaves.  PERSIST = 2: the
+// stream may begin and end inside a unit (see Params::bal_chunks).
+// CKPT = true (launches of the prefill proper): the state before every chunk and after the last one is also left in
+// Params::ckpt, for the gradient call that follows a training step's forward pass.
+template <bool SUMMARY, bool C2, int PERSIST = 0, bool CKPT = false>
 __global__ void __launch_bounds__(THREADS, 1)
 wkv6_chunked_kernel(const __grid_constant__ CUtensorMap tm_r, const __grid_constant__ CUtensorMap tm_k,
                     const __grid_constant__ CUtensorMap tm_v, const __grid_constant__ CUtensorMap tm_x,
@@ -697,12 +752,13 @@ wkv6_chunked_kernel(const __grid_constant__ CUtensorMap tm_r, const __grid_const
     const int col0 = h * 64;
     const size_t C = (size_t)p.H * 64;
     static_assert(!(PERSIST && SUMMARY), "the summary pass is a single-unit launch");
-    static_assert(!(CKPT && (PERSIST || SUMMARY)), "checkpoints of the prefill proper: single-unit launches only");
+    static_assert(!(CKPT && SUMMARY), "the summary pass keeps its checkpoints by Params::ckpt");
+    constexpr bool BAL = PERSIST == 2;
 
     // One chunk of this CTA's work.  Single-unit launches derive it from the chunk index; persistent launches
     // read the descriptor the producer warp left for the chunk, which is visible to any warp that has waited
     // on a barrier downstream of the chunk's "full" barrier.
-    struct Chunk { int row; int valid; int unit; int h; int rem; bool first; bool end; };
+    struct Chunk { int row; int valid; int unit; int h; int rem; bool first; bool last; bool end; };
     auto chunk_at = [&](int c) -> Chunk {
         Chunk ck;
         if constexpr (PERSIST) {
@@ -710,12 +766,15 @@ wkv6_chunked_kernel(const __grid_constant__ CUtensorMap tm_r, const __grid_const
             asm volatile("ld.shared.v4.s32 {%0, %1, %2, %3}, [%4];"
                          : "=r"(d.x), "=r"(d.y), "=r"(d.z), "=r"(d.w) : "r"(sbase + OFF_DESC + 16 * (c & (NSIDE - 1))) : "memory");
             ck.row = d.x; ck.valid = d.y & 0xff; ck.unit = d.z; ck.h = d.y >> 16; ck.rem = d.w;
-            ck.first = (d.y & DESC_FIRST) != 0; ck.end = (d.y & DESC_END) != 0;
+            ck.first = (d.y & DESC_FIRST) != 0; ck.last = BAL ? (d.y & DESC_LAST) != 0 : d.w == 0; ck.end = (d.y & DESC_END) != 0;
         } else {
             ck.row = (int)(row0 + (long long)c * L); ck.valid = min(L, len - c * L); ck.unit = unit; ck.h = h;
-            ck.rem = nchunks - 1 - c; ck.first = c == 0; ck.end = false;
+            ck.rem = nchunks - 1 - c; ck.first = c == 0; ck.last = ck.rem == 0; ck.end = false;
         }
         return ck;
+    };
+    auto chunk_continues = [&](int c) -> bool {      // (balanced launches) a piece of a unit that another CTA began
+        return (lds32(sbase + OFF_DESC + 16 * (c & (NSIDE - 1)) + 4) & DESC_CONT) != 0;
     };
     auto chunk_is_end = [&](int c) -> bool {
         if constexpr (PERSIST) return (lds32(sbase + OFF_DESC + 16 * (c & (NSIDE - 1)) + 4) & DESC_END) != 0;
@@ -741,7 +800,9 @@ wkv6_chunked_kernel(const __grid_constant__ CUtensorMap tm_r, const __grid_const
         mbar_init(bar(BAR_SPRE), N_GW);
         mbar_init(bar(BAR_FB_READY), N_GW);
         mbar_init(bar(BAR_FB_DONE), N_GW);
-        for (int i = 0; i < N_GW; ++i) mbar_init(bar(BAR_U2 + i), 1);
+        for (int i = 0; i < (C2 && BAL ? 2 : 1) * N_GW; ++i) mbar_init(bar(BAR_U2 + i), 1);
+        if (C2 && BAL)
+            for (int i = 0; i < NSIDE; ++i) sts32(sbase + OFF_DESC + 16 * i + 4, DESC_TAG);        // (of the turn before the first)
         sts32(abort_flag, 0u);
         sts32(abort_flag + 4, p.wait_limit_us ? p.wait_limit_us : WAIT_LIMIT_US);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -753,6 +814,16 @@ wkv6_chunked_kernel(const __grid_constant__ CUtensorMap tm_r, const __grid_const
     tc_fence_after();
     const uint32_t tmem = lds32(sbase + OFF_TMEM);
 
+    // (producer lane) leaves the descriptor of chunk gc of the stream.  Roles that wait on a barrier downstream of the
+    // chunk's copies find it complete; the tag, written last, is for the one that looks at it earlier (desc_wait).
+    auto put_desc = [&](int gc, int row, int meta, int u, int rem) {
+        const uint32_t d = sbase + OFF_DESC + 16 * (gc & (NSIDE - 1));
+        const int tag = ((gc / NSIDE) & 1) * DESC_TAG;
+        if (C2 && BAL) meta |= tag ^ DESC_TAG;
+        asm volatile("st.shared.v4.s32 [%0], {%1, %2, %3, %4};" ::"r"(d), "r"(row), "r"(meta), "r"(u), "r"(rem) : "memory");
+        if (C2 && BAL) asm volatile("st.release.cta.shared::cta.u32 [%0], %1;" ::"r"(d + 4), "r"(meta ^ DESC_TAG) : "memory");
+    };
+
     if (warp == 0) {
         // ============================== TMA producer ==============================
         if constexpr (PERSIST) {
@@ -760,8 +831,40 @@ wkv6_chunked_kernel(const __grid_constant__ CUtensorMap tm_r, const __grid_const
             int s = 0, ph = 1;                       // ring stage and the parity of its previous release
             bool alive = true;
             for (int k = 0; alive; ++k) {
-                int u = 0;
-                if (p.ticket) {
+                int u = 0, c0 = 0, c1 = 0;               // the next piece: chunks c0 .. c1-1 of unit u (balanced launches)
+                if constexpr (BAL) {
+                    // First the beginning of the unit this CTA's range ends in, then whole units, last the end of the unit
+                    // the range begins in.  (32-bit products: the host balances only calls whose chunk counts allow it.)
+                    const unsigned G = gridDim.x, nc = p.bal_chunks, rounds = p.n_units / G - 1, R = p.n_units - rounds * G, bi = blockIdx.x;
+                    const unsigned b0 = R * nc * bi / G, b1 = R * nc * (bi + 1) / G;
+                    const unsigned head = b1 % nc, tail = b0 % nc;
+                    int kk = k - (head != 0);
+                    c1 = nc;
+                    // Which unit: neighbouring heads share lines of memory, so units processed at the same time get
+                    // neighbouring indices.  The cut ones come first, by CTA (their beginnings all start the launch and
+                    // their ends all close it), then the whole ones by the time at which their CTA starts them.
+                    auto cuts_before = [&](unsigned n) {                                     // cuts at the ends of the first n CTAs
+                        int cuts = 0;
+                        for (unsigned b = lane; b < n; b += 32) cuts += R * nc * (b + 1) / G % nc != 0;
+                        return (unsigned)__reduce_add_sync(0xffffffffu, cuts);
+                    };
+                    if (kk < 0) { u = rounds * G + cuts_before(bi); c1 = head; }
+                    else if (kk < (int)rounds) u = bi + kk * G;
+                    else {
+                        kk -= rounds;
+                        const bool whole = b1 / nc > (b0 + nc - 1) / nc;                     // (a range holds at most one whole unit)
+                        if (whole && kk == 0) {
+                            int before = 0;
+                            for (unsigned b = lane; b < G; b += 32) {
+                                const unsigned e0 = R * nc * b / G, e1 = R * nc * (b + 1) / G, eh = e1 % nc;
+                                before += e1 / nc > (e0 + nc - 1) / nc && (eh < head || (eh == head && b < bi));
+                            }
+                            u = rounds * G + cuts_before(G) + __reduce_add_sync(0xffffffffu, before);
+                        } else if (kk == (whole ? 1 : 0) && tail != 0) {
+                            u = rounds * G + cuts_before(bi) - 1; c0 = tail;
+                        } else break;
+                    }
+                } else if (p.ticket) {
                     if (lane == 0) u = (int)atomicAdd(p.ticket, 1u);
                     u = __shfl_sync(0xffffffffu, u, 0);
                 } else {
@@ -789,23 +892,29 @@ wkv6_chunked_kernel(const __grid_constant__ CUtensorMap tm_r, const __grid_const
                     if (p.state_out && p.state_out != p.state_in)
                         for (int i = lane; i < 4096; i += 32)
                             p.state_out[(size_t)u * 4096 + i] = p.state_in ? p.state_in[(size_t)u * 4096 + i] : 0.f;
+                    if constexpr (CKPT) {                    // (its only checkpoint, in the packed layout of ckpt_slot above)
+                        const size_t slot = (size_t)uh * p.ckpt_slots + (size_t)(p.cu_seqlens[useq] >> 6) + 2 * (size_t)useq;
+                        for (int i = lane; i < 4096; i += 32)
+                            reinterpret_cast<__nv_bfloat16*>(p.ckpt)[slot * 4096 + i] = __float2bfloat16_rn(p.state_in ? p.state_in[(size_t)u * 4096 + i] : 0.f);
+                    }
                     continue;
                 }
-                if (p.state_in) {
+                if (!BAL) c1 = unch;
+                if (p.state_in && (!BAL || c0 == 0)) {
                     // the state warps read this unit's start state a few chunks from now: have it in L2 by then
                     const char* sp0 = reinterpret_cast<const char*>(p.state_in + (size_t)u * 4096);
 #pragma unroll
                     for (int i = 0; i < 4; ++i)
                         asm volatile("prefetch.global.L2 [%0];" ::"l"(sp0 + 128 * (lane + 32 * i)));
                 }
-                for (int c = 0; c < unch; ++c, ++gc) {
+                for (int c = c0; c < c1; ++c, ++gc) {
                     if (gc >= NS && !mbar_wait_warp(bar(BAR_EMPTY_RKV + s), ph, abort_flag)) { alive = false; break; }
                     const int row = (int)(urow0 + (long long)c * L);
                     const uint32_t dst = sbase + OFF_RING + s * STAGE;
                     if (elect_one()) {
-                        const int meta = min(L, ulen - c * L) | (c == 0 ? DESC_FIRST : 0) | (uh << 16);
-                        asm volatile("st.shared.v4.s32 [%0], {%1, %2, %3, %4};" ::"r"(sbase + OFF_DESC + 16 * (gc & (NSIDE - 1))),
-                                     "r"(row), "r"(meta), "r"(u), "r"(unch - 1 - c) : "memory");
+                        int meta = min(L, ulen - c * L) | (c == c0 ? DESC_FIRST : 0) | (uh << 16);
+                        if (BAL) meta |= (c == c0 && c0 > 0 ? DESC_CONT : 0) | (c == c1 - 1 ? DESC_LAST : 0);
+                        put_desc(gc, row, meta, u, unch - 1 - c);
                         mbar_expect_tx(bar(BAR_FULL_RKV + s), STAGE);      // (release: the descriptor is visible to the waiters)
                         tma_load_2d(dst, &tm_x, uh * 64, row, bar(BAR_FULL_RKV + s));
                         tma_load_2d(dst + TILE, &tm_r, uh * 64, row, bar(BAR_FULL_RKV + s));
@@ -822,8 +931,7 @@ wkv6_chunked_kernel(const __grid_constant__ CUtensorMap tm_r, const __grid_const
                 for (int e = 0; e < 2 && alive; ++e, ++gc) {
                     if (gc >= NS && !mbar_wait_warp(bar(BAR_EMPTY_RKV + s), ph, abort_flag)) { alive = false; break; }
                     if (elect_one()) {
-                        asm volatile("st.shared.v4.s32 [%0], {%1, %2, %3, %4};" ::"r"(sbase + OFF_DESC + 16 * (gc & (NSIDE - 1))),
-                                     "r"(0), "r"(DESC_END), "r"(0), "r"(0) : "memory");
+                        put_desc(gc, 0, DESC_END, 0, 0);
                         mbar_arrive(bar(BAR_FULL_RKV + s));                 // no copy: the arrival alone completes the phase
                     }
                     __syncwarp();
@@ -1001,9 +1109,9 @@ wkv6_chunked_kernel(const __grid_constant__ CUtensorMap tm_r, const __grid_const
         // warp sends its 16 rows of the tile to the checkpoint array by TMA (tm_ck16: the array as [slots * 64][64]).
         constexpr bool CK_TMA = CKPT || SUMMARY;
         const bool ck_on = CKPT || (SUMMARY && p.ckpt);
-        auto ckpt_tile = [&](int tile, int c_abs) {      // after the tile's rows are written, fenced and the warp synchronised
+        auto ckpt_tile = [&](int tile, size_t slot) {    // after the tile's rows are written, fenced and the warp synchronised
             if (lane == 0) {
-                tma_store_2d(&tm_ck16, 0, (int)(ckpt_slot(c_abs) * 64) + 16 * sp, sbase + OFF_SB + tile * TILE + 16 * sp * 128);
+                tma_store_2d(&tm_ck16, 0, (int)(slot * 64) + 16 * sp, sbase + OFF_SB + tile * TILE + 16 * sp * 128);
                 bulk_commit();
             }
         };
@@ -1012,14 +1120,15 @@ wkv6_chunked_kernel(const __grid_constant__ CUtensorMap tm_r, const __grid_const
             fence_proxy_async();
             __syncwarp();
             mbar_arrive_if(bar(BAR_S_READY), lane == 0);
-            if (CKPT) ckpt_tile(0, seg * p.seg_chunks);
+            if (CKPT) ckpt_tile(0, ckpt_slot(seg * p.seg_chunks));
         }
         if (SUMMARY && ck_on && nchunks > 0) {
             store_acc_bf16(sbase + OFF_SB, 16 * sp, st, lane);
             fence_proxy_async();
             __syncwarp();
-            ckpt_tile(0, seg * p.seg_chunks);
+            ckpt_tile(0, ckpt_slot(seg * p.seg_chunks));
         }
+        int pslot = 0;                           // (persistent launches) checkpoint slot of the current chunk's start state
         for (int c = 0; PERSIST || c < nchunks; ++c) {
             const int tb = c & 1, pt = (c >> 1) & 1, sd = c & (NSIDE - 1);
             if (!mbar_wait(bar(BAR_F_FULL + tb), pt, abort_flag)) break;
@@ -1037,12 +1146,37 @@ wkv6_chunked_kernel(const __grid_constant__ CUtensorMap tm_r, const __grid_const
             if (PERSIST && ck.first) {
                 // a new unit starts with this chunk: its state replaces the registers, and the operand tile of
                 // this chunk (last read by the products of chunk c-2) takes its bf16 copy
-                load_state((size_t)ck.unit * 4096);
+                if (BAL && chunk_continues(c)) {
+                    // ... or continues one whose beginning another CTA has: the state at the cut, from state_out
+                    bool ok = true;
+                    if (lane == 0) {
+                        ok = word_wait(reinterpret_cast<const unsigned long long*>(p.y + (size_t)ck.row * C + ck.h * 64) + sp, p.nonce, abort_flag);
+                        asm volatile("fence.proxy.async.global;" ::: "memory");       // (the y tile that replaces the word goes by TMA)
+                    }
+                    if (!__all_sync(0xffffffffu, ok)) break;
+                    const float* src = p.state_out + (size_t)ck.unit * 4096 + 2 * q;
+#pragma unroll
+                    for (int n = 0; n < 8; ++n) {
+                        const float2 lo = __ldcg(reinterpret_cast<const float2*>(src + (size_t)c_lo * 64 + 8 * n));
+                        const float2 hi = __ldcg(reinterpret_cast<const float2*>(src + (size_t)(c_lo + 8) * 64 + 8 * n));
+                        st[n][0] = lo.x; st[n][1] = lo.y; st[n][2] = hi.x; st[n][3] = hi.y;
+                    }
+                } else {
+                    load_state((size_t)ck.unit * 4096);
+                }
                 if (c >= 2 && !mbar_wait(bar(BAR_B_DONE + tb), ((c - 2) >> 1) & 1, abort_flag)) break;
+                if (CKPT) {
+                    const int useq = ck.unit / p.H;
+                    if (p.cu_seqlens) pslot = (int)((ck.unit - useq * p.H) * p.ckpt_slots) + (p.cu_seqlens[useq] >> 6) + 2 * useq;
+                    else pslot = ck.unit * ((p.T + L - 1) / L + 1) + (BAL ? p.bal_chunks - 1 - ck.rem : 0);
+                    if (lane == 0) bulk_wait_read<1>();      // the checkpoint copy of chunk c - 2 has finished reading this tile
+                    __syncwarp();
+                }
                 store_acc_bf16(sbase + OFF_SB + tb * TILE, 16 * sp, st, lane);
                 fence_proxy_async();
                 __syncwarp();
                 mbar_arrive_if(bar(BAR_S_READY + tb), lane == 0);
+                if (CKPT) ckpt_tile(tb, pslot);
             }
             bool next_tile_free = c == 0;        // the products of chunk c-1 have finished reading operand tile tb^1
             const uint32_t dl = sbase + OFF_DL + 4 * (sd * 64 + c_lo);
@@ -1106,7 +1240,7 @@ wkv6_chunked_kernel(const __grid_constant__ CUtensorMap tm_r, const __grid_const
                 if (!mbar_wait(bar(BAR_SSYNC), fb_uses & 1, abort_flag)) break;
                 ++fb_uses;
             }
-            if (!SUMMARY && ck.rem > 0) {
+            if (!SUMMARY && !ck.last) {
                 const int nb = tb ^ 1;
                 if (!next_tile_free && !mbar_wait(bar(BAR_B_DONE + nb), ((c - 1) >> 1) & 1, abort_flag)) break;
                 if (CKPT) {                          // the checkpoint copy of chunk c - 1 has finished reading this tile
@@ -1117,7 +1251,7 @@ wkv6_chunked_kernel(const __grid_constant__ CUtensorMap tm_r, const __grid_const
                 fence_proxy_async();
                 __syncwarp();
                 mbar_arrive_if(bar(BAR_S_READY + nb), lane == 0);
-                if (CKPT) ckpt_tile(nb, seg * p.seg_chunks + c + 1);
+                if (CKPT) ckpt_tile(nb, PERSIST ? (size_t)++pslot : ckpt_slot(seg * p.seg_chunks + c + 1));
             }
             if (SUMMARY && ck_on && ck.rem > 0) {    // (no product reads these tiles in a summary pass)
                 const int nb = tb ^ 1;
@@ -1126,12 +1260,22 @@ wkv6_chunked_kernel(const __grid_constant__ CUtensorMap tm_r, const __grid_const
                 store_acc_bf16(sbase + OFF_SB + nb * TILE, 16 * sp, st, lane);
                 fence_proxy_async();
                 __syncwarp();
-                ckpt_tile(nb, seg * p.seg_chunks + c + 1);
+                ckpt_tile(nb, ckpt_slot(seg * p.seg_chunks + c + 1));
             }
-            if (PERSIST && ck.rem == 0 && p.state_out && !lds32(abort_flag)) store_state((size_t)ck.unit * 4096);
+            if (PERSIST && ck.last && !lds32(abort_flag)) {
+                if (BAL || p.state_out) store_state((size_t)ck.unit * 4096);
+                if (CKPT && ck.rem == 0) store_ckpt(pslot + 1);
+                if (BAL && ck.rem > 0) {             // a cut: the CTA that holds the rest of the unit may have the state
+                    __threadfence();
+                    __syncwarp();
+                    if (lane == 0)
+                        asm volatile("st.release.gpu.global.u64 [%0], %1;"
+                                     ::"l"(reinterpret_cast<unsigned long long*>(p.y + (size_t)(ck.row + L) * C + ck.h * 64) + sp), "l"(p.nonce) : "memory");
+                }
+            }
         }
         if (CK_TMA && ck_on && lane == 0) bulk_wait<0>();          // this warp's checkpoint copies have reached memory
-        if (CKPT && seg == p.nseg - 1 && !lds32(abort_flag)) store_ckpt(ckpt_slot(ckpt_chunks()));
+        if (CKPT && !PERSIST && seg == p.nseg - 1 && !lds32(abort_flag)) store_ckpt(ckpt_slot(ckpt_chunks()));
         if (SUMMARY && p.ckpt) {
             if (seg == p.nseg - 1 && !lds32(abort_flag))     // the state after the last token
                 store_ckpt(ckpt_slot(ckpt_chunks()));
@@ -1234,25 +1378,60 @@ wkv6_chunked_kernel(const __grid_constant__ CUtensorMap tm_r, const __grid_const
             ++u2_loads;
         };
         if (!PERSIST && has_u2 && nchunks > 0) load_u2((int)row0, col0, nchunks - 1);
-        for (int c = 0; PERSIST || c < (SUMMARY ? 0 : nchunks); ++c) {
+        // Balanced launches keep every SM streaming, so a chunk's time does not hide that load: two slabs per warp (by chunk
+        // parity), second-value rows in and y rows out in their place, the load a chunk ahead and across units.  (5 x 2011
+        // tokens x 32 heads: 69.6 us with one slab, 62.3 with the pair.  With fewer SMs streaming it loses 3-5 %.)
+        constexpr bool PAIR = C2 && BAL;
+        int u2_issued = 0, u2_used = 0;          // one load per chunk: the i-th completes phase i / 2 of the barrier of slab i % 2
+        auto u2_bar = [&](int i) { return bar(BAR_U2 + N_GW * (i & 1) + sp); };
+        auto slab_of = [&](int i) { return (i & 1) ? u2slab : slab; };
+        auto load_pair = [&](int row, int col, int rem) {
+            if (elect_one()) {
+                mbar_expect_tx(u2_bar(u2_issued), 2048);
+                tma_load_2d(slab_of(u2_issued), &tm_u2_16, col, row + 16 * sp, u2_bar(u2_issued));
+                if (rem >= 2) tma_prefetch_2d(&tm_u2_16, col, row + 2 * L + 16 * sp);
+            }
+            __syncwarp();
+            ++u2_issued;
+        };
+        // the first chunk of the next unit of the stream, if there is one.  The producer is a ring ahead, so its descriptor
+        // is there or about to be; it cannot be replaced before this warp has output the chunk.  (Not a wait on the
+        // chunk's "full" barrier: this role lags behind it, and by more than one phase a parity means nothing.)
+        auto load_pair_unit = [&](int c) -> bool {
+            if (!__all_sync(0xffffffffu, desc_wait(sbase + OFF_DESC + 16 * (c & (NSIDE - 1)) + 4, ((c / NSIDE) & 1) * DESC_TAG, abort_flag))) return false;
+            const Chunk nk = chunk_at(c);
+            if (!nk.end) load_pair(nk.row, nk.h * 64, nk.rem);
+            return true;
+        };
+        bool go = true;
+        if (PAIR && has_u2) go = load_pair_unit(0);
+        for (int c = 0; (!PAIR || go) && (PERSIST || c < (SUMMARY ? 0 : nchunks)); ++c) {
             const int tb = c & 1;
             if (!mbar_wait(bar(BAR_B_DONE + tb), (c >> 1) & 1, abort_flag)) break;
             tc_fence_after();
             const Chunk ck = chunk_at(c);
             if (PERSIST && ck.end) break;
             const int ccol = PERSIST ? ck.h * 64 : col0;                  // this chunk's head column
-            if (PERSIST && has_u2 && ck.first) load_u2(ck.row, ccol, ck.rem);   // (a unit's first slab is not fetched ahead)
+            if (PERSIST && !PAIR && has_u2 && ck.first) load_u2(ck.row, ccol, ck.rem);   // (a unit's first slab is not fetched ahead)
             const bool safe = safe_at(c & (NSIDE - 1));
-            if (lane == 0) bulk_wait_read<0>();   // this warp's previous store has finished reading the slab
+            if (lane == 0) bulk_wait_read<0>();   // this warp's previous store has finished reading its slab
             __syncwarp();
+            if (PAIR && has_u2) {                 // ... which (chunk c - 1's) takes the rows of chunk c + 1
+                if (!ck.last) load_pair(ck.row + L, ccol, ck.rem - 1);
+                else if (!load_pair_unit(c + 1)) break;
+            }
+            const uint32_t out = PAIR ? slab_of(c) : slab;
             if (!safe) {
                 // decay too strong for the tensor-core formulation: exact recurrence on the fp32 state copy
                 // the state warps put in shared memory; writes this chunk's y rows itself
                 mbar_arrive_if(bar(BAR_Y_EMPTY + tb), lane == 0);
-                if (has_u2) {                     // keep the slab's phase in step: consume, then request the next
+                if (PAIR && has_u2) {             // keep the slab's phase in step
+                    if (!mbar_wait(u2_bar(c), (c >> 1) & 1, abort_flag)) break;
+                    ++u2_used;
+                } else if (has_u2) {              // ... consume, then request the next
                     if (!mbar_wait(bar(BAR_U2 + sp), u2_parity, abort_flag)) break;
                     u2_pending = false;
-                    if (ck.rem > 0) load_u2(ck.row + L, ccol, ck.rem - 1);
+                    if (!ck.last) load_u2(ck.row + L, ccol, ck.rem - 1);
                 }
                 if (!mbar_wait(bar(BAR_FB_READY), fb_uses & 1, abort_flag)) break;
                 exact_chunk<true>(reinterpret_cast<float*>(smem + OFF_SB), p, ck.h, sp, lane, ck.row, ck.valid, C, ccol);
@@ -1266,22 +1445,28 @@ wkv6_chunked_kernel(const __grid_constant__ CUtensorMap tm_r, const __grid_const
                 const uint32_t ta = tmem + ((uint32_t)(32 * sp) << 16) + TM_Y + 64 * tb;
                 float ya[4][4];
                 tmem_ld_16x32(ta, ya);
-                if (has_u2) {
+                if (PAIR && has_u2) {
+                    if (!mbar_wait(u2_bar(c), (c >> 1) & 1, abort_flag)) break;
+                    ++u2_used;
+                    add_slab_bf16<0>(ya, out, lane);
+                } else if (has_u2) {
                     if (!mbar_wait(bar(BAR_U2 + sp), u2_parity, abort_flag)) break;
                     u2_pending = false;
                     add_slab_bf16<0>(ya, u2slab, lane);
                 }
-                store_half_bf16<0>(slab, 0, ya, lane);
+                store_half_bf16<0>(out, 0, ya, lane);
                 tmem_ld_16x32(ta + 32, ya);
                 tc_fence_before();
                 __syncwarp();
                 mbar_arrive_if(bar(BAR_Y_EMPTY + tb), lane == 0);
                 if (has_u2) {
-                    add_slab_bf16<1>(ya, u2slab, lane);
-                    __syncwarp();
-                    if (ck.rem > 0) load_u2(ck.row + L, ccol, ck.rem - 1);
+                    add_slab_bf16<1>(ya, PAIR ? out : u2slab, lane);
+                    if (!PAIR) {
+                        __syncwarp();
+                        if (!ck.last) load_u2(ck.row + L, ccol, ck.rem - 1);
+                    }
                 }
-                store_half_bf16<1>(slab, 0, ya, lane);
+                store_half_bf16<1>(out, 0, ya, lane);
             }
             fence_proxy_async();
             __syncwarp();
@@ -1289,7 +1474,7 @@ wkv6_chunked_kernel(const __grid_constant__ CUtensorMap tm_r, const __grid_const
             const long long grow = (long long)ck.row + 16 * sp;
             if (rows >= 16) {
                 if (lane == 0) {
-                    tma_store_2d(&tm_y16, ccol, (int)grow, slab);
+                    tma_store_2d(&tm_y16, ccol, (int)grow, out);
                     bulk_commit();
                 }
             } else {
@@ -1298,7 +1483,7 @@ wkv6_chunked_kernel(const __grid_constant__ CUtensorMap tm_r, const __grid_const
                     const int t = i >> 3, ch = i & 7;
                     uint4 val;
                     asm volatile("ld.shared.v4.u32 {%0,%1,%2,%3}, [%4];"
-                                 : "=r"(val.x), "=r"(val.y), "=r"(val.z), "=r"(val.w) : "r"(slab + swz(t, ch << 4)));
+                                 : "=r"(val.x), "=r"(val.y), "=r"(val.z), "=r"(val.w) : "r"(out + swz(t, ch << 4)));
                     *reinterpret_cast<uint4*>(p.y + (size_t)(grow + t) * C + ccol + ch * 8) = val;
                 }
                 __syncwarp();
@@ -1307,6 +1492,7 @@ wkv6_chunked_kernel(const __grid_constant__ CUtensorMap tm_r, const __grid_const
         if (lane == 0) bulk_wait<0>();
         // leaving early (abort) with a slab copy still in flight: wait for it, it targets this CTA's memory
         if (u2_pending) mbar_wait(bar(BAR_U2 + sp), u2_parity, abort_flag, false);
+        for (; PAIR && u2_used < u2_issued; ++u2_used) mbar_wait(u2_bar(u2_used), (u2_used >> 1) & 1, abort_flag, false);
     } else {
         // ============================== elementwise warps ==============================
         const int eset = (warp - WARP_E0) / N_EW;        // this set takes chunks eset, eset + 2, ...
@@ -1572,7 +1758,7 @@ inline int choose_split(long long units, int T, int n_sm, int* seg_chunks, size_
     return 1;
 }
 
-// Opts the eight instantiations of the chunked kernel in to their dynamic shared-memory size, once per device.
+// Opts the instantiations of the chunked kernel in to their dynamic shared-memory size, once per device.
 inline bool chunked_kernel_attributes()
 {
     static PerDeviceFlag attr_set;                   // zero-initialised
@@ -1586,7 +1772,13 @@ inline bool chunked_kernel_attributes()
             cudaFuncSetAttribute(ck::wkv6_chunked_kernel<false, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, ck::SMEM_ALLOC) != cudaSuccess ||
             cudaFuncSetAttribute(ck::wkv6_chunked_kernel<false, true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, ck::SMEM_ALLOC) != cudaSuccess ||
             cudaFuncSetAttribute(ck::wkv6_chunked_kernel<false, false, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, ck::SMEM_ALLOC) != cudaSuccess ||
-            cudaFuncSetAttribute(ck::wkv6_chunked_kernel<false, true, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, ck::SMEM_ALLOC) != cudaSuccess)
+            cudaFuncSetAttribute(ck::wkv6_chunked_kernel<false, true, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, ck::SMEM_ALLOC) != cudaSuccess ||
+            cudaFuncSetAttribute(ck::wkv6_chunked_kernel<false, false, 1, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, ck::SMEM_ALLOC) != cudaSuccess ||
+            cudaFuncSetAttribute(ck::wkv6_chunked_kernel<false, true, 1, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, ck::SMEM_ALLOC) != cudaSuccess ||
+            cudaFuncSetAttribute(ck::wkv6_chunked_kernel<false, false, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, ck::SMEM_ALLOC) != cudaSuccess ||
+            cudaFuncSetAttribute(ck::wkv6_chunked_kernel<false, true, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, ck::SMEM_ALLOC) != cudaSuccess ||
+            cudaFuncSetAttribute(ck::wkv6_chunked_kernel<false, false, 2, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, ck::SMEM_ALLOC) != cudaSuccess ||
+            cudaFuncSetAttribute(ck::wkv6_chunked_kernel<false, true, 2, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, ck::SMEM_ALLOC) != cudaSuccess)
             return false;
         attr_set.set(dev);
     }
@@ -1628,6 +1820,47 @@ inline std::atomic<uint32_t>& wait_limit_us()
 {
     static std::atomic<uint32_t> v{0};
     return v;
+}
+
+// A number no earlier launch of this process has used, and that memory left by anything else holds with probability 2^-64.
+inline unsigned long long launch_nonce()
+{
+    static std::atomic<unsigned long long> next{((unsigned long long)std::random_device{}() << 32) ^ std::random_device{}()};
+    unsigned long long z = next.fetch_add(0x9e3779b97f4a7c15ull, std::memory_order_relaxed);     // (Weyl sequence, then a bijective mix)
+    z = (z ^ (z >> 30)) * 0xbf58476d1ce4e5b9ull;
+    z = (z ^ (z >> 27)) * 0x94d049bb133111ebull;
+    return z ^ (z >> 31);
+}
+
+// Whether cutting units between CTAs (Params::bal_chunks) shortens a dense launch of more units than SMs: whole units end
+// with a round that not every SM has one for.  The cut itself costs about two chunk times (its chunk enters the stream like
+// a unit's first one), and while all SMs stream, a chunk takes a fifth longer than with the SMs of a last round idle; so
+// it is taken where it saves more than four chunk times and more than a fifth of the launch.  Measured (us, whole units ->
+// balanced): 160 units of 128 chunks 258 -> 163, of 20 chunks 53 -> 39; 156 of 39 chunks 93 -> 61; 192 of 63 chunks
+// 135 -> 106; 320 of 47 chunks 159 -> 130; not taken: 256 of 32 chunks 79.7 -> 80.5.
+inline bool balance_pays(long long units, int n_chunks, int n_sm)
+{
+    const long long rounds = (units + n_sm - 1) / n_sm, idle = rounds * n_sm - units;
+    return idle * n_chunks > 4LL * n_sm && idle * 5 > rounds * n_sm && 2LL * n_sm * n_sm * n_chunks < (1LL << 32);   // (32-bit ranges)
+}
+
+// Launches a persistent instantiation with one CTA per SM; cooperative if its CTAs wait for one another.
+template <typename Kernel>
+inline cudaError_t launch_persistent(Kernel kernel, int n_sm, bool cooperative, cudaStream_t st, const CUtensorMap& tr, const CUtensorMap& tk,
+                                     const CUtensorMap& tv, const CUtensorMap& tx, const CUtensorMap& ty, const CUtensorMap& tu2,
+                                     const ck::Params& p, const CUtensorMap& tck)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)n_sm);
+    cfg.blockDim = dim3(ck::THREADS);
+    cfg.dynamicSmemBytes = ck::SMEM_ALLOC;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeCooperative;
+    attr[0].val.cooperative = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = cooperative ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, kernel, tr, tk, tv, tx, ty, tu2, p, tck);
 }
 
 inline gf_status_t chunked_prefill(const __nv_bfloat16* r, const __nv_bfloat16* k, const __nv_bfloat16* v,
@@ -1672,6 +1905,39 @@ inline gf_status_t chunked_prefill(const __nv_bfloat16* r, const __nv_bfloat16* 
             if (cudaGetLastError() != cudaSuccess) return GF_ERR_CUDA;
         }
         p.ckpt = ckpt;
+        const int n_sm_ck = sm_count(), unit_chunks = (T + ck::L - 1) / ck::L;
+        if (!cu && nseg == 1 && state_out && n_sm_ck > 0 && units > n_sm_ck && balance_pays(units, unit_chunks, n_sm_ck)) {
+            p.n_units = (int)units;                  // a balanced stream per SM (see below)
+            p.bal_chunks = unit_chunks;
+            p.nonce = launch_nonce();
+            const cudaError_t e = c2 ? launch_persistent(ck::wkv6_chunked_kernel<false, true, 2, true>, n_sm_ck, true, st, tr, tk, tv, tx, ty, tu2, p, tck)
+                                     : launch_persistent(ck::wkv6_chunked_kernel<false, false, 2, true>, n_sm_ck, true, st, tr, tk, tv, tx, ty, tu2, p, tck);
+            if (e != cudaErrorCooperativeLaunchTooLarge) {
+                launches->fetch_add(1, std::memory_order_relaxed);
+                return e == cudaSuccess ? GF_OK : GF_ERR_CUDA;
+            }
+            cudaGetLastError();                      // (fewer SMs to be had than the device has: whole units below)
+            p.bal_chunks = 0;
+        }
+        if (nseg == 1 && n_sm_ck > 0 && units > n_sm_ck && (units >= 6LL * n_sm_ck || (unit_chunks <= 48 && units >= 3LL * n_sm_ck)) &&
+            (!cu || (scratch && scratch_bytes >= persistent_scratch_bytes(n_seq)))) {
+            // A stream of whole units per SM; packed: the longest sequences first, as in the prefill without checkpoints.
+            // (Packed, 768 units of 2..47 chunks: the training pair 662 -> 650 us.  Dense, 256 units of 32 chunks: 84.0 us
+            // with one CTA per unit, 85.3 with the stream, which therefore wants three units per SM.)
+            p.n_units = (int)units;
+            if (cu) {
+                p.ticket = reinterpret_cast<unsigned int*>(scratch);
+                int32_t* order = n_seq <= ORDER_MAX_SEQ ? reinterpret_cast<int32_t*>(reinterpret_cast<char*>(scratch) + ORDER_OFFSET) : nullptr;
+                p.order = order;
+                wkv6_order_kernel<<<1, 1024, 0, st>>>(cu, n_seq, p.ticket, order);
+                launches->fetch_add(1, std::memory_order_relaxed);
+                if (cudaGetLastError() != cudaSuccess) return GF_ERR_CUDA;
+            }
+            const cudaError_t e = c2 ? launch_persistent(ck::wkv6_chunked_kernel<false, true, 1, true>, n_sm_ck, false, st, tr, tk, tv, tx, ty, tu2, p, tck)
+                                     : launch_persistent(ck::wkv6_chunked_kernel<false, false, 1, true>, n_sm_ck, false, st, tr, tk, tv, tx, ty, tu2, p, tck);
+            launches->fetch_add(1, std::memory_order_relaxed);
+            return e == cudaSuccess ? GF_OK : GF_ERR_CUDA;
+        }
         if (c2) ck::wkv6_chunked_kernel<false, true, false, true><<<(unsigned)(units * nseg), ck::THREADS, ck::SMEM_ALLOC, st>>>(tr, tk, tv, tx, ty, tu2, p, tck);
         else ck::wkv6_chunked_kernel<false, false, false, true><<<(unsigned)(units * nseg), ck::THREADS, ck::SMEM_ALLOC, st>>>(tr, tk, tv, tx, ty, tu2, p, tck);
         launches->fetch_add(1, std::memory_order_relaxed);
@@ -1685,6 +1951,20 @@ inline gf_status_t chunked_prefill(const __nv_bfloat16* r, const __nv_bfloat16* 
     // their units from a counter in the scratch (their lengths differ); dense calls take every gridDim-th unit
     // (drawing them from the counter too was measured 3 % slower).
     const int max_chunks = (T + ck::L - 1) / ck::L;
+    // Where whole units would leave SMs idle in the last round, dense calls cut units between CTAs (balance_pays).
+    if (!cu && state_out && nseg == 1 && n_sm > 0 && units > n_sm && balance_pays(units, max_chunks, n_sm)) {
+        p.n_units = (int)units;
+        p.bal_chunks = max_chunks;
+        p.nonce = launch_nonce();
+        const cudaError_t e = c2 ? launch_persistent(ck::wkv6_chunked_kernel<false, true, 2>, n_sm, true, st, tr, tk, tv, tx, ty, tu2, p, tck)
+                                 : launch_persistent(ck::wkv6_chunked_kernel<false, false, 2>, n_sm, true, st, tr, tk, tv, tx, ty, tu2, p, tck);
+        if (e != cudaErrorCooperativeLaunchTooLarge) {
+            launches->fetch_add(1, std::memory_order_relaxed);
+            return e == cudaSuccess ? GF_OK : GF_ERR_CUDA;
+        }
+        cudaGetLastError();                          // (fewer SMs to be had than the device has: whole units below)
+        p.bal_chunks = 0;
+    }
     if (nseg == 1 && n_sm > 0 && units > n_sm && (units >= 6LL * n_sm || max_chunks <= 48) &&
         (!cu || (scratch && scratch_bytes >= sizeof(unsigned int)))) {
         p.n_units = (int)units;

@@ -1,0 +1,106 @@
+"""Dense calls with more (sequence, head) units than SMs whose units are cut between CTAs (balanced persistent launches).
+
+The state at a cut is handed over in fp32 at a chunk boundary, so every result must equal, bit for bit, that of the same
+sequences run one at a time without a cut (one CTA per unit); the smallest shapes are also compared with the oracle."""
+import pytest
+import torch
+
+import paper_2407_12077_b200 as gf
+from oracle import wkv6_oracle as orc
+from paper_2407_12077_b200 import synth
+
+pytestmark = pytest.mark.gpu
+DEV = "cuda:0"
+
+# (B, T, H), on 148 SMs: 160 units of 5 ragged chunks; 222 of 11; 308 of 6 (one whole round, then the cut ones); 157 of 64
+SHAPES = [(5, 300, 32), (3, 641, 74), (11, 321, 28), (1, 4096, 157)]
+
+
+@pytest.mark.parametrize("B,T,H", SHAPES)
+@pytest.mark.parametrize("c2,in_place,x_hi", [(False, False, -1.0), (False, True, 2.5), (True, False, -1.0), (True, True, 2.5)])
+def test_units_cut_between_ctas(B, T, H, c2, in_place, x_hi):
+    # x_hi = 2.5: some chunks decay by more than 2^-96 and take the token-by-token path
+    i = synth.make_dense(B, T, H, 64, "bf16", seed=B * T + H, device=DEV, state_std=0.1, x_hi=x_hi)
+    u2 = torch.randn(i.r.shape, device=DEV, generator=torch.Generator(device=DEV).manual_seed(3)).bfloat16()
+
+    def run(sl, state, out=None, **kw):
+        t = [x[sl].contiguous() for x in (i.r, i.k, i.v, i.x, u2)]
+        if c2:
+            return gf.prefill_c2(*t, state, state_out=out, **kw)
+        return gf.prefill(*t[:4], i.u, state, state_out=out, **kw)
+
+    s0 = i.state_in.clone()
+    y, s = run(slice(None), s0, s0 if in_place else None)
+    gf.last_device_status()
+    if B > 1:
+        for b in range(B):                       # few units each, never split: one CTA per unit
+            yb, sb = run(slice(b, b + 1), i.state_in[b:b + 1].contiguous(), split=False)
+            assert torch.equal(yb[0], y[b]) and torch.equal(sb[0], s[b])
+        gf.last_device_status()
+    if T <= 321 and not c2:
+        y_ref, s_ref = orc.prefill(*(t.cpu() for t in (i.r, i.k, i.v, i.x, i.u, i.state_in)))
+        assert orc.rel_l2(y.float().cpu().numpy(), y_ref) <= 5e-3      # the contract's tolerance
+        assert orc.rel_l2(s.cpu().numpy(), s_ref) <= 5e-3
+
+
+@pytest.mark.parametrize("c2", [False, True])
+def test_cut_call_repeats_and_replays(c2):
+    # the announcement words lie in y: neither a reused y nor a replayed graph may see an old one
+    i = synth.make_dense(5, 700, 32, 64, "bf16", seed=8, device=DEV, state_std=0.1)
+    y, s = torch.empty_like(i.r), torch.empty_like(i.state_in)
+    fn = (lambda st=None: gf.prefill_c2(i.r, i.k, i.v, i.x, i.r, i.state_in, state_out=s, y=y, stream=st)) if c2 else \
+         (lambda st=None: gf.prefill(i.r, i.k, i.v, i.x, i.u, i.state_in, state_out=s, y=y, stream=st))
+    fn()
+    y0, s0 = y.clone(), s.clone()
+    for _ in range(20):
+        fn()
+        assert torch.equal(y, y0) and torch.equal(s, s0)
+    st, g = torch.cuda.Stream(), torch.cuda.CUDAGraph()
+    with torch.cuda.stream(st):
+        torch.cuda.synchronize()
+        with torch.cuda.graph(g, stream=st):
+            fn(st)
+    for _ in range(5):
+        g.replay()
+        torch.cuda.synchronize()
+        assert torch.equal(y, y0) and torch.equal(s, s0)
+    gf.last_device_status()
+
+
+@pytest.mark.parametrize("c2", [False, True])
+@pytest.mark.parametrize("B,T,H", SHAPES[:3] + [(40, 90, 32)])
+def test_training_forward_of_many_units(B, T, H, c2):
+    # the checkpoints of cut (and, in the last shape, of streamed whole) units: the gradient from them equals the gradient
+    # that makes its own
+    i = synth.make_dense(B, T, H, 64, "bf16", seed=B + T + H, device=DEV, state_std=0.1)
+    dy = torch.randn(i.r.shape, device=DEV, generator=torch.Generator(device=DEV).manual_seed(4)).bfloat16()
+    ws = torch.empty(gf.backward_workspace_bytes(B, T, H, 64), dtype=torch.uint8, device=DEV)
+    y, s = gf.prefill_train(i.r, i.k, i.v, i.x, i.u, ws, i.state_in, c2=c2)
+    y1, s1 = (gf.prefill_c2(i.r, i.k, i.v, i.x, None, i.state_in) if c2 else gf.prefill(i.r, i.k, i.v, i.x, i.u, i.state_in))
+    assert torch.equal(y, y1) and torch.equal(s, s1)
+    back = (lambda **kw: gf.backward_c2(i.r, i.k, i.v, i.x, dy, i.state_in, **kw)) if c2 else \
+           (lambda **kw: gf.backward(i.r, i.k, i.v, i.x, i.u, dy, i.state_in, **kw))
+    for a, b in zip(back(workspace=ws, saved=True), back()):
+        assert torch.equal(a, b)
+    gf.last_device_status()
+
+
+@pytest.mark.parametrize("c2", [False, True])
+def test_packed_training_forward_as_a_stream(c2):
+    # more units than SMs: the packed training forward walks units from a counter, empty sequences included
+    lens = [0, 130, 64, 1, 700, 63, 0, 65, 200, 128]
+    cu = torch.tensor([0] + torch.tensor(lens).cumsum(0).tolist(), dtype=torch.int32)
+    i = synth.make_varlen(cu, 20, 64, "bf16", seed=11, device=DEV, state_std=0.1)
+    total, S = int(cu[-1]), len(lens)
+    u2 = i.v if c2 else None
+    dy = torch.randn(i.r.shape, device=DEV, generator=torch.Generator(device=DEV).manual_seed(5)).bfloat16()
+    ws = torch.empty(gf.backward_varlen_workspace_bytes(S, total, 20, 64), dtype=torch.uint8, device=DEV)
+    y, s = gf.prefill_varlen_train(i.r, i.k, i.v, i.x, i.u, i.cu_seqlens, 700, ws, i.state_in, c2=c2, u2=u2)
+    y1, s1 = (gf.prefill_varlen_c2(i.r, i.k, i.v, i.x, u2, i.cu_seqlens, 700, i.state_in) if c2 else
+              gf.prefill_varlen(i.r, i.k, i.v, i.x, i.u, i.cu_seqlens, 700, i.state_in))
+    assert torch.equal(y, y1) and torch.equal(s, s1)
+    kw = dict(c2=c2)
+    for a, b in zip(gf.backward_varlen(i.r, i.k, i.v, i.x, i.u, dy, i.cu_seqlens, 700, i.state_in, workspace=ws, saved=True, **kw),
+                    gf.backward_varlen(i.r, i.k, i.v, i.x, i.u, dy, i.cu_seqlens, 700, i.state_in, **kw)):
+        assert a is None and b is None or torch.equal(a, b)
+    gf.last_device_status()
