@@ -136,7 +136,8 @@ constexpr int OFF_DESC = (OFF_BAR + BAR_COUNT * 8 + 15) & ~15;   // [NSIDE] int4
 // a unit another CTA began, last chunk of a piece
 constexpr int DESC_FIRST = 0x100, DESC_END = 0x200, DESC_CONT = 0x400, DESC_LAST = 0x800;
 constexpr int DESC_TAG = 0x1000;                                 // (balanced launches) parity of the ring's turn: (chunk / NSIDE) & 1
-constexpr int SMEM_BYTES = OFF_DESC + NSIDE * 16;
+constexpr int OFF_MARK = OFF_DESC + NSIDE * 16;                  // int: the segment's state became non-finite (Params::trail)
+constexpr int SMEM_BYTES = OFF_MARK + 16;
 constexpr int SMEM_ALLOC = SMEM_BYTES + 1024;              // slack for manual 1024-byte alignment
 static_assert(SMEM_ALLOC <= 232448, "shared memory budget of one sm_100 CTA");
 
@@ -540,8 +541,17 @@ struct Params {
     // output overwrites.  The launch is cooperative: every CTA a cut waits for is resident.
     int bal_chunks;
     unsigned long long nonce;
+    // Summary launch of a split call: nonzero lets a CTA start late in its segment.  dS forgets what lies before a run of
+    // tokens over which every channel decays by more than 2^-TRAIL_LOG2, far below fp32's rounding of what comes after,
+    // and D is then zero to the same degree: so the CTA first sums the decays of its segment's last TRAIL_CHUNKS chunks
+    // and runs from the last chunk boundary after which every channel has decayed that far, if there is one.  (Segments of
+    // 512 chunks with w in [0.69, 0.998]: 16 chunks run, the launch takes 25 us instead of 292.)  What rounding forgets, a
+    // NaN or infinity before that boundary does not: see poison_later_segments.
+    int trail;
 };
 constexpr int SUMMARY_FLOATS = 64 + 64 * 64;
+constexpr float TRAIL_LOG2 = 96.f;
+constexpr int TRAIL_CHUNKS = 30;       // (one per warp)
 
 // Writes a warp's 16 x 64 fp32 accumulator block (acc[n][0..1] = row g, cols 8n+2q,+1;
 // acc[n][2..3] = row g+8) as bf16 into rows row0 .. row0+15 of a 128B-swizzled [rows][64] tile.
@@ -687,6 +697,59 @@ __device__ __forceinline__ void exact_chunk(float* scr, const Params& p, int h, 
     }
 }
 
+// Main launch of a split call whose summary launch may have started late in its segments (Params::trail): a segment's state
+// that has become non-finite goes on being so, although the summary did not see it.  A CTA whose segment ends like that
+// writes NaN over those elements of its summary's dS (from_marks) and says so in the sign of D[1]; every CTA says in the
+// sign of D[0] of the summary before its segment that its outputs are written (D is a decay, readers drop the signs).
+// Whichever of two CTAs of a unit comes second sees the other's word (both sequentially consistent) and makes the marked
+// columns of the later segment's outputs NaN, and the marked elements of the final state.  Runs after the CTA's last
+// barrier; without a mark it costs a few words of memory traffic per CTA.
+__device__ __forceinline__ void poison_later_segments(const Params& p, int unit, int seg, bool marked, int* mark, int* todo)
+{
+    const int tid = threadIdx.x, nseg = p.nseg;
+    unsigned* base = reinterpret_cast<unsigned*>(p.summaries) + (size_t)unit * (nseg - 1) * SUMMARY_FLOATS;
+    if (tid == 0) {
+        // todo: bit g (g < seg): this segment takes the marks of segment g; bit g > seg: segment g takes this one's
+        int t = 0;
+        asm volatile("fence.sc.gpu;" ::: "memory");
+        if (marked && seg < nseg - 1) atomicOr(base + (size_t)seg * SUMMARY_FLOATS + 1, 0x80000000u);
+        if (seg > 0) atomicOr(base + (size_t)(seg - 1) * SUMMARY_FLOATS, 0x80000000u);
+        asm volatile("fence.sc.gpu;" ::: "memory");
+        for (int g = 0; g < nseg; ++g) {
+            if (g < seg && (atomicOr(base + (size_t)g * SUMMARY_FLOATS + 1, 0u) >> 31)) t |= 1 << g;
+            if (marked && g > seg && (atomicOr(base + (size_t)(g - 1) * SUMMARY_FLOATS, 0u) >> 31)) t |= 1 << g;
+        }
+        asm volatile("fence.sc.gpu;" ::: "memory");
+        *todo = t;
+    }
+    __syncthreads();
+    const int t = *todo;
+    if (t == 0) return;
+    const int seq = unit / p.H, h = unit % p.H;
+    const long long row0 = p.cu_seqlens ? p.cu_seqlens[seq] : (long long)seq * p.T;
+    const int len = p.cu_seqlens ? p.cu_seqlens[seq + 1] - p.cu_seqlens[seq] : p.T;
+    const float nan = __int_as_float(0x7fc00000);
+    for (int g = 0; g < nseg; ++g) {
+        if (!(t >> g & 1)) continue;
+        const int from = g < seg ? g : seg, to = g < seg ? seg : g;
+        const float* ds = reinterpret_cast<const float*>(base + (size_t)from * SUMMARY_FLOATS + 64);
+        __syncthreads();
+        if (tid < 64) mark[tid] = 0;
+        __syncthreads();
+        for (int i = tid; i < 4096; i += blockDim.x) {
+            const float v = __ldcg(ds + i);
+            if (v != v) {
+                mark[i & 63] = 1;
+                if (to == nseg - 1 && p.state_out) p.state_out[(size_t)unit * 4096 + i] = nan;
+            }
+        }
+        __syncthreads();
+        const int first = min(len, to * p.seg_chunks * L), end = to == nseg - 1 ? len : min(len, first + p.seg_chunks * L);
+        for (long long i = (long long)first * 64 + tid; i < (long long)end * 64; i += blockDim.x)
+            if (mark[i & 63]) p.y[(size_t)(row0 + (i >> 6)) * p.H * 64 + h * 64 + (i & 63)] = __float2bfloat16_rn(nan);
+    }
+}
+
 // ---------------------------------------------------------------- the kernel
 // SUMMARY = false: the prefill proper.  SUMMARY = true: the first pass of a split call, which only
 // carries the state over a segment from a zero start (no r, no scores, no outputs: the score warps and
@@ -698,7 +761,8 @@ __device__ __forceinline__ void exact_chunk(float* scr, const Params& p, int h, 
 // stream may begin and end inside a unit (see Params::bal_chunks).
 // CKPT = true (launches of the prefill proper): the state before every chunk and after the last one is also left in
 // Params::ckpt, for the gradient call that follows a training step's forward pass.
-template <bool SUMMARY, bool C2, int PERSIST = 0, bool CKPT = false>
+// TRAIL = true (main launches of split calls): the summary launch may have started late in its segments (see Params::trail).
+template <bool SUMMARY, bool C2, int PERSIST = 0, bool CKPT = false, bool TRAIL = false>
 __global__ void __launch_bounds__(THREADS, 1)
 wkv6_chunked_kernel(const __grid_constant__ CUtensorMap tm_r, const __grid_constant__ CUtensorMap tm_k,
                     const __grid_constant__ CUtensorMap tm_v, const __grid_constant__ CUtensorMap tm_x,
@@ -733,6 +797,39 @@ wkv6_chunked_kernel(const __grid_constant__ CUtensorMap tm_r, const __grid_const
         row0 += first;
         len = (seg == p.nseg - 1) ? len - first : min(len - first, p.seg_chunks * L);
     }
+    int trail_cut = 0;                     // (see Params::trail) chunks of the segment that need not be run
+    if constexpr (SUMMARY) {
+        // only whole, full segments (of which all but the last chunks may go); one warp per chunk sums it: lane = 4 channels
+        // (lane % 16) of every other row
+        const int n_full = len / L, look = min(TRAIL_CHUNKS, n_full - 1);
+        if (p.trail && len % L == 0 && look > 0) {
+            float* tot = reinterpret_cast<float*>(smem);           // [TRAIL_CHUNKS][64] (the ring: nothing has been loaded yet)
+            if (warp < look) {                                     // chunk n_full - 1 - warp
+                const __nv_bfloat16* xp = p.x + (size_t)(row0 + (long long)(n_full - 1 - warp) * L + (lane >> 4)) * ((size_t)p.H * 64) + h * 64 + 4 * (lane & 15);
+                float e[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll 16
+                for (int t = 0; t < L / 2; ++t) {
+                    const uint2 w = *reinterpret_cast<const uint2*>(xp + (size_t)(2 * t) * ((size_t)p.H * 64));
+                    e[0] += ex2(fmaf(bf_lo(w.x), LOG2E, LOG2_LOG2E)); e[1] += ex2(fmaf(bf_hi(w.x), LOG2E, LOG2_LOG2E));
+                    e[2] += ex2(fmaf(bf_lo(w.y), LOG2E, LOG2_LOG2E)); e[3] += ex2(fmaf(bf_hi(w.y), LOG2E, LOG2_LOG2E));
+                }
+#pragma unroll
+                for (int i = 0; i < 4; ++i) e[i] += __shfl_xor_sync(0xffffffffu, e[i], 16);
+                if (lane < 16) *reinterpret_cast<float4*>(tot + warp * 64 + 4 * lane) = make_float4(e[0], e[1], e[2], e[3]);
+            }
+            __syncthreads();
+            // every warp finds the same answer: two channels per lane, chunks from the last one back
+            float a0 = 0.f, a1 = 0.f;
+            for (int k = 0; k < look; ++k) {
+                a0 += tot[k * 64 + 2 * lane]; a1 += tot[k * 64 + 2 * lane + 1];
+                if (__all_sync(0xffffffffu, a0 > TRAIL_LOG2 && a1 > TRAIL_LOG2)) { trail_cut = n_full - 1 - k; break; }     // (false for NaN)
+            }
+            row0 += (long long)trail_cut * L;
+            len -= trail_cut * L;
+            __syncthreads();                                       // (the sums are read before the ring is loaded)
+            fence_proxy_async();
+        }
+    }
     const int nchunks = PERSIST ? 0 : (len + L - 1) / L;
     // checkpoint slots of this unit: the first one, and how many chunks the whole sequence has
     auto ckpt_slot = [&](int c_abs) -> size_t {       // (the packed form recomputes what it needs: nothing stays live for it)
@@ -753,6 +850,7 @@ wkv6_chunked_kernel(const __grid_constant__ CUtensorMap tm_r, const __grid_const
     const size_t C = (size_t)p.H * 64;
     static_assert(!(PERSIST && SUMMARY), "the summary pass is a single-unit launch");
     static_assert(!(CKPT && SUMMARY), "the summary pass keeps its checkpoints by Params::ckpt");
+    static_assert(!(TRAIL && (PERSIST || SUMMARY)), "the main launch of a split call");
     constexpr bool BAL = PERSIST == 2;
 
     // One chunk of this CTA's work.  Single-unit launches derive it from the chunk index; persistent launches
@@ -805,6 +903,7 @@ wkv6_chunked_kernel(const __grid_constant__ CUtensorMap tm_r, const __grid_const
             for (int i = 0; i < NSIDE; ++i) sts32(sbase + OFF_DESC + 16 * i + 4, DESC_TAG);        // (of the turn before the first)
         sts32(abort_flag, 0u);
         sts32(abort_flag + 4, p.wait_limit_us ? p.wait_limit_us : WAIT_LIMIT_US);
+        if (TRAIL) sts32(sbase + OFF_MARK, 0u);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         fence_proxy_async();
     }
@@ -1092,7 +1191,8 @@ wkv6_chunked_kernel(const __grid_constant__ CUtensorMap tm_r, const __grid_const
             // start state of a later segment: fold the summaries of the segments before it, in order
             for (int gg = 0; gg < seg; ++gg) {
                 const float* sm = p.summaries + ((size_t)unit * (p.nseg - 1) + gg) * SUMMARY_FLOATS;
-                const float d_lo = sm[c_lo], d_hi = sm[c_lo + 8];
+                float d_lo = sm[c_lo], d_hi = sm[c_lo + 8];
+                if (TRAIL) { d_lo = fabsf(d_lo); d_hi = fabsf(d_hi); }               // (signs: see poison_later_segments)
 #pragma unroll
                 for (int n = 0; n < 8; ++n) {
                     const float2 lo = *reinterpret_cast<const float2*>(sm + 64 + c_lo * 64 + 8 * n + 2 * q);
@@ -1282,6 +1382,7 @@ wkv6_chunked_kernel(const __grid_constant__ CUtensorMap tm_r, const __grid_const
         } else if (SUMMARY) {
             if (!lds32(abort_flag)) {
                 float* sm = p.summaries + ((size_t)unit * (p.nseg - 1) + seg) * SUMMARY_FLOATS;
+                if (trail_cut) dprod_lo = dprod_hi = 0.f;
                 if (q == 0) { sm[c_lo] = dprod_lo; sm[c_lo + 8] = dprod_hi; }
 #pragma unroll
                 for (int n = 0; n < 8; ++n) {
@@ -1291,6 +1392,23 @@ wkv6_chunked_kernel(const __grid_constant__ CUtensorMap tm_r, const __grid_const
             }
         } else if (!PERSIST && p.state_out && seg == p.nseg - 1 && !lds32(abort_flag)) {
             store_state(sb);
+        } else if (TRAIL && seg < p.nseg - 1) {
+            // a state that is no longer finite: marked in the segment's summary (see poison_later_segments)
+            float z = 0.f;
+#pragma unroll
+            for (int n = 0; n < 8; ++n)
+#pragma unroll
+                for (int e = 0; e < 4; ++e) z = fmaf(st[n][e], 0.f, z);
+            if (z != 0.f) {
+                float* sm = p.summaries + ((size_t)unit * (p.nseg - 1) + seg) * SUMMARY_FLOATS + 64;
+#pragma unroll
+                for (int n = 0; n < 8; ++n)
+#pragma unroll
+                    for (int e = 0; e < 4; ++e)
+                        if (st[n][e] * 0.f != 0.f) sm[(size_t)(e < 2 ? c_lo : c_lo + 8) * 64 + 8 * n + 2 * q + (e & 1)] = __int_as_float(0x7fc00000);
+                __threadfence();
+                sts32(sbase + OFF_MARK, 1u);
+            }
         }
     } else if (warp < WARP_Y0) {
         // ============================== score warps ==============================
@@ -1671,6 +1789,8 @@ wkv6_chunked_kernel(const __grid_constant__ CUtensorMap tm_r, const __grid_const
         tc_fence_after();
         tmem_dealloc(tmem, TM_COLS);
     }
+    if (TRAIL)
+        poison_later_segments(p, unit, seg, lds32(sbase + OFF_MARK) != 0, reinterpret_cast<int*>(smem + OFF_TOT), reinterpret_cast<int*>(smem + OFF_TOT) + 64);
 }
 
 // One warp that waits, with the kernel's own bounded wait, on a barrier nobody arrives on: the wait runs out after
@@ -1775,6 +1895,10 @@ inline bool chunked_kernel_attributes()
             cudaFuncSetAttribute(ck::wkv6_chunked_kernel<false, true, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, ck::SMEM_ALLOC) != cudaSuccess ||
             cudaFuncSetAttribute(ck::wkv6_chunked_kernel<false, false, 1, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, ck::SMEM_ALLOC) != cudaSuccess ||
             cudaFuncSetAttribute(ck::wkv6_chunked_kernel<false, true, 1, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, ck::SMEM_ALLOC) != cudaSuccess ||
+            cudaFuncSetAttribute(ck::wkv6_chunked_kernel<false, false, 0, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, ck::SMEM_ALLOC) != cudaSuccess ||
+            cudaFuncSetAttribute(ck::wkv6_chunked_kernel<false, true, 0, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, ck::SMEM_ALLOC) != cudaSuccess ||
+            cudaFuncSetAttribute(ck::wkv6_chunked_kernel<false, false, 0, true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, ck::SMEM_ALLOC) != cudaSuccess ||
+            cudaFuncSetAttribute(ck::wkv6_chunked_kernel<false, true, 0, true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, ck::SMEM_ALLOC) != cudaSuccess ||
             cudaFuncSetAttribute(ck::wkv6_chunked_kernel<false, false, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, ck::SMEM_ALLOC) != cudaSuccess ||
             cudaFuncSetAttribute(ck::wkv6_chunked_kernel<false, true, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, ck::SMEM_ALLOC) != cudaSuccess ||
             cudaFuncSetAttribute(ck::wkv6_chunked_kernel<false, false, 2, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, ck::SMEM_ALLOC) != cudaSuccess ||
@@ -1891,6 +2015,10 @@ inline gf_status_t chunked_prefill(const __nv_bfloat16* r, const __nv_bfloat16* 
     ck::Params p{r, k, v, x, y, u, state_in, state_out, cu, T, H, scratch, seg_chunks, nseg, u2, c2};
     CUtensorMap tck = ty;                            // (read only by the launches that keep checkpoints)
     if (nseg > 1 && state_in) p.state_copy = scratch + (size_t)units * (nseg - 1) * ck::SUMMARY_FLOATS;
+    // A late start (Params::trail) costs the summary launch 5 us of looking and the main launch's CTAs 2 us at their end: it
+    // is allowed where segments are long enough to gain (us, without -> with: segments of 512 chunks 776 -> 537, of 64
+    // 113 -> 101, of 48 89 -> 85, of 15 39 -> 46).
+    p.trail = nseg > 1 && seg_chunks >= 48;
     p.wait_limit_us = wait_limit_us().load(std::memory_order_relaxed);
     if (ckpt) {
         // a training step's forward pass: one CTA per unit and segment, the chunk-start states kept for the gradient
@@ -1938,8 +2066,9 @@ inline gf_status_t chunked_prefill(const __nv_bfloat16* r, const __nv_bfloat16* 
             launches->fetch_add(1, std::memory_order_relaxed);
             return e == cudaSuccess ? GF_OK : GF_ERR_CUDA;
         }
-        if (c2) ck::wkv6_chunked_kernel<false, true, false, true><<<(unsigned)(units * nseg), ck::THREADS, ck::SMEM_ALLOC, st>>>(tr, tk, tv, tx, ty, tu2, p, tck);
-        else ck::wkv6_chunked_kernel<false, false, false, true><<<(unsigned)(units * nseg), ck::THREADS, ck::SMEM_ALLOC, st>>>(tr, tk, tv, tx, ty, tu2, p, tck);
+        const auto kernel = p.trail ? (c2 ? ck::wkv6_chunked_kernel<false, true, 0, true, true> : ck::wkv6_chunked_kernel<false, false, 0, true, true>)
+                                    : (c2 ? ck::wkv6_chunked_kernel<false, true, 0, true> : ck::wkv6_chunked_kernel<false, false, 0, true>);
+        kernel<<<(unsigned)(units * nseg), ck::THREADS, ck::SMEM_ALLOC, st>>>(tr, tk, tv, tx, ty, tu2, p, tck);
         launches->fetch_add(1, std::memory_order_relaxed);
         return cudaGetLastError() == cudaSuccess ? GF_OK : GF_ERR_CUDA;
     }
@@ -2001,8 +2130,9 @@ inline gf_status_t chunked_prefill(const __nv_bfloat16* r, const __nv_bfloat16* 
         attr[0].val.programmaticStreamSerializationAllowed = 1;
         cfg.attrs = attr;
         cfg.numAttrs = 1;
-        const cudaError_t e = c2 ? cudaLaunchKernelEx(&cfg, ck::wkv6_chunked_kernel<false, true, false>, tr, tk, tv, tx, ty, tu2, p, tck)
-                                 : cudaLaunchKernelEx(&cfg, ck::wkv6_chunked_kernel<false, false, false>, tr, tk, tv, tx, ty, tu2, p, tck);
+        const auto kernel = p.trail ? (c2 ? ck::wkv6_chunked_kernel<false, true, 0, false, true> : ck::wkv6_chunked_kernel<false, false, 0, false, true>)
+                                    : (c2 ? ck::wkv6_chunked_kernel<false, true> : ck::wkv6_chunked_kernel<false, false>);
+        const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, tr, tk, tv, tx, ty, tu2, p, tck);
         launches->fetch_add(1, std::memory_order_relaxed);
         return e == cudaSuccess ? GF_OK : GF_ERR_CUDA;
     }

@@ -1,0 +1,62 @@
+"""Split calls (few (sequence, head) units) whose summary launch may start late in its segments: decays on both sides of
+the threshold, and non-finite inputs before the point where it starts."""
+import pytest
+import torch
+
+import paper_2407_12077_b200 as gf
+from oracle import wkv6_oracle as orc
+from paper_2407_12077_b200 import synth
+
+pytestmark = pytest.mark.gpu
+DEV = "cuda:0"
+NAN, INF = float("nan"), float("inf")
+
+
+@pytest.mark.parametrize("T", [24576, 25000])
+@pytest.mark.parametrize("x_lo,x_hi", [(-6.0, -1.0), (-4.5, -4.0), (-5.4, -5.1), (-7.0, -6.5), (-1.0, -0.5)])
+def test_late_start_against_oracle(T, x_lo, x_hi):
+    # about 16 / 95 / 280 / 1200 / 2 chunks until every channel has decayed by 2^-96: within a few chunks, around the 30 that
+    # are looked at and beyond.  One slow channel in head 1.  Tolerance: the contract's.
+    inp = synth.make_dense(1, T, 3, 64, "bf16", seed=T, state_std=1.0, x_lo=x_lo, x_hi=x_hi)
+    inp.x[:, :, 1, 17] = -11.0
+    d = inp.to(DEV)
+    assert gf.workspace_bytes(1, T, 3, 64) > 0
+    y, s = gf.prefill(d.r, d.k, d.v, d.x, d.u, d.state_in)
+    gf.last_device_status()
+    y_ref, s_ref = orc.prefill(inp.r, inp.k, inp.v, inp.x, inp.u, inp.state_in)
+    for h in range(3):
+        assert orc.rel_l2(y[:, :, h].float().cpu().numpy(), y_ref[:, :, h]) <= 5e-3
+        assert orc.rel_l2(s[:, h].cpu().numpy(), s_ref[:, h]) <= 5e-3
+
+
+@pytest.mark.parametrize("c2", [False, True])
+@pytest.mark.parametrize("train", [False, True])
+def test_non_finite_values_are_not_forgotten(c2, train):
+    # one call per place: the tokens after it and the final state are non-finite where the unsplit call's are, the other
+    # head is untouched
+    T, H = 24576, 2
+    clean = synth.make_dense(1, T, H, 64, "bf16", seed=5, device=DEV, state_std=0.1)
+    ws = torch.empty(gf.backward_workspace_bytes(1, T, H, 64), dtype=torch.uint8, device=DEV)
+
+    def run(i, split):
+        if train and split:
+            return gf.prefill_train(i.r, i.k, i.v, i.x, i.u, ws, i.state_in, c2=c2)
+        if c2:
+            return gf.prefill_c2(i.r, i.k, i.v, i.x, None, i.state_in, split=split)
+        return gf.prefill(i.r, i.k, i.v, i.x, i.u, i.state_in, split=split)
+
+    y0, s0 = run(clean, True)
+    for name, t, value in [("k", 70, NAN), ("v", 4500, NAN), ("x", 9000, NAN), ("v", 10, INF), ("k", 6300, INF), ("v", T - 700, NAN)]:
+        i = synth.make_dense(1, T, H, 64, "bf16", seed=5, device=DEV, state_std=0.1)
+        getattr(i, name)[0, t, 1, 9] = value
+        y, s = run(i, True)
+        y1, s1 = run(i, False)
+        gf.last_device_status()
+        assert torch.equal(y[:, :, 0], y0[:, :, 0]) and torch.equal(s[:, 0], s0[:, 0]), name
+        bad, bad1 = ~torch.isfinite(y[0, :, 1]), ~torch.isfinite(y1[0, :, 1])
+        assert torch.equal(bad.any(1), bad1.any(1)), (name, t)               # the same tokens
+        assert bool((bad | ~bad1).all()), (name, t)                          # and at least the same elements
+        sb, sb1 = ~torch.isfinite(s[0, 1]), ~torch.isfinite(s1[0, 1])
+        assert bool((sb | ~sb1).all()), (name, t)
+    y, s = run(clean, True)                                                  # nothing stays behind
+    assert torch.equal(y, y0) and torch.equal(s, s0)
