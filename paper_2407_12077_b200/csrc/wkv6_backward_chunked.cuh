@@ -30,15 +30,19 @@
 // Layout inside a group: warp (sp = warp % 4, cx = warp / 4 % 2) owns rows 16 sp .. +15 and columns 32 cx .. +31 of
 // every 64x64 tile; lane (g = lane / 4, q = lane % 4) rows 16 sp + g and + 8, columns 32 cx + 8 n + 2 q + e (n < 4,
 // e < 2): 16 cells, the accumulator layout of the 64-row products, in which bf16 tiles move through ldmatrix /
-// stmatrix, so nothing is transposed and a lane's cells are the same in every phase.  (G_NB = 2 gives groups of 16
-// warps with 8 cells per lane at 64 registers instead: measured slower, the spills cost more than the warps bring.)
+// stmatrix.  For everything per token and channel (decays, operands, epilogue, dx) the rows are channels and the columns
+// tokens: the [token][channel] tiles pass through the transposing forms of those instructions, and dR^ and dK^ are formed
+// transposed (dR^^T = S_0 dY^T + K^^T dP'^T, dK^^T = G^ V^T + R^^T dP'; the transposition costs nothing, it is a bit of the
+// descriptor).  The sums along the tokens then run over a lane's own eight tokens and three neighbouring lanes, 24
+// shuffles per lane and scan where tokens along the lanes took 104, and per-channel values (bonus, E, du) are two
+// registers.  The adjoint G and the scores keep [channel][value] and [token][token].  Measured with the gradient of
+// 8 x 2048 tokens x 32 heads in the training pair: 330 -> 310 us, packed 650 -> 616.
 // Each group has its own input stage (x, v, dy and r, k by TMA, each part re-filled as soon as its tiles fall free),
 // operand tiles, tensor-memory columns (three accumulators that the second group of products reuses once the first
 // group's have been read) and barriers; the four staging tiles of the gradients lie over operand tiles that are dead
 // by the time they are written.  One lane of a group issues its copies, two others (in other warps) its two groups of
 // products, so that no warp carries all the issuing.  Sums along the tokens (the
-// cumulative decay; the suffix sums of the decay gradient) run over lanes by shuffles and across the four row groups
-// through shared memory.  Waits are per thread and bounded; their outcome is made uniform over the group at its next
+// cumulative decay; the suffix sums of the decay gradient) cross the two column slabs through shared memory.  Waits are per thread and bounded; their outcome is made uniform over the group at its next
 // barrier, and the hand-over waits watch the CTA's abort word, so after a wait that ran out both groups leave.
 // A chunk in which a channel decays by more than 2^-96 runs token by token in fp32 on its group's warps (its 64
 // states recomputed into a scratch slot of the workspace), so any decay logit gives the gradient of the exact
@@ -52,6 +56,7 @@ namespace bc {
 using namespace ck;          // PTX wrappers, descriptors, layout helpers of the forward kernel
 
 constexpr float LN2 = 0.6931471805599453f;
+constexpr uint32_t IDESC_MN_K = IDESC | (1u << 15);
 constexpr size_t FB_SLOT_FLOATS = (size_t)64 * 4096;      // scratch of the token-by-token path per SM and group: 64 states
 
 struct BParams {
@@ -111,11 +116,15 @@ __device__ __forceinline__ unsigned smid()
 }
 
 // 1 - 2^l for l <= 0 without the cancellation of the direct form near l = 0 (slow decays): the series of -expm1 there.
-__device__ __forceinline__ float one_minus_ex2(float l)
+__device__ __forceinline__ float2 one_minus_ex2_2(float2 l)
 {
-    const float t = l * LN2;
-    const float series = -t * (1.f + t * (0.5f + t * (0.16666667f + t * 0.041666668f)));
-    return l > -0.125f ? series : 1.f - ex2(l);
+    const float2 t = mul2(l, make_float2(LN2, LN2)), one = make_float2(1.f, 1.f);
+    float2 s = fma2(t, make_float2(0.041666668f, 0.041666668f), make_float2(0.16666667f, 0.16666667f));
+    s = fma2(t, s, make_float2(0.5f, 0.5f));
+    s = fma2(t, s, one);
+    s = mul2(make_float2(-t.x, -t.y), s);
+    const float2 d = sub2(one, ex2_2(l));
+    return make_float2(l.x > -0.125f ? s.x : d.x, l.y > -0.125f ? s.y : d.y);
 }
 
 __device__ __forceinline__ void tmem_ld_done() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
@@ -199,6 +208,31 @@ __device__ __forceinline__ void st_half(uint32_t addr, const float (&v)[2][4])
 {
     stsm_x4(addr, pack_bf16(v[0][0], v[0][1]), pack_bf16(v[0][2], v[0][3]), pack_bf16(v[1][0], v[1][1]), pack_bf16(v[1][2], v[1][3]));
 }
+// The same blocks transposed on the way: the tile is [token][channel], the lane's cells are [channel][token]
+__device__ __forceinline__ void ld_half_t(uint32_t addr, float (&v)[2][4])
+{
+    uint32_t w0, w1, w2, w3;
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(w0), "=r"(w1), "=r"(w2), "=r"(w3) : "r"(addr) : "memory");
+    v[0][0] = bf_lo(w0); v[0][1] = bf_hi(w0); v[0][2] = bf_lo(w1); v[0][3] = bf_hi(w1);
+    v[1][0] = bf_lo(w2); v[1][1] = bf_hi(w2); v[1][2] = bf_lo(w3); v[1][3] = bf_hi(w3);
+}
+__device__ __forceinline__ void st_half_t(uint32_t addr, const float (&v)[2][4])
+{
+    asm volatile("stmatrix.sync.aligned.m8n8.x4.trans.shared.b16 [%0], {%1,%2,%3,%4};"
+                 ::"r"(addr), "r"(pack_bf16(v[0][0], v[0][1])), "r"(pack_bf16(v[0][2], v[0][3])),
+                   "r"(pack_bf16(v[1][0], v[1][1])), "r"(pack_bf16(v[1][2], v[1][3])) : "memory");
+}
+__device__ __forceinline__ void ld_tile_t(uint32_t tile, const uint32_t (&moff)[G_H2], float (&v)[G_NB][4])
+{
+#pragma unroll
+    for (int h2 = 0; h2 < G_H2; ++h2) ld_half_t(tile + moff[h2], reinterpret_cast<float (&)[2][4]>(v[2 * h2]));
+}
+__device__ __forceinline__ void st_tile_t(uint32_t tile, const uint32_t (&moff)[G_H2], const float (&v)[G_NB][4])
+{
+#pragma unroll
+    for (int h2 = 0; h2 < G_H2; ++h2) st_half_t(tile + moff[h2], reinterpret_cast<const float (&)[2][4]>(v[2 * h2]));
+}
 __device__ __forceinline__ void ld_tile(uint32_t tile, const uint32_t (&moff)[G_H2], float (&v)[G_NB][4])
 {
 #pragma unroll
@@ -210,68 +244,62 @@ __device__ __forceinline__ void st_tile(uint32_t tile, const uint32_t (&moff)[G_
     for (int h2 = 0; h2 < G_H2; ++h2) st_half(tile + moff[h2], reinterpret_cast<const float (&)[2][4]>(v[2 * h2]));
 }
 
-// Inclusive sums along the 64 rows of a tile in the group's layout, forwards (rows <= t) or backwards (rows >= t).
-// tot: [4][64] floats of the group's shared memory.  Contains one barrier of the group, which also forms the AND of
-// `ok` over it (returned).
+// Inclusive sums along the tokens (columns) of the lane's cells, forwards (tokens <= t) or backwards (tokens >= t): a
+// lane's pairs, then the four lanes of a quad (two shuffles of a pair's sum), then the lane's 8-token blocks, then the
+// column slabs through shared memory.  tot: [G_NSLAB][64] floats of the group's shared memory, left with each slab's total
+// per channel.  Contains one barrier of the group, which also forms the AND of `ok` over it (returned).
 template <bool REV>
-__device__ __forceinline__ bool scan_rows(float (&v)[G_NB][4], uint32_t tot, int grp, int sp, int cb, int lane, bool ok)
+__device__ __forceinline__ bool scan_tokens(float (&v)[G_NB][4], uint32_t tot, int grp, int cx, int R0, int lane, bool ok)
 {
-    const int g = lane >> 2, q = lane & 3;           // (cb: the lane's first column, a multiple of 2)
-    // (the additions run on the pairs of neighbouring columns: one two-lane instruction for two cells)
+    const int q = lane & 3;
+    float pair[G_NB][2], ex[G_NB][2];                // the lane's pair of an 8-token block; the pairs before (after) it in the block
 #pragma unroll
-    for (int d = 4; d < 32; d <<= 1) {
-        const bool take = REV ? lane + d < 32 : lane >= d;
+    for (int n = 0; n < G_NB; ++n)
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            pair[n][h] = v[n][2 * h] + v[n][2 * h + 1];
+            const float o1 = REV ? __shfl_down_sync(0xffffffffu, pair[n][h], 1, 4) : __shfl_up_sync(0xffffffffu, pair[n][h], 1, 4);
+            ex[n][h] = (REV ? q < 3 : q > 0) ? o1 : 0.f;
+        }
+#pragma unroll
+    for (int n = 0; n < G_NB; ++n)
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const float s = pair[n][h] + ex[n][h];
+            const float o2 = REV ? __shfl_down_sync(0xffffffffu, s, 2, 4) : __shfl_up_sync(0xffffffffu, s, 2, 4);
+            ex[n][h] += (REV ? q < 2 : q > 1) ? o2 : 0.f;
+            pair[n][h] += ex[n][h];                  // inclusive; the block's total on the quad's last (first) lane
+        }
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        float run = 0.f;                             // the lane's blocks before (after) this one
+#pragma unroll
+        for (int k = 0; k < G_NB; ++k) {
+            const int n = REV ? G_NB - 1 - k : k;
+            const float base = ex[n][h] + run;
+            run += __shfl_sync(0xffffffffu, pair[n][h], REV ? 0 : 3, 4);
+            const int e0 = 2 * h + (REV ? 1 : 0), e1 = 2 * h + (REV ? 0 : 1);
+            v[n][e0] += base;
+            v[n][e1] += v[n][e0];
+        }
+        if (q == 0) stsf(tot + 4 * (cx * 64 + R0 + 8 * h), run);
+    }
+    ok = gbar_and(grp, ok);
+    // the totals of the column slabs before (after) this one
+    float t[2] = {0.f, 0.f};
+#pragma unroll
+    for (int o = 0; o < G_NSLAB; ++o)
+        if (REV ? o > cx : o < cx)
+#pragma unroll
+            for (int h = 0; h < 2; ++h) t[h] += ldsf(tot + 4 * (o * 64 + R0 + 8 * h));
+    if (REV ? cx < G_NSLAB - 1 : cx > 0) {
 #pragma unroll
         for (int n = 0; n < G_NB; ++n)
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
-                float2 o;
-                o.x = REV ? __shfl_down_sync(0xffffffffu, v[n][2 * h], d) : __shfl_up_sync(0xffffffffu, v[n][2 * h], d);
-                o.y = REV ? __shfl_down_sync(0xffffffffu, v[n][2 * h + 1], d) : __shfl_up_sync(0xffffffffu, v[n][2 * h + 1], d);
-                if (take) {
-                    const float2 r = add2(make_float2(v[n][2 * h], v[n][2 * h + 1]), o);
-                    v[n][2 * h] = r.x; v[n][2 * h + 1] = r.y;
-                }
+                const float2 r = add2(make_float2(v[n][2 * h], v[n][2 * h + 1]), make_float2(t[h], t[h]));
+                v[n][2 * h] = r.x; v[n][2 * h + 1] = r.y;
             }
-    }
-#pragma unroll
-    for (int n = 0; n < G_NB; ++n) {
-        float2 o;
-        if (REV) {
-            o.x = __shfl_sync(0xffffffffu, v[n][2], q); o.y = __shfl_sync(0xffffffffu, v[n][3], q);
-            const float2 r = add2(make_float2(v[n][0], v[n][1]), o);
-            v[n][0] = r.x; v[n][1] = r.y;
-        } else {
-            o.x = __shfl_sync(0xffffffffu, v[n][0], 28 + q); o.y = __shfl_sync(0xffffffffu, v[n][1], 28 + q);
-            const float2 r = add2(make_float2(v[n][2], v[n][3]), o);
-            v[n][2] = r.x; v[n][3] = r.y;
-        }
-    }
-    if (g == (REV ? 0 : 7)) {
-#pragma unroll
-        for (int n = 0; n < G_NB; ++n)
-            stsf2(tot + 4 * (sp * 64 + cb + 8 * n), REV ? make_float2(v[n][0], v[n][1]) : make_float2(v[n][2], v[n][3]));
-    }
-    ok = gbar_and(grp, ok);
-    // the totals of the row groups before (after) this one: summed first, then added to both rows
-    float2 t[G_NB];
-#pragma unroll
-    for (int n = 0; n < G_NB; ++n) t[n] = make_float2(0.f, 0.f);
-    bool any = false;
-#pragma unroll
-    for (int o = 0; o < 4; ++o) {
-        if (REV ? o > sp : o < sp) {
-#pragma unroll
-            for (int n = 0; n < G_NB; ++n) t[n] = add2(t[n], ldsf2(tot + 4 * (o * 64 + cb + 8 * n)));
-            any = true;
-        }
-    }
-    if (any) {
-#pragma unroll
-        for (int n = 0; n < G_NB; ++n) {
-            const float2 lo = add2(make_float2(v[n][0], v[n][1]), t[n]), hi = add2(make_float2(v[n][2], v[n][3]), t[n]);
-            v[n][0] = lo.x; v[n][1] = lo.y; v[n][2] = hi.x; v[n][3] = hi.y;
-        }
     }
     return ok;
 }
@@ -325,20 +353,25 @@ wkv6_backward_chunked_kernel(const __grid_constant__ CUtensorMap tm_x, const __g
 #pragma unroll
     for (int h2 = 0; h2 < G_H2; ++h2)
         moff[h2] = swz(16 * sp + (lane & 7) + 8 * ((lane >> 3) & 1), (G_NB * cx + 2 * h2 + (lane >> 4)) << 4);
+    // the same for the [token][channel] tiles, read and written transposed: the warp's rows are channels 16 sp .. +15, its
+    // columns tokens 8 G_NB cx ..
+    uint32_t tmoff[G_H2];
+#pragma unroll
+    for (int h2 = 0; h2 < G_H2; ++h2)
+        tmoff[h2] = swz(8 * (G_NB * cx + 2 * h2) + (lane & 7) + 8 * (lane >> 4), (2 * sp + ((lane >> 3) & 1)) << 4);
     const uint32_t gbase = sbase + grp * GO_BYTES;   // this group's shared memory
     auto gsm = [&](int off) { return reinterpret_cast<float*>(smem + grp * GO_BYTES + off); };
-    // the adjoint tiles handed between the groups: [buffer][cell of the lane][thread of the group] (conflict-free)
+    // the adjoint tiles handed between the groups: [buffer][column block of the lane][thread of the group] (16 bytes per thread)
     auto g_put = [&](int b, const float (&v)[G_NB][4]) {
 #pragma unroll
-        for (int n = 0; n < G_NB; ++n)
-#pragma unroll
-            for (int e = 0; e < 4; ++e) stsf(sbase + GS_GBUF + 4 * ((b * 4 * G_NB + 4 * n + e) * G_GT + gt), v[n][e]);
+        for (int n = 0; n < G_NB; ++n) stsf4(sbase + GS_GBUF + 16 * ((b * G_NB + n) * G_GT + gt), make_float4(v[n][0], v[n][1], v[n][2], v[n][3]));
     };
     auto g_get = [&](int b, float (&v)[G_NB][4]) {
 #pragma unroll
-        for (int n = 0; n < G_NB; ++n)
-#pragma unroll
-            for (int e = 0; e < 4; ++e) v[n][e] = ldsf(sbase + GS_GBUF + 4 * ((b * 4 * G_NB + 4 * n + e) * G_GT + gt));
+        for (int n = 0; n < G_NB; ++n) {
+            const float4 t = ldsf4(sbase + GS_GBUF + 16 * ((b * G_NB + n) * G_GT + gt));
+            v[n][0] = t.x; v[n][1] = t.y; v[n][2] = t.z; v[n][3] = t.w;
+        }
     };
     auto gld = [&](int off) { return ldsf(gbase + off); };           // a float of this group's small arrays
     const float* ub = reinterpret_cast<const float*>(smem + GS_U);
@@ -421,9 +454,8 @@ wkv6_backward_chunked_kernel(const __grid_constant__ CUtensorMap tm_x, const __g
             v[n][0] = lo.x; v[n][1] = lo.y; v[n][2] = hi.x; v[n][3] = hi.y;
         }
     };
-    float du_acc[G_NB][2];
-#pragma unroll
-    for (int n = 0; n < G_NB; ++n) du_acc[n][0] = du_acc[n][1] = 0.f;
+    float du_acc[2] = {0.f, 0.f};                    // bonus gradient of channels R0, R1 over this lane's tokens
+    const float2 u_lh = (C2 || GSUM) ? make_float2(0.f, 0.f) : make_float2(ub[R0], ub[R1]);      // the bonus of those channels
     if (gt == 0 && grp < nit) { issue_loads_a(grp); issue_loads_b(grp); }
     int mph = 0;                                     // phase bit of this group's two product barriers
     float dprod_lo = 1.f, dprod_hi = 1.f;            // summary variant: product of this group's chunk decays (rows R0, R1)
@@ -449,24 +481,24 @@ wkv6_backward_chunked_kernel(const __grid_constant__ CUtensorMap tm_x, const __g
         float a[G_NB][4], lw2[G_NB][4];
         {
             float xv[G_NB][4];
-            ld_tile(tx, moff, xv);
+            ld_tile_t(tx, tmoff, xv);
 #pragma unroll
             for (int n = 0; n < G_NB; ++n)
 #pragma unroll
                 for (int e = 0; e < 4; ++e) {
-                    const bool live = (e < 2 ? R0 : R1) < valid;
+                    const bool live = cb + 8 * n + (e & 1) < valid;
                     lw2[n][e] = live ? -ex2(fmaf(xv[n][e], LOG2E, LOG2_LOG2E)) : 0.f;
                     a[n][e] = lw2[n][e];
                 }
         }
-        ok = scan_rows<false>(a, gbase + GO_TOT, grp, sp, cb, lane, ok);      // (barrier: the zeroed rows are visible after it)
+        ok = scan_tokens<false>(a, gbase + GO_TOT, grp, cx, R0, lane, ok);      // (barrier: the zeroed rows are visible after it)
         if (!ok) { alive = false; break; }
         float d_lo, d_hi;                            // the chunk's decay for the channels that are this lane's rows of G
         bool safe;
         {
             float al0 = 0.f, al1 = 0.f;
 #pragma unroll
-            for (int o = 0; o < 4; ++o) { al0 += gld(GO_TOT + 4 * (o * 64 + R0)); al1 += gld(GO_TOT + 4 * (o * 64 + R1)); }
+            for (int o = 0; o < G_NSLAB; ++o) { al0 += gld(GO_TOT + 4 * (o * 64 + R0)); al1 += gld(GO_TOT + 4 * (o * 64 + R1)); }
             d_lo = ex2(al0); d_hi = ex2(al1);
             safe = GSUM || ((al0 >= -A2_MAX) && (al1 >= -A2_MAX));         // false for NaN as well
             if (GSUM) { dprod_lo *= d_lo; dprod_hi *= d_hi; }
@@ -483,33 +515,42 @@ wkv6_backward_chunked_kernel(const __grid_constant__ CUtensorMap tm_x, const __g
         }
         {
             float rv[G_NB][4], kv[G_NB][4];
-            ld_tile(tr, moff, rv);
-            ld_tile(tk, moff, kv);
-            float b0 = 0.f, b1 = 0.f;
+            ld_tile_t(tr, tmoff, rv);
+            ld_tile_t(tk, tmoff, kv);
+            float bt[2 * G_NB];                                        // bonus terms of the lane's tokens over its two channels
             // (two-lane fp32 arithmetic on the pairs of neighbouring columns: half the multiply / add instructions)
 #pragma unroll
             for (int n = 0; n < G_NB; ++n) {
-                const float2 u2 = (!C2 && !GSUM) ? ldsf2(sbase + GS_U + 4 * (cb + 8 * n)) : make_float2(0.f, 0.f);
 #pragma unroll
-                for (int h = 0; h < 2; ++h) {                          // h = 0: row R0, h = 1: row R1
+                for (int h = 0; h < 2; ++h) {                          // h = 0: channel R0, h = 1: channel R1
                     float2 rr = make_float2(rv[n][2 * h], rv[n][2 * h + 1]), kk = make_float2(kv[n][2 * h], kv[n][2 * h + 1]);
                     const float2 aa = make_float2(a[n][2 * h], a[n][2 * h + 1]), ll = make_float2(lw2[n][2 * h], lw2[n][2 * h + 1]);
-                    if (C2) kk = mul2(kk, make_float2(one_minus_ex2(ll.x), one_minus_ex2(ll.y)));      // the key that enters the state
+                    if (C2) kk = mul2(kk, one_minus_ex2_2(ll));      // the key that enters the state
                     if (!C2 && !GSUM) {
-                        const float2 t = mul2(mul2(rr, kk), u2);
-                        if (h == 0) b0 += t.x + t.y; else b1 += t.x + t.y;
+                        const float uc = h ? u_lh.y : u_lh.x;
+                        const float2 t = mul2(mul2(rr, kk), make_float2(uc, uc));
+                        if (h == 0) { bt[2 * n] = t.x; bt[2 * n + 1] = t.y; }
+                        else { bt[2 * n] += t.x; bt[2 * n + 1] += t.y; }
                     }
                     rr = mul2(rr, ex2_2(sub2(aa, ll)));
                     kk = mul2(kk, make_float2(ex2(-aa.x), ex2(-aa.y)));
                     rv[n][2 * h] = rr.x; rv[n][2 * h + 1] = rr.y; kv[n][2 * h] = kk.x; kv[n][2 * h + 1] = kk.y;
                 }
             }
-            st_tile(t_rh, moff, rv);
-            if (!GSUM) st_tile(t_kh, moff, kv);
+            st_tile_t(t_rh, tmoff, rv);
+            if (!GSUM) st_tile_t(t_kh, tmoff, kv);
             if (!C2 && !GSUM) {
-                b0 += __shfl_xor_sync(0xffffffffu, b0, 1); b1 += __shfl_xor_sync(0xffffffffu, b1, 1);
-                b0 += __shfl_xor_sync(0xffffffffu, b0, 2); b1 += __shfl_xor_sync(0xffffffffu, b1, 2);
-                if (q == 0) { stsf(gbase + GO_BP + 4 * (cx * 64 + R0), b0); stsf(gbase + GO_BP + 4 * (cx * 64 + R1), b1); }
+                // over the warp's 16 channels: transposing butterfly over the eight lanes of a column (lane g ends with
+                // column block (g4, g2), token e = g1 of its pair)
+                static_assert(G_NB == 4, "eight tokens per lane");
+                const bool g4 = g & 4, g2 = g & 2, g1 = g & 1;
+                float h4[4], h2[2];
+#pragma unroll
+                for (int m = 0; m < 4; ++m) h4[m] = (g4 ? bt[4 + m] : bt[m]) + __shfl_xor_sync(0xffffffffu, g4 ? bt[m] : bt[4 + m], 16);
+#pragma unroll
+                for (int m = 0; m < 2; ++m) h2[m] = (g2 ? h4[2 + m] : h4[m]) + __shfl_xor_sync(0xffffffffu, g2 ? h4[m] : h4[2 + m], 8);
+                const float h1 = (g1 ? h2[1] : h2[0]) + __shfl_xor_sync(0xffffffffu, g1 ? h2[0] : h2[1], 4);
+                stsf(gbase + GO_BP + 4 * (sp * 64 + cb + 8 * (g >> 1) + (g & 1)), h1);
             }
         }
         if (!GSUM && !mbar_wait(gb(GB_S0), use & 1, abort_flag)) ok = false;       // the chunk-start state is in its tile
@@ -777,7 +818,7 @@ wkv6_backward_chunked_kernel(const __grid_constant__ CUtensorMap tm_x, const __g
                     float bon0 = 0.f, bon1 = 0.f;
                     if (!C2) {
 #pragma unroll
-                        for (int o = 0; o < G_NSLAB; ++o) { bon0 += gld(GO_BP + 4 * (o * 64 + R0)); bon1 += gld(GO_BP + 4 * (o * 64 + R1)); }
+                        for (int o = 0; o < 4; ++o) { bon0 += gld(GO_BP + 4 * (o * 64 + R0)); bon1 += gld(GO_BP + 4 * (o * 64 + R1)); }
                     }
                     tmem_ld_done();
 #pragma unroll
@@ -805,14 +846,14 @@ wkv6_backward_chunked_kernel(const __grid_constant__ CUtensorMap tm_x, const __g
 #pragma unroll
                 for (int kk = 0; kk < 4; ++kk) {
                     const uint64_t ks = 2 * kk;
-                    tc_mma(tmem + GT_DR, dY + ks, dS + ks, IDESC_K_K, kk > 0);         // dR[t][c] = dY S_0^T
-                    tc_mma(tmem + GT_DK, dV + ks, dG + ks, IDESC_K_K, kk > 0);         // dK[i][c] = V G^^T
+                    tc_mma(tmem + GT_DR, dS + ks, dY + ks, IDESC_K_K, kk > 0);         // dR^T[c][t] = S_0 dY^T
+                    tc_mma(tmem + GT_DK, dG + ks, dV + ks, IDESC_K_K, kk > 0);         // dK^T[c][i] = G^ V^T
                 }
 #pragma unroll
                 for (int kk = 0; kk < 4; ++kk) {
                     const uint64_t ks = 2 * kk, ms = 128 * kk;
-                    tc_mma(tmem + GT_DR, dD + ks, dK + ms, IDESC_K_MN, 1);             // dR += dP' K^
-                    tc_mma(tmem + GT_DK, dD + ms, dR + ms, IDESC_MN_MN, 1);            // dK += dP'^T R^
+                    tc_mma(tmem + GT_DR, dK + ms, dD + ks, IDESC_MN_K, 1);             // dR^T += K^^T dP'^T
+                    tc_mma(tmem + GT_DK, dR + ms, dD + ms, IDESC_MN_MN, 1);            // dK^T += R^^T dP'
                 }
                 tc_commit(gb(GB_MRK));
 #pragma unroll
@@ -836,20 +877,19 @@ wkv6_backward_chunked_kernel(const __grid_constant__ CUtensorMap tm_x, const __g
                 // q and m take the operands as the tensor core saw them (rounded to bf16): the pair terms that q and
                 // m share, and that cancel in the suffix sums, are then the same products on both sides
                 float acc[2][4], o[2][4], hat[2][4], rv[2][4], kv[2][4];
-                const float pd0 = C2 ? 0.f : gld(GO_DPD + 4 * R0), pd1 = C2 ? 0.f : gld(GO_DPD + 4 * R1);
                 tmem_ld_16x16_async2(tacc + GT_DR + 16 * h2, acc);
-                ld_half(tr + moff[h2], rv);
-                ld_half(tk + moff[h2], kv);
-                ld_half(t_rh + moff[h2], hat);
+                ld_half_t(tr + tmoff[h2], rv);
+                ld_half_t(tk + tmoff[h2], kv);
+                ld_half_t(t_rh + tmoff[h2], hat);
                 tmem_ld_done();
                 // (two-lane fp32 arithmetic on the pairs of neighbouring columns)
 #pragma unroll
                 for (int n = 0; n < 2; ++n) {
                     const int nn = 2 * h2 + n;
-                    const float2 u2 = C2 ? make_float2(0.f, 0.f) : ldsf2(sbase + GS_U + 4 * (cb + 8 * nn));
+                    const float2 pd = C2 ? make_float2(0.f, 0.f) : ldsf2(gbase + GO_DPD + 4 * (cb + 8 * nn));
 #pragma unroll
                     for (int h = 0; h < 2; ++h) {
-                        const float2 pd = h ? make_float2(pd1, pd1) : make_float2(pd0, pd0);
+                        const float2 u2 = h ? make_float2(u_lh.y, u_lh.y) : make_float2(u_lh.x, u_lh.x);
                         const float2 ac = make_float2(acc[n][2 * h], acc[n][2 * h + 1]), kk = make_float2(kv[n][2 * h], kv[n][2 * h + 1]);
                         const float2 sr = ex2_2(sub2(make_float2(a[nn][2 * h], a[nn][2 * h + 1]), make_float2(lw2[nn][2 * h], lw2[nn][2 * h + 1])));
                         const float2 oo = C2 ? mul2(ac, sr) : fma2(mul2(u2, kk), pd, mul2(ac, sr));
@@ -857,22 +897,22 @@ wkv6_backward_chunked_kernel(const __grid_constant__ CUtensorMap tm_x, const __g
                         o[n][2 * h] = oo.x; o[n][2 * h + 1] = oo.y;
                         qv[nn][2 * h] = qq.x; qv[nn][2 * h + 1] = qq.y;
                         if (!C2) {
-                            const float2 dd = fma2(mul2(make_float2(rv[n][2 * h], rv[n][2 * h + 1]), kk), pd, make_float2(du_acc[nn][0], du_acc[nn][1]));
-                            du_acc[nn][0] = dd.x; du_acc[nn][1] = dd.y;
+                            const float2 dd = mul2(mul2(make_float2(rv[n][2 * h], rv[n][2 * h + 1]), kk), pd);
+                            du_acc[h] += dd.x + dd.y;
                         }
                     }
                 }
                 tmem_ld_16x16_async2(tacc + GT_DK + 16 * h2, acc);
-                ld_half(t_kh + moff[h2], hat);
+                ld_half_t(t_kh + tmoff[h2], hat);
                 tmem_ld_done();
-                st_half(o_dr + moff[h2], o);
+                st_half_t(o_dr + tmoff[h2], o);
 #pragma unroll
                 for (int n = 0; n < 2; ++n) {
                     const int nn = 2 * h2 + n;
-                    const float2 u2 = C2 ? make_float2(0.f, 0.f) : ldsf2(sbase + GS_U + 4 * (cb + 8 * nn));
+                    const float2 pd = C2 ? make_float2(0.f, 0.f) : ldsf2(gbase + GO_DPD + 4 * (cb + 8 * nn));
 #pragma unroll
                     for (int h = 0; h < 2; ++h) {
-                        const float2 pd = h ? make_float2(pd1, pd1) : make_float2(pd0, pd0);
+                        const float2 u2 = h ? make_float2(u_lh.y, u_lh.y) : make_float2(u_lh.x, u_lh.x);
                         const float2 ac = make_float2(acc[n][2 * h], acc[n][2 * h + 1]);
                         const float2 sk = make_float2(ex2(-a[nn][2 * h]), ex2(-a[nn][2 * h + 1]));
                         float2 oo = C2 ? mul2(ac, sk) : fma2(mul2(u2, make_float2(rv[n][2 * h], rv[n][2 * h + 1])), pd, mul2(ac, sk));
@@ -881,7 +921,7 @@ wkv6_backward_chunked_kernel(const __grid_constant__ CUtensorMap tm_x, const __g
                         if (C2) {
                             // oo is the gradient of k (1 - w): the key gets (1 - w) of it, and the decay logit its
                             // share through the key factor, folded into the term that leaves the suffix sums
-                            const float2 omw = make_float2(one_minus_ex2(lw2[nn][2 * h]), one_minus_ex2(lw2[nn][2 * h + 1]));
+                            const float2 omw = one_minus_ex2_2(make_float2(lw2[nn][2 * h], lw2[nn][2 * h + 1]));
                             const float2 qq = fma2(mul2(oo, make_float2(kv[n][2 * h], kv[n][2 * h + 1])), sub2(make_float2(1.f, 1.f), omw),
                                                    make_float2(qv[nn][2 * h], qv[nn][2 * h + 1]));
                             qv[nn][2 * h] = qq.x; qv[nn][2 * h + 1] = qq.y;
@@ -890,7 +930,7 @@ wkv6_backward_chunked_kernel(const __grid_constant__ CUtensorMap tm_x, const __g
                         o[n][2 * h] = oo.x; o[n][2 * h + 1] = oo.y;
                     }
                 }
-                st_half(o_dk + moff[h2], o);
+                st_half_t(o_dk + tmoff[h2], o);
             }
             // dV: every product of the chunk has completed, so x, v, dy can take the group's next chunk
             if (!mbar_wait(gb(GB_MV), mph, abort_flag)) ok = false;
@@ -905,22 +945,22 @@ wkv6_backward_chunked_kernel(const __grid_constant__ CUtensorMap tm_x, const __g
                 st_tile(o_dv, moff, acc);
             }
             tc_fence_before();
-            ok = scan_rows<true>(z, gbase + GO_TOT, grp, sp, cb, lane, ok);
+            ok = scan_tokens<true>(z, gbase + GO_TOT, grp, cx, R0, lane, ok);
             if (!ok) { alive = false; break; }
             if (gt == 0 && it + 2 < nit) issue_loads_b(it + 2);      // (r, k were last read before the barrier of the sums)
+            float E[2] = {0.f, 0.f};
+#pragma unroll
+            for (int o = 0; o < G_NSLAB; ++o) { E[0] += gld(GO_EP + 4 * (o * 64 + R0)); E[1] += gld(GO_EP + 4 * (o * 64 + R1)); }
 #pragma unroll
             for (int n = 0; n < G_NB; ++n) {
-                float E0 = 0.f, E1 = 0.f;
-#pragma unroll
-                for (int o = 0; o < G_NSLAB; ++o) { const float2 ev = ldsf2(gbase + GO_EP + 4 * (o * 64 + cb + 8 * n)); E0 += ev.x; E1 += ev.y; }
 #pragma unroll
                 for (int h = 0; h < 2; ++h) {
-                    const float2 dl = sub2(add2(make_float2(E0, E1), make_float2(z[n][2 * h], z[n][2 * h + 1])), make_float2(qv[n][2 * h], qv[n][2 * h + 1]));
+                    const float2 dl = sub2(add2(make_float2(E[h], E[h]), make_float2(z[n][2 * h], z[n][2 * h + 1])), make_float2(qv[n][2 * h], qv[n][2 * h + 1]));
                     const float2 dx2 = mul2(dl, mul2(make_float2(lw2[n][2 * h], lw2[n][2 * h + 1]), make_float2(LN2, LN2)));
                     z[n][2 * h] = dx2.x; z[n][2 * h + 1] = dx2.y;
                 }
             }
-            st_tile(o_dx, moff, z);
+            st_tile_t(o_dx, tmoff, z);
         }
         // ---- the chunk's four gradient tiles leave: TMA for a whole chunk, plain stores for a ragged one
         fence_proxy_async();
@@ -971,18 +1011,12 @@ wkv6_backward_chunked_kernel(const __grid_constant__ CUtensorMap tm_x, const __g
     if (!alive && gt == 0) sts32(abort_flag, 1u);    // (the other group's waits see it)
     if (GSUM && cx == 0 && q == 0) { stsf(gbase + GO_REDV + 4 * R0, dprod_lo); stsf(gbase + GO_REDV + 4 * R1, dprod_hi); }
     if (!C2 && !GSUM) {
+        // (over the four lanes of a channel; the column slabs are added below)
 #pragma unroll
-        for (int d = 4; d < 32; d <<= 1)
+        for (int d = 1; d < 4; d <<= 1)
 #pragma unroll
-            for (int n = 0; n < G_NB; ++n)
-#pragma unroll
-                for (int e = 0; e < 2; ++e) du_acc[n][e] += __shfl_xor_sync(0xffffffffu, du_acc[n][e], d);
-        if (g == 0) {
-#pragma unroll
-            for (int n = 0; n < G_NB; ++n)
-#pragma unroll
-                for (int e = 0; e < 2; ++e) gsm(GO_REDV)[sp * 64 + cb + 8 * n + e] = du_acc[n][e];
-        }
+            for (int h = 0; h < 2; ++h) du_acc[h] += __shfl_xor_sync(0xffffffffu, du_acc[h], d);
+        if (q == 0) { gsm(GO_REDV)[cx * 64 + R0] = du_acc[0]; gsm(GO_REDV)[cx * 64 + R1] = du_acc[1]; }
     }
     if (gt == 0) {
         bulk_wait<0>();                              // the gradient tiles have reached memory
@@ -1002,7 +1036,7 @@ wkv6_backward_chunked_kernel(const __grid_constant__ CUtensorMap tm_x, const __g
         for (int gg = 0; gg < 2; ++gg) {
             const float* rv4 = reinterpret_cast<const float*>(smem + gg * GO_BYTES + GO_REDV);
             const float* fb = reinterpret_cast<const float*>(smem + gg * GO_BYTES + GO_DUFB);
-            s += ((rv4[tid] + rv4[64 + tid]) + (rv4[128 + tid] + rv4[192 + tid])) + fb[tid];
+            s += (rv4[tid] + rv4[64 + tid]) + fb[tid];
         }
         p.du_part[((size_t)unit * p.nseg + seg) * 64 + tid] = s;
     }
