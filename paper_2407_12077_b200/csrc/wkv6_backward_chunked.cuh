@@ -88,8 +88,24 @@ struct BParamsPacked : BParams {
     // does not end on a long one while the other SMs idle); NULL: in index order.
     const int32_t* order;
 };
-template <bool PACKED> struct BParamsOf { using type = BParams; };
-template <> struct BParamsOf<true> { using type = BParamsPacked; };
+// Balanced launches (dense calls whose whole units would leave SMs idle in a last round): a CTA walks a stream of pieces of
+// units without draining in between.  While at least two units per CTA are left they go whole, unit b + k gridDim to CTA b;
+// the chunks of the rest, in order, are cut into gridDim equal ranges of one to two units each.  A CTA takes the later part
+// (in time) of the unit its range begins in first of all and the earlier part of the unit it ends in last, so the adjoint at
+// a cut is there long before it is wanted: it is handed over in `hand` (one [64][64] fp32 block per CTA that ends with an
+// earlier part), announced by a word equal to `nonce` (a number no earlier launch has used).  The launch is cooperative.
+struct BParamsBal : BParams {
+    int n_units;
+    float* hand;                 // [gridDim][64][64]
+    unsigned long long* words;   // [gridDim]
+    unsigned long long nonce;
+};
+template <bool PACKED, bool BAL> struct BParamsOf { using type = BParams; };
+template <> struct BParamsOf<true, false> { using type = BParamsPacked; };
+template <> struct BParamsOf<false, true> { using type = BParamsBal; };
+constexpr int BAL_MAX_ROUNDS = 12;                        // whole units per CTA before the cut ones
+constexpr int BAL_PIECES = BAL_MAX_ROUNDS + 4;
+constexpr int BAL_DU_SLOTS = 8;                           // bonus-gradient partial sums per unit: two parts x two groups x two column slabs
 constexpr int GSUM_FLOATS = 64 + 64 * 64;
 constexpr size_t CKPT_FLOATS = 64 * 64 / 2;               // a checkpoint (one bf16 [64][64] state) in units of the workspace's floats
 
@@ -161,7 +177,10 @@ constexpr int GS_TMEM = GS_ABORT + 8;
 // mbarriers, per group: inputs x, v, dy / inputs r, k / first group of products / dR^ and dK^ / dV; then the hand-over pair
 constexpr int GS_BAR = GS_TMEM + 8;
 enum { GB_INA = 0, GB_INB = 1, GB_MA = 2, GB_MRK = 3, GB_MV = 4, GB_S0 = 5, GB_PER_GROUP = 6, GB_GREADY = 12, GB_COUNT = 14 };
-constexpr int G_SMEM_BYTES = GS_BAR + 8 * GB_COUNT;
+// balanced launches: the CTA's pieces, {end of the piece (iteration), row of iteration 0, column, checkpoint slot of iteration
+// 0, unit, chunk of iteration 0, kind (0 whole, 1 later part, 2 earlier part), first iteration}
+constexpr int GS_PT = (GS_BAR + 8 * GB_COUNT + 15) & ~15;
+constexpr int G_SMEM_BYTES = GS_PT + 32 * BAL_PIECES;
 constexpr int G_SMEM_ALLOC = G_SMEM_BYTES + 1024;
 static_assert(G_SMEM_ALLOC <= 232448, "shared memory budget of one sm_100 CTA");
 
@@ -308,14 +327,15 @@ __device__ __forceinline__ bool scan_tokens(float (&v)[G_NB][4], uint32_t tot, i
 // G <- diag(D) G + R^^T dY over a segment, from zero, and the product of the chunk decays; it reads x, r, dy only and
 // needs no token-by-token path (R^ never exceeds r: no exponent can overflow).
 // PACKED: packed variable-length sequences (BParams::cu), one CTA per sequence and head.
-template <bool C2, bool GSUM = false, bool PACKED = false>
+// BAL: one CTA per SM, pieces of units (BParamsBal).
+template <bool C2, bool GSUM = false, bool PACKED = false, bool BAL = false>
 __global__ void __launch_bounds__(G_THREADS, 1)
 wkv6_backward_chunked_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ CUtensorMap tm_r,
                             const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ CUtensorMap tm_v,
                             const __grid_constant__ CUtensorMap tm_dy, const __grid_constant__ CUtensorMap tm_dr,
                             const __grid_constant__ CUtensorMap tm_dk, const __grid_constant__ CUtensorMap tm_dv,
                             const __grid_constant__ CUtensorMap tm_dx, const __grid_constant__ CUtensorMap tm_ck,
-                            const typename BParamsOf<PACKED>::type p)
+                            const typename BParamsOf<PACKED, BAL>::type p)
 {
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -343,7 +363,7 @@ wkv6_backward_chunked_kernel(const __grid_constant__ CUtensorMap tm_x, const __g
     const int nchunks = (T + L - 1) / L;
     const int c_lo = p.nseg > 1 ? min(nchunks, seg * p.seg_chunks) : 0;                      // this CTA's chunks: c_lo .. c_hi-1,
     const int c_hi = (p.nseg > 1 && seg < p.nseg - 1) ? min(nchunks, c_lo + p.seg_chunks) : nchunks;   // walked from the last
-    const int nit = c_hi - c_lo;
+    const int nit_unit = c_hi - c_lo;
     const int col0 = h * 64;
     const size_t C = (size_t)p.H * 64;
     const int R0 = 16 * sp + g, R1 = R0 + 8;         // this lane's two rows
@@ -386,7 +406,28 @@ wkv6_backward_chunked_kernel(const __grid_constant__ CUtensorMap tm_x, const __g
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         fence_proxy_async();
     }
-    if (tid < 64) reinterpret_cast<float*>(smem + GS_U)[tid] = (C2 || GSUM) ? 0.f : p.u[col0 + tid];
+    if (!BAL && tid < 64) reinterpret_cast<float*>(smem + GS_U)[tid] = (C2 || GSUM) ? 0.f : p.u[col0 + tid];
+    if constexpr (BAL) {
+        // this CTA's pieces, by one thread (32-bit products: the host balances only calls whose chunk counts allow it)
+        if (tid == 0) {
+            const unsigned G = gridDim.x, nc = nchunks, rounds = p.n_units / G - 1, R = p.n_units - rounds * G, bi = blockIdx.x;
+            const unsigned b0 = R * nc * bi / G, b1 = R * nc * (bi + 1) / G;
+            int n = 0, it0 = 0;
+            auto put = [&](int un, int lo, int hi, int kind) {             // chunks hi-1 .. lo of unit un
+                const int cs = hi - 1 + it0;                               // chunk of iteration it: cs - it
+                int* e = reinterpret_cast<int*>(smem + GS_PT + 32 * n);
+                e[0] = it0 + hi - lo; e[1] = (un / p.H) * T + cs * L; e[2] = (un % p.H) * 64; e[3] = un * (int)(nc + 1) + cs;
+                e[4] = un; e[5] = cs; e[6] = kind; e[7] = it0;
+                it0 += hi - lo; ++n;
+            };
+            const unsigned w0 = (b0 + nc - 1) / nc, w1 = b1 / nc;          // whole units of the range
+            if (b0 % nc) put(rounds * G + w0 - 1, b0 % nc, nc, 1);
+            for (unsigned k = 0; k < rounds; ++k) put(bi + k * G, 0, nc, 0);
+            for (unsigned w = w0; w < w1; ++w) put(rounds * G + w, 0, nc, 0);
+            if (b1 % nc) put(rounds * G + w1, 0, b1 % nc, 2);
+            for (; n < BAL_PIECES; ++n) reinterpret_cast<int*>(smem + GS_PT + 32 * n)[0] = 0x7fffffff, reinterpret_cast<int*>(smem + GS_PT + 32 * n)[5] = it0;
+        }
+    }
     if (gt < 64) gsm(GO_DUFB)[gt] = 0.f;
     if (warp == 1) tmem_alloc(sbase + GS_TMEM, GT_COLS);
     tc_fence_before();
@@ -395,7 +436,32 @@ wkv6_backward_chunked_kernel(const __grid_constant__ CUtensorMap tm_x, const __g
     const uint32_t tmem = lds32(sbase + GS_TMEM) + 256 * grp;                 // this group's columns
     const uint32_t tacc = tmem + ((uint32_t)(32 * sp) << 16) + 8 * G_NB * cx;      // this warp's block of an accumulator
 
+    // where iteration it lies: chunk, first row, column, checkpoint slot of its start state (balanced launches: from the piece
+    // table, looked up from piece k on)
+    auto pt = [&](int k, int f) -> int { return (int)lds32(sbase + GS_PT + 32 * k + 4 * f); };
+    auto piece_of = [&](int it, int k) -> int { while (it >= pt(k, 0)) ++k; return k; };
+    int nit = nit_unit;
+    int pc = 0;                                      // (balanced launches) the piece of this group's current iteration
+    if constexpr (BAL) {
+        for (int k = 0; k < BAL_PIECES && pt(k, 0) != 0x7fffffff; ++k) nit = pt(k, 0);
+        // the bonus partial sums of this CTA's pieces start at zero: a group may have no chunk in a piece
+        if (!C2) {
+            for (int k = 0; k < BAL_PIECES && pt(k, 0) != 0x7fffffff; ++k) {
+                const int kind = pt(k, 6), n = kind == 0 ? 512 : 256;
+                if (tid < n) p.du_part[(size_t)pt(k, 4) * 512 + (kind == 1 ? 256 : 0) + tid] = 0.f;
+            }
+            __syncthreads();
+        }
+    }
     auto chunk_of = [&](int it) { return c_hi - 1 - it; };
+    auto row_at = [&](int it) -> int {
+        if constexpr (BAL) return pt(piece_of(it, pc), 1) - it * L;
+        return (int)(row0 + (long long)chunk_of(it) * L);
+    };
+    auto col_at = [&](int it) -> int {
+        if constexpr (BAL) return pt(piece_of(it, pc), 2);
+        return col0;
+    };
     const uint32_t tin = gbase + GO_IN;
     const uint32_t tx = tin, tr = tin + TILE, tk = tin + 2 * TILE, tv = tin + 3 * TILE, tdy = tin + 4 * TILE;
     const uint32_t t_rh = gbase + GO_RH, t_kh = gbase + GO_KH;
@@ -407,18 +473,18 @@ wkv6_backward_chunked_kernel(const __grid_constant__ CUtensorMap tm_x, const __g
     // chunk before (of this group) has finished its products, r, k once its epilogue has read them.
     int last_a = -1, last_b = -1, last_s = -1;       // (thread 0 of the group) the last iterations whose copies were issued
     auto issue_loads_a = [&](int it) {               // thread 0 of the group
-        const int row = (int)(row0 + (long long)chunk_of(it) * L);
+        const int row = row_at(it), col = col_at(it);
         mbar_expect_tx(gb(GB_INA), 3 * TILE);
-        tma_load_2d(tx, &tm_x, col0, row, gb(GB_INA));
-        tma_load_2d(tv, &tm_v, col0, row, gb(GB_INA));
-        tma_load_2d(tdy, &tm_dy, col0, row, gb(GB_INA));
+        tma_load_2d(tx, &tm_x, col, row, gb(GB_INA));
+        tma_load_2d(tv, &tm_v, col, row, gb(GB_INA));
+        tma_load_2d(tdy, &tm_dy, col, row, gb(GB_INA));
         last_a = it;
     };
     auto issue_loads_b = [&](int it) {
-        const int row = (int)(row0 + (long long)chunk_of(it) * L);
+        const int row = row_at(it), col = col_at(it);
         mbar_expect_tx(gb(GB_INB), 2 * TILE);
-        tma_load_2d(tr, &tm_r, col0, row, gb(GB_INB));
-        tma_load_2d(tk, &tm_k, col0, row, gb(GB_INB));
+        tma_load_2d(tr, &tm_r, col, row, gb(GB_INB));
+        tma_load_2d(tk, &tm_k, col, row, gb(GB_INB));
         last_b = it;
     };
     auto load_f32_block = [&](const float* src, float (&v)[G_NB][4]) {      // [64][64] fp32 block, the lane's cells
@@ -438,12 +504,15 @@ wkv6_backward_chunked_kernel(const __grid_constant__ CUtensorMap tm_x, const __g
     };
 
     const size_t ck_slot0 = PACKED ? ck_first : (size_t)unit * (nchunks + 1);       // this unit's first checkpoint
-    const __nv_bfloat16* ck_unit = p.ckpt + ck_slot0 * 4096;
+    auto slot_at = [&](int it) -> size_t {           // checkpoint of the iteration's start state
+        if constexpr (BAL) return (size_t)(pt(piece_of(it, pc), 3) - it);
+        return ck_slot0 + (size_t)chunk_of(it);
+    };
     // the chunk-start state is a bf16 [64][64] tile in memory: it lands in its operand tile by TMA (rows of the
     // checkpoint array seen as [slots * 64][64])
     auto issue_load_s = [&](int it) {                // thread 0 of the group
         mbar_expect_tx(gb(GB_S0), TILE);
-        tma_load_2d(t_sb, &tm_ck, 0, (int)((ck_slot0 + (size_t)chunk_of(it)) * 64), gb(GB_S0));
+        tma_load_2d(t_sb, &tm_ck, 0, (int)(slot_at(it) * 64), gb(GB_S0));
         last_s = it;
     };
     auto load_bf16_block = [&](const __nv_bfloat16* src, float (&v)[G_NB][4]) {     // a checkpoint, the lane's cells
@@ -455,22 +524,50 @@ wkv6_backward_chunked_kernel(const __grid_constant__ CUtensorMap tm_x, const __g
         }
     };
     float du_acc[2] = {0.f, 0.f};                    // bonus gradient of channels R0, R1 over this lane's tokens
-    const float2 u_lh = (C2 || GSUM) ? make_float2(0.f, 0.f) : make_float2(ub[R0], ub[R1]);      // the bonus of those channels
+    float2 u_lh = (C2 || GSUM || BAL) ? make_float2(0.f, 0.f) : make_float2(ub[R0], ub[R1]);      // the bonus of those channels
+    // (balanced launches) this group's part of a piece's bonus gradient: over the four lanes of a channel, plus what the
+    // token-by-token path left
+    auto flush_du = [&]() {
+        float d[2] = {du_acc[0], du_acc[1]};
+#pragma unroll
+        for (int o = 1; o < 4; o <<= 1)
+#pragma unroll
+            for (int h = 0; h < 2; ++h) d[h] += __shfl_xor_sync(0xffffffffu, d[h], o);
+        if (q == 0) {
+            if (cx == 0) {
+                d[0] += gsm(GO_DUFB)[R0]; d[1] += gsm(GO_DUFB)[R1];
+                gsm(GO_DUFB)[R0] = 0.f; gsm(GO_DUFB)[R1] = 0.f;
+            }
+            float* dst = p.du_part + (size_t)pt(pc, 4) * 512 + (pt(pc, 6) == 1 ? 256 : 0) + (2 * grp + cx) * 64;
+            dst[R0] = d[0]; dst[R1] = d[1];
+        }
+        du_acc[0] = du_acc[1] = 0.f;
+    };
+    if (BAL) pc = 0;
     if (gt == 0 && grp < nit) { issue_loads_a(grp); issue_loads_b(grp); }
+    if (BAL) pc = -1;
     int mph = 0;                                     // phase bit of this group's two product barriers
     float dprod_lo = 1.f, dprod_hi = 1.f;            // summary variant: product of this group's chunk decays (rows R0, R1)
     bool alive = true;
 
     for (int it = grp; it < nit; it += 2) {
-        const int c = chunk_of(it), valid = min(L, T - c * L);
+        if constexpr (BAL) {
+            const int k = piece_of(it, max(pc, 0));
+            if (k != pc) {
+                pc = k;
+                if (!C2) { u_lh.x = p.u[pt(k, 2) + R0]; u_lh.y = p.u[pt(k, 2) + R1]; }
+            }
+        }
+        const int c = BAL ? pt(pc, 5) - it : chunk_of(it), valid = min(L, T - c * L);
+        const bool first = BAL ? it == pt(pc, 7) : it == 0, last = BAL ? it + 1 == pt(pc, 0) : it + 1 == nit;      // of the piece
         const int use = it >> 1;                     // how often this group's input stage has been filled before
         if (it + 2 < nit && gt == 128) {
             // this group's next chunk: its start state and its input tiles into L2 now, so that the copies issued
             // later find them there
-            const int row = (int)(row0 + (long long)(c - 2) * L);
-            tma_prefetch_2d(&tm_x, col0, row); tma_prefetch_2d(&tm_r, col0, row); tma_prefetch_2d(&tm_k, col0, row);
-            tma_prefetch_2d(&tm_v, col0, row); tma_prefetch_2d(&tm_dy, col0, row);
-            if (!GSUM) tma_prefetch_2d(&tm_ck, 0, (int)((ck_slot0 + (size_t)(c - 2)) * 64));
+            const int row = row_at(it + 2), col = col_at(it + 2);
+            tma_prefetch_2d(&tm_x, col, row); tma_prefetch_2d(&tm_r, col, row); tma_prefetch_2d(&tm_k, col, row);
+            tma_prefetch_2d(&tm_v, col, row); tma_prefetch_2d(&tm_dy, col, row);
+            if (!GSUM) tma_prefetch_2d(&tm_ck, 0, (int)(slot_at(it + 2) * 64));
         }
         // ---- decay: log2-domain magnitudes, cumulative sums over the tokens
         bool ok = mbar_wait(gb(GB_INA), use & 1, abort_flag);
@@ -573,8 +670,26 @@ wkv6_backward_chunked_kernel(const __grid_constant__ CUtensorMap tm_x, const __g
         }
         // ---- the adjoint at the chunk's end, from the other group (the call's dstate_out for the last chunk)
         float G[G_NB][4];
-        if (it == 0) {
-            if (!GSUM && p.dstate_out) load_f32_block(p.dstate_out + (size_t)unit * 4096, G);
+        if (BAL && it > 0 && first) {
+            // (the wait keeps this group from running ahead of the other one's reads of the hand-over tiles)
+            if (!mbar_wait(bar(GB_GREADY + ((it - 1) & 1)), ((it - 1) >> 1) & 1, abort_flag)) ok = false;
+        }
+        if (BAL && first && pt(pc, 6) == 2) {
+            // the earlier part of a unit whose later part the next CTA has taken: the adjoint at the cut
+            if constexpr (BAL) {
+                bool there = true;
+                if (lane == 0) there = word_wait(p.words + blockIdx.x, p.nonce, abort_flag);
+                if (!__all_sync(0xffffffffu, there)) ok = false;
+                const float* src = p.hand + (size_t)blockIdx.x * 4096;
+#pragma unroll
+                for (int n = 0; n < G_NB; ++n) {
+                    const float2 lo = __ldcg(reinterpret_cast<const float2*>(src + (size_t)R0 * 64 + cb + 8 * n));
+                    const float2 hi = __ldcg(reinterpret_cast<const float2*>(src + (size_t)R1 * 64 + cb + 8 * n));
+                    G[n][0] = lo.x; G[n][1] = lo.y; G[n][2] = hi.x; G[n][3] = hi.y;
+                }
+            }
+        } else if (first) {
+            if (!GSUM && p.dstate_out) load_f32_block(p.dstate_out + (size_t)(BAL ? pt(pc, 4) : unit) * 4096, G);
             else {
 #pragma unroll
                 for (int n = 0; n < G_NB; ++n) G[n][0] = G[n][1] = G[n][2] = G[n][3] = 0.f;
@@ -611,13 +726,27 @@ wkv6_backward_chunked_kernel(const __grid_constant__ CUtensorMap tm_x, const __g
             if (q == 0) { stsf(dst + 4 * (cx * 64 + R0), e0); stsf(dst + 4 * (cx * 64 + R1), e1); }
         };
         if (GSUM) {
-        } else if (it == 0) {
+        } else if (first) {
             float SL[G_NB][4];
-            load_bf16_block(ck_unit + (size_t)(c + 1) * 4096, SL);
+            load_bf16_block(p.ckpt + (slot_at(it) + 1) * 4096, SL);
             e_put(gbase + GO_EP, G, SL);
         } else if (gt < G_NSLAB * 64) {
             stsf(gbase + GO_EP + 4 * gt, ldsf(sbase + GS_EH + 4 * (((it - 1) & 1) * G_NSLAB * 64 + gt)));      // (a private copy: the slot is rewritten two chunks on)
         }
+
+        // the adjoint at the start of the piece: the unit's, or a cut's
+        auto end_of_piece = [&](const float (&Gm)[G_NB][4]) {
+            if constexpr (BAL) {
+                if (pt(pc, 6) == 1) {
+                    store_f32_block(p.hand + (size_t)(blockIdx.x - 1) * 4096, Gm);      // (announced at the end of the iteration)
+                    __threadfence();
+                } else if (p.dstate_in) {
+                    store_f32_block(p.dstate_in + (size_t)pt(pc, 4) * 4096, Gm);
+                }
+            } else {
+                if (p.dstate_in && seg == 0) store_f32_block(p.dstate_in + (size_t)unit * 4096, Gm);
+            }
+        };
 
         if (unsafe) {
             // ---- token by token: the chunk's states recomputed into this group's scratch, then the reverse recurrence
@@ -630,7 +759,7 @@ wkv6_backward_chunked_kernel(const __grid_constant__ CUtensorMap tm_x, const __g
             if (!gbar_and(grp, ok)) { alive = false; break; }
             float* scr = p.fb_scratch + (size_t)slot * FB_SLOT_FLOATS + (size_t)gt * (4 * G_NB);
             float S[G_NB][4];
-            load_bf16_block(ck_unit + (size_t)c * 4096, S);
+            load_bf16_block(p.ckpt + slot_at(it) * 4096, S);
             for (int t = 0; t < valid; ++t) {
 #pragma unroll
                 for (int n = 0; n < G_NB; ++n)
@@ -706,7 +835,7 @@ wkv6_backward_chunked_kernel(const __grid_constant__ CUtensorMap tm_x, const __g
                     for (int e = 0; e < 2; ++e) {
                         const int cc = 2 * lane + e;
                         vd = fmaf(lds_bf16(tv + swz(t, 2 * cc)), lds_bf16(tdy + swz(t, 2 * cc)), vd);
-                        if (!C2) ruk = fmaf(lds_bf16(tr + swz(t, 2 * cc)) * ub[cc], lds_bf16(tk + swz(t, 2 * cc)), ruk);
+                        if (!C2) ruk = fmaf(lds_bf16(tr + swz(t, 2 * cc)) * (BAL ? p.u[col_at(it) + cc] : ub[cc]), lds_bf16(tk + swz(t, 2 * cc)), ruk);
                     }
 #pragma unroll
                     for (int d = 1; d < 32; d <<= 1) {
@@ -728,7 +857,7 @@ wkv6_backward_chunked_kernel(const __grid_constant__ CUtensorMap tm_x, const __g
                         sts_bf16(o_dk + swz(t, 2 * cc), s_k * -expm1f(-ec));
                         sts_bf16(o_dx + swz(t, 2 * cc), (s_g - s_k * kc) * (-wc * ec));
                     } else {
-                        const float uc = ub[cc], vd = scal[0];
+                        const float uc = BAL ? p.u[col_at(it) + cc] : ub[cc], vd = scal[0];
                         sts_bf16(o_dr + swz(t, 2 * cc), fmaf(uc * kc, vd, s_r));
                         sts_bf16(o_dk + swz(t, 2 * cc), fmaf(rc * uc, vd, s_k));
                         sts_bf16(o_dx + swz(t, 2 * cc), s_g * (-wc * ec));
@@ -742,14 +871,14 @@ wkv6_backward_chunked_kernel(const __grid_constant__ CUtensorMap tm_x, const __g
                 gbar(grp);
             }
             // hand the adjoint on (and the row sums the next chunk needs, from the fp32 state: the operand tile is gone)
-            if (it + 1 < nit) {
+            if (!last) {
                 g_put(it & 1, G);
-                load_bf16_block(ck_unit + (size_t)c * 4096, S);
+                load_bf16_block(p.ckpt + slot_at(it) * 4096, S);
                 e_put(sbase + GS_EH + 4 * ((it & 1) * G_NSLAB * 64), G, S);
-                mbar_arrive(bar(GB_GREADY + (it & 1)));
-            } else if (p.dstate_in && seg == 0) {
-                store_f32_block(p.dstate_in + (size_t)unit * 4096, G);
+            } else {
+                end_of_piece(G);
             }
+            if (it + 1 < nit) mbar_arrive(bar(GB_GREADY + (it & 1)));
         } else {
             // ---- G^ as an operand; G_0 = G^ + R^^T dY handed on
             if (!GSUM) {
@@ -776,19 +905,19 @@ wkv6_backward_chunked_kernel(const __grid_constant__ CUtensorMap tm_x, const __g
                     G[n][0] = lo.x; G[n][1] = lo.y; G[n][2] = hi.x; G[n][3] = hi.y;
                 }
             }
-            if (it + 1 < nit) {
+            if (!last) {
                 g_put(it & 1, G);
                 if (!GSUM) {
                     float sb[G_NB][4];               // this chunk's start state is the next chunk's end state (bf16 copy: the operand tile)
                     ld_tile(t_sb, moff, sb);
                     e_put(sbase + GS_EH + 4 * ((it & 1) * G_NSLAB * 64), G, sb);
                 }
-                mbar_arrive(bar(GB_GREADY + (it & 1)));
             } else if (GSUM) {
                 store_f32_block(p.gsum_out + ((size_t)unit * (p.nseg - 1) + (seg - 1)) * GSUM_FLOATS + 64, G);      // the segment's dG
-            } else if (p.dstate_in && seg == 0) {
-                store_f32_block(p.dstate_in + (size_t)unit * 4096, G);
+            } else {
+                end_of_piece(G);
             }
+            if (it + 1 < nit) mbar_arrive(bar(GB_GREADY + (it & 1)));
             if (GSUM) {
                 // nothing else in the summary variant: once every lane is done with the tiles, the next chunk's copies
                 mph ^= 1;
@@ -971,7 +1100,7 @@ wkv6_backward_chunked_kernel(const __grid_constant__ CUtensorMap tm_x, const __g
                 const int tile = i / (valid * 8), rem = i % (valid * 8), t = rem >> 3, blk = rem & 7;
                 uint32_t w[4];
                 lds_v4(t_sb + tile * TILE + swz(t, blk << 4), w);
-                *reinterpret_cast<uint4*>(outs[tile] + (size_t)(row0 + (long long)c * L + t) * C + col0 + 8 * blk) = make_uint4(w[0], w[1], w[2], w[3]);
+                *reinterpret_cast<uint4*>(outs[tile] + (size_t)(row_at(it) + t) * C + col_at(it) + 8 * blk) = make_uint4(w[0], w[1], w[2], w[3]);
             }
             // every thread has read the staging tiles: the first of them takes the next chunk's start state by TMA at
             // the top of the group's next iteration, issued by one thread that would otherwise not wait for the others
@@ -979,15 +1108,22 @@ wkv6_backward_chunked_kernel(const __grid_constant__ CUtensorMap tm_x, const __g
         }
         if (gt == 0) {
             if (valid == L) {
-                const int row = (int)(row0 + (long long)c * L);
-                tma_store_2d(&tm_dr, col0, row, o_dr);
-                tma_store_2d(&tm_dk, col0, row, o_dk);
-                tma_store_2d(&tm_dv, col0, row, o_dv);
-                tma_store_2d(&tm_dx, col0, row, o_dx);
+                const int row = row_at(it), col = col_at(it);
+                tma_store_2d(&tm_dr, col, row, o_dr);
+                tma_store_2d(&tm_dk, col, row, o_dk);
+                tma_store_2d(&tm_dv, col, row, o_dv);
+                tma_store_2d(&tm_dx, col, row, o_dx);
                 bulk_commit();
             }
             if (unsafe && it + 2 < nit) { issue_loads_a(it + 2); issue_loads_b(it + 2); }      // (the other path has issued them)
+            if constexpr (BAL) {
+                if (last && pt(pc, 6) == 1) {
+                    __threadfence();                 // (the group's barrier above: every lane's part of the adjoint is written)
+                    asm volatile("st.release.gpu.global.u64 [%0], %1;" ::"l"(p.words + blockIdx.x - 1), "l"(p.nonce) : "memory");
+                }
+            }
         }
+        if (BAL && !C2 && (it + 2 >= nit || it + 2 >= pt(pc, 0))) flush_du();
     }
 
     if (PACKED && GSUM && nit == 0 && grp == 0) {
@@ -1010,7 +1146,7 @@ wkv6_backward_chunked_kernel(const __grid_constant__ CUtensorMap tm_x, const __g
     // ---- the bonus gradient of this unit: over the lanes' rows, the row groups and the two groups, in a fixed order
     if (!alive && gt == 0) sts32(abort_flag, 1u);    // (the other group's waits see it)
     if (GSUM && cx == 0 && q == 0) { stsf(gbase + GO_REDV + 4 * R0, dprod_lo); stsf(gbase + GO_REDV + 4 * R1, dprod_hi); }
-    if (!C2 && !GSUM) {
+    if (!C2 && !GSUM && !BAL) {
         // (over the four lanes of a channel; the column slabs are added below)
 #pragma unroll
         for (int d = 1; d < 4; d <<= 1)
@@ -1030,7 +1166,7 @@ wkv6_backward_chunked_kernel(const __grid_constant__ CUtensorMap tm_x, const __g
     if (GSUM && tid < 64 && !lds32(abort_flag))       // the segment's decay: the product over both groups' chunks
         p.gsum_out[((size_t)unit * (p.nseg - 1) + (seg - 1)) * GSUM_FLOATS + tid] =
             ldsf(sbase + GO_REDV + 4 * tid) * ldsf(sbase + GO_BYTES + GO_REDV + 4 * tid);
-    if (!C2 && !GSUM && tid < 64 && !lds32(abort_flag)) {
+    if (!C2 && !GSUM && !BAL && tid < 64 && !lds32(abort_flag)) {
         float s = 0.f;
 #pragma unroll
         for (int gg = 0; gg < 2; ++gg) {
@@ -1075,13 +1211,26 @@ inline int backward_split(long long units, int T, int n_sm, int* seg_chunks)
 
 // Workspace of the chunked gradient: checkpoints, bonus gradients per unit and segment, the adjoint's segment
 // summaries, the token-by-token path's scratch (one slot of 64 states per SM and group of warps).
+// Whether a dense gradient call of more units than SMs cuts units between CTAs (BParamsBal); the same rule as the forward
+// pass's (balance_pays), here too because a chunk takes longer the more SMs are at work.  Measured (us, one CTA per unit ->
+// balanced): 160 units of 32 chunks 222 -> 145, of 128 chunks 913 -> 595; not taken: 256 of 32 chunks 223 -> 231.
+inline bool backward_balance_pays(long long units, int n_chunks, int n_sm)
+{
+    if (units <= n_sm || units / n_sm - 1 > bc::BAL_MAX_ROUNDS) return false;
+    const long long rounds = (units + n_sm - 1) / n_sm, idle = rounds * n_sm - units;
+    return idle * n_chunks > 4LL * n_sm && idle * 5 > rounds * n_sm && 2LL * n_sm * n_sm * n_chunks < (1LL << 32);
+}
+// Floats of the bonus partial sums of a dense call, and of a balanced launch's hand-over blocks and words behind them.
+inline size_t backward_du_floats(long long units, int nseg, bool balanced) { return (size_t)units * (balanced ? bc::BAL_DU_SLOTS : nseg) * 64; }
+inline size_t backward_hand_floats(int n_sm, bool balanced) { return balanced ? (size_t)n_sm * 4096 + (size_t)(2 * n_sm + 3) / 4 * 4 : 0; }
 inline size_t chunked_backward_workspace_bytes(long long units, int T, int n_sm)
 {
     const size_t nck = (size_t)((T + ck::L - 1) / ck::L) + 1;
     int seg_chunks = 0;
     const int nseg = backward_split(units, T, n_sm, &seg_chunks);
-    return ((size_t)units * nck * bc::CKPT_FLOATS + (size_t)units * nseg * 64 + (size_t)units * (nseg - 1) * bc::GSUM_FLOATS +
-            (size_t)2 * n_sm * bc::FB_SLOT_FLOATS) * sizeof(float);
+    const bool bal = backward_balance_pays(units, (int)nck - 1, n_sm);
+    return ((size_t)units * nck * bc::CKPT_FLOATS + backward_du_floats(units, nseg, bal) + (size_t)units * (nseg - 1) * bc::GSUM_FLOATS +
+            backward_hand_floats(n_sm, bal) + (size_t)2 * n_sm * bc::FB_SLOT_FLOATS) * sizeof(float);
 }
 
 // The same for packed sequences: checkpoints in the packed layout, [H][total_rows / 64 + 2 S] states.
@@ -1113,7 +1262,9 @@ inline float* backward_workspace_forward_scratch(float* ws, long long units, int
     int seg_chunks = 0;
     const int nseg = backward_split(units, T, n_sm, &seg_chunks);
     *bytes = (size_t)2 * n_sm * bc::FB_SLOT_FLOATS * sizeof(float);
-    return ws + (size_t)units * nck * bc::CKPT_FLOATS + (size_t)units * nseg * 64 + (size_t)units * (nseg - 1) * bc::GSUM_FLOATS;
+    const bool bal = backward_balance_pays(units, (int)nck - 1, n_sm);
+    return ws + (size_t)units * nck * bc::CKPT_FLOATS + backward_du_floats(units, nseg, bal) + (size_t)units * (nseg - 1) * bc::GSUM_FLOATS +
+           backward_hand_floats(n_sm, bal);
 }
 
 // The part of the packed gradient's workspace that its forward pass may use for the counter and the sequence order of a
@@ -1147,6 +1298,8 @@ inline gf_status_t chunked_backward(const __nv_bfloat16* r, const __nv_bfloat16*
             cudaFuncSetAttribute(bc::wkv6_backward_chunked_kernel<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, bc::G_SMEM_ALLOC) != cudaSuccess ||
             cudaFuncSetAttribute(bc::wkv6_backward_chunked_kernel<false, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, bc::G_SMEM_ALLOC) != cudaSuccess ||
             cudaFuncSetAttribute(bc::wkv6_backward_chunked_kernel<true, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, bc::G_SMEM_ALLOC) != cudaSuccess ||
+            cudaFuncSetAttribute(bc::wkv6_backward_chunked_kernel<false, false, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, bc::G_SMEM_ALLOC) != cudaSuccess ||
+            cudaFuncSetAttribute(bc::wkv6_backward_chunked_kernel<true, false, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, bc::G_SMEM_ALLOC) != cudaSuccess ||
             cudaFuncSetAttribute(bc::wkv6_backward_chunked_kernel<false, true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, bc::G_SMEM_ALLOC) != cudaSuccess)
             return GF_ERR_CUDA;
         attr_set.set(dev);
@@ -1161,8 +1314,10 @@ inline gf_status_t chunked_backward(const __nv_bfloat16* r, const __nv_bfloat16*
     const size_t n_ckpt = cu ? (size_t)H * ckpt_slots : (size_t)units * nck;       // checkpoints: bf16 [64][64] tiles
     if (n_ckpt * 64 >= (1ull << 31)) return GF_ERR_UNSUPPORTED;                    // (32-bit TMA row coordinates)
     float* du_part = ckpt + n_ckpt * bc::CKPT_FLOATS;
-    float* gsum = du_part + (size_t)units * nalloc * 64;
-    float* fb = gsum + (size_t)units * (nalloc - 1) * bc::GSUM_FLOATS;
+    bool bal = !cu && backward_balance_pays(units, (int)nck - 1, n_sm);
+    float* gsum = du_part + (cu ? (size_t)units * nalloc * 64 : backward_du_floats(units, nseg, bal));
+    float* hand = gsum + (size_t)units * (nalloc - 1) * bc::GSUM_FLOATS;
+    float* fb = hand + (cu ? 0 : backward_hand_floats(n_sm, bal));
     const int32_t* order = nullptr;
     if (cu) {
         // packed: the sequences longest first (the order array lies between the bonus partial sums and the scratch slots)
@@ -1184,8 +1339,10 @@ inline gf_status_t chunked_backward(const __nv_bfloat16* r, const __nv_bfloat16*
     const long long C = (long long)H * 64;
     CUtensorMap tx, tr, tk, tv, tdy, tdr, tdk, tdv, tdx, tck;
     if (!ck::make_map(&tck, ckpt, (long long)n_ckpt * 64, 64, 64)) return GF_ERR_CUDA;
-    if (!ck::make_map(&tx, x, rows, C, 64) || !ck::make_map(&tr, r, rows, C, 64) || !ck::make_map(&tk, k, rows, C, 64) ||
-        !ck::make_map(&tv, v, rows, C, 64) || !ck::make_map(&tdy, dy, rows, C, 64) || !ck::make_map(&tdr, dr, rows, C, 64) ||
+    // (in a balanced launch neighbouring heads are at different places: no fetching of a neighbour's line along)
+    const CUtensorMapL2promotion pr = bal ? CU_TENSOR_MAP_L2_PROMOTION_L2_128B : CU_TENSOR_MAP_L2_PROMOTION_L2_256B;
+    if (!ck::make_map(&tx, x, rows, C, 64, pr) || !ck::make_map(&tr, r, rows, C, 64, pr) || !ck::make_map(&tk, k, rows, C, 64, pr) ||
+        !ck::make_map(&tv, v, rows, C, 64, pr) || !ck::make_map(&tdy, dy, rows, C, 64, pr) || !ck::make_map(&tdr, dr, rows, C, 64) ||
         !ck::make_map(&tdk, dk, rows, C, 64) || !ck::make_map(&tdv, dv, rows, C, 64) || !ck::make_map(&tdx, dx, rows, C, 64))
         return GF_ERR_CUDA;
     bc::BParams p{u, dstate_out, dstate_in, reinterpret_cast<const __nv_bfloat16*>(ckpt), du_part, fb, dr, dk, dv, dx, T, H, 2 * n_sm,
@@ -1198,14 +1355,34 @@ inline gf_status_t chunked_backward(const __nv_bfloat16* r, const __nv_bfloat16*
         launches->fetch_add(1, std::memory_order_relaxed);
         if (cudaGetLastError() != cudaSuccess) return GF_ERR_CUDA;
     }
-    if (cu && c2) bc::wkv6_backward_chunked_kernel<true, false, true><<<(unsigned)(units * nseg), bc::G_THREADS, bc::G_SMEM_ALLOC, st>>>(tx, tr, tk, tv, tdy, tdr, tdk, tdv, tdx, tck, pp);
+    if (bal) {
+        bc::BParamsBal pb{p, (int)units, hand, reinterpret_cast<unsigned long long*>(hand + (size_t)n_sm * 4096), launch_nonce()};
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3((unsigned)n_sm);
+        cfg.blockDim = dim3(bc::G_THREADS);
+        cfg.dynamicSmemBytes = bc::G_SMEM_ALLOC;
+        cfg.stream = st;
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeCooperative;
+        attr[0].val.cooperative = 1;
+        cfg.attrs = attr;
+        cfg.numAttrs = 1;
+        const cudaError_t e = c2 ? cudaLaunchKernelEx(&cfg, bc::wkv6_backward_chunked_kernel<true, false, false, true>, tx, tr, tk, tv, tdy, tdr, tdk, tdv, tdx, tck, pb)
+                                 : cudaLaunchKernelEx(&cfg, bc::wkv6_backward_chunked_kernel<false, false, false, true>, tx, tr, tk, tv, tdy, tdr, tdk, tdv, tdx, tck, pb);
+        if (e == cudaErrorCooperativeLaunchTooLarge) {
+            cudaGetLastError();                      // (fewer SMs to be had than the device has: one CTA per unit)
+            bal = false;
+        } else if (e != cudaSuccess) return GF_ERR_CUDA;
+    }
+    if (bal) {
+    } else if (cu && c2) bc::wkv6_backward_chunked_kernel<true, false, true><<<(unsigned)(units * nseg), bc::G_THREADS, bc::G_SMEM_ALLOC, st>>>(tx, tr, tk, tv, tdy, tdr, tdk, tdv, tdx, tck, pp);
     else if (cu) bc::wkv6_backward_chunked_kernel<false, false, true><<<(unsigned)(units * nseg), bc::G_THREADS, bc::G_SMEM_ALLOC, st>>>(tx, tr, tk, tv, tdy, tdr, tdk, tdv, tdx, tck, pp);
     else if (c2) bc::wkv6_backward_chunked_kernel<true><<<(unsigned)(units * nseg), bc::G_THREADS, bc::G_SMEM_ALLOC, st>>>(tx, tr, tk, tv, tdy, tdr, tdk, tdv, tdx, tck, p);
     else bc::wkv6_backward_chunked_kernel<false><<<(unsigned)(units * nseg), bc::G_THREADS, bc::G_SMEM_ALLOC, st>>>(tx, tr, tk, tv, tdy, tdr, tdk, tdv, tdx, tck, p);
     launches->fetch_add(1, std::memory_order_relaxed);
     if (cudaGetLastError() != cudaSuccess) return GF_ERR_CUDA;
     if (c2) return GF_OK;                            // no bonus, no bonus gradient
-    bc::wkv6_backward_chunked_du_kernel<<<(unsigned)H, 512, 0, st>>>(du_part, B, H, nseg, du);
+    bc::wkv6_backward_chunked_du_kernel<<<(unsigned)H, 512, 0, st>>>(du_part, B, H, bal ? bc::BAL_DU_SLOTS : nseg, du);
     launches->fetch_add(1, std::memory_order_relaxed);
     return cudaGetLastError() == cudaSuccess ? GF_OK : GF_ERR_CUDA;
 }

@@ -1829,7 +1829,8 @@ inline EncodeTiledFn encode_fn()
 }
 
 // [rows][C] bf16 tensor, box = box_rows rows x 64 channels (128 bytes), 128-byte swizzle
-inline bool make_map(CUtensorMap* tm, const void* base, long long rows, long long C, int box_rows)
+inline bool make_map(CUtensorMap* tm, const void* base, long long rows, long long C, int box_rows,
+                     CUtensorMapL2promotion promotion = CU_TENSOR_MAP_L2_PROMOTION_L2_256B)
 {
     EncodeTiledFn enc = encode_fn();
     if (!enc) return false;
@@ -1838,7 +1839,7 @@ inline bool make_map(CUtensorMap* tm, const void* base, long long rows, long lon
     cuuint32_t box[2] = {64, (cuuint32_t)box_rows};
     cuuint32_t estr[2] = {1, 1};
     return enc(tm, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(base), dims, strides, box, estr,
-               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, promotion,
                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 

@@ -104,3 +104,36 @@ def test_packed_training_forward_as_a_stream(c2):
                     gf.backward_varlen(i.r, i.k, i.v, i.x, i.u, dy, i.cu_seqlens, 700, i.state_in, **kw)):
         assert a is None and b is None or torch.equal(a, b)
     gf.last_device_status()
+
+
+@pytest.mark.parametrize("B,T,H", SHAPES[:3] + [(6, 200, 32)])
+@pytest.mark.parametrize("c2", [False, True])
+@pytest.mark.parametrize("x_hi,with_dstate", [(-1.0, True), (2.5, False)])
+def test_gradient_units_cut_between_ctas(B, T, H, c2, x_hi, with_dstate):
+    # each sequence on its own (few units and short: one CTA per unit) gives the same bits; the bonus gradient, summed over
+    # the batch, to fp32 rounding of its B * T terms
+    i = synth.make_dense(B, T, H, 64, "bf16", seed=B + 3 * T + H, device=DEV, state_std=0.1, x_hi=x_hi)
+    g = torch.Generator(device=DEV).manual_seed(6)
+    dy = torch.randn(i.r.shape, device=DEV, generator=g).bfloat16()
+    ds = torch.randn(i.state_in.shape, device=DEV, generator=g) if with_dstate else None
+
+    def grad(sl):
+        t = [x[sl].contiguous() for x in (i.r, i.k, i.v, i.x)]
+        kw = dict(state_in=i.state_in[sl].contiguous(), dstate_out=None if ds is None else ds[sl].contiguous(), want_dstate=with_dstate)
+        if c2:
+            return gf.backward_c2(*t, dy[sl].contiguous(), **kw)
+        return gf.backward(*t, i.u, dy[sl].contiguous(), **kw)
+
+    full = grad(slice(None))
+    du = torch.zeros_like(i.u, dtype=torch.float64)
+    for b in range(B):
+        one = grad(slice(b, b + 1))
+        for n in range(4):
+            assert torch.equal(one[n][0], full[n][b]), (b, n)
+        if with_dstate:
+            assert torch.equal(one[-1][0], full[-1][b])
+        if not c2:
+            du += one[4].double()
+    if not c2:
+        assert float((full[4].double() - du).norm() / du.norm()) < 1e-5
+    gf.last_device_status()
