@@ -48,6 +48,25 @@ def test_shapes_tails_and_ranks(B, T, D, Rd, Rw):
     print(_run(B, T, D, Rd, Rw, seed=100 + T + D))
 
 
+@pytest.mark.parametrize("rows,D", [(63, 64), (64, 64), (65, 64), (129, 64), (127, 192), (64 * 148, 192), (64 * 149 + 1, 192),
+                                    (64 * 300 - 1, 192)])
+def test_shares_of_rows_and_slices(rows, D):
+    """A CTA's share in units of 64 rows (half tiles, one CTA more or less than SMs), one slice (the second worker set has
+    none) and three (two and one)."""
+    _run(1, rows, D, 32, 64, seed=rows + D)
+
+
+def test_repeats_bit_for_bit():
+    """Two worker sets with rings of their own: no set may pass on a phase of the other's."""
+    x, xp = synth.make_block_input(4, 16384, 1024, seed=31, device=DEV)
+    w = synth.make_decay_lora(1024, 32, 64, seed=32, device=DEV)
+    run = lambda: gf.decay_logit(x, w["mu_x"], w["A_d"], w["B_d"], w["lambda_d"], w["A_w"], w["B_w"], w["lambda_w"], x_prev=xp)
+    d = run()
+    outs = [run() for _ in range(20)]
+    gf.last_device_status()
+    assert all(torch.equal(d, o) for o in outs)
+
+
 def test_without_x_prev_and_many_tiles_per_cta():
     print(_run(2, 12000, 256, 32, 64, seed=7, with_prev=False))      # 188 tiles over the persistent CTAs
 
