@@ -5,12 +5,17 @@
 // With Dc = D/16 the product does 2*Dc = 256 flops per 2-byte element of x it reads (D = 2048): it sits at
 // the crossing of the HBM and tensor rooflines, so x is read exactly once and W (D*Dc*2 bytes, L2-resident)
 // as rarely as tensor memory allows.  One persistent CTA per SM walks row tiles of MBLK*128 tokens; a tile's
-// MBLK x NB accumulators (128 rows x 64 fp32 columns each, NB = ceil(Dc/64)) take, up to Dc = 128, at most 256
+// MBLK accumulators (128 rows x NB*64 fp32 columns each, NB = ceil(Dc/64)) take, up to Dc = 128, at most 256
 // of the 512 columns of tensor memory, so there are two sets: the products of the next tile run while the
 // epilogue drains this one (wider outputs fill all 512 columns with one set).  Every 64-row slice of W that
-// enters shared memory serves MBLK*128 tokens.
+// enters shared memory serves MBLK*128 tokens, and one instruction multiplies 128 of them by all NB*64 columns, so that
+// the x operand is read from shared memory once (D = 2048, Dc = 128: 65536 rows 53.3 -> 50.6 us, 5.3 TB/s of x;
+// D = 4096, Dc = 256: 148 -> 118; 658 rows 14.8 -> 12.1).
+// What bounds a call: many rows, HBM (262144 rows 175 us, 6.5 TB/s); few rows, the 64 bytes per cycle that one SM gets
+// from L2, so a short call spreads a tile over a cluster of SMs (SPLIT): each takes a share of the input channels,
+// leaves its fp32 sums in shared memory, and adds up a share of the rows over the cluster in a fixed order.
 //   warp 0      TMA producer: per 64 input channels, 2*MBLK tiles of x and NB tiles of W into a ring stage
-//   warp 1      tensor-memory allocation; an elected lane issues the MBLK*NB*4 tcgen05.mma (128x64x16) of a stage
+//   warp 1      tensor-memory allocation; an elected lane issues the MBLK*4 tcgen05.mma (128 x NB*64 x 16) of a stage
 //   warps 2-5   epilogue: the 32 accumulator rows of the own sub-partition -> bf16 slab -> TMA store (32-row
 //               boxes; rows past the end of the tensor are clipped by the store, rows read past it are zero)
 // Operands are 128-byte swizzled as TMA delivers them: two stacked 64-token x tiles form the 128-row K-major
@@ -33,12 +38,17 @@ constexpr int KC_OFF_MISC = KC_OFF_SLAB + 4 * 4096;   // abort word, tensor-memo
 constexpr int KC_SMEM = KC_OFF_MISC + 256 + 1024;     // + slack for manual 1024-byte alignment
 enum { KC_FULL = 0, KC_EMPTY = KC_MAX_NS, KC_ACC_FULL = 2 * KC_MAX_NS, KC_ACC_EMPTY = KC_ACC_FULL + 2, KC_BAR_COUNT = KC_ACC_EMPTY + 2 };
 static_assert(16 + 8 * KC_BAR_COUNT <= 256, "barrier block");
-// instruction descriptor: fp32 accumulator, bf16 A (K-major) and B (MN-major), M = 128, N = 64
-constexpr uint32_t KC_IDESC = (1u << 4) | (1u << 7) | (1u << 10) | (1u << 16) | ((64u >> 3) << 17) | ((128u >> 4) << 24);
+// instruction descriptor: fp32 accumulator, bf16 A (K-major) and B (MN-major), M = 128, N = n
+constexpr uint32_t kc_idesc(int n) { return (1u << 4) | (1u << 7) | (1u << 10) | (1u << 16) | ((uint32_t)(n >> 3) << 17) | ((128u >> 4) << 24); }
+// B operand of several W tiles side by side: the leading byte offset is the step between 64-column blocks
+__device__ __forceinline__ uint64_t kc_desc_w(uint32_t saddr) { return smem_desc(saddr) + ((uint64_t)((TILE >> 4) - 1) << 16); }
 
 struct KcParams {
+    __nv_bfloat16* c;
     long long rows;
+    int cols;
     int ksteps;                                       // ceil(D / 64)
+    int shares;                                       // an equal share of the rows per CTA instead of every gridDim-th tile
 };
 
 // One accumulator row per lane: 32 consecutive fp32 columns of the lane's row in this warp's sub-partition.
@@ -56,7 +66,39 @@ __device__ __forceinline__ void tmem_ld_row32(uint32_t taddr, uint32_t (&v)[32])
         : "r"(taddr) : "memory");
 }
 
-template <int MBLK, int NB>
+// A 16-byte load from the shared memory of CTA `rank` of the cluster, at the address that `saddr` has in this CTA.
+__device__ __forceinline__ float4 ld_cluster(uint32_t saddr, uint32_t rank)
+{
+    float4 v;
+    asm volatile("{\n\t.reg .b32 a;\n\tmapa.shared::cluster.u32 a, %4, %5;\n\t"
+                 "ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [a];\n\t}"
+                 : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(saddr), "r"(rank) : "memory");
+    return v;
+}
+__device__ __forceinline__ void cluster_sync()
+{
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
+// Adds this CTA's share of a tile's rows over the cluster's CS sets of partial sums; all loads of a thread are in flight together.
+template <int CS, int NB>
+__device__ __forceinline__ void add_up(uint32_t sums, uint32_t rank, long long r_first, int tid, const KcParams& p)
+{
+    constexpr int SHARE = 128 / CS;
+    for (int i = tid; i < SHARE * 16 * NB; i += KC_THREADS) {
+        const int row = SHARE * (int)rank + i / (16 * NB), col = i % (16 * NB) * 4;
+        const uint32_t a = sums + (row * (64 * NB + 4) + col) * 4;
+        float4 v[CS];
+#pragma unroll
+        for (int q = 0; q < CS; ++q) v[q] = ld_cluster(a, q);
+#pragma unroll
+        for (int q = 1; q < CS; ++q) { v[0].x += v[q].x; v[0].y += v[q].y; v[0].z += v[q].z; v[0].w += v[q].w; }
+        if (r_first + row < p.rows && col < p.cols)
+            *reinterpret_cast<uint2*>(p.c + (r_first + row) * p.cols + col) = make_uint2(pack_bf16(v[0].x, v[0].y), pack_bf16(v[0].z, v[0].w));
+    }
+}
+
+template <int MBLK, int NB, bool SPLIT>
 __global__ void __launch_bounds__(KC_THREADS, 1)
 key_compress_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ CUtensorMap tm_w,
                     const __grid_constant__ CUtensorMap tm_c32, const KcParams p)
@@ -75,9 +117,31 @@ key_compress_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_const
     const uint32_t abort_flag = sbase + KC_OFF_MISC;
     auto bar = [&](int i) { return sbase + KC_OFF_MISC + 16 + 8 * i; };
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const long long tile_rows = (long long)MBLK * 128;
-    const long long n_tiles = (p.rows + tile_rows - 1) / tile_rows;
+    static_assert(!SPLIT || MBLK == 1, "one block of rows per cluster");
+    constexpr int PART_LD = 64 * NB + 4;             // SPLIT: row of partial sums in shared memory, fp32
+    static_assert(!SPLIT || 128 * PART_LD * 4 <= KC_RING, "partial sums");
+    // This CTA's rows [r_first, r_end), r_step apart, and its input channels [k_first, k_end) in units of 64
+    const long long n_half = (p.rows + 63) / 64;
+    long long r_first, r_end = n_half * 64, r_step = (long long)gridDim.x * MBLK * 128;
+    int k_first = 0, k_end = p.ksteps;
+    uint32_t c_rank = 0, c_size = 1;
+    if constexpr (SPLIT) {
+        asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(c_rank));
+        asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(c_size));
+        r_first = (long long)(blockIdx.x / c_size) * 128;            // one tile
+        k_first = p.ksteps * (int)c_rank / (int)c_size;
+        k_end = p.ksteps * (int)(c_rank + 1) / (int)c_size;
+    } else if (p.shares) {
+        r_first = n_half * blockIdx.x / gridDim.x * 64;
+        r_end = n_half * (blockIdx.x + 1) / gridDim.x * 64;
+        r_step = MBLK * 128;
+    } else {
+        r_first = (long long)blockIdx.x * MBLK * 128;
+    }
 
+    // Launched with programmatic stream serialisation: the set-up below overlaps the end of the kernel ahead, and no
+    // global memory is touched before that kernel has completed and flushed (back-to-back calls: 0.5 to 1 us each).
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     if (tid == 0) {
         for (int i = 0; i < KC_NS; ++i) {
             mbar_init(bar(KC_FULL + i), 1);
@@ -98,20 +162,22 @@ key_compress_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_const
     tc_fence_after();
     const uint32_t tmem = lds32(sbase + KC_OFF_MISC + 8);
 
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     if (warp == 0) {
         // ============================== TMA producer ==============================
         int it = 0, issued = 0;
         bool alive = true;
-        for (long long t = blockIdx.x; t < n_tiles && alive; t += gridDim.x) {
-            const int row0 = (int)(t * tile_rows);
-            for (int ks = 0; ks < p.ksteps; ++ks, ++it) {
+        for (long long r = r_first; r < r_end && alive; r += r_step) {
+            const int row0 = (int)r, nx = (int)min(2LL * MBLK, (r_end - r) / 64);       // x tiles
+            for (int ks = k_first; ks < k_end; ++ks, ++it) {
                 const int s = it % KC_NS;
                 if (it >= KC_NS && !mbar_wait_warp(bar(KC_EMPTY + s), ((it / KC_NS) + 1) & 1, abort_flag)) { alive = false; break; }
                 const uint32_t dst = sbase + s * KC_STAGE;
                 if (elect_one()) {
-                    mbar_expect_tx(bar(KC_FULL + s), (2 * MBLK + NB) * TILE);
+                    mbar_expect_tx(bar(KC_FULL + s), (nx + NB) * TILE);
 #pragma unroll
-                    for (int mb = 0; mb < 2 * MBLK; ++mb) tma_load_2d(dst + mb * TILE, &tm_x, ks * 64, row0 + 64 * mb, bar(KC_FULL + s));
+                    for (int mb = 0; mb < 2 * MBLK; ++mb)
+                        if (mb < nx) tma_load_2d(dst + mb * TILE, &tm_x, ks * 64, row0 + 64 * mb, bar(KC_FULL + s));
 #pragma unroll
                     for (int nb = 0; nb < NB; ++nb) tma_load_2d(dst + (2 * MBLK + nb) * TILE, &tm_w, nb * 64, ks * 64, bar(KC_FULL + s));
                 }
@@ -126,12 +192,13 @@ key_compress_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_const
         // ============================== MMA issuer ==============================
         int it = 0, ti = 0;
         bool alive = true;
-        for (long long t = blockIdx.x; t < n_tiles && alive; t += gridDim.x, ++ti) {
+        for (long long r = r_first; r < r_end && alive; r += r_step, ++ti) {
+            const int nx = (int)min(2LL * MBLK, (r_end - r) / 64);
             const int ab = NSETS == 2 ? (ti & 1) : 0, use = NSETS == 2 ? (ti >> 1) : ti;   // accumulator set and its use count
             // the epilogue has read this set's previous tile out of tensor memory
             if (use >= 1 && !mbar_wait_warp(bar(KC_ACC_EMPTY + ab), (use + 1) & 1, abort_flag)) break;
             tc_fence_after();
-            for (int ks = 0; ks < p.ksteps; ++ks, ++it) {
+            for (int ks = k_first; ks < k_end; ++ks, ++it) {
                 const int s = it % KC_NS;
                 if (!mbar_wait_warp(bar(KC_FULL + s), (it / KC_NS) & 1, abort_flag)) { alive = false; break; }
                 tc_fence_after();
@@ -139,34 +206,52 @@ key_compress_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_const
                     const uint32_t st = sbase + s * KC_STAGE;
 #pragma unroll
                     for (int mb = 0; mb < MBLK; ++mb) {
+                        if (2 * mb >= nx) break;
                         const uint64_t da = smem_desc(st + 2 * mb * TILE);       // 128 rows: two stacked x tiles
+                        const uint64_t db = kc_desc_w(st + 2 * MBLK * TILE);
 #pragma unroll
-                        for (int nb = 0; nb < NB; ++nb) {
-                            const uint64_t db = smem_desc(st + (2 * MBLK + nb) * TILE);
-#pragma unroll
-                            for (int kk = 0; kk < 4; ++kk)
-                                tc_mma(tmem + ACC_COLS * ab + 64 * (mb * NB + nb), da + (uint64_t)(2 * kk), db + (uint64_t)(128 * kk),
-                                       KC_IDESC, (ks > 0 || kk > 0) ? 1u : 0u);
-                        }
+                        for (int kk = 0; kk < 4; ++kk)
+                            tc_mma(tmem + ACC_COLS * ab + 64 * NB * mb, da + (uint64_t)(2 * kk), db + (uint64_t)(128 * kk),
+                                   kc_idesc(64 * NB), (ks > k_first || kk > 0) ? 1u : 0u);
                     }
                     tc_commit(bar(KC_EMPTY + s));                    // the stage is free once these products are done
-                    if (ks == p.ksteps - 1) tc_commit(bar(KC_ACC_FULL + ab));
+                    if (ks == k_end - 1) tc_commit(bar(KC_ACC_FULL + ab));
                 }
                 __syncwarp();
             }
         }
+    } else if constexpr (SPLIT) {
+        // ============================== partial sums to shared memory ==============================
+        // The ring is free: every slice that was loaded has been multiplied.
+        const int sp = warp & 3;
+        if (mbar_wait(bar(KC_ACC_FULL), 0, abort_flag)) {
+            __syncwarp();
+            tc_fence_after();
+#pragma unroll
+            for (int half = 0; half < 2 * NB; ++half) {
+                uint32_t v[32];
+                tmem_ld_row32(tmem + ((uint32_t)(32 * sp) << 16) + 32 * half, v);
+#pragma unroll
+                for (int q = 0; q < 8; ++q)
+                    asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};"
+                                 ::"r"(sbase + ((32 * sp + lane) * PART_LD + 32 * half + 4 * q) * 4),
+                                   "r"(v[4 * q]), "r"(v[4 * q + 1]), "r"(v[4 * q + 2]), "r"(v[4 * q + 3]) : "memory");
+            }
+        }
+        __syncwarp();
     } else {
         // ============================== epilogue warps ==============================
         const int sp = warp & 3;                     // tensor-memory sub-partition: accumulator rows 32*sp .. 32*sp+31
         const uint32_t slab = sbase + KC_OFF_SLAB + (warp - 2) * 4096;
         int ti = 0;
-        for (long long t = blockIdx.x; t < n_tiles; t += gridDim.x, ++ti) {
+        for (long long r = r_first; r < r_end; r += r_step, ++ti) {
             const int ab = NSETS == 2 ? (ti & 1) : 0, use = NSETS == 2 ? (ti >> 1) : ti;
             if (!mbar_wait(bar(KC_ACC_FULL + ab), use & 1, abort_flag)) break;
             tc_fence_after();
-            const long long row0 = t * tile_rows;
 #pragma unroll
             for (int mb = 0; mb < MBLK; ++mb) {
+                const long long grow = r + 128 * mb + 32 * sp;
+                if (grow >= r_end) break;
 #pragma unroll
                 for (int nb = 0; nb < NB; ++nb) {
                     const uint32_t ta = tmem + ((uint32_t)(32 * sp) << 16) + ACC_COLS * ab + 64 * (mb * NB + nb);
@@ -188,7 +273,6 @@ key_compress_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_const
                     }
                     fence_proxy_async();
                     __syncwarp();
-                    const long long grow = row0 + 128 * mb + 32 * sp;
                     if (lane == 0 && grow < p.rows) {
                         tma_store_2d(&tm_c32, nb * 64, (int)grow, slab);
                         bulk_commit();
@@ -208,6 +292,16 @@ key_compress_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_const
         tc_fence_after();
         tmem_dealloc(tmem, 512);
     }
+    if constexpr (SPLIT) {
+        // Each CTA adds up its share of the tile's rows over the cluster, in the order of the channels.
+        __syncwarp();
+        cluster_sync();
+        if (c_size == 8) add_up<8, NB>(sbase, c_rank, r_first, tid, p);
+        else if (c_size == 4) add_up<4, NB>(sbase, c_rank, r_first, tid, p);
+        else add_up<2, NB>(sbase, c_rank, r_first, tid, p);
+        __syncwarp();
+        cluster_sync();                              // no CTA leaves while another reads its sums
+    }
 }
 
 }  // namespace kc
@@ -222,43 +316,57 @@ inline gf_status_t key_compress(const __nv_bfloat16* x, const __nv_bfloat16* w, 
     const int n_sm = sm_count();
     const int dev = current_device();
     if (n_sm <= 0 || dev < 0) return GF_ERR_CUDA;
+    using Kernel = void (*)(CUtensorMap, CUtensorMap, CUtensorMap, kc::KcParams);
+    static const Kernel kernels[3][4] = {
+        {kc::key_compress_kernel<1, 1, true>, kc::key_compress_kernel<1, 2, true>, kc::key_compress_kernel<1, 3, true>, kc::key_compress_kernel<1, 4, true>},
+        {kc::key_compress_kernel<1, 1, false>, kc::key_compress_kernel<1, 2, false>, kc::key_compress_kernel<1, 3, false>, kc::key_compress_kernel<1, 4, false>},
+        {kc::key_compress_kernel<2, 1, false>, kc::key_compress_kernel<2, 2, false>, kc::key_compress_kernel<2, 3, false>, kc::key_compress_kernel<2, 4, false>}};
     static PerDeviceFlag attr_set;
     if (!attr_set.is_set(dev)) {
-        if (cudaFuncSetAttribute(kc::key_compress_kernel<1, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, kc::KC_SMEM) != cudaSuccess ||
-            cudaFuncSetAttribute(kc::key_compress_kernel<1, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, kc::KC_SMEM) != cudaSuccess ||
-            cudaFuncSetAttribute(kc::key_compress_kernel<2, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, kc::KC_SMEM) != cudaSuccess ||
-            cudaFuncSetAttribute(kc::key_compress_kernel<2, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, kc::KC_SMEM) != cudaSuccess ||
-            cudaFuncSetAttribute(kc::key_compress_kernel<1, 3>, cudaFuncAttributeMaxDynamicSharedMemorySize, kc::KC_SMEM) != cudaSuccess ||
-            cudaFuncSetAttribute(kc::key_compress_kernel<1, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, kc::KC_SMEM) != cudaSuccess ||
-            cudaFuncSetAttribute(kc::key_compress_kernel<2, 3>, cudaFuncAttributeMaxDynamicSharedMemorySize, kc::KC_SMEM) != cudaSuccess ||
-            cudaFuncSetAttribute(kc::key_compress_kernel<2, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, kc::KC_SMEM) != cudaSuccess)
-            return GF_ERR_CUDA;
+        for (const auto& row : kernels)
+            for (const Kernel k : row)
+                if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kc::KC_SMEM) != cudaSuccess) return GF_ERR_CUDA;
         attr_set.set(dev);
     }
     CUtensorMap tx, tw, tc;
     if (!ck::make_map(&tx, x, rows, D, 64) || !ck::make_map(&tw, w, D, Dc, 64) || !ck::make_map(&tc, c, rows, Dc, 32)) return GF_ERR_CUDA;
-    // 256-row tiles halve the re-reads of W but need enough rows to give every SM a tile
-    const int nb = (Dc + 63) / 64, mblk = rows >= 256LL * n_sm ? 2 : 1;
+    kc::KcParams p{c, rows, Dc, (D + 63) / 64, 0};
+    const int nb = (Dc + 63) / 64;
+    // 256-row tiles halve the re-reads of W but need more than 128 rows per SM.
+    const int mblk = rows > 128LL * n_sm ? 2 : 1;
     const long long n_tiles = (rows + 128LL * mblk - 1) / (128LL * mblk);
-    const unsigned grid = (unsigned)(n_tiles < n_sm ? n_tiles : n_sm);
-    kc::KcParams p{rows, (D + 63) / 64};
-    if (mblk == 2) {
-        switch (nb) {
-        case 1: kc::key_compress_kernel<2, 1><<<grid, kc::KC_THREADS, kc::KC_SMEM, st>>>(tx, tw, tc, p); break;
-        case 2: kc::key_compress_kernel<2, 2><<<grid, kc::KC_THREADS, kc::KC_SMEM, st>>>(tx, tw, tc, p); break;
-        case 3: kc::key_compress_kernel<2, 3><<<grid, kc::KC_THREADS, kc::KC_SMEM, st>>>(tx, tw, tc, p); break;
-        default: kc::key_compress_kernel<2, 4><<<grid, kc::KC_THREADS, kc::KC_SMEM, st>>>(tx, tw, tc, p); break;
-        }
-    } else {
-        switch (nb) {
-        case 1: kc::key_compress_kernel<1, 1><<<grid, kc::KC_THREADS, kc::KC_SMEM, st>>>(tx, tw, tc, p); break;
-        case 2: kc::key_compress_kernel<1, 2><<<grid, kc::KC_THREADS, kc::KC_SMEM, st>>>(tx, tw, tc, p); break;
-        case 3: kc::key_compress_kernel<1, 3><<<grid, kc::KC_THREADS, kc::KC_SMEM, st>>>(tx, tw, tc, p); break;
-        default: kc::key_compress_kernel<1, 4><<<grid, kc::KC_THREADS, kc::KC_SMEM, st>>>(tx, tw, tc, p); break;
-        }
+    // Few tiles: clusters of up to 8 SMs per tile with at least two slices of the channels for each.  Clusters must lie
+    // within one GPC, so not every SM finds a place in one (14 clusters of 8 run at once on 148 SMs, 16 do not); four
+    // fifths of the SMs do.  D = 2048, Dc = 128, us, whole tiles -> clusters of 8: 658 rows 12.1 -> 6.2, 1792 rows 12.2 -> 6.9
+    // (of 4: 7.2); of 4: 2500 rows 12.3 -> 7.4; of 2: 5000 rows 12.4 -> 10.2.  Past the limit: 2000 rows in 16 clusters of 8
+    // 12.4 (of 4: 7.1), 4700 rows in 37 clusters of 4 14.1 (whole 12.5).
+    int split = 1;
+    while (split < 8 && n_tiles * split * 2 * 5 <= n_sm * 4LL && p.ksteps >= 4 * split) split *= 2;
+    long long grid = n_tiles < n_sm ? n_tiles * split : n_sm;
+    // Whole tiles leave more than a fifth of the last round idle: equal shares of the rows, in units of 64, instead (us at
+    // D = 2048, Dc = 128: 20000 rows 27.9 -> 21.0, 30000 rows 31.2 -> 26.5, 40000 rows 45.0 -> 40.5).  Otherwise whole tiles: a CTA
+    // with rows left over after its last whole tile reads all of W once more for them (262144 rows 175.5, in shares 177.7).
+    const long long slots = (n_tiles + n_sm - 1) / n_sm * n_sm;
+    if (mblk == 2 && (slots - n_tiles) * 5 > slots) {
+        p.shares = 1;
+        grid = n_sm;
     }
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)grid);
+    cfg.blockDim = dim3(kc::KC_THREADS);
+    cfg.dynamicSmemBytes = kc::KC_SMEM;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[2];
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = (unsigned)split;
+    attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = split > 1 ? 2 : 1;
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, kernels[split > 1 ? 0 : mblk][nb - 1], tx, tw, tc, p);
     launches->fetch_add(1, std::memory_order_relaxed);
-    return cudaGetLastError() == cudaSuccess ? GF_OK : GF_ERR_CUDA;
+    return e == cudaSuccess ? GF_OK : GF_ERR_CUDA;
 }
 
 }  // namespace gf

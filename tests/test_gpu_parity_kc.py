@@ -84,3 +84,40 @@ def test_benchmark_size_on_sampled_rows():
     assert np.isfinite(c.float().cpu().numpy()).all()
     compare(c[idx.to(DEV)], ref, "65536 rows, sampled")
     assert (np.abs(got - ref) <= 2.0 ** -8 * np.abs(ref) + 1e-3).all()
+
+
+@pytest.mark.parametrize("D,Dc", [(136, 24), (512, 128), (1536, 192), (2048, 256)])
+def test_row_counts_where_the_division_between_sms_changes(D, Dc):
+    """Clusters of 8, 4 and 2 SMs per 128-row tile, whole tiles, equal shares of 64-row units, whole 256-row tiles: the last
+    row count of each and the first of the next.  (Few channels end the doubling of the cluster earlier.)"""
+    n_sm = torch.cuda.get_device_properties(0).multi_processor_count
+    g = torch.Generator().manual_seed(23)
+    w = (torch.randn(D, Dc, generator=g) / D ** 0.5).bfloat16()
+    x = torch.randn(256 * n_sm + 1, D, generator=g).bfloat16()
+    xd, wd = x.to(DEV), w.to(DEV)
+    edges = [128 * (n_sm * 4 // (5 * s)) for s in (8, 4, 2)] + [128 * n_sm, 256 * (n_sm * 4 // 5), 256 * n_sm]
+    for rows in [r + d for r in edges for d in (-64, 0, 1)]:
+        if rows > x.shape[0]:
+            continue
+        c = torch.full((rows + 1, Dc), 777.0, dtype=torch.bfloat16, device=DEV)
+        gf.key_compress(xd[:rows], wd, out=c[:rows])
+        gf.last_device_status()
+        assert torch.all(c[rows] == 777.0)
+        idx = torch.cat([torch.randint(0, rows, (60,), generator=g), torch.tensor([0, 63, 64, rows // 2, rows - 65, rows - 64, rows - 1])])
+        compare(c[idx.to(DEV)], orc.key_compress(x[idx], w), f"rows {rows} D {D} Dc {Dc}, sampled")
+        assert torch.isfinite(c.float()).all()
+
+
+@pytest.mark.parametrize("rows", [300, 9000, 40000])
+def test_a_call_sees_the_result_of_the_one_before(rows):
+    """Calls back to back on one stream, each reading what the one before wrote: the same as with a synchronisation between."""
+    x, w = draw(rows, 256, 256, seed=rows)
+    x, w = x.to(DEV), w.to(DEV)
+    a, b = x, x
+    for _ in range(8):
+        a = gf.key_compress(a, w)
+    for _ in range(8):
+        b = gf.key_compress(b, w)
+        torch.cuda.synchronize()
+    gf.last_device_status()
+    assert torch.equal(a, b)
