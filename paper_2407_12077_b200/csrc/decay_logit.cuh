@@ -171,6 +171,7 @@ decay_logit_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_consta
     // this CTA's rows, in units of 64: tiles of 128, the last of 64 if the number is odd
     const long long n_half = (p.rows + 63) / 64, r_first = n_half * blockIdx.x / gridDim.x * 64, r_end = n_half * (blockIdx.x + 1) / gridDim.x * 64;
     const int S = p.nslices;
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 
     if (tid == 0) {
         for (int i = 0; i < DL_NSET * DL_NSX; ++i) {
@@ -202,6 +203,7 @@ decay_logit_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_consta
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = lds32(sbase + DL_OFF_MISC + 8);
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     // ring positions: the set's n-th slice over all passes and tiles
     auto xslot = [&](int set, int n) { return set * DL_NSX + n % DL_NSX; };
     auto wslot = [&](int set, int n) { return set * DL_NSW + n % DL_NSW; };
@@ -620,9 +622,9 @@ inline gf_status_t decay_logit(const __nv_bfloat16* x, const __nv_bfloat16* x_pr
     const long long n_half = (rows + 63) / 64;
     const int n_sm = sm_count();
     const unsigned grid = (unsigned)(n_half < n_sm ? n_half : n_sm);
-    dl::decay_logit_kernel<<<grid, dl::DL_THREADS, dl::DL_SMEM, st>>>(tx, tx1, tad, tbd, taw, tbw, td, p);
+    const cudaError_t e = launch_pdl(dl::decay_logit_kernel, grid, dl::DL_THREADS, dl::DL_SMEM, st, tx, tx1, tad, tbd, taw, tbw, td, p);
     launches->fetch_add(1, std::memory_order_relaxed);
-    return cudaGetLastError() == cudaSuccess ? GF_OK : GF_ERR_CUDA;
+    return e == cudaSuccess ? GF_OK : GF_ERR_CUDA;
 }
 
 }  // namespace gf

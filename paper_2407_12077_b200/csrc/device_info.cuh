@@ -5,6 +5,7 @@
 #include <cuda_runtime.h>
 
 #include <atomic>
+#include <utility>
 
 namespace gf {
 
@@ -39,5 +40,25 @@ struct PerDeviceFlag {
     bool is_set(int dev) const { return done[dev].load(std::memory_order_acquire); }
     void set(int dev) { done[dev].store(true, std::memory_order_release); }
 };
+
+// Launches with programmatic stream serialisation: the grid may be scheduled while the kernel ahead of it in the stream drains
+// (from the moment all of that kernel's CTAs have executed griddepcontrol.launch_dependents or left), sets itself up meanwhile, and
+// holds at its griddepcontrol.wait, which a kernel launched this way executes before its first access to global memory, until
+// that kernel has completed and flushed.
+template <typename... Params, typename... Args>
+inline cudaError_t launch_pdl(void (*kernel)(Params...), unsigned grid, unsigned block, size_t smem, cudaStream_t st, Args&&... args)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(block);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
+}
 
 }  // namespace gf

@@ -132,6 +132,7 @@ layernorm_heads_kernel(const IO* __restrict__ y, const float* __restrict__ gamma
     __shared__ float cnt[MAX_WARPS];                // channels that each warp holds
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int team = warp / W, wt = warp % W, tl = wt * 32 + lane;
+    asm volatile("griddepcontrol.launch_dependents;\n\tgriddepcontrol.wait;" ::: "memory");
 
     for (int idx = tid; idx < VPL * 2 * TL; idx += THREADS) {
         const int j = idx / (2 * TL), half = (idx / TL) & 1, l = idx % TL;
@@ -273,8 +274,7 @@ inline cudaError_t launch(const IO* y, const float* gamma, const float* beta, fl
     }
     const long long groups = (rows + (long long)R * TEAMS - 1) / ((long long)R * TEAMS);
     const unsigned grid = (unsigned)(groups < n_sm ? groups : n_sm);      // one resident CTA per SM walks the rows
-    layernorm_heads_kernel<IO, VPL, W><<<grid, cta_threads<IO>(), SMEM, st>>>(y, gamma, beta, eps, out, rows, D);
-    return cudaGetLastError();
+    return launch_pdl(layernorm_heads_kernel<IO, VPL, W>, grid, cta_threads<IO>(), SMEM, st, y, gamma, beta, eps, out, rows, D);
 }
 
 }  // namespace ln

@@ -89,17 +89,7 @@ template <typename IO, bool C2>
 inline cudaError_t launch_step(unsigned grid, cudaStream_t st, const IO* r, const IO* k, const IO* v, const IO* x, const float* u,
                                const float* state_in, float* state_out, IO* y, int H, const IO* u2)
 {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(grid);
-    cfg.blockDim = dim3(ST_THREADS);
-    cfg.dynamicSmemBytes = 0;
-    cfg.stream = st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, wkv6_step_kernel<IO, C2>, r, k, v, x, u, state_in, state_out, y, H, u2);
+    return launch_pdl(wkv6_step_kernel<IO, C2>, grid, ST_THREADS, 0, st, r, k, v, x, u, state_in, state_out, y, H, u2);
 }
 
 }  // namespace gf
