@@ -115,6 +115,15 @@ __device__ __forceinline__ void sts128(uint32_t a, uint4 v)
 {
     asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(a), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w) : "memory");
 }
+// (ax + x, ay + y) rounded to a bf16 pair, the two sums in one instruction (8680 tokens x 768: 19.9 -> 19.65 us, 16982 x 1280:
+// 31.4 -> 31.05)
+__device__ __forceinline__ uint32_t pack_sum(float ax, float ay, uint32_t x, uint32_t y)
+{
+    uint32_t r;
+    asm("{\n\t.reg .b64 a, b;\n\t.reg .b32 lo, hi;\n\tmov.b64 a, {%1, %2};\n\tmov.b64 b, {%3, %4};\n\tadd.rn.f32x2 a, a, b;\n\t"
+        "mov.b64 {lo, hi}, a;\n\tcvt.rn.bf16x2.f32 %0, hi, lo;\n\t}" : "=r"(r) : "f"(ax), "f"(ay), "r"(x), "r"(y));
+    return r;
+}
 __device__ __forceinline__ float tanh_fast(float v)
 {
     float y;
@@ -458,8 +467,8 @@ decay_logit_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_consta
 #pragma unroll
                             for (int q = 0; q < 8; ++q) {
                                 const float4 v4 = ldsf4(stage + DL_OFF_VEC + 128 * hf + 16 * q);
-                                mixw[2 * q] = pack_bf16(v4.x + __uint_as_float(l[4 * q]), v4.y + __uint_as_float(l[4 * q + 1]));
-                                mixw[2 * q + 1] = pack_bf16(v4.z + __uint_as_float(l[4 * q + 2]), v4.w + __uint_as_float(l[4 * q + 3]));
+                                mixw[2 * q] = pack_sum(v4.x, v4.y, l[4 * q], l[4 * q + 1]);
+                                mixw[2 * q + 1] = pack_sum(v4.z, v4.w, l[4 * q + 2], l[4 * q + 3]);
                             }
                         } else {
 #pragma unroll
@@ -550,10 +559,8 @@ decay_logit_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_consta
                     for (int q = 0; q < 4; ++q) {
                         const float4 la = ldsf4(stage + DL_OFF_VEC + 128 * hf + 32 * q), lb = ldsf4(stage + DL_OFF_VEC + 128 * hf + 32 * q + 16);
                         sts128(slab0 + swz(lane, (4 * hf + q) << 4),
-                               make_uint4(pack_bf16(__uint_as_float(v[8 * q]) + la.x, __uint_as_float(v[8 * q + 1]) + la.y),
-                                          pack_bf16(__uint_as_float(v[8 * q + 2]) + la.z, __uint_as_float(v[8 * q + 3]) + la.w),
-                                          pack_bf16(__uint_as_float(v[8 * q + 4]) + lb.x, __uint_as_float(v[8 * q + 5]) + lb.y),
-                                          pack_bf16(__uint_as_float(v[8 * q + 6]) + lb.z, __uint_as_float(v[8 * q + 7]) + lb.w)));
+                               make_uint4(pack_sum(la.x, la.y, v[8 * q], v[8 * q + 1]), pack_sum(la.z, la.w, v[8 * q + 2], v[8 * q + 3]),
+                                          pack_sum(lb.x, lb.y, v[8 * q + 4], v[8 * q + 5]), pack_sum(lb.z, lb.w, v[8 * q + 6], v[8 * q + 7])));
                     }
                 }
                 __syncwarp();
