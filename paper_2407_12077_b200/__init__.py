@@ -172,6 +172,11 @@ def _dev(t: torch.Tensor | None, name: str, dtype=None, shape=None):
     return t.data_ptr()
 
 
+def _new_states(n, H, N, device) -> torch.Tensor:
+    """Uninitialised [n, H, N, N] fp32 states (empty_strided takes half the host time of empty: 1.4 us against 2.8)."""
+    return torch.empty_strided((n, H, N, N), (H * N * N, N * N, N, 1), dtype=torch.float32, device=device)
+
+
 def _suffix(dtype) -> str:
     if dtype == torch.bfloat16:
         return ""
@@ -243,16 +248,24 @@ def prefill(r, k, v, x, u, state_in=None, state_out=None, y=None, stream=None, w
     both are allocated here unless passed in (state_out may be state_in).  split=False unregisters
     the scratch workspace first, so that a call with few (b,h) units runs as a single launch."""
     lib = load_library()
-    B, T, H, N = r.shape
-    sfx = _suffix(r.dtype)
+    shape = r.shape
+    B, T, H, N = shape
+    dt = r.dtype
+    sfx = _suffix(dt)
     if y is None:
         y = torch.empty_like(r)
+        y_ptr = y.data_ptr()
+    else:
+        y_ptr = _dev(y, "y", dt, shape)
     if state_out is None and want_state:
-        state_out = torch.empty((B, H, N, N), device=r.device, dtype=torch.float32)
-    args = [_dev(r, "r", shape=(B, T, H, N)), _dev(k, "k", r.dtype, r.shape), _dev(v, "v", r.dtype, r.shape),
-            _dev(x, "x", r.dtype, r.shape), _dev(u, "u", torch.float32, (H, N)),
+        state_out = _new_states(B, H, N, r.device)
+        s_ptr = state_out.data_ptr()
+    else:
+        s_ptr = _dev(state_out, "state_out", torch.float32, (B, H, N, N))
+    args = [_dev(r, "r", shape=shape), _dev(k, "k", dt, shape), _dev(v, "v", dt, shape),
+            _dev(x, "x", dt, shape), _dev(u, "u", torch.float32, (H, N)),
             _dev(state_in, "state_in", torch.float32, (B, H, N, N)),
-            _dev(state_out, "state_out", torch.float32, (B, H, N, N)), _dev(y, "y", r.dtype, r.shape)]
+            s_ptr, y_ptr]
     with _on(r):
         if sfx == "" and split:
             _ensure_workspace(B, T, H, N, r.device)
@@ -354,13 +367,14 @@ def prefill_train(r, k, v, x, u, workspace, state_in=None, c2=False, u2=None, st
     backward_workspace_bytes(B,T,H,N) bytes) receives the chunk-start states for backward(..., saved=True).
     Returns (y, state_out)."""
     lib = load_library()
-    B, T, H, N = r.shape
+    shape = r.shape
+    B, T, H, N = shape
     bf, f32 = torch.bfloat16, torch.float32
     y = torch.empty_like(r)
-    s_out = torch.empty((B, H, N, N), device=r.device, dtype=f32)
+    s_out = _new_states(B, H, N, r.device)
     with _on(r):
-        base = [_dev(r, "r", bf), _dev(k, "k", bf, r.shape), _dev(v, "v", bf, r.shape), _dev(x, "x", bf, r.shape)]
-        mid = _dev(u2, "u2", bf, r.shape) if c2 else _dev(u, "u", f32, (H, N))
+        base = [_dev(r, "r", bf), _dev(k, "k", bf, shape), _dev(v, "v", bf, shape), _dev(x, "x", bf, shape)]
+        mid = _dev(u2, "u2", bf, shape) if c2 else _dev(u, "u", f32, (H, N))
         fn = "gf_wkv6_prefill_c2_train" if c2 else "gf_wkv6_prefill_train"
         _check(getattr(lib, fn)(*base, mid, _dev(state_in, "state_in", f32, (B, H, N, N)), _dev(s_out, "state_out"),
                                 _dev(y, "y"), B, T, H, N, _dev(workspace, "workspace"), workspace.numel(), _stream(stream)), fn)
@@ -380,14 +394,15 @@ def prefill_varlen_train(r, k, v, x, u, cu_seqlens, max_seqlen, workspace, state
     backward_varlen_workspace_bytes(S,total_T,H,N) bytes) receives the chunk-start states for
     backward_varlen(..., saved=True).  Returns (y, state_out)."""
     lib = load_library()
-    total_T, H, N = r.shape
+    shape = r.shape
+    total_T, H, N = shape
     S = cu_seqlens.numel() - 1
     bf, f32 = torch.bfloat16, torch.float32
     y = torch.empty_like(r)
-    s_out = torch.empty((S, H, N, N), device=r.device, dtype=f32)
+    s_out = _new_states(S, H, N, r.device)
     with _on(r):
-        base = [_dev(r, "r", bf), _dev(k, "k", bf, r.shape), _dev(v, "v", bf, r.shape), _dev(x, "x", bf, r.shape)]
-        mid = _dev(u2, "u2", bf, r.shape) if c2 else _dev(u, "u", f32, (H, N))
+        base = [_dev(r, "r", bf), _dev(k, "k", bf, shape), _dev(v, "v", bf, shape), _dev(x, "x", bf, shape)]
+        mid = _dev(u2, "u2", bf, shape) if c2 else _dev(u, "u", f32, (H, N))
         fn = "gf_wkv6_prefill_varlen_c2_train" if c2 else "gf_wkv6_prefill_varlen_train"
         _check(getattr(lib, fn)(*base, mid, _dev(state_in, "state_in", f32, (S, H, N, N)), _dev(s_out, "state_out"),
                                 _dev(y, "y"), _dev(cu_seqlens, "cu_seqlens", torch.int32), S, total_T, int(max_seqlen), H, N,
@@ -404,15 +419,22 @@ def prefill_c2(r, k, v, x, u2=None, state_in=None, state_out=None, y=None, strea
     """gf_wkv6_prefill_c2: the Finch-C2 form.  r,k,v,x (and u2, the per-token second-value vector, or
     None): [B,T,H,N] bf16 CUDA tensors; k is the key before the (1 - w) factor.  Returns (y, state_out)."""
     lib = load_library()
-    B, T, H, N = r.shape
+    shape = r.shape
+    B, T, H, N = shape
     bf = torch.bfloat16
     if y is None:
         y = torch.empty_like(r)
+        y_ptr = y.data_ptr()
+    else:
+        y_ptr = _dev(y, "y", bf, shape)
     if state_out is None and want_state:
-        state_out = torch.empty((B, H, N, N), device=r.device, dtype=torch.float32)
-    args = [_dev(r, "r", bf), _dev(k, "k", bf, r.shape), _dev(v, "v", bf, r.shape), _dev(x, "x", bf, r.shape),
-            _dev(u2, "u2", bf, r.shape), _dev(state_in, "state_in", torch.float32, (B, H, N, N)),
-            _dev(state_out, "state_out", torch.float32, (B, H, N, N)), _dev(y, "y", bf, r.shape)]
+        state_out = _new_states(B, H, N, r.device)
+        s_ptr = state_out.data_ptr()
+    else:
+        s_ptr = _dev(state_out, "state_out", torch.float32, (B, H, N, N))
+    args = [_dev(r, "r", bf), _dev(k, "k", bf, shape), _dev(v, "v", bf, shape), _dev(x, "x", bf, shape),
+            _dev(u2, "u2", bf, shape), _dev(state_in, "state_in", torch.float32, (B, H, N, N)),
+            s_ptr, y_ptr]
     with _on(r):
         if split:
             _ensure_workspace(B, T, H, N, r.device)
@@ -426,16 +448,23 @@ def prefill_varlen_c2(r, k, v, x, u2, cu_seqlens, max_seqlen, state_in=None, sta
                       stream=None, want_state=True, split=True):
     """gf_wkv6_prefill_varlen_c2: packed Finch-C2 prefill.  r,k,v,x,u2 (u2 may be None): [total_T,H,N] bf16."""
     lib = load_library()
-    total_T, H, N = r.shape
+    shape = r.shape
+    total_T, H, N = shape
     S = cu_seqlens.numel() - 1
     bf = torch.bfloat16
     if y is None:
         y = torch.empty_like(r)
+        y_ptr = y.data_ptr()
+    else:
+        y_ptr = _dev(y, "y", bf, shape)
     if state_out is None and want_state:
-        state_out = torch.empty((S, H, N, N), device=r.device, dtype=torch.float32)
-    args = [_dev(r, "r", bf), _dev(k, "k", bf, r.shape), _dev(v, "v", bf, r.shape), _dev(x, "x", bf, r.shape),
-            _dev(u2, "u2", bf, r.shape), _dev(state_in, "state_in", torch.float32, (S, H, N, N)),
-            _dev(state_out, "state_out", torch.float32, (S, H, N, N)), _dev(y, "y", bf, r.shape),
+        state_out = _new_states(S, H, N, r.device)
+        s_ptr = state_out.data_ptr()
+    else:
+        s_ptr = _dev(state_out, "state_out", torch.float32, (S, H, N, N))
+    args = [_dev(r, "r", bf), _dev(k, "k", bf, shape), _dev(v, "v", bf, shape), _dev(x, "x", bf, shape),
+            _dev(u2, "u2", bf, shape), _dev(state_in, "state_in", torch.float32, (S, H, N, N)),
+            s_ptr, y_ptr,
             _dev(cu_seqlens, "cu_seqlens", torch.int32)]
     with _on(r):
         if split:
@@ -451,15 +480,16 @@ def step_c2(r, k, v, x, u2, state_in, state_out=None, y=None, stream=None):
     """gf_wkv6_step_c2: one Finch-C2 decode token per sequence.  r,k,v,x,u2 (u2 may be None): [B,H,N] bf16;
     state_out defaults to state_in (in-place update)."""
     lib = load_library()
-    B, H, N = r.shape
+    shape = r.shape
+    B, H, N = shape
     bf = torch.bfloat16
     if y is None:
         y = torch.empty_like(r)
     if state_out is None:
-        state_out = state_in if state_in is not None else torch.empty((B, H, N, N), device=r.device, dtype=torch.float32)
-    args = [_dev(r, "r", bf), _dev(k, "k", bf, r.shape), _dev(v, "v", bf, r.shape), _dev(x, "x", bf, r.shape),
-            _dev(u2, "u2", bf, r.shape), _dev(state_in, "state_in", torch.float32, (B, H, N, N)),
-            _dev(state_out, "state_out", torch.float32, (B, H, N, N)), _dev(y, "y", bf, r.shape)]
+        state_out = state_in if state_in is not None else _new_states(B, H, N, r.device)
+    args = [_dev(r, "r", bf), _dev(k, "k", bf, shape), _dev(v, "v", bf, shape), _dev(x, "x", bf, shape),
+            _dev(u2, "u2", bf, shape), _dev(state_in, "state_in", torch.float32, (B, H, N, N)),
+            _dev(state_out, "state_out", torch.float32, (B, H, N, N)), _dev(y, "y", bf, shape)]
     with _on(r):
         _check(lib.gf_wkv6_step_c2(*args, B, H, N, _stream(stream)), "gf_wkv6_step_c2")
     return y, state_out
@@ -573,17 +603,25 @@ def prefill_varlen(r, k, v, x, u, cu_seqlens, max_seqlen, state_in=None, state_o
     """gf_wkv6_prefill_varlen(_f32).  r,k,v,x: [total_T,H,N]; cu_seqlens: int32 CUDA [S+1];
     states [S,H,N,N].  Returns (y, state_out).  split as for prefill (cut by max_seqlen)."""
     lib = load_library()
-    total_T, H, N = r.shape
+    shape = r.shape
+    total_T, H, N = shape
     S = cu_seqlens.numel() - 1
-    sfx = _suffix(r.dtype)
+    dt = r.dtype
+    sfx = _suffix(dt)
     if y is None:
         y = torch.empty_like(r)
+        y_ptr = y.data_ptr()
+    else:
+        y_ptr = _dev(y, "y", dt, shape)
     if state_out is None and want_state:
-        state_out = torch.empty((S, H, N, N), device=r.device, dtype=torch.float32)
-    args = [_dev(r, "r"), _dev(k, "k", r.dtype, r.shape), _dev(v, "v", r.dtype, r.shape),
-            _dev(x, "x", r.dtype, r.shape), _dev(u, "u", torch.float32, (H, N)),
+        state_out = _new_states(S, H, N, r.device)
+        s_ptr = state_out.data_ptr()
+    else:
+        s_ptr = _dev(state_out, "state_out", torch.float32, (S, H, N, N))
+    args = [_dev(r, "r"), _dev(k, "k", dt, shape), _dev(v, "v", dt, shape),
+            _dev(x, "x", dt, shape), _dev(u, "u", torch.float32, (H, N)),
             _dev(state_in, "state_in", torch.float32, (S, H, N, N)),
-            _dev(state_out, "state_out", torch.float32, (S, H, N, N)), _dev(y, "y", r.dtype, r.shape),
+            s_ptr, y_ptr,
             _dev(cu_seqlens, "cu_seqlens", torch.int32)]
     with _on(r):
         if sfx == "" and split:
@@ -599,16 +637,18 @@ def step(r, k, v, x, u, state_in, state_out=None, y=None, stream=None):
     """gf_wkv6_step(_f32): one decode token per sequence.  r,k,v,x: [B,H,N]; state [B,H,N,N].
     state_out defaults to state_in (in-place update).  Returns (y, state_out)."""
     lib = load_library()
-    B, H, N = r.shape
-    sfx = _suffix(r.dtype)
+    shape = r.shape
+    B, H, N = shape
+    dt = r.dtype
+    sfx = _suffix(dt)
     if y is None:
         y = torch.empty_like(r)
     if state_out is None:
-        state_out = state_in if state_in is not None else torch.empty((B, H, N, N), device=r.device, dtype=torch.float32)
-    args = [_dev(r, "r"), _dev(k, "k", r.dtype, r.shape), _dev(v, "v", r.dtype, r.shape),
-            _dev(x, "x", r.dtype, r.shape), _dev(u, "u", torch.float32, (H, N)),
+        state_out = state_in if state_in is not None else _new_states(B, H, N, r.device)
+    args = [_dev(r, "r"), _dev(k, "k", dt, shape), _dev(v, "v", dt, shape),
+            _dev(x, "x", dt, shape), _dev(u, "u", torch.float32, (H, N)),
             _dev(state_in, "state_in", torch.float32, (B, H, N, N)),
-            _dev(state_out, "state_out", torch.float32, (B, H, N, N)), _dev(y, "y", r.dtype, r.shape)]
+            _dev(state_out, "state_out", torch.float32, (B, H, N, N)), _dev(y, "y", dt, shape)]
     with _on(r):
         _check(getattr(lib, "gf_wkv6_step" + sfx)(*args, B, H, N, _stream(stream)), "gf_wkv6_step" + sfx)
     return y, state_out
