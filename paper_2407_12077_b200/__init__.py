@@ -532,16 +532,19 @@ def layernorm_heads(y, gamma=None, beta=None, eps=1e-5, out=None, stream=None):
     (bf16 or fp32, contiguous); gamma, beta: fp32 [H*N] (or [H, N]) or None.  out defaults to a new tensor
     (pass out=y for in place).  Returns out."""
     lib = load_library()
-    H, N = y.shape[-2], y.shape[-1]
+    H, N = y.shape[-2:]
     rows = y.numel() // (H * N) if H * N else 0
     sfx = _suffix(y.dtype)
     if out is None:
         out = torch.empty_like(y)
+        out_ptr = out.data_ptr()
+    else:
+        out_ptr = _dev(out, "out", y.dtype, y.shape)
     with _on(y):
         _check(getattr(lib, "gf_c2_layernorm" + sfx)(
             _dev(y, "y"), _dev(None if gamma is None else gamma.reshape(H * N), "gamma", torch.float32),
             _dev(None if beta is None else beta.reshape(H * N), "beta", torch.float32), float(eps),
-            _dev(out, "out", y.dtype, y.shape), rows, H, N, _stream(stream)), "gf_c2_layernorm" + sfx)
+            out_ptr, rows, H, N, _stream(stream)), "gf_c2_layernorm" + sfx)
     return out
 
 
@@ -550,13 +553,18 @@ def key_compress(x, w_kd, out=None, stream=None):
     Returns c [..., Dc] bf16 (allocated here unless passed as out)."""
     lib = load_library()
     D, Dc = w_kd.shape
-    assert x.shape[-1] == D
+    c_shape = x.shape
+    assert c_shape[-1] == D
+    c_shape = c_shape[:-1] + (Dc,)
     rows = x.numel() // D if D else 0
     bf = torch.bfloat16
     if out is None:
-        out = torch.empty(x.shape[:-1] + (Dc,), device=x.device, dtype=bf)
+        out = torch.empty(c_shape, device=x.device, dtype=bf)
+        c_ptr = out.data_ptr()
+    else:
+        c_ptr = _dev(out, "c", bf, c_shape)
     with _on(x):
-        _check(lib.gf_gold_key_compress(_dev(x, "x", bf), _dev(w_kd, "w_kd", bf, (D, Dc)), _dev(out, "c", bf, x.shape[:-1] + (Dc,)),
+        _check(lib.gf_gold_key_compress(_dev(x, "x", bf), _dev(w_kd, "w_kd", bf), c_ptr,
                                         rows, D, Dc, _stream(stream)), "gf_gold_key_compress")
     return out
 
