@@ -93,12 +93,12 @@ struct BParamsPacked : BParams {
 // the chunks of the rest, in order, are cut into gridDim equal ranges of one to two units each.  A CTA takes the later part
 // (in time) of the unit its range begins in first of all and the earlier part of the unit it ends in last, so the adjoint at
 // a cut is there long before it is wanted: it is handed over in `hand` (one [64][64] fp32 block per CTA that ends with an
-// earlier part), announced by a word equal to `nonce` (a number no earlier launch has used).  The launch is cooperative.
+// earlier part), announced by a word that becomes 1.  The words keep that value when the kernel ends, and a replayed graph
+// launches it with the same arguments again: the call clears them, on the stream, ahead of every launch.  The launch is cooperative.
 struct BParamsBal : BParams {
     int n_units;
     float* hand;                 // [gridDim][64][64]
     unsigned long long* words;   // [gridDim]
-    unsigned long long nonce;
 };
 template <bool PACKED, bool BAL> struct BParamsOf { using type = BParams; };
 template <> struct BParamsOf<true, false> { using type = BParamsPacked; };
@@ -678,7 +678,7 @@ wkv6_backward_chunked_kernel(const __grid_constant__ CUtensorMap tm_x, const __g
             // the earlier part of a unit whose later part the next CTA has taken: the adjoint at the cut
             if constexpr (BAL) {
                 bool there = true;
-                if (lane == 0) there = word_wait(p.words + blockIdx.x, p.nonce, abort_flag);
+                if (lane == 0) there = word_wait(p.words + blockIdx.x, 1ull, abort_flag);
                 if (!__all_sync(0xffffffffu, there)) ok = false;
                 const float* src = p.hand + (size_t)blockIdx.x * 4096;
 #pragma unroll
@@ -1119,7 +1119,7 @@ wkv6_backward_chunked_kernel(const __grid_constant__ CUtensorMap tm_x, const __g
             if constexpr (BAL) {
                 if (last && pt(pc, 6) == 1) {
                     __threadfence();                 // (the group's barrier above: every lane's part of the adjoint is written)
-                    asm volatile("st.release.gpu.global.u64 [%0], %1;" ::"l"(p.words + blockIdx.x - 1), "l"(p.nonce) : "memory");
+                    asm volatile("st.release.gpu.global.u64 [%0], %1;" ::"l"(p.words + blockIdx.x - 1), "l"(1ull) : "memory");
                 }
             }
         }
@@ -1356,7 +1356,8 @@ inline gf_status_t chunked_backward(const __nv_bfloat16* r, const __nv_bfloat16*
         if (cudaGetLastError() != cudaSuccess) return GF_ERR_CUDA;
     }
     if (bal) {
-        bc::BParamsBal pb{p, (int)units, hand, reinterpret_cast<unsigned long long*>(hand + (size_t)n_sm * 4096), launch_nonce()};
+        bc::BParamsBal pb{p, (int)units, hand, reinterpret_cast<unsigned long long*>(hand + (size_t)n_sm * 4096)};
+        if (cudaMemsetAsync(pb.words, 0, (size_t)n_sm * sizeof(unsigned long long), st) != cudaSuccess) return GF_ERR_CUDA;
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3((unsigned)n_sm);
         cfg.blockDim = dim3(bc::G_THREADS);

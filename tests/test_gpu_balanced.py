@@ -68,6 +68,43 @@ def test_cut_call_repeats_and_replays(c2):
 
 
 @pytest.mark.parametrize("c2", [False, True])
+@pytest.mark.parametrize("saved", [False, True])
+def test_cut_gradient_replays_with_new_inputs(c2, saved):
+    # a graph's launches carry the same arguments every time, and the workspace still holds the cuts' words and adjoints of the
+    # replay before; token-by-token chunks in the units' later parts make the CTA that hands over the slower one
+    B, T, H = 5, 641, 32
+
+    def draw(seed):
+        i = synth.make_dense(B, T, H, 64, "bf16", seed=seed, device=DEV, state_std=0.1)
+        i.x[:, 2 * T // 3:, :, seed % 7::9] = 2.5
+        return [i.r, i.k, i.v, i.x, i.u, i.state_in, torch.randn(i.r.shape, device=DEV, generator=torch.Generator(device=DEV).manual_seed(seed)).bfloat16()]
+
+    def step(t, ws):
+        r, k, v, x, u, s0, dy = t
+        out = gf.prefill_train(r, k, v, x, u, ws, s0, c2=c2) if saved else ()
+        if c2:
+            return (*out, *gf.backward_c2(r, k, v, x, dy, s0, workspace=ws, saved=saved))
+        return (*out, *gf.backward(r, k, v, x, u, dy, s0, workspace=ws, saved=saved))
+
+    n = gf.backward_workspace_bytes(B, T, H, 64)
+    held, ws, ws_eager = draw(20), torch.empty(n, dtype=torch.uint8, device=DEV), torch.empty(n, dtype=torch.uint8, device=DEV)
+    step(held, ws)
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        out = step(held, ws)
+    for seed in (20, 21, 22, 23):
+        for t, new in zip(held, draw(seed)):
+            t.copy_(new)
+        g.replay()
+        torch.cuda.synchronize()
+        gf.last_device_status()
+        for a, b in zip(out, step(held, ws_eager)):
+            assert torch.equal(a, b), seed
+    gf.last_device_status()
+
+
+@pytest.mark.parametrize("c2", [False, True])
 @pytest.mark.parametrize("B,T,H", SHAPES[:3] + [(40, 90, 32)])
 def test_training_forward_of_many_units(B, T, H, c2):
     # the checkpoints of cut (and, in the last shape, of streamed whole) units: the gradient from them equals the gradient

@@ -1,0 +1,69 @@
+"""What the library's host code asks of the CUDA runtime, seen through a stand-in for it (fake_cuda_runtime.cpp; no GPU, no
+device code runs): the launches of a call, and what a call does when one of them is refused."""
+import json
+import os
+import shutil
+import subprocess
+import sys
+
+import pytest
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+CSRC = os.path.join(ROOT, "paper_2407_12077_b200", "csrc")
+NVCC = shutil.which("nvcc") or "/usr/local/cuda/bin/nvcc"
+pytestmark = pytest.mark.skipif(not os.path.exists(NVCC), reason="no nvcc")
+
+CALLER = """
+import ctypes, json, sys
+lib = ctypes.CDLL(sys.argv[1])
+lib.fake_log.restype = ctypes.c_char_p
+P = lambda i: ctypes.c_void_p(0x10000000 * (i + 1))      # never dereferenced
+WS = 0x700000000000
+out = []
+for name, args, refuse in json.loads(sys.stdin.read()):
+    lib.fake_reset(*refuse)
+    conv = []
+    for i, a in enumerate(args):
+        conv.append(P(i) if a == "p" else ctypes.c_void_p(WS) if a == "ws" else ctypes.c_size_t(a[0]) if isinstance(a, list) else
+                    ctypes.c_longlong(a["ll"]) if isinstance(a, dict) else a if a is None else ctypes.c_int(a))
+    status = getattr(lib, name)(*conv)
+    out.append([status, lib.fake_log().decode().splitlines()])
+print(json.dumps(out))
+"""
+
+
+@pytest.fixture(scope="module")
+def host_library(tmp_path_factory):
+    d = tmp_path_factory.mktemp("host")
+    lib = str(d / "libhost.so")
+    subprocess.run(["g++", "-shared", "-fPIC", "-I/usr/local/cuda/include", "-o", str(d / "libfake.so"),
+                    os.path.join(ROOT, "tests", "fake_cuda_runtime.cpp")], check=True)
+    subprocess.run([NVCC, "-gencode", "arch=compute_100a,code=compute_100a", "-std=c++17", "--expt-relaxed-constexpr", "-w",
+                    "-Xcompiler", "-fPIC", "-shared", "-cudart", "none", "-I", os.path.join(ROOT, "include"), "-I", CSRC, "-o", lib,
+                    os.path.join(CSRC, "gf_wkv6_api.cu"), "-L", str(d), "-lfake", "-Xlinker", "-rpath", "-Xlinker", str(d)], check=True)
+    return lib
+
+
+def calls(lib, *todo):
+    """[(status, log lines)] of the calls, made one after another in a process of their own."""
+    r = subprocess.run([sys.executable, "-c", CALLER, lib], input=json.dumps(todo), capture_output=True, text=True, timeout=120)
+    assert r.returncode == 0, r.stderr[-500:]
+    return json.loads(r.stdout)
+
+
+def backward(c2, B, T, H, bytes_):
+    ins = ["p"] * 4 + ([] if c2 else ["p"]) + ["p"] * 3 + ["p"] * 4 + ([] if c2 else ["p"]) + ["p"]
+    return ["gf_wkv6_backward" + ("_c2" if c2 else "") + "_saved", ins + [B, T, H, 64, "ws", [bytes_], None]]
+
+
+@pytest.mark.parametrize("c2", [False, True])
+def test_gradient_clears_the_words_of_its_cuts(host_library, c2):
+    # a replayed graph repeats the call's launches with the arguments of the first time: the words that announce the adjoint at
+    # a cut have to be cleared by the call itself, every time, before the launch that waits for them
+    for s, log in calls(host_library, backward(c2, 5, 700, 32, 1 << 40) + [[0, 0]], backward(c2, 5, 700, 32, 1 << 40) + [[0, 0]]):
+        assert s == 0
+        cut = [i for i, line in enumerate(log) if " cooperative " in line]
+        assert len(cut) == 1 and log[cut[0]].startswith("grid 148 "), log
+        cleared = [line.split() for line in log[:cut[0]] if line.startswith("memset")]
+        assert len(cleared) == 1 and cleared[0][2:] == ["0", str(8 * 148)], log
+        assert int(cleared[0][1]) > 0x700000000000          # (in the workspace, behind the checkpoints)
