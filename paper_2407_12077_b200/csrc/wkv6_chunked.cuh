@@ -541,17 +541,18 @@ struct Params {
     // output overwrites.  The launch is cooperative: every CTA a cut waits for is resident.
     int bal_chunks;
     unsigned long long nonce;
-    // Summary launch of a split call: nonzero lets a CTA start late in its segment.  dS forgets what lies before a run of
-    // tokens over which every channel decays by more than 2^-TRAIL_LOG2, far below fp32's rounding of what comes after,
-    // and D is then zero to the same degree: so the CTA first sums the decays of its segment's last TRAIL_CHUNKS chunks
-    // and runs from the last chunk boundary after which every channel has decayed that far, if there is one.  (Segments of
-    // 512 chunks with w in [0.69, 0.998]: 16 chunks run, the launch takes 25 us instead of 292.)  What rounding forgets, a
-    // NaN or infinity before that boundary does not: see poison_later_segments.
+    // Summary launch of a split call: nonzero lets a CTA start late in its segment.  Over a run of tokens in which every
+    // channel decays by more than 2^-TRAIL_LOG2 any finite fp32 value, 2^128 at most, falls below half of the smallest
+    // subnormal, 2^-150, whatever comes after it: dS forgets what lies before such a run, and D is zero.  So the CTA first
+    // sums the decays of its segment's last chunks, TRAIL_CHUNKS at a time and at most TRAIL_LOOKS times, and runs from the
+    // last chunk boundary after which every channel has decayed that far, if there is one.  What no finite value survives, a
+    // NaN or infinity before that boundary does: see poison_later_segments.
     int trail;
 };
 constexpr int SUMMARY_FLOATS = 64 + 64 * 64;
-constexpr float TRAIL_LOG2 = 96.f;
+constexpr float TRAIL_LOG2 = 280.f;    // (278, and a margin for the rounding of the sums)
 constexpr int TRAIL_CHUNKS = 30;       // (one per warp)
+constexpr int TRAIL_LOOKS = 3;
 
 // Writes a warp's 16 x 64 fp32 accumulator block (acc[n][0..1] = row g, cols 8n+2q,+1;
 // acc[n][2..3] = row g+8) as bf16 into rows row0 .. row0+15 of a 128B-swizzled [rows][64] tile.
@@ -807,32 +808,36 @@ wkv6_chunked_kernel(const __grid_constant__ CUtensorMap tm_r, const __grid_const
     if constexpr (SUMMARY) {
         // only whole, full segments (of which all but the last chunks may go); one warp per chunk sums it: lane = 4 channels
         // (lane % 16) of every other row
-        const int n_full = len / L, look = min(TRAIL_CHUNKS, n_full - 1);
-        if (p.trail && len % L == 0 && look > 0) {
+        const int n_full = len / L;
+        if (p.trail && len % L == 0 && n_full > 1) {
             float* tot = reinterpret_cast<float*>(smem);           // [TRAIL_CHUNKS][64] (the ring: nothing has been loaded yet)
-            if (warp < look) {                                     // chunk n_full - 1 - warp
-                const __nv_bfloat16* xp = p.x + (size_t)(row0 + (long long)(n_full - 1 - warp) * L + (lane >> 4)) * ((size_t)p.H * 64) + h * 64 + 4 * (lane & 15);
-                float e[4] = {0.f, 0.f, 0.f, 0.f};
+            float a0 = 0.f, a1 = 0.f;                              // every warp finds the same answer: two channels per lane
+            for (int k0 = 0; k0 < min(TRAIL_LOOKS * TRAIL_CHUNKS, n_full - 1) && !trail_cut; k0 += TRAIL_CHUNKS) {
+                const int look = min(TRAIL_CHUNKS, n_full - 1 - k0), cw = n_full - 1 - k0 - warp;        // (this warp's chunk)
+                if (warp < look) {
+                    const __nv_bfloat16* xp = p.x + (size_t)(row0 + (long long)cw * L + (lane >> 4)) * ((size_t)p.H * 64) + h * 64 + 4 * (lane & 15);
+                    float e[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll 16
-                for (int t = 0; t < L / 2; ++t) {
-                    const uint2 w = *reinterpret_cast<const uint2*>(xp + (size_t)(2 * t) * ((size_t)p.H * 64));
-                    e[0] += ex2(fmaf(bf_lo(w.x), LOG2E, LOG2_LOG2E)); e[1] += ex2(fmaf(bf_hi(w.x), LOG2E, LOG2_LOG2E));
-                    e[2] += ex2(fmaf(bf_lo(w.y), LOG2E, LOG2_LOG2E)); e[3] += ex2(fmaf(bf_hi(w.y), LOG2E, LOG2_LOG2E));
-                }
+                    for (int t = 0; t < L / 2; ++t) {
+                        const uint2 w = *reinterpret_cast<const uint2*>(xp + (size_t)(2 * t) * ((size_t)p.H * 64));
+                        e[0] += ex2(fmaf(bf_lo(w.x), LOG2E, LOG2_LOG2E)); e[1] += ex2(fmaf(bf_hi(w.x), LOG2E, LOG2_LOG2E));
+                        e[2] += ex2(fmaf(bf_lo(w.y), LOG2E, LOG2_LOG2E)); e[3] += ex2(fmaf(bf_hi(w.y), LOG2E, LOG2_LOG2E));
+                    }
 #pragma unroll
-                for (int i = 0; i < 4; ++i) e[i] += __shfl_xor_sync(0xffffffffu, e[i], 16);
-                if (lane < 16) *reinterpret_cast<float4*>(tot + warp * 64 + 4 * lane) = make_float4(e[0], e[1], e[2], e[3]);
-            }
-            __syncthreads();
-            // every warp finds the same answer: two channels per lane, chunks from the last one back
-            float a0 = 0.f, a1 = 0.f;
-            for (int k = 0; k < look; ++k) {
-                a0 += tot[k * 64 + 2 * lane]; a1 += tot[k * 64 + 2 * lane + 1];
-                if (__all_sync(0xffffffffu, a0 > TRAIL_LOG2 && a1 > TRAIL_LOG2)) { trail_cut = n_full - 1 - k; break; }     // (false for NaN)
+                    for (int i = 0; i < 4; ++i) e[i] += __shfl_xor_sync(0xffffffffu, e[i], 16);
+                    if (lane < 16) *reinterpret_cast<float4*>(tot + warp * 64 + 4 * lane) = make_float4(e[0], e[1], e[2], e[3]);
+                }
+                __syncthreads();
+                for (int k = 0; k < look; ++k) {                   // chunks from the last one back
+                    a0 += tot[k * 64 + 2 * lane]; a1 += tot[k * 64 + 2 * lane + 1];
+                    if (__all_sync(0xffffffffu, a0 > TRAIL_LOG2 && a1 > TRAIL_LOG2)) { trail_cut = n_full - 1 - k0 - k; break; }     // (false for NaN)
+                }
+                __syncthreads();                                   // (the sums are read before they, or the ring, are written again)
+                // (decays that one look leaves below a third of the way are too slow for the others)
+                if (!__all_sync(0xffffffffu, a0 > TRAIL_LOG2 / TRAIL_LOOKS && a1 > TRAIL_LOG2 / TRAIL_LOOKS)) break;
             }
             row0 += (long long)trail_cut * L;
             len -= trail_cut * L;
-            __syncthreads();                                       // (the sums are read before the ring is loaded)
             fence_proxy_async();
         }
     }

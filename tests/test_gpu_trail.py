@@ -12,11 +12,12 @@ DEV = "cuda:0"
 NAN, INF = float("nan"), float("inf")
 
 
-@pytest.mark.parametrize("T", [24576, 25000])
-@pytest.mark.parametrize("x_lo,x_hi", [(-6.0, -1.0), (-4.5, -4.0), (-5.4, -5.1), (-7.0, -6.5), (-1.0, -0.5)])
+@pytest.mark.parametrize("T", [24576, 25000, 51200, 51300])
+@pytest.mark.parametrize("x_lo,x_hi", [(-6.0, -1.0), (-4.5, -4.0), (-5.4, -5.1), (-7.0, -6.5), (-1.0, -0.5), (-3.6, -3.2), (-3.4, -3.0)])
 def test_late_start_against_oracle(T, x_lo, x_hi):
-    # about 16 / 95 / 280 / 1200 / 2 chunks until every channel has decayed by 2^-96: within a few chunks, around the 30 that
-    # are looked at and beyond.  One slow channel in head 1.  Tolerance: the contract's.
+    # about 42 / 210 / 580 / 2600 / 7 / 90 / 74 chunks until every channel has decayed by 2^-280: within the first look of 30
+    # chunks, the second, the third and beyond; segments of 48, 49, 100 and 101 chunks.  One slow channel in head 1.
+    # Tolerance: the contract's.
     inp = synth.make_dense(1, T, 3, 64, "bf16", seed=T, state_std=1.0, x_lo=x_lo, x_hi=x_hi)
     inp.x[:, :, 1, 17] = -11.0
     d = inp.to(DEV)
@@ -27,6 +28,29 @@ def test_late_start_against_oracle(T, x_lo, x_hi):
     for h in range(3):
         assert orc.rel_l2(y[:, :, h].float().cpu().numpy(), y_ref[:, :, h]) <= 5e-3
         assert orc.rel_l2(s[:, h].cpu().numpy(), s_ref[:, h]) <= 5e-3
+
+
+@pytest.mark.parametrize("log2_kv,chunks", [(0, 20), (0, 23), (100, 30), (100, 36), (100, 41)])
+def test_what_lies_before_an_empty_tail_is_kept(log2_kv, chunks):
+    # the keys and values of the segments' last chunks are zero, every channel decays by about 2^-5.6 in each of them, and the
+    # last segment, without keys and without decay, hands the state on: what the tails leave of k v 2^log2_kv, down to
+    # 2^-130, is the whole of it.  Against the unsplit call, whose products are the same and whose sums differ in what a segment
+    # starts from: fp32 rounding of the sums of a channel's row, twice 2^-24 in each of the segment's chunks, and a subnormal.
+    H, seg = 4, 128
+    T = 8 * seg * 64
+    assert gf.split_plan(1, T, H, torch.cuda.get_device_properties(0).multi_processor_count)[:2] == (8, seg)
+    i = synth.make_dense(1, T, H, 64, "bf16", seed=31, device=DEV)
+    i.x.copy_((-2.735 + 0.02 * i.x.float()).bfloat16())                      # (x around -3.5, so about -2.8)
+    for t in (i.k, i.v):
+        t.mul_(2.0 ** (log2_kv / 2))
+        t.view(8, seg * 64, H, 64)[:, (seg - chunks) * 64:] = 0
+    for t, value in ((i.k, 0), (i.v, 0), (i.x, -30)):
+        t[:, 7 * seg * 64:] = value
+    y, s = gf.prefill(i.r, i.k, i.v, i.x, i.u, None)
+    y1, s1 = gf.prefill(i.r, i.k, i.v, i.x, i.u, None, split=False)
+    gf.last_device_status()
+    assert int((s1 != 0).sum()) > 0.99 * s1.numel()
+    assert bool(((s - s1).abs() <= 2 * seg * 2.0 ** -24 * s1.abs().amax(-1, keepdim=True) + 2.0 ** -149).all())
 
 
 @pytest.mark.parametrize("c2", [False, True])
