@@ -703,9 +703,11 @@ __device__ __forceinline__ void exact_chunk(float* scr, const Params& p, int h, 
 // writes NaN over those elements of its summary's dS (from_marks) and says so in the sign of D[1]; every CTA says in the
 // sign of D[0] of the summary before its segment that its outputs are written (D is a decay, readers drop the signs).
 // Whichever of two CTAs of a unit comes second sees the other's word (both sequentially consistent) and makes the marked
-// columns of the later segment's outputs NaN, and the marked elements of the final state.  Runs after the CTA's last
-// barrier; without a mark it costs a few words of memory traffic per CTA.
-__device__ __forceinline__ void poison_later_segments(const Params& p, int unit, int seg, bool marked, int* mark, int* todo)
+// columns of the later segment's outputs NaN, and the marked elements of the final state and (CKPT) of the segment's
+// checkpoints.  Runs after the CTA's last barrier; without a mark it costs a few words of memory traffic per CTA.
+// first_slot: the unit's first checkpoint slot.
+template <bool CKPT>
+__device__ __forceinline__ void poison_later_segments(const Params& p, int unit, int seg, bool marked, int* mark, int* todo, size_t first_slot)
 {
     const int tid = threadIdx.x, nseg = p.nseg;
     unsigned* base = reinterpret_cast<unsigned*>(p.summaries) + (size_t)unit * (nseg - 1) * SUMMARY_FLOATS;
@@ -734,6 +736,9 @@ __device__ __forceinline__ void poison_later_segments(const Params& p, int unit,
         if (!(t >> g & 1)) continue;
         const int from = g < seg ? g : seg, to = g < seg ? seg : g;
         const float* ds = reinterpret_cast<const float*>(base + (size_t)from * SUMMARY_FLOATS + 64);
+        const int first = min(len, to * p.seg_chunks * L), end = to == nseg - 1 ? len : min(len, first + p.seg_chunks * L);
+        // the states before the segment's chunks, and after the last one of the unit
+        const int ck_first = (first + L - 1) / L, ck_end = (end + L - 1) / L + (to == nseg - 1 ? 1 : 0);
         __syncthreads();
         if (tid < 64) mark[tid] = 0;
         __syncthreads();
@@ -742,10 +747,12 @@ __device__ __forceinline__ void poison_later_segments(const Params& p, int unit,
             if (v != v) {
                 mark[i & 63] = 1;
                 if (to == nseg - 1 && p.state_out) p.state_out[(size_t)unit * 4096 + i] = nan;
+                if (CKPT)
+                    for (int c = ck_first; c < ck_end; ++c)
+                        reinterpret_cast<__nv_bfloat16*>(p.ckpt)[(first_slot + c) * 4096 + i] = __float2bfloat16_rn(nan);
             }
         }
         __syncthreads();
-        const int first = min(len, to * p.seg_chunks * L), end = to == nseg - 1 ? len : min(len, first + p.seg_chunks * L);
         for (long long i = (long long)first * 64 + tid; i < (long long)end * 64; i += blockDim.x)
             if (mark[i & 63]) p.y[(size_t)(row0 + (i >> 6)) * p.H * 64 + h * 64 + (i & 63)] = __float2bfloat16_rn(nan);
     }
@@ -1802,7 +1809,8 @@ wkv6_chunked_kernel(const __grid_constant__ CUtensorMap tm_r, const __grid_const
         tmem_dealloc(tmem, TM_COLS);
     }
     if (TRAIL)
-        poison_later_segments(p, unit, seg, lds32(sbase + OFF_MARK) != 0, reinterpret_cast<int*>(smem + OFF_TOT), reinterpret_cast<int*>(smem + OFF_TOT) + 64);
+        poison_later_segments<CKPT>(p, unit, seg, lds32(sbase + OFF_MARK) != 0, reinterpret_cast<int*>(smem + OFF_TOT),
+                                    reinterpret_cast<int*>(smem + OFF_TOT) + 64, CKPT ? ckpt_slot(0) : 0);
 }
 
 // One warp that waits, with the kernel's own bounded wait, on a barrier nobody arrives on: the wait runs out after

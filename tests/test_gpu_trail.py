@@ -55,10 +55,11 @@ def test_what_lies_before_an_empty_tail_is_kept(log2_kv, chunks):
 
 @pytest.mark.parametrize("c2", [False, True])
 @pytest.mark.parametrize("train", [False, True])
-def test_non_finite_values_are_not_forgotten(c2, train):
+@pytest.mark.parametrize("T", [24576, 61440])
+def test_non_finite_values_are_not_forgotten(T, c2, train):
     # one call per place: the tokens after it and the final state are non-finite where the unsplit call's are, the other
-    # head is untouched
-    T, H = 24576, 2
+    # head is untouched (segments of 48 chunks and of 120)
+    H = 2
     clean = synth.make_dense(1, T, H, 64, "bf16", seed=5, device=DEV, state_std=0.1)
     ws = torch.empty(gf.backward_workspace_bytes(1, T, H, 64), dtype=torch.uint8, device=DEV)
 
@@ -82,5 +83,13 @@ def test_non_finite_values_are_not_forgotten(c2, train):
         assert bool((bad | ~bad1).all()), (name, t)                          # and at least the same elements
         sb, sb1 = ~torch.isfinite(s[0, 1]), ~torch.isfinite(s1[0, 1])
         assert bool((sb | ~sb1).all()), (name, t)
+        if train:                            # the states the gradient takes from the forward pass: as those it makes itself
+            back = (lambda **kw: gf.backward_c2(i.r, i.k, i.v, i.x, i.r, i.state_in, **kw)) if c2 else \
+                   (lambda **kw: gf.backward(i.r, i.k, i.v, i.x, i.u, i.r, i.state_in, **kw))
+            for a, b in zip(back(workspace=ws, saved=True), back()):
+                assert bool((~torch.isfinite(a) | torch.isfinite(b)).all()), (name, t)        # non-finite wherever the other is
+                if a.dim() == 4 and a.shape[1] == T:
+                    assert bool(torch.isfinite(a[:, :, 0]).all()), (name, t)
+            gf.last_device_status()
     y, s = run(clean, True)                                                  # nothing stays behind
     assert torch.equal(y, y0) and torch.equal(s, s0)
