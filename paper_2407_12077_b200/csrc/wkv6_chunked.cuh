@@ -72,6 +72,12 @@ namespace ck {
 constexpr int L = 64;                  // tokens per chunk
 constexpr int TILE = 64 * 64 * 2;      // one bf16 [64 x 64] tile
 constexpr int NS = 5;                  // {x,r,k,v} ring depth
+// Copies in flight per CTA at most: the producer requests chunk c once the copy of chunk c - LOAD_AHEAD has landed.  A set of
+// elementwise warps takes every N_ESET-th chunk and so meets only every other phase of a stage (the ring's depth is odd); by its
+// parity alone it would also be let through to chunk c while the copy of chunk c - NS, which had the stage before, is still
+// landing.  When it waits for chunk c it has scaled chunk c - N_ESET, which was requested after chunk c - N_ESET - LOAD_AHEAD
+// had landed, and with it all chunks up to c - NS.
+constexpr int LOAD_AHEAD = 3;
 constexpr int NSB = 2;                 // bf16 chunk-start state operand tiles (by chunk parity)
 constexpr int NPP = 2;                 // bf16 masked-score operand tiles (by chunk parity)
 constexpr int NSIDE = 8;               // ring of per-chunk side vectors (chunk decay, bonus, safety flag): deeper than
@@ -79,6 +85,7 @@ constexpr int NSIDE = 8;               // ring of per-chunk side vectors (chunk 
 constexpr int NTOT = 4;                // per-warp decay-total buffers (two per elementwise set)
 constexpr int N_EW = 8;                // elementwise warps per set
 constexpr int N_ESET = 2;              // elementwise sets (alternate chunks)
+static_assert(LOAD_AHEAD + N_ESET <= NS, "a set may be let through to a stage whose previous copy has not landed");
 constexpr int N_GW = 4;                // warps per tensor-memory reader group (one per sub-partition)
 constexpr int WARP_MMA_F = 1;          // issues P = R^ K^^T and dS = K^^T V; owns the tensor-memory allocation
 constexpr int WARP_MMA_B = 2;          // issues Y = R^ S_0 + P' V
@@ -947,6 +954,7 @@ wkv6_chunked_kernel(const __grid_constant__ CUtensorMap tm_r, const __grid_const
         if constexpr (PERSIST) {
             int gc = 0, real_end = -1;               // chunks of the stream issued so far; index of the first end marker
             int s = 0, ph = 1;                       // ring stage and the parity of its previous release
+            int fs = 0, fph = 0;                     // stage and phase bit of the copy that has to have landed (LOAD_AHEAD)
             bool alive = true;
             for (int k = 0; alive; ++k) {
                 int u = 0, c0 = 0, c1 = 0;               // the next piece: chunks c0 .. c1-1 of unit u (balanced launches)
@@ -1027,6 +1035,10 @@ wkv6_chunked_kernel(const __grid_constant__ CUtensorMap tm_r, const __grid_const
                 }
                 for (int c = c0; c < c1; ++c, ++gc) {
                     if (gc >= NS && !mbar_wait_warp(bar(BAR_EMPTY_RKV + s), ph, abort_flag)) { alive = false; break; }
+                    if (gc >= LOAD_AHEAD) {
+                        if (!mbar_wait_warp(bar(BAR_FULL_RKV + fs), fph, abort_flag)) { alive = false; break; }
+                        if (++fs == NS) { fs = 0; fph ^= 1; }
+                    }
                     const int row = (int)(urow0 + (long long)c * L);
                     const uint32_t dst = sbase + OFF_RING + s * STAGE;
                     if (elect_one()) {
@@ -1065,9 +1077,14 @@ wkv6_chunked_kernel(const __grid_constant__ CUtensorMap tm_r, const __grid_const
         } else {
             int issued = 0;
             int s = 0, ph = 1;                       // ring stage and the parity of its previous release
+            int fs = 0, fph = 0;                     // stage and phase bit of the copy that has to have landed (LOAD_AHEAD)
             int row = (int)row0;
             for (int c = 0; c < nchunks; ++c, row += L) {
                 if (c >= NS && !mbar_wait_warp(bar(BAR_EMPTY_RKV + s), ph, abort_flag)) break;
+                if (c >= LOAD_AHEAD) {
+                    if (!mbar_wait_warp(bar(BAR_FULL_RKV + fs), fph, abort_flag)) break;
+                    if (++fs == NS) { fs = 0; fph ^= 1; }
+                }
                 const uint32_t dst = sbase + OFF_RING + s * STAGE;
                 if (elect_one()) {
                     mbar_expect_tx(bar(BAR_FULL_RKV + s), SUMMARY ? 3 * TILE : STAGE);
