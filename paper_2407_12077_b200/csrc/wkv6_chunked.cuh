@@ -138,6 +138,7 @@ enum {
 };
 // persistent launches: one descriptor per chunk of the CTA's chunk stream
 // {first row, valid tokens | flags | head << 16, unit, chunks left in the unit}
+constexpr int STREAM_MAX_HEADS = 65536;                          // (a descriptor's upper 16 bits; more heads: one CTA per unit)
 constexpr int OFF_DESC = (OFF_BAR + BAR_COUNT * 8 + 15) & ~15;   // [NSIDE] int4
 // flags beside the valid-token count (low byte): first chunk of a unit (or piece of one), no chunk, piece that continues
 // a unit another CTA began, last chunk of a piece
@@ -888,7 +889,7 @@ wkv6_chunked_kernel(const __grid_constant__ CUtensorMap tm_r, const __grid_const
             int4 d;
             asm volatile("ld.shared.v4.s32 {%0, %1, %2, %3}, [%4];"
                          : "=r"(d.x), "=r"(d.y), "=r"(d.z), "=r"(d.w) : "r"(sbase + OFF_DESC + 16 * (c & (NSIDE - 1))) : "memory");
-            ck.row = d.x; ck.valid = d.y & 0xff; ck.unit = d.z; ck.h = d.y >> 16; ck.rem = d.w;
+            ck.row = d.x; ck.valid = d.y & 0xff; ck.unit = d.z; ck.h = (int)((unsigned)d.y >> 16); ck.rem = d.w;
             ck.first = (d.y & DESC_FIRST) != 0; ck.last = BAL ? (d.y & DESC_LAST) != 0 : d.w == 0; ck.end = (d.y & DESC_END) != 0;
         } else {
             ck.row = (int)(row0 + (long long)c * L); ck.valid = min(L, len - c * L); ck.unit = unit; ck.h = h;
@@ -1042,7 +1043,7 @@ wkv6_chunked_kernel(const __grid_constant__ CUtensorMap tm_r, const __grid_const
                     const int row = (int)(urow0 + (long long)c * L);
                     const uint32_t dst = sbase + OFF_RING + s * STAGE;
                     if (elect_one()) {
-                        int meta = min(L, ulen - c * L) | (c == c0 ? DESC_FIRST : 0) | (uh << 16);
+                        int meta = min(L, ulen - c * L) | (c == c0 ? DESC_FIRST : 0) | (int)((unsigned)uh << 16);
                         if (BAL) meta |= (c == c0 && c0 > 0 ? DESC_CONT : 0) | (c == c1 - 1 ? DESC_LAST : 0);
                         put_desc(gc, row, meta, u, unch - 1 - c);
                         mbar_expect_tx(bar(BAR_FULL_RKV + s), STAGE);      // (release: the descriptor is visible to the waiters)
@@ -1674,8 +1675,8 @@ wkv6_chunked_kernel(const __grid_constant__ CUtensorMap tm_r, const __grid_const
             if (!mbar_wait(bar(BAR_FULL_RKV + s), ph, abort_flag)) break;
             Chunk ck;                                    // (this role needs the valid-token count, the head and the end flag only)
             if constexpr (PERSIST) {
-                const int meta = (int)lds32(sbase + OFF_DESC + 16 * (c & (NSIDE - 1)) + 4);
-                ck.valid = meta & 0xff; ck.h = meta >> 16; ck.end = (meta & DESC_END) != 0;
+                const uint32_t meta = lds32(sbase + OFF_DESC + 16 * (c & (NSIDE - 1)) + 4);
+                ck.valid = (int)(meta & 0xff); ck.h = (int)(meta >> 16); ck.end = (meta & DESC_END) != 0;
             } else {
                 ck.valid = min(L, len - c * L); ck.h = h; ck.end = false;
             }
@@ -2086,7 +2087,7 @@ inline gf_status_t chunked_prefill(const __nv_bfloat16* r, const __nv_bfloat16* 
             cudaGetLastError();                      // (fewer SMs to be had than the device has: whole units below)
             p.bal_chunks = 0;
         }
-        if (nseg == 1 && n_sm_ck > 0 && units > n_sm_ck && (units >= 6LL * n_sm_ck || (unit_chunks <= 48 && units >= 3LL * n_sm_ck)) &&
+        if (nseg == 1 && n_sm_ck > 0 && units > n_sm_ck && H <= ck::STREAM_MAX_HEADS && (units >= 6LL * n_sm_ck || (unit_chunks <= 48 && units >= 3LL * n_sm_ck)) &&
             (!cu || (scratch && scratch_bytes >= persistent_scratch_bytes(n_seq)))) {
             // A stream of whole units per SM; packed: the longest sequences first, as in the prefill without checkpoints.
             // (Packed, 768 units of 2..47 chunks: the training pair 662 -> 650 us.  Dense, 256 units of 32 chunks: 84.0 us
@@ -2133,7 +2134,7 @@ inline gf_status_t chunked_prefill(const __nv_bfloat16* r, const __nv_bfloat16* 
         cudaGetLastError();                          // (fewer SMs to be had than the device has: whole units below)
         p.bal_chunks = 0;
     }
-    if (nseg == 1 && n_sm > 0 && units > n_sm && (units >= 6LL * n_sm || max_chunks <= 48) &&
+    if (nseg == 1 && n_sm > 0 && units > n_sm && H <= ck::STREAM_MAX_HEADS && (units >= 6LL * n_sm || max_chunks <= 48) &&
         (!cu || (scratch && scratch_bytes >= sizeof(unsigned int)))) {
         p.n_units = (int)units;
         if (cu) {

@@ -650,3 +650,36 @@ def test_packed_call_with_thousands_of_short_sequences(S):
     assert worst <= 6e-3, worst
     empty = [i for i, n in enumerate(lens) if n == 0]
     assert all(np.array_equal(sn[i], inp.state_in[i].numpy()) for i in empty[:200])
+
+
+@pytest.mark.parametrize("H", [32769, 65536, 65537])
+@pytest.mark.parametrize("form", ["dense", "packed", "c2", "train"])
+def test_more_heads_than_15_bits(H, form):
+    """A streamed launch hands the head on in the 16 upper bits of a chunk's descriptor; more heads run one CTA per unit."""
+    T = 3
+    i = synth.make_dense(1, T, H, 64, "bf16", seed=H, device=DEV)
+    if form == "dense":
+        y, _ = gf.prefill(i.r, i.k, i.v, i.x, i.u, None, want_state=False)
+    elif form == "packed":
+        cu = torch.tensor([0, 1, T], dtype=torch.int32, device=DEV)
+        y, _ = gf.prefill_varlen(i.r[0], i.k[0], i.v[0], i.x[0], i.u, cu, 2, None, want_state=False)
+        y = y[None]
+    elif form == "c2":
+        y, _ = gf.prefill_c2(i.r, i.k, i.v, i.x, None, None, want_state=False)
+    else:
+        ws = torch.empty(gf.backward_workspace_bytes(1, T, H, 64), dtype=torch.uint8, device=DEV)
+        y, _ = gf.prefill_train(i.r, i.k, i.v, i.x, i.u, ws, None)
+    gf.last_device_status()
+    heads = torch.tensor([0, 1, 32767, 32768, H // 2, H - 2, H - 1])
+    c = [t[:, :, heads.to(DEV)].contiguous().cpu() for t in (i.r, i.k, i.v, i.x)]
+    u = i.u[heads.to(DEV)].cpu()
+    if form == "c2":
+        ref, _ = orc.prefill_c2(*c, None, None)
+    elif form == "packed":
+        ref = np.concatenate([orc.prefill(*(t[:, a:b].contiguous() for t in c), u, None)[0] for a, b in ((0, 1), (1, T))], axis=1)
+    else:
+        ref, _ = orc.prefill(*c, u, None)
+    got = y[:, :, heads.to(DEV)].float().cpu().numpy()
+    for n in range(len(heads)):
+        assert orc.rel_l2(got[:, :, n], ref[:, :, n]) <= 2 * 2.0 ** -8, int(heads[n])      # (three tokens of one head: two bf16 roundings)
+    assert torch.isfinite(y.float()).all()

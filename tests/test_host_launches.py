@@ -67,3 +67,10 @@ def test_gradient_clears_the_words_of_its_cuts(host_library, c2):
         cleared = [line.split() for line in log[:cut[0]] if line.startswith("memset")]
         assert len(cleared) == 1 and cleared[0][2:] == ["0", str(8 * 148)], log
         assert int(cleared[0][1]) > 0x700000000000          # (in the workspace, behind the checkpoints)
+
+
+@pytest.mark.parametrize("H,streamed", [(65536, True), (65537, False)])
+def test_streams_end_where_a_head_no_longer_fits_its_descriptor(host_library, H, streamed):
+    (s, log), = calls(host_library, ["gf_wkv6_prefill", ["p"] * 8 + [1, 3, H, 64, None], [0, 0]])
+    assert s == 0 and len(log) == 1
+    assert log[0].startswith("grid 148 " if streamed else "grid %d " % H), log
