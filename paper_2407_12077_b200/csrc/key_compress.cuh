@@ -340,9 +340,10 @@ inline gf_status_t key_compress(const __nv_bfloat16* x, const __nv_bfloat16* w, 
     // fifths of the SMs do.  D = 2048, Dc = 128, us, whole tiles -> clusters of 8: 658 rows 12.1 -> 6.2, 1792 rows 12.2 -> 6.9
     // (of 4: 7.2); of 4: 2500 rows 12.3 -> 7.4; of 2: 5000 rows 12.4 -> 10.2.  Past the limit: 2000 rows in 16 clusters of 8
     // 12.4 (of 4: 7.1), 4700 rows in 37 clusters of 4 14.1 (whole 12.5).
+    // Where a cluster cannot be placed at all (a partitioned device) the launch is refused, and the call runs on whole tiles.
     int split = 1;
     while (split < 8 && n_tiles * split * 2 * 5 <= n_sm * 4LL && p.ksteps >= 4 * split) split *= 2;
-    long long grid = n_tiles < n_sm ? n_tiles * split : n_sm;
+    long long grid = n_tiles < n_sm ? n_tiles : n_sm;              // (of a short call: times the cluster size)
     // Whole tiles leave more than a fifth of the last round idle: equal shares of the rows, in units of 64, instead (us at
     // D = 2048, Dc = 128: 20000 rows 27.9 -> 21.0, 30000 rows 31.2 -> 26.5, 40000 rows 45.0 -> 40.5).  Otherwise whole tiles: a CTA
     // with rows left over after its last whole tile reads all of W once more for them (262144 rows 175.5, in shares 177.7).
@@ -352,19 +353,25 @@ inline gf_status_t key_compress(const __nv_bfloat16* x, const __nv_bfloat16* w, 
         grid = n_sm;
     }
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)grid);
     cfg.blockDim = dim3(kc::KC_THREADS);
     cfg.dynamicSmemBytes = kc::KC_SMEM;
     cfg.stream = st;
     cudaLaunchAttribute attr[2];
     attr[1].id = cudaLaunchAttributeClusterDimension;
-    attr[1].val.clusterDim.x = (unsigned)split;
     attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = split > 1 ? 2 : 1;
-    const cudaError_t e = cudaLaunchKernelEx(&cfg, kernels[split > 1 ? 0 : mblk][nb - 1], tx, tw, tc, p);
+    cudaError_t e;
+    for (;;) {
+        cfg.gridDim = dim3((unsigned)(grid * split));
+        attr[1].val.clusterDim.x = (unsigned)split;
+        cfg.numAttrs = split > 1 ? 2 : 1;
+        e = cudaLaunchKernelEx(&cfg, kernels[split > 1 ? 0 : mblk][nb - 1], tx, tw, tc, p);
+        if (e == cudaSuccess || split == 1) break;
+        cudaGetLastError();
+        split = 1;
+    }
     launches->fetch_add(1, std::memory_order_relaxed);
     return e == cudaSuccess ? GF_OK : GF_ERR_CUDA;
 }

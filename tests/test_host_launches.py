@@ -74,3 +74,17 @@ def test_streams_end_where_a_head_no_longer_fits_its_descriptor(host_library, H,
     (s, log), = calls(host_library, ["gf_wkv6_prefill", ["p"] * 8 + [1, 3, H, 64, None], [0, 0]])
     assert s == 0 and len(log) == 1
     assert log[0].startswith("grid 148 " if streamed else "grid %d " % H), log
+
+
+def key_compress(rows, D, Dc):
+    return ["gf_gold_key_compress", ["p", "p", "p", {"ll": rows}, D, Dc, None]]
+
+
+@pytest.mark.parametrize("status", [9, 701, 912])          # invalid configuration, out of resources, invalid cluster size
+def test_key_compression_without_clusters(host_library, status):
+    # where no cluster can be placed (a partitioned device) a short call runs on whole tiles instead of failing
+    (s, log), (s1, log1) = calls(host_library, key_compress(658, 2048, 128) + [[status, 0]], key_compress(658, 2048, 128) + [[0, 0]])
+    assert s1 == 0 and len(log1) == 1 and " cluster 8 " in log1[0]
+    assert s == 0
+    assert "refused" in log[0] and " cluster 8 " in log[0]
+    assert len(log) == 2 and "refused" not in log[1] and log[1].startswith("grid 6 cluster 1 ")
