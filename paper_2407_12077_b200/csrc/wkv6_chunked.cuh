@@ -43,10 +43,10 @@
 // between neighbouring CTAs, so that every CTA gets the same number of chunks: see Params::bal_chunks).
 #pragma once
 #include <atomic>
+#include <chrono>
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
-#include <random>
 #include <stdint.h>
 
 #include "device_info.cuh"
@@ -1986,10 +1986,11 @@ inline std::atomic<uint32_t>& wait_limit_us()
     return v;
 }
 
-// A number no earlier launch of this process has used, and that memory left by anything else holds with probability 2^-64.
+// A number no earlier launch of this process has used, and that memory left by anything else does not hold (from the time the
+// first one was drawn; not from std::random_device, which may throw, and nothing may be thrown through the C interface).
 inline unsigned long long launch_nonce()
 {
-    static std::atomic<unsigned long long> next{((unsigned long long)std::random_device{}() << 32) ^ std::random_device{}()};
+    static std::atomic<unsigned long long> next{(unsigned long long)std::chrono::system_clock::now().time_since_epoch().count()};
     unsigned long long z = next.fetch_add(0x9e3779b97f4a7c15ull, std::memory_order_relaxed);     // (Weyl sequence, then a bijective mix)
     z = (z ^ (z >> 30)) * 0xbf58476d1ce4e5b9ull;
     z = (z ^ (z >> 27)) * 0x94d049bb133111ebull;

@@ -13,6 +13,14 @@ CSRC = os.path.join(ROOT, "paper_2407_12077_b200", "csrc")
 NVCC = shutil.which("nvcc") or "/usr/local/cuda/bin/nvcc"
 pytestmark = pytest.mark.skipif(not os.path.exists(NVCC), reason="no nvcc")
 
+# std::random_device may throw where the system has no source of random numbers
+PRELUDE = """
+#include <random>
+#include <stdexcept>
+namespace std { struct gf_refusing_device { unsigned operator()() { throw std::runtime_error("no random device"); } }; }
+#define random_device gf_refusing_device
+"""
+
 CALLER = """
 import ctypes, json, sys
 lib = ctypes.CDLL(sys.argv[1])
@@ -35,11 +43,13 @@ print(json.dumps(out))
 @pytest.fixture(scope="module")
 def host_library(tmp_path_factory):
     d = tmp_path_factory.mktemp("host")
-    lib = str(d / "libhost.so")
+    prelude, lib = str(d / "prelude.h"), str(d / "libhost.so")
+    with open(prelude, "w") as f:
+        f.write(PRELUDE)
     subprocess.run(["g++", "-shared", "-fPIC", "-I/usr/local/cuda/include", "-o", str(d / "libfake.so"),
                     os.path.join(ROOT, "tests", "fake_cuda_runtime.cpp")], check=True)
     subprocess.run([NVCC, "-gencode", "arch=compute_100a,code=compute_100a", "-std=c++17", "--expt-relaxed-constexpr", "-w",
-                    "-Xcompiler", "-fPIC", "-shared", "-cudart", "none", "-I", os.path.join(ROOT, "include"), "-I", CSRC, "-o", lib,
+                    "-include", prelude, "-Xcompiler", "-fPIC", "-shared", "-cudart", "none", "-I", os.path.join(ROOT, "include"), "-I", CSRC, "-o", lib,
                     os.path.join(CSRC, "gf_wkv6_api.cu"), "-L", str(d), "-lfake", "-Xlinker", "-rpath", "-Xlinker", str(d)], check=True)
     return lib
 
@@ -88,3 +98,11 @@ def test_key_compression_without_clusters(host_library, status):
     assert s == 0
     assert "refused" in log[0] and " cluster 8 " in log[0]
     assert len(log) == 2 and "refused" not in log[1] and log[1].startswith("grid 6 cluster 1 ")
+
+
+def test_nothing_is_thrown_for_want_of_random_numbers(host_library):
+    # a cut prefill announces its states by a number of its own; no exception may cross the C interface while it is drawn
+    (s, log), (s1, log1) = calls(host_library, *[["gf_wkv6_prefill", ["p"] * 8 + [5, 700, 32, 64, None], [0, refused]] for refused in (0, 720)])
+    assert s == 0 and len(log) == 1 and " cooperative " in log[0]
+    # and where such a launch does not fit (cudaErrorCooperativeLaunchTooLarge) the call runs whole units
+    assert s1 == 0 and len(log1) == 2 and "refused" in log1[0] and "cooperative" not in log1[1]
