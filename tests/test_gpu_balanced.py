@@ -1,7 +1,8 @@
 """Dense calls with more (sequence, head) units than SMs whose units are cut between CTAs (balanced persistent launches).
 
 The state at a cut is handed over in fp32 at a chunk boundary, so every result must equal, bit for bit, that of the same
-sequences run one at a time without a cut (one CTA per unit); the smallest shapes are also compared with the oracle."""
+sequences (of a single one: of its heads) run a part at a time without a cut (one CTA per unit); the smallest shapes are also
+compared with the oracle."""
 import pytest
 import torch
 
@@ -16,6 +17,14 @@ DEV = "cuda:0"
 SHAPES = [(5, 300, 32), (3, 641, 74), (11, 321, 28), (1, 4096, 157)]
 
 
+def parts(B, H):
+    """Index pairs (sequences, heads) that cover a call in parts of few units: one sequence each, or halves of its heads.  Run
+    with split=False (the gradient: with more than 74 units) a part takes one CTA per unit."""
+    if B > 1:
+        return [(slice(b, b + 1), slice(None)) for b in range(B)]
+    return [(slice(None), slice(0, (H + 1) // 2)), (slice(None), slice((H + 1) // 2, H))]
+
+
 @pytest.mark.parametrize("B,T,H", SHAPES)
 @pytest.mark.parametrize("c2,in_place,x_hi", [(False, False, -1.0), (False, True, 2.5), (True, False, -1.0), (True, True, 2.5)])
 def test_units_cut_between_ctas(B, T, H, c2, in_place, x_hi):
@@ -23,20 +32,19 @@ def test_units_cut_between_ctas(B, T, H, c2, in_place, x_hi):
     i = synth.make_dense(B, T, H, 64, "bf16", seed=B * T + H, device=DEV, state_std=0.1, x_hi=x_hi)
     u2 = torch.randn(i.r.shape, device=DEV, generator=torch.Generator(device=DEV).manual_seed(3)).bfloat16()
 
-    def run(sl, state, out=None, **kw):
-        t = [x[sl].contiguous() for x in (i.r, i.k, i.v, i.x, u2)]
+    def run(b, h, state, out=None, **kw):
+        t = [x[b, :, h].contiguous() for x in (i.r, i.k, i.v, i.x, u2)]
         if c2:
             return gf.prefill_c2(*t, state, state_out=out, **kw)
-        return gf.prefill(*t[:4], i.u, state, state_out=out, **kw)
+        return gf.prefill(*t[:4], i.u[h].contiguous(), state, state_out=out, **kw)
 
     s0 = i.state_in.clone()
-    y, s = run(slice(None), s0, s0 if in_place else None)
+    y, s = run(slice(None), slice(None), s0, s0 if in_place else None)
     gf.last_device_status()
-    if B > 1:
-        for b in range(B):                       # few units each, never split: one CTA per unit
-            yb, sb = run(slice(b, b + 1), i.state_in[b:b + 1].contiguous(), split=False)
-            assert torch.equal(yb[0], y[b]) and torch.equal(sb[0], s[b])
-        gf.last_device_status()
+    for b, h in parts(B, H):
+        yb, sb = run(b, h, i.state_in[b, h].contiguous(), split=False)
+        assert torch.equal(yb, y[b, :, h]) and torch.equal(sb, s[b, h])
+    gf.last_device_status()
     if T <= 321 and not c2:
         y_ref, s_ref = orc.prefill(*(t.cpu() for t in (i.r, i.k, i.v, i.x, i.u, i.state_in)))
         assert orc.rel_l2(y.float().cpu().numpy(), y_ref) <= 5e-3      # the contract's tolerance
@@ -143,34 +151,34 @@ def test_packed_training_forward_as_a_stream(c2):
     gf.last_device_status()
 
 
-@pytest.mark.parametrize("B,T,H", SHAPES[:3] + [(6, 200, 32)])
+@pytest.mark.parametrize("B,T,H", SHAPES + [(6, 200, 32)])
 @pytest.mark.parametrize("c2", [False, True])
 @pytest.mark.parametrize("x_hi,with_dstate", [(-1.0, True), (2.5, False)])
 def test_gradient_units_cut_between_ctas(B, T, H, c2, x_hi, with_dstate):
-    # each sequence on its own (few units and short: one CTA per unit) gives the same bits; the bonus gradient, summed over
-    # the batch, to fp32 rounding of its B * T terms
+    # each part on its own (few units and short, or more than half the SMs: one CTA per unit) gives the same bits; the bonus
+    # gradient, summed over the batch, to fp32 rounding of its B * T terms
     i = synth.make_dense(B, T, H, 64, "bf16", seed=B + 3 * T + H, device=DEV, state_std=0.1, x_hi=x_hi)
     g = torch.Generator(device=DEV).manual_seed(6)
     dy = torch.randn(i.r.shape, device=DEV, generator=g).bfloat16()
     ds = torch.randn(i.state_in.shape, device=DEV, generator=g) if with_dstate else None
 
-    def grad(sl):
-        t = [x[sl].contiguous() for x in (i.r, i.k, i.v, i.x)]
-        kw = dict(state_in=i.state_in[sl].contiguous(), dstate_out=None if ds is None else ds[sl].contiguous(), want_dstate=with_dstate)
+    def grad(b, h):
+        t = [x[b, :, h].contiguous() for x in (i.r, i.k, i.v, i.x)]
+        kw = dict(state_in=i.state_in[b, h].contiguous(), dstate_out=None if ds is None else ds[b, h].contiguous(), want_dstate=with_dstate)
         if c2:
-            return gf.backward_c2(*t, dy[sl].contiguous(), **kw)
-        return gf.backward(*t, i.u, dy[sl].contiguous(), **kw)
+            return gf.backward_c2(*t, dy[b, :, h].contiguous(), **kw)
+        return gf.backward(*t, i.u[h].contiguous(), dy[b, :, h].contiguous(), **kw)
 
-    full = grad(slice(None))
+    full = grad(slice(None), slice(None))
     du = torch.zeros_like(i.u, dtype=torch.float64)
-    for b in range(B):
-        one = grad(slice(b, b + 1))
+    for b, h in parts(B, H):
+        one = grad(b, h)
         for n in range(4):
-            assert torch.equal(one[n][0], full[n][b]), (b, n)
+            assert torch.equal(one[n], full[n][b, :, h]), (b, h, n)
         if with_dstate:
-            assert torch.equal(one[-1][0], full[-1][b])
+            assert torch.equal(one[-1], full[-1][b, h])
         if not c2:
-            du += one[4].double()
+            du[h] += one[4].double()
     if not c2:
         assert float((full[4].double() - du).norm() / du.norm()) < 1e-5
     gf.last_device_status()
