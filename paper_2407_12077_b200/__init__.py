@@ -152,7 +152,7 @@ _HERE = _Here()
 
 def _on(t: torch.Tensor):
     """Context in which the tensor's device is the current one.  torch.cuda.device costs microseconds of host time per
-    call (a prefill call of one short prompt: 30 us enqueued with it, 21 us without), so it is only entered when the
+    call (the pass of one short prompt: 21.9 us with it, 15.3 us without), so it is only entered when the
     device has to change."""
     return _HERE if t.get_device() == torch.cuda.current_device() else torch.cuda.device(t.device)
 

@@ -145,8 +145,8 @@ __device__ __forceinline__ float2 one_minus_ex2_2(float2 l)
 
 __device__ __forceinline__ void tmem_ld_done() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 
-// NB = 8-column blocks per lane: 4 (groups of 8 warps, 16 cells per lane, 128 registers) or 2 (groups of 16 warps,
-// 8 cells per lane, 64 registers)
+// 8-column blocks per lane: groups of 8 warps, 16 cells per lane, 128 registers.  (Groups of 16 warps with two blocks per lane
+// and 64 registers spilled; the reduction of the bonus terms is written for four.)
 constexpr int G_NB = 4;
 constexpr int G_NSLAB = 8 / G_NB;                 // column slabs of 8 NB columns per tile = warps per row group
 constexpr int G_H2 = G_NB / 2;                    // 16-column blocks per lane
@@ -159,9 +159,9 @@ constexpr int GO_IN = 0;                          // x, r, k, v, dy
 constexpr int GO_RH = GO_IN + 5 * TILE;           // R^ [t][c]
 constexpr int GO_KH = GO_RH + TILE;               // K^ [i][c]
 constexpr int GO_T4 = GO_KH + TILE;               // S_0, G^, P', dP' operand tiles; later the dr, dk, dv, dx staging tiles
-constexpr int GO_TOT = GO_T4 + 4 * TILE;          // [4][64] float: row-group totals of a scan
+constexpr int GO_TOT = GO_T4 + 4 * TILE;          // [NSLAB][64] float: a scan's totals per channel by column slab
 constexpr int GO_EP = GO_TOT + 1024;              // [NSLAB][64] float: partial E by column slab
-constexpr int GO_BP = GO_EP + 1024;               // [NSLAB][64] float: partial bonus by column slab
+constexpr int GO_BP = GO_EP + 1024;               // [4][64] float: partial bonus per token by row group
 constexpr int GO_DPD = GO_BP + 1024;              // [64] float: dy_t . v_t
 constexpr int GO_RED = GO_DPD + 256;              // token-by-token path: [NSLAB][3][64]
 constexpr int GO_REDV = GO_RED + 4 * 3 * 64 * 4;  //   [4][64]
