@@ -72,12 +72,6 @@ namespace ck {
 constexpr int L = 64;                  // tokens per chunk
 constexpr int TILE = 64 * 64 * 2;      // one bf16 [64 x 64] tile
 constexpr int NS = 5;                  // {x,r,k,v} ring depth
-// Copies in flight per CTA at most: the producer requests chunk c once the copy of chunk c - LOAD_AHEAD has landed.  A set of
-// elementwise warps takes every N_ESET-th chunk and so meets only every other phase of a stage (the ring's depth is odd); by its
-// parity alone it would also be let through to chunk c while the copy of chunk c - NS, which had the stage before, is still
-// landing.  When it waits for chunk c it has scaled chunk c - N_ESET, which was requested after chunk c - N_ESET - LOAD_AHEAD
-// had landed, and with it all chunks up to c - NS.
-constexpr int LOAD_AHEAD = 3;
 constexpr int NSB = 2;                 // bf16 chunk-start state operand tiles (by chunk parity)
 constexpr int NPP = 2;                 // bf16 masked-score operand tiles (by chunk parity)
 constexpr int NSIDE = 8;               // ring of per-chunk side vectors (chunk decay, bonus, safety flag): deeper than
@@ -85,7 +79,12 @@ constexpr int NSIDE = 8;               // ring of per-chunk side vectors (chunk 
 constexpr int NTOT = 4;                // per-warp decay-total buffers (two per elementwise set)
 constexpr int N_EW = 8;                // elementwise warps per set
 constexpr int N_ESET = 2;              // elementwise sets (alternate chunks)
-static_assert(LOAD_AHEAD + N_ESET <= NS, "a set may be let through to a stage whose previous copy has not landed");
+// The ring is waited on by two sets that take alternate chunks, and its depth is odd: a stage belongs to either set in turn.  A
+// wait names a phase by its parity alone, so a set has to meet every phase of the barriers it waits on.  Hence a "full" barrier
+// per stage and set: chunk c completes phase c / N_FULL of barrier c % N_FULL, which only set c % N_ESET waits on.  (One barrier
+// per stage would let a set through to chunk c while the copy of chunk c - NS, which had the stage before, is still landing.)
+constexpr int N_FULL = NS % N_ESET ? N_ESET * NS : NS;
+static_assert(N_FULL % N_ESET == 0 && N_FULL % NS == 0, "a barrier belongs to one stage and one set");
 constexpr int N_GW = 4;                // warps per tensor-memory reader group (one per sub-partition)
 constexpr int WARP_MMA_F = 1;          // issues P = R^ K^^T and dS = K^^T V; owns the tensor-memory allocation
 constexpr int WARP_MMA_B = 2;          // issues Y = R^ S_0 + P' V
@@ -119,8 +118,8 @@ constexpr int OFF_ABORT = OFF_SAFE + NSIDE * 4;            // int
 constexpr int OFF_TMEM = OFF_ABORT + 8;                    // uint32: tensor-memory base address
 constexpr int OFF_BAR = OFF_ABORT + 16;                    // mbarriers (8 bytes each)
 enum {
-    BAR_FULL_RKV = 0,
-    BAR_EMPTY_RKV = BAR_FULL_RKV + NS,
+    BAR_FULL_RKV = 0,                    // copies of a chunk landed (by chunk modulo N_FULL)
+    BAR_EMPTY_RKV = BAR_FULL_RKV + N_FULL,     // (from here on by stage)
     BAR_RK_READY = BAR_EMPTY_RKV + NS,
     BAR_S_READY = BAR_RK_READY + NS,     // bf16 state operand tile written            (by chunk parity)
     BAR_PP_READY = BAR_S_READY + 2,      // masked-score operand tile written
@@ -906,8 +905,8 @@ wkv6_chunked_kernel(const __grid_constant__ CUtensorMap tm_r, const __grid_const
     };
 
     if (tid == 0) {
+        for (int i = 0; i < N_FULL; ++i) mbar_init(bar(BAR_FULL_RKV + i), 1);
         for (int i = 0; i < NS; ++i) {
-            mbar_init(bar(BAR_FULL_RKV + i), 1);
             mbar_init(bar(BAR_EMPTY_RKV + i), 1);                  // the commit after the last product that reads the stage
             mbar_init(bar(BAR_RK_READY + i), N_EW);
         }
@@ -955,7 +954,7 @@ wkv6_chunked_kernel(const __grid_constant__ CUtensorMap tm_r, const __grid_const
         if constexpr (PERSIST) {
             int gc = 0, real_end = -1;               // chunks of the stream issued so far; index of the first end marker
             int s = 0, ph = 1;                       // ring stage and the parity of its previous release
-            int fs = 0, fph = 0;                     // stage and phase bit of the copy that has to have landed (LOAD_AHEAD)
+            int fb = 0;                              // "full" barrier of the next chunk
             bool alive = true;
             for (int k = 0; alive; ++k) {
                 int u = 0, c0 = 0, c1 = 0;               // the next piece: chunks c0 .. c1-1 of unit u (balanced launches)
@@ -1036,24 +1035,22 @@ wkv6_chunked_kernel(const __grid_constant__ CUtensorMap tm_r, const __grid_const
                 }
                 for (int c = c0; c < c1; ++c, ++gc) {
                     if (gc >= NS && !mbar_wait_warp(bar(BAR_EMPTY_RKV + s), ph, abort_flag)) { alive = false; break; }
-                    if (gc >= LOAD_AHEAD) {
-                        if (!mbar_wait_warp(bar(BAR_FULL_RKV + fs), fph, abort_flag)) { alive = false; break; }
-                        if (++fs == NS) { fs = 0; fph ^= 1; }
-                    }
                     const int row = (int)(urow0 + (long long)c * L);
                     const uint32_t dst = sbase + OFF_RING + s * STAGE;
                     if (elect_one()) {
                         int meta = min(L, ulen - c * L) | (c == c0 ? DESC_FIRST : 0) | (int)((unsigned)uh << 16);
                         if (BAL) meta |= (c == c0 && c0 > 0 ? DESC_CONT : 0) | (c == c1 - 1 ? DESC_LAST : 0);
                         put_desc(gc, row, meta, u, unch - 1 - c);
-                        mbar_expect_tx(bar(BAR_FULL_RKV + s), STAGE);      // (release: the descriptor is visible to the waiters)
-                        tma_load_2d(dst, &tm_x, uh * 64, row, bar(BAR_FULL_RKV + s));
-                        tma_load_2d(dst + TILE, &tm_r, uh * 64, row, bar(BAR_FULL_RKV + s));
-                        tma_load_2d(dst + 2 * TILE, &tm_k, uh * 64, row, bar(BAR_FULL_RKV + s));
-                        tma_load_2d(dst + 3 * TILE, &tm_v, uh * 64, row, bar(BAR_FULL_RKV + s));
+                        const uint32_t full = bar(BAR_FULL_RKV + fb);
+                        mbar_expect_tx(full, STAGE);                       // (release: the descriptor is visible to the waiters)
+                        tma_load_2d(dst, &tm_x, uh * 64, row, full);
+                        tma_load_2d(dst + TILE, &tm_r, uh * 64, row, full);
+                        tma_load_2d(dst + 2 * TILE, &tm_k, uh * 64, row, full);
+                        tma_load_2d(dst + 3 * TILE, &tm_v, uh * 64, row, full);
                     }
                     __syncwarp();
                     if (++s == NS) { s = 0; ph ^= 1; }
+                    if (++fb == N_FULL) fb = 0;
                 }
             }
             if (alive) {
@@ -1063,10 +1060,11 @@ wkv6_chunked_kernel(const __grid_constant__ CUtensorMap tm_r, const __grid_const
                     if (gc >= NS && !mbar_wait_warp(bar(BAR_EMPTY_RKV + s), ph, abort_flag)) { alive = false; break; }
                     if (elect_one()) {
                         put_desc(gc, 0, DESC_END, 0, 0);
-                        mbar_arrive(bar(BAR_FULL_RKV + s));                 // no copy: the arrival alone completes the phase
+                        mbar_arrive(bar(BAR_FULL_RKV + fb));                // no copy: the arrival alone completes the phase
                     }
                     __syncwarp();
                     if (++s == NS) { s = 0; ph ^= 1; }
+                    if (++fb == N_FULL) fb = 0;
                 }
             }
             // Do not leave while copies into this CTA's shared memory may still be in flight.  A stage that an end
@@ -1074,33 +1072,31 @@ wkv6_chunked_kernel(const __grid_constant__ CUtensorMap tm_r, const __grid_const
             const int issued = real_end >= 0 ? real_end : gc;
             const int from = (real_end >= 0 && alive) ? max(0, issued - NS + 2) : max(0, issued - NS);
             for (int c = from; c < issued; ++c)
-                mbar_wait_warp(bar(BAR_FULL_RKV + c % NS), (c / NS) & 1, abort_flag, false);
+                mbar_wait_warp(bar(BAR_FULL_RKV + c % N_FULL), (c / N_FULL) & 1, abort_flag, false);
         } else {
             int issued = 0;
             int s = 0, ph = 1;                       // ring stage and the parity of its previous release
-            int fs = 0, fph = 0;                     // stage and phase bit of the copy that has to have landed (LOAD_AHEAD)
+            int fb = 0;                              // "full" barrier of the next chunk
             int row = (int)row0;
             for (int c = 0; c < nchunks; ++c, row += L) {
                 if (c >= NS && !mbar_wait_warp(bar(BAR_EMPTY_RKV + s), ph, abort_flag)) break;
-                if (c >= LOAD_AHEAD) {
-                    if (!mbar_wait_warp(bar(BAR_FULL_RKV + fs), fph, abort_flag)) break;
-                    if (++fs == NS) { fs = 0; fph ^= 1; }
-                }
                 const uint32_t dst = sbase + OFF_RING + s * STAGE;
                 if (elect_one()) {
-                    mbar_expect_tx(bar(BAR_FULL_RKV + s), SUMMARY ? 3 * TILE : STAGE);
-                    tma_load_2d(dst, &tm_x, col0, row, bar(BAR_FULL_RKV + s));
-                    if (!SUMMARY) tma_load_2d(dst + TILE, &tm_r, col0, row, bar(BAR_FULL_RKV + s));
-                    tma_load_2d(dst + 2 * TILE, &tm_k, col0, row, bar(BAR_FULL_RKV + s));
-                    tma_load_2d(dst + 3 * TILE, &tm_v, col0, row, bar(BAR_FULL_RKV + s));
+                    const uint32_t full = bar(BAR_FULL_RKV + fb);
+                    mbar_expect_tx(full, SUMMARY ? 3 * TILE : STAGE);
+                    tma_load_2d(dst, &tm_x, col0, row, full);
+                    if (!SUMMARY) tma_load_2d(dst + TILE, &tm_r, col0, row, full);
+                    tma_load_2d(dst + 2 * TILE, &tm_k, col0, row, full);
+                    tma_load_2d(dst + 3 * TILE, &tm_v, col0, row, full);
                 }
                 __syncwarp();
                 issued = c + 1;
                 if (++s == NS) { s = 0; ph ^= 1; }
+                if (++fb == N_FULL) fb = 0;
             }
             // do not leave while copies into this CTA's shared memory may still be in flight
             for (int c = max(0, issued - NS); c < issued; ++c)
-                mbar_wait_warp(bar(BAR_FULL_RKV + c % NS), (c / NS) & 1, abort_flag, false);
+                mbar_wait_warp(bar(BAR_FULL_RKV + c % N_FULL), (c / N_FULL) & 1, abort_flag, false);
         }
     } else if (warp == WARP_MMA_F) {
         // ============================== MMA issuer, input-only products ==============================
@@ -1665,14 +1661,15 @@ wkv6_chunked_kernel(const __grid_constant__ CUtensorMap tm_r, const __grid_const
 #pragma unroll
         for (int tt = 0; tt < 4; ++tt) roff[tt] = swz(8 * tq + 4 * th + tt, 8 * cq);
         const float2 kLog2e = make_float2(LOG2E, LOG2E), kLogLog = make_float2(LOG2_LOG2E, LOG2_LOG2E);
-        int s = eset, ph = 0;                            // ring stage of this set's current chunk and its phase bit
+        int s = eset;                                    // ring stage of this set's current chunk,
+        int fb = eset, ph = 0;                           // its "full" barrier and that one's phase bit
         for (int c = eset; PERSIST || c < nchunks; c += N_ESET) {
             const int sd = c & (NSIDE - 1);
             const uint32_t tx = sbase + OFF_RING + s * STAGE, tv = tx + 3 * TILE;
             uint32_t ax[4];                              // this lane's 8 bytes in its 4 rows of the x tile; r at +TILE, k at +2 TILE
 #pragma unroll
             for (int tt = 0; tt < 4; ++tt) ax[tt] = tx + roff[tt];
-            if (!mbar_wait(bar(BAR_FULL_RKV + s), ph, abort_flag)) break;
+            if (!mbar_wait(bar(BAR_FULL_RKV + fb), ph, abort_flag)) break;
             Chunk ck;                                    // (this role needs the valid-token count, the head and the end flag only)
             if constexpr (PERSIST) {
                 const uint32_t meta = lds32(sbase + OFF_DESC + 16 * (c & (NSIDE - 1)) + 4);
@@ -1815,7 +1812,9 @@ wkv6_chunked_kernel(const __grid_constant__ CUtensorMap tm_r, const __grid_const
             __syncwarp();
             mbar_arrive_if(bar(BAR_RK_READY + s), lane == 0);
             s += N_ESET;
-            if (s >= NS) { s -= NS; ph ^= 1; }
+            if (s >= NS) s -= NS;
+            fb += N_ESET;
+            if (fb >= N_FULL) { fb -= N_FULL; ph ^= 1; }
         }
     }
 
