@@ -143,8 +143,7 @@ constexpr int OFF_DESC = (OFF_BAR + BAR_COUNT * 8 + 15) & ~15;   // [NSIDE] int4
 // a unit another CTA began, last chunk of a piece
 constexpr int DESC_FIRST = 0x100, DESC_END = 0x200, DESC_CONT = 0x400, DESC_LAST = 0x800;
 constexpr int DESC_TAG = 0x1000;                                 // (balanced launches) parity of the ring's turn: (chunk / NSIDE) & 1
-constexpr int OFF_MARK = OFF_DESC + NSIDE * 16;                  // int: the segment's state became non-finite (Params::trail)
-constexpr int SMEM_BYTES = OFF_MARK + 16;
+constexpr int SMEM_BYTES = OFF_DESC + NSIDE * 16;
 constexpr int SMEM_ALLOC = SMEM_BYTES + 1024;              // slack for manual 1024-byte alignment
 static_assert(SMEM_ALLOC <= 232448, "shared memory budget of one sm_100 CTA");
 
@@ -553,13 +552,13 @@ struct Params {
     // subnormal, 2^-150, whatever comes after it: dS forgets what lies before such a run, and D is zero.  So the CTA first
     // sums the decays of its segment's last chunks, TRAIL_CHUNKS at a time and at most TRAIL_LOOKS times, and runs from the
     // last chunk boundary after which every channel has decayed that far, if there is one.  What no finite value survives, a
-    // NaN or infinity before that boundary does: see poison_later_segments.
+    // NaN or infinity before that boundary does: see wkv6_mark_kernel.
     int trail;
 };
 constexpr int SUMMARY_FLOATS = 64 + 64 * 64;
 constexpr float TRAIL_LOG2 = 280.f;    // (278, and a margin for the rounding of the sums)
-constexpr int TRAIL_CHUNKS = 30;       // (one per warp)
-constexpr int TRAIL_LOOKS = 3;
+constexpr int TRAIL_CHUNKS = 15;       // (two warps each)
+constexpr int TRAIL_LOOKS = 6;
 
 // Writes a warp's 16 x 64 fp32 accumulator block (acc[n][0..1] = row g, cols 8n+2q,+1;
 // acc[n][2..3] = row g+8) as bf16 into rows row0 .. row0+15 of a 128B-swizzled [rows][64] tile.
@@ -705,66 +704,6 @@ __device__ __forceinline__ void exact_chunk(float* scr, const Params& p, int h, 
     }
 }
 
-// Main launch of a split call whose summary launch may have started late in its segments (Params::trail): a segment's state
-// that has become non-finite goes on being so, although the summary did not see it.  A CTA whose segment ends like that
-// writes NaN over those elements of its summary's dS (from_marks) and says so in the sign of D[1]; every CTA says in the
-// sign of D[0] of the summary before its segment that its outputs are written (D is a decay, readers drop the signs).
-// Whichever of two CTAs of a unit comes second sees the other's word (both sequentially consistent) and makes the marked
-// columns of the later segment's outputs NaN, and the marked elements of the final state and (CKPT) of the segment's
-// checkpoints.  Runs after the CTA's last barrier; without a mark it costs a few words of memory traffic per CTA.
-// first_slot: the unit's first checkpoint slot.
-template <bool CKPT>
-__device__ __forceinline__ void poison_later_segments(const Params& p, int unit, int seg, bool marked, int* mark, int* todo, size_t first_slot)
-{
-    const int tid = threadIdx.x, nseg = p.nseg;
-    unsigned* base = reinterpret_cast<unsigned*>(p.summaries) + (size_t)unit * (nseg - 1) * SUMMARY_FLOATS;
-    if (tid == 0) {
-        // todo: bit g (g < seg): this segment takes the marks of segment g; bit g > seg: segment g takes this one's
-        int t = 0;
-        asm volatile("fence.sc.gpu;" ::: "memory");
-        if (marked && seg < nseg - 1) atomicOr(base + (size_t)seg * SUMMARY_FLOATS + 1, 0x80000000u);
-        if (seg > 0) atomicOr(base + (size_t)(seg - 1) * SUMMARY_FLOATS, 0x80000000u);
-        asm volatile("fence.sc.gpu;" ::: "memory");
-        for (int g = 0; g < nseg; ++g) {
-            if (g < seg && (atomicOr(base + (size_t)g * SUMMARY_FLOATS + 1, 0u) >> 31)) t |= 1 << g;
-            if (marked && g > seg && (atomicOr(base + (size_t)(g - 1) * SUMMARY_FLOATS, 0u) >> 31)) t |= 1 << g;
-        }
-        asm volatile("fence.sc.gpu;" ::: "memory");
-        *todo = t;
-    }
-    __syncthreads();
-    const int t = *todo;
-    if (t == 0) return;
-    const int seq = unit / p.H, h = unit % p.H;
-    const long long row0 = p.cu_seqlens ? p.cu_seqlens[seq] : (long long)seq * p.T;
-    const int len = p.cu_seqlens ? p.cu_seqlens[seq + 1] - p.cu_seqlens[seq] : p.T;
-    const float nan = __int_as_float(0x7fc00000);
-    for (int g = 0; g < nseg; ++g) {
-        if (!(t >> g & 1)) continue;
-        const int from = g < seg ? g : seg, to = g < seg ? seg : g;
-        const float* ds = reinterpret_cast<const float*>(base + (size_t)from * SUMMARY_FLOATS + 64);
-        const int first = min(len, to * p.seg_chunks * L), end = to == nseg - 1 ? len : min(len, first + p.seg_chunks * L);
-        // the states before the segment's chunks, and after the last one of the unit
-        const int ck_first = (first + L - 1) / L, ck_end = (end + L - 1) / L + (to == nseg - 1 ? 1 : 0);
-        __syncthreads();
-        if (tid < 64) mark[tid] = 0;
-        __syncthreads();
-        for (int i = tid; i < 4096; i += blockDim.x) {
-            const float v = __ldcg(ds + i);
-            if (v != v) {
-                mark[i & 63] = 1;
-                if (to == nseg - 1 && p.state_out) p.state_out[(size_t)unit * 4096 + i] = nan;
-                if (CKPT)
-                    for (int c = ck_first; c < ck_end; ++c)
-                        reinterpret_cast<__nv_bfloat16*>(p.ckpt)[(first_slot + c) * 4096 + i] = __float2bfloat16_rn(nan);
-            }
-        }
-        __syncthreads();
-        for (long long i = (long long)first * 64 + tid; i < (long long)end * 64; i += blockDim.x)
-            if (mark[i & 63]) p.y[(size_t)(row0 + (i >> 6)) * p.H * 64 + h * 64 + (i & 63)] = __float2bfloat16_rn(nan);
-    }
-}
-
 // ---------------------------------------------------------------- the kernel
 // SUMMARY = false: the prefill proper.  SUMMARY = true: the first pass of a split call, which only
 // carries the state over a segment from a zero start (no r, no scores, no outputs: the score warps and
@@ -776,7 +715,8 @@ __device__ __forceinline__ void poison_later_segments(const Params& p, int unit,
 // stream may begin and end inside a unit (see Params::bal_chunks).
 // CKPT = true (launches of the prefill proper): the state before every chunk and after the last one is also left in
 // Params::ckpt, for the gradient call that follows a training step's forward pass.
-// TRAIL = true (main launches of split calls): the summary launch may have started late in its segments (see Params::trail).
+// TRAIL = true (main launches of split calls): the summary launch may have started late in its segments (see Params::trail);
+// a segment that ends in a non-finite state is marked for wkv6_mark_kernel.
 template <bool SUMMARY, bool C2, int PERSIST = 0, bool CKPT = false, bool TRAIL = false>
 __global__ void __launch_bounds__(THREADS, 1)
 wkv6_chunked_kernel(const __grid_constant__ CUtensorMap tm_r, const __grid_constant__ CUtensorMap tm_k,
@@ -820,22 +760,24 @@ wkv6_chunked_kernel(const __grid_constant__ CUtensorMap tm_r, const __grid_const
     }
     int trail_cut = 0;                     // (see Params::trail) chunks of the segment that need not be run
     if constexpr (SUMMARY) {
-        // only whole, full segments (of which all but the last chunks may go); one warp per chunk sums it: lane = 4 channels
-        // (lane % 16) of every other row
+        // only whole, full segments (of which all but the last chunks may go); two warps per chunk sum it, 32 tokens each, with
+        // all their loads in flight: lane = 4 channels (lane % 16) of every other row
         const int n_full = len / L;
         if (p.trail && len % L == 0 && n_full > 1) {
-            float* tot = reinterpret_cast<float*>(smem);           // [TRAIL_CHUNKS][64] (the ring: nothing has been loaded yet)
+            float* tot = reinterpret_cast<float*>(smem);           // [TRAIL_CHUNKS][2][64] (the ring: nothing has been loaded yet)
             float a0 = 0.f, a1 = 0.f;                              // every warp finds the same answer: two channels per lane
             for (int k0 = 0; k0 < min(TRAIL_LOOKS * TRAIL_CHUNKS, n_full - 1) && !trail_cut; k0 += TRAIL_CHUNKS) {
-                const int look = min(TRAIL_CHUNKS, n_full - 1 - k0), cw = n_full - 1 - k0 - warp;        // (this warp's chunk)
-                if (warp < look) {
-                    const __nv_bfloat16* xp = p.x + (size_t)(row0 + (long long)cw * L + (lane >> 4)) * ((size_t)p.H * 64) + h * 64 + 4 * (lane & 15);
+                const int look = min(TRAIL_CHUNKS, n_full - 1 - k0), cw = n_full - 1 - k0 - (warp >> 1);      // (this warp's chunk)
+                if (warp < 2 * look) {
+                    const __nv_bfloat16* xp = p.x + (size_t)(row0 + (long long)cw * L + 32 * (warp & 1) + (lane >> 4)) * ((size_t)p.H * 64) + h * 64 + 4 * (lane & 15);
+                    uint2 w[L / 4];
+#pragma unroll
+                    for (int t = 0; t < L / 4; ++t) w[t] = *reinterpret_cast<const uint2*>(xp + (size_t)(2 * t) * ((size_t)p.H * 64));
                     float e[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll 16
-                    for (int t = 0; t < L / 2; ++t) {
-                        const uint2 w = *reinterpret_cast<const uint2*>(xp + (size_t)(2 * t) * ((size_t)p.H * 64));
-                        e[0] += ex2(fmaf(bf_lo(w.x), LOG2E, LOG2_LOG2E)); e[1] += ex2(fmaf(bf_hi(w.x), LOG2E, LOG2_LOG2E));
-                        e[2] += ex2(fmaf(bf_lo(w.y), LOG2E, LOG2_LOG2E)); e[3] += ex2(fmaf(bf_hi(w.y), LOG2E, LOG2_LOG2E));
+#pragma unroll
+                    for (int t = 0; t < L / 4; ++t) {
+                        e[0] += ex2(fmaf(bf_lo(w[t].x), LOG2E, LOG2_LOG2E)); e[1] += ex2(fmaf(bf_hi(w[t].x), LOG2E, LOG2_LOG2E));
+                        e[2] += ex2(fmaf(bf_lo(w[t].y), LOG2E, LOG2_LOG2E)); e[3] += ex2(fmaf(bf_hi(w[t].y), LOG2E, LOG2_LOG2E));
                     }
 #pragma unroll
                     for (int i = 0; i < 4; ++i) e[i] += __shfl_xor_sync(0xffffffffu, e[i], 16);
@@ -843,12 +785,13 @@ wkv6_chunked_kernel(const __grid_constant__ CUtensorMap tm_r, const __grid_const
                 }
                 __syncthreads();
                 for (int k = 0; k < look; ++k) {                   // chunks from the last one back
-                    a0 += tot[k * 64 + 2 * lane]; a1 += tot[k * 64 + 2 * lane + 1];
+                    a0 += tot[k * 128 + 2 * lane] + tot[k * 128 + 64 + 2 * lane]; a1 += tot[k * 128 + 2 * lane + 1] + tot[k * 128 + 64 + 2 * lane + 1];
                     if (__all_sync(0xffffffffu, a0 > TRAIL_LOG2 && a1 > TRAIL_LOG2)) { trail_cut = n_full - 1 - k0 - k; break; }     // (false for NaN)
                 }
                 __syncthreads();                                   // (the sums are read before they, or the ring, are written again)
-                // (decays that one look leaves below a third of the way are too slow for the others)
-                if (!__all_sync(0xffffffffu, a0 > TRAIL_LOG2 / TRAIL_LOOKS && a1 > TRAIL_LOG2 / TRAIL_LOOKS)) break;
+                // (decays that have not come their share of the way are too slow for the looks that are left)
+                const float share = TRAIL_LOG2 / TRAIL_LOOKS * (float)(k0 / TRAIL_CHUNKS + 1);
+                if (!__all_sync(0xffffffffu, a0 > 0.9f * share && a1 > 0.9f * share)) break;
             }
             row0 += (long long)trail_cut * L;
             len -= trail_cut * L;
@@ -928,7 +871,6 @@ wkv6_chunked_kernel(const __grid_constant__ CUtensorMap tm_r, const __grid_const
             for (int i = 0; i < NSIDE; ++i) sts32(sbase + OFF_DESC + 16 * i + 4, DESC_TAG);        // (of the turn before the first)
         sts32(abort_flag, 0u);
         sts32(abort_flag + 4, p.wait_limit_us ? p.wait_limit_us : WAIT_LIMIT_US);
-        if (TRAIL) sts32(sbase + OFF_MARK, 0u);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         fence_proxy_async();
     }
@@ -1225,7 +1167,7 @@ wkv6_chunked_kernel(const __grid_constant__ CUtensorMap tm_r, const __grid_const
             for (int gg = 0; gg < seg; ++gg) {
                 const float* sm = p.summaries + ((size_t)unit * (p.nseg - 1) + gg) * SUMMARY_FLOATS;
                 float d_lo = sm[c_lo], d_hi = sm[c_lo + 8];
-                if (TRAIL) { d_lo = fabsf(d_lo); d_hi = fabsf(d_hi); }               // (signs: see poison_later_segments)
+                if (TRAIL) { d_lo = fabsf(d_lo); d_hi = fabsf(d_hi); }               // (the signs are marks)
 #pragma unroll
                 for (int n = 0; n < 8; ++n) {
                     const float2 lo = *reinterpret_cast<const float2*>(sm + 64 + c_lo * 64 + 8 * n + 2 * q);
@@ -1426,7 +1368,8 @@ wkv6_chunked_kernel(const __grid_constant__ CUtensorMap tm_r, const __grid_const
         } else if (!PERSIST && p.state_out && seg == p.nseg - 1 && !lds32(abort_flag)) {
             store_state(sb);
         } else if (TRAIL && seg < p.nseg - 1) {
-            // a state that is no longer finite: marked in the segment's summary (see poison_later_segments)
+            // a state that is no longer finite: NaN over those elements of the segment's dS, and the sign of D[1] (D is a decay,
+            // readers drop the sign).  A later segment's CTA that folds this summary meanwhile may see either.
             float z = 0.f;
 #pragma unroll
             for (int n = 0; n < 8; ++n)
@@ -1439,8 +1382,7 @@ wkv6_chunked_kernel(const __grid_constant__ CUtensorMap tm_r, const __grid_const
 #pragma unroll
                     for (int e = 0; e < 4; ++e)
                         if (st[n][e] * 0.f != 0.f) sm[(size_t)(e < 2 ? c_lo : c_lo + 8) * 64 + 8 * n + 2 * q + (e & 1)] = __int_as_float(0x7fc00000);
-                __threadfence();
-                sts32(sbase + OFF_MARK, 1u);
+                atomicOr(reinterpret_cast<unsigned*>(sm) - 63, 0x80000000u);
             }
         }
     } else if (warp < WARP_Y0) {
@@ -1825,9 +1767,48 @@ wkv6_chunked_kernel(const __grid_constant__ CUtensorMap tm_r, const __grid_const
         tc_fence_after();
         tmem_dealloc(tmem, TM_COLS);
     }
-    if (TRAIL)
-        poison_later_segments<CKPT>(p, unit, seg, lds32(sbase + OFF_MARK) != 0, reinterpret_cast<int*>(smem + OFF_TOT),
-                                    reinterpret_cast<int*>(smem + OFF_TOT) + 64, CKPT ? ckpt_slot(0) : 0);
+}
+
+// Behind the main launch of a split call whose summary launch may have started late in its segments (Params::trail): a
+// segment's state that has become non-finite goes on being so, although its summary did not see it.  The main launch has marked
+// such a segment; the marked columns of the later segments' outputs become NaN, and the marked elements of their checkpoints
+// (ckpt, dense) and of the final state.  One CTA per unit and segment but the first; without a mark it reads a word per segment.
+// (The main launch's CTAs did this at their own ends before, and had to tell one another what they had marked and written.)
+constexpr int MARK_THREADS = 256;
+__global__ void __launch_bounds__(MARK_THREADS)
+wkv6_mark_kernel(const float* summaries, int nseg, int seg_chunks, const int32_t* cu, int T, int H, __nv_bfloat16* y, float* state_out,
+                 __nv_bfloat16* ckpt)
+{
+    __shared__ int mark[64];
+    asm volatile("griddepcontrol.launch_dependents;\n\tgriddepcontrol.wait;" ::: "memory");
+    const int unit = blockIdx.x / (nseg - 1), to = blockIdx.x % (nseg - 1) + 1, tid = threadIdx.x;
+    const float* sm = summaries + (size_t)unit * (nseg - 1) * SUMMARY_FLOATS;
+    auto marked = [&](int from) { return (__float_as_uint(sm[(size_t)from * SUMMARY_FLOATS + 1]) >> 31) != 0; };
+    if (!__syncthreads_or(tid < to && marked(tid))) return;
+    const int seq = unit / H, h = unit % H;
+    const long long row0 = cu ? cu[seq] : (long long)seq * T;
+    const int len = cu ? cu[seq + 1] - cu[seq] : T;
+    const int first = min(len, to * seg_chunks * L), end = to == nseg - 1 ? len : min(len, first + seg_chunks * L);
+    // the states before the segment's chunks, and after the last one of the unit
+    const int ck_first = (first + L - 1) / L, ck_end = (end + L - 1) / L + (to == nseg - 1 ? 1 : 0);
+    const size_t slot0 = (size_t)unit * ((T + L - 1) / L + 1);
+    const float nan = __int_as_float(0x7fc00000);
+    if (tid < 64) mark[tid] = 0;
+    __syncthreads();
+    for (int from = 0; from < to; ++from) {
+        if (!marked(from)) continue;
+        for (int i = tid; i < 4096; i += MARK_THREADS) {
+            const float v = sm[(size_t)from * SUMMARY_FLOATS + 64 + i];
+            if (v == v) continue;
+            mark[i & 63] = 1;
+            if (to == nseg - 1 && state_out) state_out[(size_t)unit * 4096 + i] = nan;
+            if (ckpt)
+                for (int c = ck_first; c < ck_end; ++c) ckpt[(slot0 + c) * 4096 + i] = __float2bfloat16_rn(nan);
+        }
+    }
+    __syncthreads();
+    for (long long i = (long long)first * 64 + tid; i < (long long)end * 64; i += MARK_THREADS)
+        if (mark[i & 63]) y[(size_t)(row0 + (i >> 6)) * H * 64 + h * 64 + (i & 63)] = __float2bfloat16_rn(nan);
 }
 
 // One warp that waits, with the kernel's own bounded wait, on a barrier nobody arrives on: the wait runs out after
@@ -1945,6 +1926,15 @@ inline bool chunked_kernel_attributes()
         attr_set.set(dev);
     }
     return true;
+}
+
+// wkv6_mark_kernel behind the main launch of a split call with late starts
+inline gf_status_t launch_marks(const ck::Params& p, long long units, cudaStream_t st, std::atomic<uint64_t>* launches)
+{
+    const cudaError_t e = launch_pdl(ck::wkv6_mark_kernel, (unsigned)(units * (p.nseg - 1)), ck::MARK_THREADS, 0, st, p.summaries, p.nseg, p.seg_chunks,
+                                     p.cu_seqlens, p.T, p.H, p.y, p.state_out, reinterpret_cast<__nv_bfloat16*>(p.ckpt));
+    launches->fetch_add(1, std::memory_order_relaxed);
+    return e == cudaSuccess ? GF_OK : GF_ERR_CUDA;
 }
 
 // Prepares the scratch of a packed persistent launch: zeroes the unit counter and, for up to ORDER_MAX_SEQ
@@ -2110,7 +2100,8 @@ inline gf_status_t chunked_prefill(const __nv_bfloat16* r, const __nv_bfloat16* 
                                     : (c2 ? ck::wkv6_chunked_kernel<false, true, 0, true> : ck::wkv6_chunked_kernel<false, false, 0, true>);
         kernel<<<(unsigned)(units * nseg), ck::THREADS, ck::SMEM_ALLOC, st>>>(tr, tk, tv, tx, ty, tu2, p, tck);
         launches->fetch_add(1, std::memory_order_relaxed);
-        return cudaGetLastError() == cudaSuccess ? GF_OK : GF_ERR_CUDA;
+        if (cudaGetLastError() != cudaSuccess) return GF_ERR_CUDA;
+        return p.trail ? launch_marks(p, units, st, launches) : GF_OK;
     }
     const int n_sm = sm_count();
     // More units than SMs: one CTA per SM walks a stream of units, so that a unit's pipeline fill overlaps the
@@ -2164,7 +2155,8 @@ inline gf_status_t chunked_prefill(const __nv_bfloat16* r, const __nv_bfloat16* 
                                     : (c2 ? ck::wkv6_chunked_kernel<false, true> : ck::wkv6_chunked_kernel<false, false>);
         const cudaError_t e = launch_pdl(kernel, (unsigned)(units * nseg), ck::THREADS, ck::SMEM_ALLOC, st, tr, tk, tv, tx, ty, tu2, p, tck);
         launches->fetch_add(1, std::memory_order_relaxed);
-        return e == cudaSuccess ? GF_OK : GF_ERR_CUDA;
+        if (e != cudaSuccess) return GF_ERR_CUDA;
+        return p.trail ? launch_marks(p, units, st, launches) : GF_OK;
     }
     const cudaError_t e = launch_pdl(c2 ? ck::wkv6_chunked_kernel<false, true> : ck::wkv6_chunked_kernel<false, false>, (unsigned)units, ck::THREADS,
                                      ck::SMEM_ALLOC, st, tr, tk, tv, tx, ty, tu2, p, tck);
