@@ -143,7 +143,8 @@ constexpr int OFF_DESC = (OFF_BAR + BAR_COUNT * 8 + 15) & ~15;   // [NSIDE] int4
 // a unit another CTA began, last chunk of a piece
 constexpr int DESC_FIRST = 0x100, DESC_END = 0x200, DESC_CONT = 0x400, DESC_LAST = 0x800;
 constexpr int DESC_TAG = 0x1000;                                 // (balanced launches) parity of the ring's turn: (chunk / NSIDE) & 1
-constexpr int SMEM_BYTES = OFF_DESC + NSIDE * 16;
+constexpr int OFF_MARK = OFF_DESC + NSIDE * 16;                  // int: the segment's state became non-finite (Params::trail)
+constexpr int SMEM_BYTES = OFF_MARK + 16;
 constexpr int SMEM_ALLOC = SMEM_BYTES + 1024;              // slack for manual 1024-byte alignment
 static_assert(SMEM_ALLOC <= 232448, "shared memory budget of one sm_100 CTA");
 
@@ -552,7 +553,7 @@ struct Params {
     // subnormal, 2^-150, whatever comes after it: dS forgets what lies before such a run, and D is zero.  So the CTA first
     // sums the decays of its segment's last chunks, TRAIL_CHUNKS at a time and at most TRAIL_LOOKS times, and runs from the
     // last chunk boundary after which every channel has decayed that far, if there is one.  What no finite value survives, a
-    // NaN or infinity before that boundary does: see wkv6_mark_kernel.
+    // NaN or infinity before that boundary does: see poison_later_segments.
     int trail;
 };
 constexpr int SUMMARY_FLOATS = 64 + 64 * 64;
@@ -704,6 +705,69 @@ __device__ __forceinline__ void exact_chunk(float* scr, const Params& p, int h, 
     }
 }
 
+// Main launch of a split call whose summary launch may have started late in its segments (Params::trail): a segment's state
+// that has become non-finite goes on being so, although the summary did not see it.  A CTA whose segment ends like that
+// writes NaN over those elements of its summary's dS and says so in the sign of D[1]; every CTA says in the sign of D[0] of
+// the summary before its segment that its outputs are written (D is a decay, readers drop the signs).
+// Whichever of two CTAs of a unit comes second sees the other's word (a sequentially consistent fence lies between what a CTA
+// says and what it reads) and makes the marked columns of the later segment's outputs NaN, and the marked elements of the final
+// state and (CKPT) of the segment's checkpoints.  Runs after the CTA's last barrier; without a mark it costs a fence and a load
+// of one word per segment, by one warp's lanes at once.  first_slot: the unit's first checkpoint slot.
+template <bool CKPT>
+__device__ __forceinline__ void poison_later_segments(const Params& p, int unit, int seg, bool marked, int* mark, int* todo, size_t first_slot)
+{
+    const int tid = threadIdx.x, nseg = p.nseg;
+    unsigned* base = reinterpret_cast<unsigned*>(p.summaries) + (size_t)unit * (nseg - 1) * SUMMARY_FLOATS;
+    if (tid < 32) {
+        // todo: bit g (g < seg): this segment takes the marks of segment g; bit g > seg: segment g takes this one's
+        if (tid == 0) {
+            asm volatile("fence.acq_rel.gpu;" ::: "memory");          // (the outputs and the marked elements before the words)
+            if (marked && seg < nseg - 1) atomicOr(base + (size_t)seg * SUMMARY_FLOATS + 1, 0x80000000u);
+            if (seg > 0) atomicOr(base + (size_t)(seg - 1) * SUMMARY_FLOATS, 0x80000000u);
+        }
+        __syncwarp();
+        asm volatile("fence.sc.gpu;" ::: "memory");
+        unsigned w = 0;
+        if (tid < nseg && (tid < seg || (marked && tid > seg)))
+            asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(w) : "l"(tid < seg ? base + (size_t)tid * SUMMARY_FLOATS + 1
+                                                                                        : base + (size_t)(tid - 1) * SUMMARY_FLOATS) : "memory");
+        const unsigned t = __ballot_sync(0xffffffffu, w >> 31);
+        if (tid == 0) *todo = (int)t;
+        asm volatile("fence.acq_rel.gpu;" ::: "memory");
+    }
+    __syncthreads();
+    const int t = *todo;
+    if (t == 0) return;
+    const int seq = unit / p.H, h = unit % p.H;
+    const long long row0 = p.cu_seqlens ? p.cu_seqlens[seq] : (long long)seq * p.T;
+    const int len = p.cu_seqlens ? p.cu_seqlens[seq + 1] - p.cu_seqlens[seq] : p.T;
+    const float nan = __int_as_float(0x7fc00000);
+    for (int g = 0; g < nseg; ++g) {
+        if (!(t >> g & 1)) continue;
+        const int from = g < seg ? g : seg, to = g < seg ? seg : g;
+        const float* ds = reinterpret_cast<const float*>(base + (size_t)from * SUMMARY_FLOATS + 64);
+        const int first = min(len, to * p.seg_chunks * L), end = to == nseg - 1 ? len : min(len, first + p.seg_chunks * L);
+        // the states before the segment's chunks, and after the last one of the unit
+        const int ck_first = (first + L - 1) / L, ck_end = (end + L - 1) / L + (to == nseg - 1 ? 1 : 0);
+        __syncthreads();
+        if (tid < 64) mark[tid] = 0;
+        __syncthreads();
+        for (int i = tid; i < 4096; i += blockDim.x) {
+            const float v = __ldcg(ds + i);
+            if (v != v) {
+                mark[i & 63] = 1;
+                if (to == nseg - 1 && p.state_out) p.state_out[(size_t)unit * 4096 + i] = nan;
+                if (CKPT)
+                    for (int c = ck_first; c < ck_end; ++c)
+                        reinterpret_cast<__nv_bfloat16*>(p.ckpt)[(first_slot + c) * 4096 + i] = __float2bfloat16_rn(nan);
+            }
+        }
+        __syncthreads();
+        for (long long i = (long long)first * 64 + tid; i < (long long)end * 64; i += blockDim.x)
+            if (mark[i & 63]) p.y[(size_t)(row0 + (i >> 6)) * p.H * 64 + h * 64 + (i & 63)] = __float2bfloat16_rn(nan);
+    }
+}
+
 // ---------------------------------------------------------------- the kernel
 // SUMMARY = false: the prefill proper.  SUMMARY = true: the first pass of a split call, which only
 // carries the state over a segment from a zero start (no r, no scores, no outputs: the score warps and
@@ -715,8 +779,7 @@ __device__ __forceinline__ void exact_chunk(float* scr, const Params& p, int h, 
 // stream may begin and end inside a unit (see Params::bal_chunks).
 // CKPT = true (launches of the prefill proper): the state before every chunk and after the last one is also left in
 // Params::ckpt, for the gradient call that follows a training step's forward pass.
-// TRAIL = true (main launches of split calls): the summary launch may have started late in its segments (see Params::trail);
-// a segment that ends in a non-finite state is marked for wkv6_mark_kernel.
+// TRAIL = true (main launches of split calls): the summary launch may have started late in its segments (see Params::trail).
 template <bool SUMMARY, bool C2, int PERSIST = 0, bool CKPT = false, bool TRAIL = false>
 __global__ void __launch_bounds__(THREADS, 1)
 wkv6_chunked_kernel(const __grid_constant__ CUtensorMap tm_r, const __grid_constant__ CUtensorMap tm_k,
@@ -871,6 +934,7 @@ wkv6_chunked_kernel(const __grid_constant__ CUtensorMap tm_r, const __grid_const
             for (int i = 0; i < NSIDE; ++i) sts32(sbase + OFF_DESC + 16 * i + 4, DESC_TAG);        // (of the turn before the first)
         sts32(abort_flag, 0u);
         sts32(abort_flag + 4, p.wait_limit_us ? p.wait_limit_us : WAIT_LIMIT_US);
+        if (TRAIL) sts32(sbase + OFF_MARK, 0u);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         fence_proxy_async();
     }
@@ -1167,7 +1231,7 @@ wkv6_chunked_kernel(const __grid_constant__ CUtensorMap tm_r, const __grid_const
             for (int gg = 0; gg < seg; ++gg) {
                 const float* sm = p.summaries + ((size_t)unit * (p.nseg - 1) + gg) * SUMMARY_FLOATS;
                 float d_lo = sm[c_lo], d_hi = sm[c_lo + 8];
-                if (TRAIL) { d_lo = fabsf(d_lo); d_hi = fabsf(d_hi); }               // (the signs are marks)
+                if (TRAIL) { d_lo = fabsf(d_lo); d_hi = fabsf(d_hi); }               // (signs: see poison_later_segments)
 #pragma unroll
                 for (int n = 0; n < 8; ++n) {
                     const float2 lo = *reinterpret_cast<const float2*>(sm + 64 + c_lo * 64 + 8 * n + 2 * q);
@@ -1368,8 +1432,8 @@ wkv6_chunked_kernel(const __grid_constant__ CUtensorMap tm_r, const __grid_const
         } else if (!PERSIST && p.state_out && seg == p.nseg - 1 && !lds32(abort_flag)) {
             store_state(sb);
         } else if (TRAIL && seg < p.nseg - 1) {
-            // a state that is no longer finite: NaN over those elements of the segment's dS, and the sign of D[1] (D is a decay,
-            // readers drop the sign).  A later segment's CTA that folds this summary meanwhile may see either.
+            // a state that is no longer finite: marked in the segment's summary (see poison_later_segments; a later segment's CTA
+            // that folds this summary meanwhile may see either)
             float z = 0.f;
 #pragma unroll
             for (int n = 0; n < 8; ++n)
@@ -1382,7 +1446,7 @@ wkv6_chunked_kernel(const __grid_constant__ CUtensorMap tm_r, const __grid_const
 #pragma unroll
                     for (int e = 0; e < 4; ++e)
                         if (st[n][e] * 0.f != 0.f) sm[(size_t)(e < 2 ? c_lo : c_lo + 8) * 64 + 8 * n + 2 * q + (e & 1)] = __int_as_float(0x7fc00000);
-                atomicOr(reinterpret_cast<unsigned*>(sm) - 63, 0x80000000u);
+                sts32(sbase + OFF_MARK, 1u);
             }
         }
     } else if (warp < WARP_Y0) {
@@ -1767,48 +1831,9 @@ wkv6_chunked_kernel(const __grid_constant__ CUtensorMap tm_r, const __grid_const
         tc_fence_after();
         tmem_dealloc(tmem, TM_COLS);
     }
-}
-
-// Behind the main launch of a split call whose summary launch may have started late in its segments (Params::trail): a
-// segment's state that has become non-finite goes on being so, although its summary did not see it.  The main launch has marked
-// such a segment; the marked columns of the later segments' outputs become NaN, and the marked elements of their checkpoints
-// (ckpt, dense) and of the final state.  One CTA per unit and segment but the first; without a mark it reads a word per segment.
-// (The main launch's CTAs did this at their own ends before, and had to tell one another what they had marked and written.)
-constexpr int MARK_THREADS = 256;
-__global__ void __launch_bounds__(MARK_THREADS)
-wkv6_mark_kernel(const float* summaries, int nseg, int seg_chunks, const int32_t* cu, int T, int H, __nv_bfloat16* y, float* state_out,
-                 __nv_bfloat16* ckpt)
-{
-    __shared__ int mark[64];
-    asm volatile("griddepcontrol.launch_dependents;\n\tgriddepcontrol.wait;" ::: "memory");
-    const int unit = blockIdx.x / (nseg - 1), to = blockIdx.x % (nseg - 1) + 1, tid = threadIdx.x;
-    const float* sm = summaries + (size_t)unit * (nseg - 1) * SUMMARY_FLOATS;
-    auto marked = [&](int from) { return (__float_as_uint(sm[(size_t)from * SUMMARY_FLOATS + 1]) >> 31) != 0; };
-    if (!__syncthreads_or(tid < to && marked(tid))) return;
-    const int seq = unit / H, h = unit % H;
-    const long long row0 = cu ? cu[seq] : (long long)seq * T;
-    const int len = cu ? cu[seq + 1] - cu[seq] : T;
-    const int first = min(len, to * seg_chunks * L), end = to == nseg - 1 ? len : min(len, first + seg_chunks * L);
-    // the states before the segment's chunks, and after the last one of the unit
-    const int ck_first = (first + L - 1) / L, ck_end = (end + L - 1) / L + (to == nseg - 1 ? 1 : 0);
-    const size_t slot0 = (size_t)unit * ((T + L - 1) / L + 1);
-    const float nan = __int_as_float(0x7fc00000);
-    if (tid < 64) mark[tid] = 0;
-    __syncthreads();
-    for (int from = 0; from < to; ++from) {
-        if (!marked(from)) continue;
-        for (int i = tid; i < 4096; i += MARK_THREADS) {
-            const float v = sm[(size_t)from * SUMMARY_FLOATS + 64 + i];
-            if (v == v) continue;
-            mark[i & 63] = 1;
-            if (to == nseg - 1 && state_out) state_out[(size_t)unit * 4096 + i] = nan;
-            if (ckpt)
-                for (int c = ck_first; c < ck_end; ++c) ckpt[(slot0 + c) * 4096 + i] = __float2bfloat16_rn(nan);
-        }
-    }
-    __syncthreads();
-    for (long long i = (long long)first * 64 + tid; i < (long long)end * 64; i += MARK_THREADS)
-        if (mark[i & 63]) y[(size_t)(row0 + (i >> 6)) * H * 64 + h * 64 + (i & 63)] = __float2bfloat16_rn(nan);
+    if (TRAIL)
+        poison_later_segments<CKPT>(p, unit, seg, lds32(sbase + OFF_MARK) != 0, reinterpret_cast<int*>(smem + OFF_TOT),
+                                    reinterpret_cast<int*>(smem + OFF_TOT) + 64, CKPT ? ckpt_slot(0) : 0);
 }
 
 // One warp that waits, with the kernel's own bounded wait, on a barrier nobody arrives on: the wait runs out after
@@ -1926,15 +1951,6 @@ inline bool chunked_kernel_attributes()
         attr_set.set(dev);
     }
     return true;
-}
-
-// wkv6_mark_kernel behind the main launch of a split call with late starts
-inline gf_status_t launch_marks(const ck::Params& p, long long units, cudaStream_t st, std::atomic<uint64_t>* launches)
-{
-    const cudaError_t e = launch_pdl(ck::wkv6_mark_kernel, (unsigned)(units * (p.nseg - 1)), ck::MARK_THREADS, 0, st, p.summaries, p.nseg, p.seg_chunks,
-                                     p.cu_seqlens, p.T, p.H, p.y, p.state_out, reinterpret_cast<__nv_bfloat16*>(p.ckpt));
-    launches->fetch_add(1, std::memory_order_relaxed);
-    return e == cudaSuccess ? GF_OK : GF_ERR_CUDA;
 }
 
 // Prepares the scratch of a packed persistent launch: zeroes the unit counter and, for up to ORDER_MAX_SEQ
@@ -2100,8 +2116,7 @@ inline gf_status_t chunked_prefill(const __nv_bfloat16* r, const __nv_bfloat16* 
                                     : (c2 ? ck::wkv6_chunked_kernel<false, true, 0, true> : ck::wkv6_chunked_kernel<false, false, 0, true>);
         kernel<<<(unsigned)(units * nseg), ck::THREADS, ck::SMEM_ALLOC, st>>>(tr, tk, tv, tx, ty, tu2, p, tck);
         launches->fetch_add(1, std::memory_order_relaxed);
-        if (cudaGetLastError() != cudaSuccess) return GF_ERR_CUDA;
-        return p.trail ? launch_marks(p, units, st, launches) : GF_OK;
+        return cudaGetLastError() == cudaSuccess ? GF_OK : GF_ERR_CUDA;
     }
     const int n_sm = sm_count();
     // More units than SMs: one CTA per SM walks a stream of units, so that a unit's pipeline fill overlaps the
@@ -2155,8 +2170,7 @@ inline gf_status_t chunked_prefill(const __nv_bfloat16* r, const __nv_bfloat16* 
                                     : (c2 ? ck::wkv6_chunked_kernel<false, true> : ck::wkv6_chunked_kernel<false, false>);
         const cudaError_t e = launch_pdl(kernel, (unsigned)(units * nseg), ck::THREADS, ck::SMEM_ALLOC, st, tr, tk, tv, tx, ty, tu2, p, tck);
         launches->fetch_add(1, std::memory_order_relaxed);
-        if (e != cudaSuccess) return GF_ERR_CUDA;
-        return p.trail ? launch_marks(p, units, st, launches) : GF_OK;
+        return e == cudaSuccess ? GF_OK : GF_ERR_CUDA;
     }
     const cudaError_t e = launch_pdl(c2 ? ck::wkv6_chunked_kernel<false, true> : ck::wkv6_chunked_kernel<false, false>, (unsigned)units, ck::THREADS,
                                      ck::SMEM_ALLOC, st, tr, tk, tv, tx, ty, tu2, p, tck);
