@@ -81,10 +81,18 @@ constexpr int N_EW = 8;                // elementwise warps per set
 constexpr int N_ESET = 2;              // elementwise sets (alternate chunks)
 // The ring is waited on by two sets that take alternate chunks, and its depth is odd: a stage belongs to either set in turn.  A
 // wait names a phase by its parity alone, so a set has to meet every phase of the barriers it waits on.  Hence a "full" barrier
-// per stage and set: chunk c completes phase c / N_FULL of barrier c % N_FULL, which only set c % N_ESET waits on.  (One barrier
-// per stage would let a set through to chunk c while the copy of chunk c - NS, which had the stage before, is still landing.)
-constexpr int N_FULL = NS % N_ESET ? N_ESET * NS : NS;
-static_assert(N_FULL % N_ESET == 0 && N_FULL % NS == 0, "a barrier belongs to one stage and one set");
+// per set and stage, which only that set waits on.  (One barrier per stage would let a set through to chunk c while the copy of
+// chunk c - NS, which had the stage before, is still landing.)  Chunk c takes stage 3 c mod 5, so that a set's next chunk takes
+// the next stage and its phase bit flips where the stage wraps; set 1 begins at stage 3, so its barriers of the stages before
+// that start one phase ahead.
+constexpr int STAGE_STEP = 3;
+static_assert(NS == 5 && N_ESET == 2 && STAGE_STEP * N_ESET % NS == 1, "the stages of a set's chunks follow one another");
+__device__ __forceinline__ void next_stage(int& s, int& ph)      // for the roles that take every chunk: the phase flips every NS chunks
+{
+    s += STAGE_STEP;
+    if (s >= NS) s -= NS;
+    if (s == 0) ph ^= 1;
+}
 constexpr int N_GW = 4;                // warps per tensor-memory reader group (one per sub-partition)
 constexpr int WARP_MMA_F = 1;          // issues P = R^ K^^T and dS = K^^T V; owns the tensor-memory allocation
 constexpr int WARP_MMA_B = 2;          // issues Y = R^ S_0 + P' V
@@ -118,8 +126,8 @@ constexpr int OFF_ABORT = OFF_SAFE + NSIDE * 4;            // int
 constexpr int OFF_TMEM = OFF_ABORT + 8;                    // uint32: tensor-memory base address
 constexpr int OFF_BAR = OFF_ABORT + 16;                    // mbarriers (8 bytes each)
 enum {
-    BAR_FULL_RKV = 0,                    // copies of a chunk landed (by chunk modulo N_FULL)
-    BAR_EMPTY_RKV = BAR_FULL_RKV + N_FULL,     // (from here on by stage)
+    BAR_FULL_RKV = 0,                    // copies of a chunk landed (by set and stage)
+    BAR_EMPTY_RKV = BAR_FULL_RKV + N_ESET * NS,
     BAR_RK_READY = BAR_EMPTY_RKV + NS,
     BAR_S_READY = BAR_RK_READY + NS,     // bf16 state operand tile written            (by chunk parity)
     BAR_PP_READY = BAR_S_READY + 2,      // masked-score operand tile written
@@ -911,7 +919,8 @@ wkv6_chunked_kernel(const __grid_constant__ CUtensorMap tm_r, const __grid_const
     };
 
     if (tid == 0) {
-        for (int i = 0; i < N_FULL; ++i) mbar_init(bar(BAR_FULL_RKV + i), 1);
+        for (int i = 0; i < N_ESET * NS; ++i) mbar_init(bar(BAR_FULL_RKV + i), 1);
+        for (int i = 0; i < STAGE_STEP; ++i) mbar_arrive(bar(BAR_FULL_RKV + NS + i));      // (see STAGE_STEP)
         for (int i = 0; i < NS; ++i) {
             mbar_init(bar(BAR_EMPTY_RKV + i), 1);                  // the commit after the last product that reads the stage
             mbar_init(bar(BAR_RK_READY + i), N_EW);
@@ -957,10 +966,11 @@ wkv6_chunked_kernel(const __grid_constant__ CUtensorMap tm_r, const __grid_const
 
     if (warp == 0) {
         // ============================== TMA producer ==============================
+        auto full_bar = [&](int c) { return bar(BAR_FULL_RKV + (c & 1) * NS + STAGE_STEP * c % NS); };
+        auto full_parity = [&](int c) { return (uint32_t)(((c >> 1) + (c & 1) * STAGE_STEP) / NS & 1); };
         if constexpr (PERSIST) {
             int gc = 0, real_end = -1;               // chunks of the stream issued so far; index of the first end marker
             int s = 0, ph = 1;                       // ring stage and the parity of its previous release
-            int fb = 0;                              // "full" barrier of the next chunk
             bool alive = true;
             for (int k = 0; alive; ++k) {
                 int u = 0, c0 = 0, c1 = 0;               // the next piece: chunks c0 .. c1-1 of unit u (balanced launches)
@@ -1047,7 +1057,7 @@ wkv6_chunked_kernel(const __grid_constant__ CUtensorMap tm_r, const __grid_const
                         int meta = min(L, ulen - c * L) | (c == c0 ? DESC_FIRST : 0) | (int)((unsigned)uh << 16);
                         if (BAL) meta |= (c == c0 && c0 > 0 ? DESC_CONT : 0) | (c == c1 - 1 ? DESC_LAST : 0);
                         put_desc(gc, row, meta, u, unch - 1 - c);
-                        const uint32_t full = bar(BAR_FULL_RKV + fb);
+                        const uint32_t full = bar(BAR_FULL_RKV + (gc & 1) * NS + s);
                         mbar_expect_tx(full, STAGE);                       // (release: the descriptor is visible to the waiters)
                         tma_load_2d(dst, &tm_x, uh * 64, row, full);
                         tma_load_2d(dst + TILE, &tm_r, uh * 64, row, full);
@@ -1055,8 +1065,7 @@ wkv6_chunked_kernel(const __grid_constant__ CUtensorMap tm_r, const __grid_const
                         tma_load_2d(dst + 3 * TILE, &tm_v, uh * 64, row, full);
                     }
                     __syncwarp();
-                    if (++s == NS) { s = 0; ph ^= 1; }
-                    if (++fb == N_FULL) fb = 0;
+                    next_stage(s, ph);
                 }
             }
             if (alive) {
@@ -1066,11 +1075,10 @@ wkv6_chunked_kernel(const __grid_constant__ CUtensorMap tm_r, const __grid_const
                     if (gc >= NS && !mbar_wait_warp(bar(BAR_EMPTY_RKV + s), ph, abort_flag)) { alive = false; break; }
                     if (elect_one()) {
                         put_desc(gc, 0, DESC_END, 0, 0);
-                        mbar_arrive(bar(BAR_FULL_RKV + fb));                // no copy: the arrival alone completes the phase
+                        mbar_arrive(bar(BAR_FULL_RKV + (gc & 1) * NS + s)); // no copy: the arrival alone completes the phase
                     }
                     __syncwarp();
-                    if (++s == NS) { s = 0; ph ^= 1; }
-                    if (++fb == N_FULL) fb = 0;
+                    next_stage(s, ph);
                 }
             }
             // Do not leave while copies into this CTA's shared memory may still be in flight.  A stage that an end
@@ -1078,17 +1086,16 @@ wkv6_chunked_kernel(const __grid_constant__ CUtensorMap tm_r, const __grid_const
             const int issued = real_end >= 0 ? real_end : gc;
             const int from = (real_end >= 0 && alive) ? max(0, issued - NS + 2) : max(0, issued - NS);
             for (int c = from; c < issued; ++c)
-                mbar_wait_warp(bar(BAR_FULL_RKV + c % N_FULL), (c / N_FULL) & 1, abort_flag, false);
+                mbar_wait_warp(full_bar(c), full_parity(c), abort_flag, false);
         } else {
             int issued = 0;
             int s = 0, ph = 1;                       // ring stage and the parity of its previous release
-            int fb = 0;                              // "full" barrier of the next chunk
             int row = (int)row0;
             for (int c = 0; c < nchunks; ++c, row += L) {
                 if (c >= NS && !mbar_wait_warp(bar(BAR_EMPTY_RKV + s), ph, abort_flag)) break;
                 const uint32_t dst = sbase + OFF_RING + s * STAGE;
                 if (elect_one()) {
-                    const uint32_t full = bar(BAR_FULL_RKV + fb);
+                    const uint32_t full = bar(BAR_FULL_RKV + (c & 1) * NS + s);
                     mbar_expect_tx(full, SUMMARY ? 3 * TILE : STAGE);
                     tma_load_2d(dst, &tm_x, col0, row, full);
                     if (!SUMMARY) tma_load_2d(dst + TILE, &tm_r, col0, row, full);
@@ -1097,12 +1104,11 @@ wkv6_chunked_kernel(const __grid_constant__ CUtensorMap tm_r, const __grid_const
                 }
                 __syncwarp();
                 issued = c + 1;
-                if (++s == NS) { s = 0; ph ^= 1; }
-                if (++fb == N_FULL) fb = 0;
+                next_stage(s, ph);
             }
             // do not leave while copies into this CTA's shared memory may still be in flight
             for (int c = max(0, issued - NS); c < issued; ++c)
-                mbar_wait_warp(bar(BAR_FULL_RKV + c % N_FULL), (c / N_FULL) & 1, abort_flag, false);
+                mbar_wait_warp(full_bar(c), full_parity(c), abort_flag, false);
         }
     } else if (warp == WARP_MMA_F) {
         // ============================== MMA issuer, input-only products ==============================
@@ -1136,7 +1142,7 @@ wkv6_chunked_kernel(const __grid_constant__ CUtensorMap tm_r, const __grid_const
                 if (SUMMARY) tc_commit(bar(BAR_EMPTY_RKV + s));    // no other product reads the stage
             }
             __syncwarp();
-            if (++s == NS) { s = 0; ph ^= 1; }
+            next_stage(s, ph);
         }
     } else if (warp == WARP_MMA_B) {
         // ============================== MMA issuer, state-dependent products ==============================
@@ -1173,7 +1179,8 @@ wkv6_chunked_kernel(const __grid_constant__ CUtensorMap tm_r, const __grid_const
                 tc_commit(bar(BAR_EMPTY_RKV + s));
             }
             __syncwarp();
-            if (++s == NS) s = 0;
+            s += STAGE_STEP;
+            if (s >= NS) s -= NS;
         }
     } else if (warp < WARP_P0) {
         // ============================== state warps ==============================
@@ -1667,15 +1674,14 @@ wkv6_chunked_kernel(const __grid_constant__ CUtensorMap tm_r, const __grid_const
 #pragma unroll
         for (int tt = 0; tt < 4; ++tt) roff[tt] = swz(8 * tq + 4 * th + tt, 8 * cq);
         const float2 kLog2e = make_float2(LOG2E, LOG2E), kLogLog = make_float2(LOG2_LOG2E, LOG2_LOG2E);
-        int s = eset;                                    // ring stage of this set's current chunk,
-        int fb = eset, ph = 0;                           // its "full" barrier and that one's phase bit
+        int s = STAGE_STEP * eset, ph = 0;               // ring stage of this set's current chunk and its "full" barrier's phase bit
         for (int c = eset; PERSIST || c < nchunks; c += N_ESET) {
             const int sd = c & (NSIDE - 1);
             const uint32_t tx = sbase + OFF_RING + s * STAGE, tv = tx + 3 * TILE;
             uint32_t ax[4];                              // this lane's 8 bytes in its 4 rows of the x tile; r at +TILE, k at +2 TILE
 #pragma unroll
             for (int tt = 0; tt < 4; ++tt) ax[tt] = tx + roff[tt];
-            if (!mbar_wait(bar(BAR_FULL_RKV + fb), ph, abort_flag)) break;
+            if (!mbar_wait(bar(BAR_FULL_RKV + eset * NS + s), ph, abort_flag)) break;
             Chunk ck;                                    // (this role needs the valid-token count, the head and the end flag only)
             if constexpr (PERSIST) {
                 const uint32_t meta = lds32(sbase + OFF_DESC + 16 * (c & (NSIDE - 1)) + 4);
@@ -1817,10 +1823,7 @@ wkv6_chunked_kernel(const __grid_constant__ CUtensorMap tm_r, const __grid_const
             fence_proxy_async();                  // the scaled tiles are read by the tensor core (async proxy)
             __syncwarp();
             mbar_arrive_if(bar(BAR_RK_READY + s), lane == 0);
-            s += N_ESET;
-            if (s >= NS) s -= NS;
-            fb += N_ESET;
-            if (fb >= N_FULL) { fb -= N_FULL; ph ^= 1; }
+            if (++s == NS) { s = 0; ph ^= 1; }
         }
     }
 
