@@ -2064,10 +2064,13 @@ inline gf_status_t chunked_prefill(const __nv_bfloat16* r, const __nv_bfloat16* 
     ck::Params p{r, k, v, x, y, u, state_in, state_out, cu, T, H, scratch, seg_chunks, nseg, u2, c2};
     CUtensorMap tck = ty;                            // (read only by the launches that keep checkpoints)
     if (nseg > 1 && state_in) p.state_copy = scratch + (size_t)units * (nseg - 1) * ck::SUMMARY_FLOATS;
-    // A late start (Params::trail) costs the summary launch 5 us of looking and the main launch's CTAs 2 us at their end: it
-    // is allowed where segments are long enough to gain (us, without -> with: segments of 512 chunks 776 -> 537, of 64
-    // 113 -> 101, of 48 89 -> 85, of 15 39 -> 46).
-    p.trail = nseg > 1 && seg_chunks >= 48;
+    // A late start (Params::trail) runs about 42 chunks of a segment at the decays of a trained model (w in [0.69, 0.998]), and
+    // costs 5 to 10 us of looking and marking where the decays are too slow for one: it is allowed where segments are long enough
+    // to gain more than that.  (us without -> with a late start at such decays / at slow ones; 32 units of 4 segments of 48 chunks
+    // 91 -> 107 / 91 -> 99, of 64 115 -> 124 / 115 -> 123, of 96 163 -> 155 / 163 -> 171, of 128 218 -> 189 / 218 -> 222, of 192
+    // 317 -> 261 / 320 -> 332, of 512 847 -> 596 / 900 -> 910; 8 units of 8 segments of 96 160 -> 153 / 160 -> 168, of 128
+    // 206 -> 181 / 206 -> 215.)
+    p.trail = nseg > 1 && seg_chunks >= 128;
     p.wait_limit_us = wait_limit_us().load(std::memory_order_relaxed);
     if (ckpt) {
         // a training step's forward pass: one CTA per unit and segment, the chunk-start states kept for the gradient
