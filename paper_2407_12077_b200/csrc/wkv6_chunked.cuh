@@ -2099,11 +2099,17 @@ inline gf_status_t chunked_prefill(const __nv_bfloat16* r, const __nv_bfloat16* 
             cudaGetLastError();                      // (fewer SMs to be had than the device has: whole units below)
             p.bal_chunks = 0;
         }
-        if (nseg == 1 && n_sm_ck > 0 && units > n_sm_ck && H <= ck::STREAM_MAX_HEADS && (units >= 6LL * n_sm_ck || (unit_chunks <= 48 && units >= 3LL * n_sm_ck)) &&
+        if (nseg == 1 && n_sm_ck > 0 && units > n_sm_ck && H <= ck::STREAM_MAX_HEADS &&
+            (cu ? units >= 6LL * n_sm_ck || (unit_chunks <= 48 && units >= 3LL * n_sm_ck) : unit_chunks <= 32 && units >= 3LL * n_sm_ck) &&
             (!cu || (scratch && scratch_bytes >= persistent_scratch_bytes(n_seq)))) {
             // A stream of whole units per SM; packed: the longest sequences first, as in the prefill without checkpoints.
-            // (Packed, 768 units of 2..47 chunks: the training pair 662 -> 650 us.  Dense, 256 units of 32 chunks: 84.0 us
-            // with one CTA per unit, 85.3 with the stream, which therefore wants three units per SM.)
+            // Dense (us, one CTA per unit -> stream, classic; Finch-C2): 448 units of 8..64 chunks the same; 576 of 8 chunks 69 ->
+            // 57; 82 -> 65, of 16 105 -> 98; 124 -> 111, of 32 179 -> 182; 209 -> 204, of 48 257 -> 262; 288 -> 301, of 64
+            // 334 -> 347; 372 -> 392; 896 of 32 312 -> 319; 349 -> 347, of 48 430 -> 466; 469 -> 498; 1184 of 32 348 -> 346;
+            // 395 -> 396, of 48 508 -> 510; 560 -> 606: up to 32 chunks.
+            // Packed, where a stream also hands out the longest first: 768 units of up to 14 chunks 96 -> 84 us, 45 175 -> 150, 89
+            // 380 -> 365 (all long, 32..47: 290 -> 298); 1280 of up to 63 409 -> 392; 2048 of up to 64 657 -> 671 (Finch-C2
+            // 755 -> 750).
             p.n_units = (int)units;
             if (cu) {
                 p.ticket = reinterpret_cast<unsigned int*>(scratch);
