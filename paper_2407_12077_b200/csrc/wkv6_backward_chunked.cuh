@@ -1001,6 +1001,7 @@ wkv6_backward_chunked_kernel(const __grid_constant__ CUtensorMap tm_x, const __g
             tc_fence_after();
             // ---- epilogue (the staging tiles take the place of the operand tiles S_0, G^, P', dP': all read by now)
             float z[G_NB][4], qv[G_NB][4];
+            float2 du_c[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};      // the chunk's part of du_acc
 #pragma unroll
             for (int h2 = 0; h2 < G_H2; ++h2) {
                 // q and m take the operands as the tensor core saw them (rounded to bf16): the pair terms that q and
@@ -1026,8 +1027,8 @@ wkv6_backward_chunked_kernel(const __grid_constant__ CUtensorMap tm_x, const __g
                         o[n][2 * h] = oo.x; o[n][2 * h + 1] = oo.y;
                         qv[nn][2 * h] = qq.x; qv[nn][2 * h + 1] = qq.y;
                         if (!C2) {
-                            const float2 dd = mul2(mul2(make_float2(rv[n][2 * h], rv[n][2 * h + 1]), kk), pd);
-                            du_acc[h] += dd.x + dd.y;
+                            du_c[h] = fma2(mul2(make_float2(rv[n][2 * h], rv[n][2 * h + 1]), kk), pd, du_c[h]);
+                            if (nn == G_NB - 1) du_acc[h] += du_c[h].x + du_c[h].y;      // (one rounding of the long sum per chunk)
                         }
                     }
                 }

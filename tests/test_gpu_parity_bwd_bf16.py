@@ -283,3 +283,18 @@ def test_long_context_shape_at_the_benchmarked_size_two_heads_in_full():
                 den = (r * r).sum(axis=(1, 3))
                 tok = np.sqrt(row.max(axis=1) / (den / T))
                 assert tok.max() <= TOK_TOL, (h, name, float(tok.max()))
+
+
+@pytest.mark.parametrize("H", [96, 157])
+def test_bonus_gradient_of_many_tokens(H):
+    """The bonus gradient is an fp32 sum over all tokens.  A lane adds one number per chunk, T / 128 of them: an addition rounds
+    by 2^-25 of what has been summed at the most, and errors of either sign grow as the root of their number.  (157 heads: units
+    cut between SMs.)"""
+    T = 16384
+    i = synth.make_dense(1, T, H, 64, "bf16", seed=H, device=DEV, state_std=0.1)
+    dy = torch.randn(i.r.shape, device=DEV, generator=torch.Generator(device=DEV).manual_seed(H)).bfloat16()
+    du = gf.backward(i.r, i.k, i.v, i.x, i.u, dy, i.state_in)[4]
+    gf.last_device_status()
+    vd = (i.v[0].double() * dy[0].double()).sum(-1, keepdim=True)
+    ref = (i.r[0].double() * i.k[0].double() * vd).sum(0)
+    assert float((du.double() - ref).norm() / ref.norm()) <= 2.0 ** -25 * (T / 128) ** 0.5
