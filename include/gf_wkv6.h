@@ -370,7 +370,9 @@ GF_API gf_status_t gf_wkv6_set_kernel(gf_kernel_t kernel);
 
 /* Synchronises `stream`, then returns GF_ERR_TIMEOUT if any kernel launched by this
  * library since the last query gave up on a bounded wait (its outputs are then
- * undefined), GF_ERR_CUDA if the stream reports an error, else GF_OK.  Clears the flag. */
+ * undefined), GF_ERR_CUDA if the stream reports an error, else GF_OK.  Clears the flag.  A CUDA graph that holds a
+ * dense prefill is captured again after a time-out, or its y cleared before the next replay: the words with which a call
+ * that cuts units announces a state (see gf_wkv6_workspace_bytes) may be left in y, and a replay carries the same ones. */
 GF_API gf_status_t gf_wkv6_last_device_status(gf_stream_t stream);
 
 /* Every device-side wait of the prefill kernels (on a copy, a tensor-core product, another warp) is bounded: when
