@@ -902,7 +902,8 @@ wkv6_chunked_kernel(const __grid_constant__ CUtensorMap tm_r, const __grid_const
             int4 d;
             asm volatile("ld.shared.v4.s32 {%0, %1, %2, %3}, [%4];"
                          : "=r"(d.x), "=r"(d.y), "=r"(d.z), "=r"(d.w) : "r"(sbase + OFF_DESC + 16 * (c & (NSIDE - 1))) : "memory");
-            ck.row = d.x; ck.valid = d.y & 0xff; ck.unit = d.z; ck.h = (int)((unsigned)d.y >> 16); ck.rem = d.w;
+            ck.row = d.x; ck.valid = d.y & 0xff; ck.unit = d.z; ck.rem = d.w;
+            ck.h = BAL ? d.y >> 16 : (int)((unsigned)d.y >> 16);      // (a balanced call has fewer than five units per SM: no sign; spills)
             ck.first = (d.y & DESC_FIRST) != 0; ck.last = BAL ? (d.y & DESC_LAST) != 0 : d.w == 0; ck.end = (d.y & DESC_END) != 0;
         } else {
             ck.row = (int)(row0 + (long long)c * L); ck.valid = min(L, len - c * L); ck.unit = unit; ck.h = h;
@@ -1681,7 +1682,8 @@ wkv6_chunked_kernel(const __grid_constant__ CUtensorMap tm_r, const __grid_const
             uint32_t ax[4];                              // this lane's 8 bytes in its 4 rows of the x tile; r at +TILE, k at +2 TILE
 #pragma unroll
             for (int tt = 0; tt < 4; ++tt) ax[tt] = tx + roff[tt];
-            if (!mbar_wait(bar(BAR_FULL_RKV + eset * NS + s), ph, abort_flag)) break;
+            // (c & 1 is eset: the one that leaves fewer spills in the variant)
+            if (!mbar_wait(bar(BAR_FULL_RKV + (TRAIL || SUMMARY ? eset : c & 1) * NS + s), ph, abort_flag)) break;
             Chunk ck;                                    // (this role needs the valid-token count, the head and the end flag only)
             if constexpr (PERSIST) {
                 const uint32_t meta = lds32(sbase + OFF_DESC + 16 * (c & (NSIDE - 1)) + 4);
