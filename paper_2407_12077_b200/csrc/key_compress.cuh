@@ -10,7 +10,7 @@
 // epilogue drains this one (wider outputs fill all 512 columns with one set).  Every 64-row slice of W that
 // enters shared memory serves MBLK*128 tokens, and one instruction multiplies 128 of them by all NB*64 columns, so that
 // the x operand is read from shared memory once (D = 2048, Dc = 128: 65536 rows 53.3 -> 50.6 us, 5.3 TB/s of x;
-// D = 4096, Dc = 256: 148 -> 118; 658 rows 14.8 -> 12.1).
+// D = 4096, Dc = 256: 148 -> 124; 658 rows 14.8 -> 12.1).
 // What bounds a call: many rows, HBM (262144 rows 175 us, 6.5 TB/s); few rows, the 64 bytes per cycle that one SM gets
 // from L2, so a short call spreads a tile over a cluster of SMs (SPLIT): each takes a share of the input channels,
 // leaves its fp32 sums in shared memory, and adds up a share of the rows over the cluster in a fixed order.
