@@ -15,22 +15,28 @@
 //   pass 1: z slice -> operand rows -> acc1 += z A_d[slice]                then h1 = tanh(acc1) -> operand
 //   pass 2: l = h1 B_d[:, slice] -> m slice -> operand rows -> acc3 += m A_w[slice]      then h2 = tanh(acc3) -> operand
 //   pass 3: d slice = lambda_w + h2 B_w[:, slice] -> bf16 -> TMA store
-// Two sets of four worker warps take alternate slices, each with stages, accumulators and issuing warps of its own:
-//   warp 0       TMA producer of the x rings (3 stages per set): per slice the x rows of the tile (plus the one row above
-//                it) and the 64 per-channel constants of the pass; a stage is free as soon as its rows are in registers
-//   warp 3       TMA producer of the weight rings (2 stages per set): free when the products that read a stage are done
-//   warps 1, 2   (warp 1: tensor-memory allocation) an elected lane issues a set's z A_d, h1 B_d, h2 B_w products
-//                (tcgen05.mma 128 x 64 x 16, bf16 -> fp32)
-//   warps 4, 5   an elected lane issues a set's m A_w, the product that waits for the workers inside pass 2 (an issuer of
-//                its own, so that the l products of later slices are not held up behind it)
-//   warps 6-13   the two sets; a lane owns one token row (the accumulator row of its tensor-memory sub-partition): reads its
-//                row and the row above from the swizzled x tiles, forms z / m / d for the 64 channels of the slice, 32 at a
+// Four sets of four worker warps take the slices in turn, each with a tensor-memory operand and accumulator of its own:
+//   warp 0       TMA producer of the x ring (8 stages, two per set): per slice the x rows of the tile (plus the one row above
+//                it) and the 64 per-channel constants of the pass; a stage is free as soon as its rows are in registers (pass 3: its
+//                room takes the output rows, and it is free when the store has read them)
+//   warps 1, 20  TMA producers of the weight rings (A_d, A_w: 5 stages; B_d, B_w: 3 per issuer): free when the product that reads a stage is done
+//   warp 2       an elected lane issues the products that wait for the workers, z A_d and m A_w (tcgen05.mma 128 x 64 x 16,
+//                bf16 -> fp32; tensor-memory allocation)
+//   warps 3, 21  an elected lane issues h1 B_d and h2 B_w of the even, the odd slices
+//   warps 4-19   the four sets; a lane owns one token row (the accumulator row of its tensor-memory sub-partition): reads its
+//                row and the row above from the swizzled x tiles, forms z / m / d for the 64 channels of the slice, 16 at a
 //                time, and writes the bf16 operand row or the output slab
 // z, m, h1 and h2 are A operands in tensor memory (a lane's row, two channels per column): through shared memory they were
-// a third of its traffic (16 KB written and 16 KB read per slice).  A sum over slices lies in two halves, one per set.
-// What bounds a slice is the chain load -> registers -> operand -> product of which two run at a time (65536 tokens x 2048
-// channels: 194 us; 159 with every load left out, 160 with the stores left out).  Before (one issuer for both sets, operands
-// in shared memory): 206 us; 1000 tokens 51 -> 46 us.  Twice the warps per set at half the channels each: 210 us.
+// a third of its traffic (16 KB written and 16 KB read per slice).
+// What bounds a slice is the chain load -> registers -> operand -> product, through warps that each spend 300-400 cycles per slice on
+// their part: 870 cycles a slice and pass with every set in flight, and 780 with one tile on an idle SM.  us per call, two sets of four warps on
+// rings of two weight stages each -> four sets -> a weight ring per issuer -> a producer and an issuer more (the present form):
+//   65536 tokens x 2048 channels 191 -> 196 -> 179 -> 175;  1000 x 2048 46.4 -> 43.5 -> 41.4 -> 40.0;  32 x 271 x 2048 50.5 -> 46.3 -> 45.7 -> 43.6;
+//   8680 x 768 20.1 -> 20.5 -> 19.6 -> 19.3.
+// (With one ring for both kinds of weights a slice's B_d, which its l needs early, waited for the slot of an A_w whose product comes a worker's
+// time later.)  Not better: the sum of pass 1 in an accumulator per set (175.6), rings of 5 + 6 stages with one producer (181), asking for the
+// operand rows after more of the slice (174 to 205: registers), an extra commit saved per slice at rings of 4 (192).  The three passes
+// as a pipeline over tiles, with pass 1 a product of raw rows with scaled weights, ran at 215: rings of two stages are all that fits then.
 // Weight tiles are the 128-byte-swizzled [64 rows][64 bf16] tiles of the prefill kernel; narrower ones (R < 64) are
 // zero-filled by TMA beyond their extent.  Every wait is bounded, as in the prefill kernel.
 #pragma once
@@ -42,50 +48,44 @@ namespace dl {
 
 using namespace ck;
 
-constexpr int DL_NSET = 2;                             // worker sets
-constexpr int DL_W0 = 6;                               // first worker warp
+constexpr int DL_NSET = 4;                             // worker sets
+constexpr int DL_W0 = 4;                               // first worker warp
 constexpr int DL_NWS = 4;                              // warps of a set, one per tensor-memory sub-partition
-constexpr int DL_NH = 2;                               // a warp's channels of a slice come in halves of 32 (registers)
-constexpr int DL_THREADS = 32 * (DL_W0 + DL_NWS * DL_NSET);
-// Two rings.  The x ring holds, per slice, the tile's x rows (two swizzled 64-row tiles), the row above the tile and the
-// pass's 64 per-channel constants; a worker set frees its stage as soon as the rows are in registers, so that ring
-// runs a load latency ahead of the arithmetic.  The weight ring holds up to two weight tiles per slice and is freed
-// by the products that read them (weights come from L2).
-// Each set has rings of its own: a waiter names a phase by its parity alone, so whoever waits for a stage has to wait for
-// every one of its phases (with stages that two sets use in turn, one of them asks for a phase while the other's
-// before it may not have landed, and is let through).
-constexpr int DL_NSX = 3, DL_NSW = 2;                  // stages per set
-constexpr int DL_NACC = 2;                             // l / d accumulators in tensor memory per set: the products h1 B_d and h2 B_w
-                                                       // depend on nothing the workers make, so they run this many slices ahead
+constexpr int DL_WB = DL_W0 + DL_NWS * DL_NSET;        // last warp: the producer of the B weights
+constexpr int DL_THREADS = 32 * (DL_WB + 2);
+// Slices are counted through all passes and tiles; slice n belongs to set n mod 4 and takes stage n mod 8 of the x ring, so a stage
+// always serves the same set.  (A wait names a phase by its parity alone, so whoever waits on a barrier has to wait for every one of its phases.)
+constexpr int DL_NSX = 8, DL_NSA = 5, DL_NSB = 3;
+static_assert(DL_NSX % DL_NSET == 0, "a stage serves one set");
 constexpr int DL_XSTAGE = 2 * TILE + 1024;
 constexpr int DL_OFF_PREV = 2 * TILE;                  // [64] bf16: the x row just above the tile (this slice)
 constexpr int DL_OFF_VEC = 2 * TILE + 256;             // [64] fp32: mu_x / lambda_d / lambda_w of this slice
-constexpr int DL_WSTAGE = 2 * TILE;
-constexpr int DL_OFF_W = DL_NSET * DL_NSX * DL_XSTAGE;           // weight rings
-constexpr int DL_OFF_OUT = DL_OFF_W + DL_NSET * DL_NSW * DL_WSTAGE;        // [sets][row groups][32 rows x 128 B]: output slabs of pass 3
-constexpr int DL_OFF_MISC = DL_OFF_OUT + DL_NSET * 2 * TILE;     // abort word + limit, tensor-memory address, barriers
+constexpr int DL_OFF_A = DL_NSX * DL_XSTAGE;           // weight rings: A_d, A_w slices; B_d, B_w slices
+constexpr int DL_OFF_B = DL_OFF_A + DL_NSA * TILE;
+constexpr int DL_OFF_MISC = DL_OFF_B + 2 * DL_NSB * TILE;       // abort word + limit, tensor-memory address, barriers
 constexpr int DL_SMEM = DL_OFF_MISC + 512 + 1024;      // + slack for manual 1024-byte alignment
 enum {
     DL_XFULL = 0,                      // x stage loaded
-    DL_XEMPTY = DL_XFULL + DL_NSET * DL_NSX,     // ... and read into registers by the warps of its set
-    DL_WFULL = DL_XEMPTY + DL_NSET * DL_NSX,     // weight stage loaded
-    DL_WEMPTY = DL_WFULL + DL_NSET * DL_NSW,     // ... and the last product that reads it is done
-    DL_OP_READY = DL_WEMPTY + DL_NSET * DL_NSW,  // per set: operand rows written
+    DL_XEMPTY = DL_XFULL + DL_NSX,     // ... and read into registers by the warps of its set
+    DL_AFULL = DL_XEMPTY + DL_NSX,     // A weight stage loaded
+    DL_AEMPTY = DL_AFULL + DL_NSA,     // ... and the product that reads it is done
+    DL_BFULL = DL_AEMPTY + DL_NSA,     // B weights
+    DL_BEMPTY = DL_BFULL + 2 * DL_NSB,
+    DL_OP_READY = DL_BEMPTY + 2 * DL_NSB,  // per set: operand rows written
     DL_OP_FREE = DL_OP_READY + DL_NSET,    // per set: the product that read them is done
-    DL_ACC_FULL = DL_OP_FREE + DL_NSET,    // per set and accumulator: l (pass 2) or d (pass 3) of a slice is in tensor memory
-    DL_ACC_FREE = DL_ACC_FULL + DL_NSET * DL_NACC,   // ... and read back by the warps of the set
-    DL_SUM_FULL = DL_ACC_FREE + DL_NSET * DL_NACC,   // both sets' partial sums of a pass complete
+    DL_ACC_FULL = DL_OP_FREE + DL_NSET,    // per set: l (pass 2) or d (pass 3) of a slice is in tensor memory
+    DL_ACC_FREE = DL_ACC_FULL + DL_NSET,   // ... and read back by the warps of the set
+    DL_SUM_FULL = DL_ACC_FREE + DL_NSET,   // the sum of a pass complete
     DL_H_READY = DL_SUM_FULL + 1,      // h1 / h2 operand written by all worker warps
-    DL_PASS2 = DL_H_READY + 1,         // per set: pass 2 of a tile has begun (its first issuer -> its second: one phase per tile)
-    DL_BAR_COUNT = DL_PASS2 + DL_NSET
+    DL_H_FREE = DL_H_READY + 1,        // the last product of a tile that reads h2 is done
+    DL_BAR_COUNT = DL_H_FREE + 1
 };
 static_assert(16 + 8 * DL_BAR_COUNT <= 512, "barrier block");
 static_assert(DL_SMEM <= 232448, "shared memory budget of one sm_100 CTA");
-// per set: its half of the pass's sum (acc1, then acc3: every warp has read acc1 before a product of pass 2's is issued,
-// and acc3 before one of the next tile's), and a ring of l (pass 2) / d (pass 3)
-constexpr int DL_TM_SUM = 0, DL_TM_RING = 64 * DL_NSET;
-// the A operands (lane = row, a 32-bit column = two neighbouring channels in bf16): z / m of a set, h1 / h2
-constexpr int DL_TM_OP = DL_TM_RING + 64 * DL_NSET * DL_NACC, DL_TM_H = DL_TM_OP + 32 * DL_NSET;
+// the sum of a pass (acc1, then acc3: every warp has read acc1 before a product of pass 2's is issued, and acc3 before one of
+// the next tile's); per set l (pass 2) / d (pass 3); the A operands (lane = row, a 32-bit column = two neighbouring channels
+// in bf16): z / m of a set, h1 / h2
+constexpr int DL_TM_SUM = 0, DL_TM_ACC = 64, DL_TM_OP = DL_TM_ACC + 64 * DL_NSET, DL_TM_H = DL_TM_OP + 32 * DL_NSET;
 static_assert(DL_TM_H + 32 <= 512, "tensor memory columns");
 // fp32 accumulator, bf16 A (K-major) and B (MN-major), M = 128, N = 64
 constexpr uint32_t DL_IDESC = (1u << 4) | (1u << 7) | (1u << 10) | (1u << 16) | ((64u >> 3) << 17) | ((128u >> 4) << 24);
@@ -183,53 +183,49 @@ decay_logit_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_consta
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 
     if (tid == 0) {
-        for (int i = 0; i < DL_NSET * DL_NSX; ++i) {
+        for (int i = 0; i < DL_NSX; ++i) {
             mbar_init(bar(DL_XFULL + i), 1);
             mbar_init(bar(DL_XEMPTY + i), DL_NWS);
         }
-        for (int i = 0; i < DL_NSET * DL_NSW; ++i) {
-            mbar_init(bar(DL_WFULL + i), 1);
-            mbar_init(bar(DL_WEMPTY + i), 1);
-        }
+        for (int i = 0; i < 2 * DL_NSA; ++i) mbar_init(bar(DL_AFULL + i), 1);
+        for (int i = 0; i < 4 * DL_NSB; ++i) mbar_init(bar(DL_BFULL + i), 1);
         for (int i = 0; i < DL_NSET; ++i) {
             mbar_init(bar(DL_OP_READY + i), DL_NWS);
             mbar_init(bar(DL_OP_FREE + i), 1);
-            mbar_init(bar(DL_PASS2 + i), 1);
-        }
-        for (int i = 0; i < DL_NSET * DL_NACC; ++i) {
             mbar_init(bar(DL_ACC_FULL + i), 1);
             mbar_init(bar(DL_ACC_FREE + i), DL_NWS);
         }
-        mbar_init(bar(DL_SUM_FULL), DL_NSET);
+        mbar_init(bar(DL_SUM_FULL), 1);
         mbar_init(bar(DL_H_READY), DL_NWS * DL_NSET);
+        mbar_init(bar(DL_H_FREE), 2);
         sts32(abort_flag, 0u);
         sts32(abort_flag + 4, WAIT_LIMIT_US);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         fence_proxy_async();
     }
-    if (warp == 1) tmem_alloc(sbase + DL_OFF_MISC + 8, 512);
+    if (warp == 2) tmem_alloc(sbase + DL_OFF_MISC + 8, 512);
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = lds32(sbase + DL_OFF_MISC + 8);
     asm volatile("griddepcontrol.wait;" ::: "memory");
-    // ring positions: the set's n-th slice over all passes and tiles
-    auto xslot = [&](int set, int n) { return set * DL_NSX + n % DL_NSX; };
-    auto wslot = [&](int set, int n) { return set * DL_NSW + n % DL_NSW; };
-    auto wstage = [&](int slot) { return sbase + DL_OFF_W + slot * DL_WSTAGE; };
+    auto wait = [&](int b, int phase) { return mbar_wait(bar(b), phase & 1, abort_flag); };
+    auto wait_warp = [&](int b, int phase) { return mbar_wait_warp(bar(b), phase & 1, abort_flag); };
+    auto xstage = [&](int n) { return sbase + (n & (DL_NSX - 1)) * DL_XSTAGE; };
+    auto astage = [&](int i) { return sbase + DL_OFF_A + i * TILE; };
+    auto bstage = [&](int i) { return sbase + DL_OFF_B + i * TILE; };
 
     if (warp == 0) {
         // ============================== TMA producer: x rows and per-channel constants ==============================
-        int n[DL_NSET] = {};                                 // slices issued so far, per set
+        int n = 0;
         bool alive = true;
         for (long long r = r_first; r < r_end && alive; r += 128) {
             const int row0 = (int)r;
             const bool whole = r_end - r > 64;
             for (int pass = 0; pass < 3 && alive; ++pass)
-                for (int s = 0; s < S; ++s) {
-                    const int set = s % DL_NSET, c = set ? n[1] : n[0], slot = xslot(set, c);
-                    if (c >= DL_NSX && !mbar_wait_warp(bar(DL_XEMPTY + slot), ((c / DL_NSX) + 1) & 1, abort_flag)) { alive = false; break; }
-                    const uint32_t dst = sbase + slot * DL_XSTAGE, full = bar(DL_XFULL + slot);
+                for (int s = 0; s < S; ++s, ++n) {
+                    if (n >= DL_NSX && !wait_warp(DL_XEMPTY + (n & (DL_NSX - 1)), n / DL_NSX - 1)) { alive = false; break; }
+                    const uint32_t dst = xstage(n), full = bar(DL_XFULL + (n & (DL_NSX - 1)));
                     if (elect_one()) {
                         const float* vec = pass == 0 ? p.mu_x : pass == 1 ? p.lambda_d : p.lambda_w;
                         if (pass < 2) {
@@ -243,344 +239,290 @@ decay_logit_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_consta
                         bulk_load_1d(dst + DL_OFF_VEC, vec + 64 * s, 256, full);
                     }
                     __syncwarp();
-                    if (set) ++n[1]; else ++n[0];
                 }
         }
         // do not leave while copies into this CTA's shared memory may still be in flight
-        for (int set = 0; set < DL_NSET; ++set)
-            for (int c = max(0, n[set] - DL_NSX); c < n[set]; ++c)
-                mbar_wait_warp(bar(DL_XFULL + xslot(set, c)), (c / DL_NSX) & 1, abort_flag, false);
-    } else if (warp == 3) {
-        // ============================== TMA producer: weight tiles ==============================
-        int n[DL_NSET] = {};
+        for (int c = max(0, n - DL_NSX); c < n; ++c) mbar_wait_warp(bar(DL_XFULL + (c & (DL_NSX - 1))), (c / DL_NSX) & 1, abort_flag, false);
+    } else if (warp == 1) {
+        // ============================== TMA producer: A_d, A_w tiles ==============================
+        int n = 0, ia = 0, pa = 1;                           // tiles issued; ring position and the parity of its last release
         bool alive = true;
         for (long long r = r_first; r < r_end && alive; r += 128)
-            for (int pass = 0; pass < 3 && alive; ++pass)
-                for (int s = 0; s < S; ++s) {
-                    const int set = s % DL_NSET, c = set ? n[1] : n[0], slot = wslot(set, c);
-                    if (c >= DL_NSW && !mbar_wait_warp(bar(DL_WEMPTY + slot), ((c / DL_NSW) + 1) & 1, abort_flag)) { alive = false; break; }
-                    const uint32_t dst = wstage(slot), full = bar(DL_WFULL + slot);
+            for (int pass = 0; pass < 2 && alive; ++pass)
+                for (int s = 0; s < S; ++s, ++n) {
+                    if (n >= DL_NSA && !wait_warp(DL_AEMPTY + ia, pa)) { alive = false; break; }
                     if (elect_one()) {
-                        if (pass == 0) {
-                            mbar_expect_tx(full, TILE);
-                            tma_load_2d(dst, &tm_ad, 0, 64 * s, full);
-                        } else if (pass == 1) {
-                            mbar_expect_tx(full, 2 * TILE);
-                            tma_load_2d(dst, &tm_bd, 64 * s, 0, full);
-                            tma_load_2d(dst + TILE, &tm_aw, 0, 64 * s, full);
-                        } else {
-                            mbar_expect_tx(full, TILE);
-                            tma_load_2d(dst, &tm_bw, 64 * s, 0, full);
-                        }
+                        const uint32_t full = bar(DL_AFULL + ia);
+                        mbar_expect_tx(full, TILE);
+                        tma_load_2d(astage(ia), pass == 0 ? &tm_ad : &tm_aw, 0, 64 * s, full);
                     }
                     __syncwarp();
-                    if (set) ++n[1]; else ++n[0];
+                    if (++ia == DL_NSA) { ia = 0; pa ^= 1; }
                 }
-        for (int set = 0; set < DL_NSET; ++set)
-            for (int c = max(0, n[set] - DL_NSW); c < n[set]; ++c)
-                mbar_wait_warp(bar(DL_WFULL + wslot(set, c)), (c / DL_NSW) & 1, abort_flag, false);
-    } else if (warp == 1 || warp == 2) {
-        // ============================== MMA issuers: z A_d, h1 B_d, h2 B_w of one set's slices ==============================
-        const int set = warp - 1;
-        const int n_own = (S - set + DL_NSET - 1) / DL_NSET;         // slices of this set (set, set + 2, ...)
-        const uint32_t tsum = tmem + DL_TM_SUM + 64 * set, tring = tmem + DL_TM_RING + 64 * DL_NACC * set;
-        int n = 0;                                           // ring position
-        int op_uses = 0;                                     // operand tiles of this set consumed
-        int an = 0;                                          // l / d accumulators of this set produced so far
+        for (int c = max(0, n - DL_NSA); c < n; ++c) mbar_wait_warp(bar(DL_AFULL + c % DL_NSA), (c / DL_NSA) & 1, abort_flag, false);
+    } else if (warp == DL_WB) {
+        // ============================== TMA producer: B_d, B_w tiles ==============================
+        int n = 0, i0 = 0, i1 = 0, m0 = 0, m1 = 0;           // per issuer: tiles issued, ring position
         bool alive = true;
-        auto weights_in = [&](int c) { return mbar_wait_warp(bar(DL_WFULL + wslot(set, c)), (c / DL_NSW) & 1, abort_flag); };
-        auto acc_free = [&](int n) { return n < DL_NACC || mbar_wait_warp(bar(DL_ACC_FREE + DL_NACC * set + n % DL_NACC), ((n / DL_NACC) + 1) & 1, abort_flag); };
-        const uint32_t th = tmem + DL_TM_H, ta = tmem + DL_TM_OP + 32 * set;
+        auto phase = [](int m) { return m / DL_NSB; };
         for (long long r = r_first; r < r_end && alive; r += 128) {
-            // ---- pass 1: acc1 += z A_d[slice]
-            for (int s = set; s < S; s += DL_NSET, ++n) {
-                const int i = wslot(set, n);
-                if (!weights_in(n) || !mbar_wait_warp(bar(DL_OP_READY + set), op_uses & 1, abort_flag)) { alive = false; break; }
-                ++op_uses;
-                tc_fence_after();
-                if (elect_one()) {
-                    const uint64_t db = smem_desc(wstage(i));
-#pragma unroll
-                    for (int kk = 0; kk < 4; ++kk)
-                        tc_mma_ta(tsum, ta + 8 * kk, db + (uint64_t)(128 * kk), DL_IDESC, (s > set || kk > 0) ? 1u : 0u);
-                    tc_commit(bar(DL_OP_FREE + set));
-                    tc_commit(bar(DL_WEMPTY + i));
-                    if (s + DL_NSET >= S) tc_commit(bar(DL_SUM_FULL));
+            n += S;
+            for (int pass = 1; pass < 3 && alive; ++pass)
+                for (int s = 0; s < S; ++s, ++n) {
+                    const bool odd = n & 1;
+                    const int m = odd ? m1 : m0, slot = odd ? DL_NSB + i1 : i0;
+                    if (m >= DL_NSB && !wait_warp(DL_BEMPTY + slot, phase(m) - 1)) { alive = false; break; }
+                    if (elect_one()) {
+                        const uint32_t full = bar(DL_BFULL + slot);
+                        mbar_expect_tx(full, TILE);
+                        tma_load_2d(bstage(slot), pass == 1 ? &tm_bd : &tm_bw, 64 * s, 0, full);
+                    }
+                    __syncwarp();
+                    if (odd) { ++m1; if (++i1 == DL_NSB) i1 = 0; }
+                    else { ++m0; if (++i0 == DL_NSB) i0 = 0; }
                 }
-                __syncwarp();
-            }
-            if (!alive) break;
-            if (n_own == 0 && elect_one()) mbar_arrive(bar(DL_SUM_FULL));        // (one slice: the other set's sum is all)
-            __syncwarp();
-            // ---- pass 2: l = h1 B_d[:, slice] (the set's other issuer follows with acc3 += m A_w[slice] and frees the stage)
-            if (!mbar_wait_warp(bar(DL_H_READY), 0, abort_flag)) break;          // (two uses per tile: parities 0, 1)
-            tc_fence_after();
-            if (elect_one()) mbar_arrive(bar(DL_PASS2 + set));                    // every operand-row phase of pass 1 is over
-            __syncwarp();
-            for (int s = set; s < S; s += DL_NSET, ++an, ++n) {
-                const int i = wslot(set, n), a = an % DL_NACC;
-                if (!weights_in(n) || !acc_free(an)) { alive = false; break; }
-                tc_fence_after();
-                if (elect_one()) {
-                    const uint64_t db = smem_desc(wstage(i));
-#pragma unroll
-                    for (int kk = 0; kk < 4; ++kk)
-                        if (kk < p.kd) tc_mma_ta(tring + 64 * a, th + 8 * kk, db + (uint64_t)(128 * kk), DL_IDESC, kk > 0 ? 1u : 0u);
-                    tc_commit(bar(DL_ACC_FULL + DL_NACC * set + a));
-                }
-                __syncwarp();
-            }
-            op_uses += n_own;                                 // (the set's other issuer consumes these slices' operand rows)
-            if (!alive) break;
-            // ---- pass 3: d slice = h2 B_w[:, slice]
-            if (!mbar_wait_warp(bar(DL_H_READY), 1, abort_flag)) break;
-            tc_fence_after();
-            for (int s = set; s < S; s += DL_NSET, ++an, ++n) {
-                const int i = wslot(set, n), a = an % DL_NACC;
-                if (!weights_in(n) || !acc_free(an)) { alive = false; break; }
-                tc_fence_after();
-                if (elect_one()) {
-                    const uint64_t db = smem_desc(wstage(i));
-#pragma unroll
-                    for (int kk = 0; kk < 4; ++kk)
-                        if (kk < p.kw) tc_mma_ta(tring + 64 * a, th + 8 * kk, db + (uint64_t)(128 * kk), DL_IDESC, kk > 0 ? 1u : 0u);
-                    tc_commit(bar(DL_ACC_FULL + DL_NACC * set + a));
-                    tc_commit(bar(DL_WEMPTY + i));
-                }
-                __syncwarp();
-            }
         }
-    } else if (warp == 4 || warp == 5) {
-        // ============================== MMA issuers: m A_w (pass 2) of one set's slices ==============================
-        const int set = warp - 4;
-        const int n_own = (S - set + DL_NSET - 1) / DL_NSET;
-        const uint32_t tsum = tmem + DL_TM_SUM + 64 * set;
-        const uint32_t ta = tmem + DL_TM_OP + 32 * set;
-        int ti = 0, op_uses = 0;
+        for (int c = max(0, m0 - DL_NSB); c < m0; ++c) mbar_wait_warp(bar(DL_BFULL + c % DL_NSB), phase(c) & 1, abort_flag, false);
+        for (int c = max(0, m1 - DL_NSB); c < m1; ++c) mbar_wait_warp(bar(DL_BFULL + DL_NSB + c % DL_NSB), phase(c) & 1, abort_flag, false);
+    } else if (warp == 2) {
+        // ============================== MMA issuer: sum += z A_d (pass 1), sum += m A_w (pass 2) ==============================
+        int n = 0, ia = 0, pa = 0;                           // (A ring position and its phase)
+        uint32_t phases = 0;                                 // bit: parity of the set's next operand
         bool alive = true;
-        for (long long r = r_first; r < r_end && alive; r += 128, ++ti) {
-            // A wait names a phase by its parity alone, so it must not start more than one phase ahead of the barrier:
-            // the operand-row barriers go through pass 1's phases first (the other issuer's), hence the go-ahead.
-            if (!mbar_wait_warp(bar(DL_PASS2 + set), ti & 1, abort_flag)) break;
-            op_uses += n_own;                                            // pass 1's uses of the operand rows
-            int n = (ti * 3 + 1) * n_own;                                 // ring position of pass 2, first slice
-            for (int s = set; s < S; s += DL_NSET, ++n) {
-                const int i = wslot(set, n);
-                if (!mbar_wait_warp(bar(DL_OP_READY + set), op_uses & 1, abort_flag)) { alive = false; break; }
-                ++op_uses;
-                // (its weights are there: the other issuer saw this phase complete before it made the l this operand was built
-                // from, and the next one waits for this product)
-                if (!mbar_wait_warp(bar(DL_WFULL + i), (n / DL_NSW) & 1, abort_flag)) { alive = false; break; }
-                tc_fence_after();
-                if (elect_one()) {
-                    const uint64_t db = smem_desc(wstage(i) + TILE);
+        for (long long r = r_first; r < r_end && alive; r += 128) {
+            for (int pass = 0; pass < 2 && alive; ++pass)
+                for (int s = 0; s < S; ++s, ++n) {
+                    const int set = n & (DL_NSET - 1);
+                    if (!wait_warp(DL_OP_READY + set, phases >> set)) { alive = false; break; }
+                    phases ^= 1u << set;
+                    if (!wait_warp(DL_AFULL + ia, pa)) { alive = false; break; }
+                    tc_fence_after();
+                    if (elect_one()) {
+                        const uint64_t db = smem_desc(astage(ia));
+                        const uint32_t ta = tmem + DL_TM_OP + 32 * set;
 #pragma unroll
-                    for (int kk = 0; kk < 4; ++kk)
-                        tc_mma_ta(tsum, ta + 8 * kk, db + (uint64_t)(128 * kk), DL_IDESC, (s > set || kk > 0) ? 1u : 0u);
-                    tc_commit(bar(DL_OP_FREE + set));
-                    tc_commit(bar(DL_WEMPTY + i));
-                    if (s + DL_NSET >= S) tc_commit(bar(DL_SUM_FULL));
+                        for (int kk = 0; kk < 4; ++kk)
+                            tc_mma_ta(tmem + DL_TM_SUM, ta + 8 * kk, db + (uint64_t)(128 * kk), DL_IDESC, (s > 0 || kk > 0) ? 1u : 0u);
+                        tc_commit(bar(DL_OP_FREE + set));
+                        tc_commit(bar(DL_AEMPTY + ia));
+                        if (s == S - 1) tc_commit(bar(DL_SUM_FULL));
+                    }
+                    __syncwarp();
+                    if (++ia == DL_NSA) { ia = 0; pa ^= 1; }
                 }
-                __syncwarp();
+            n += S;
+        }
+    } else if (warp == 3 || warp > DL_WB) {
+        // ============================== MMA issuers: l = h1 B_d (pass 2), d = h2 B_w (pass 3) of the even / odd slices ==============================
+        const int odd = warp > DL_WB;
+        int n0 = 0, ib = 0, pb = 0;                          // (B ring position and its phase)
+        uint32_t phases = (1u << DL_NSET) - 1;               // bit: parity of the set's accumulator's last release
+        bool alive = true;
+        for (long long r = r_first; r < r_end && alive; r += 128) {
+            n0 += S;
+            for (int pass = 1; pass < 3 && alive; ++pass, n0 += S) {
+                if (!wait_warp(DL_H_READY, pass - 1)) { alive = false; break; }      // (two uses per tile: parities 0, 1)
+                const int kn = pass == 1 ? p.kd : p.kw;
+                for (int n = n0 + ((n0 ^ odd) & 1); n < n0 + S; n += 2) {
+                    const int set = n & (DL_NSET - 1), slot = odd * DL_NSB + ib;
+                    // (before its first use an accumulator is free: the phase before the barrier's first)
+                    if (!wait_warp(DL_BFULL + slot, pb) || !wait_warp(DL_ACC_FREE + set, phases >> set)) { alive = false; break; }
+                    phases ^= 1u << set;
+                    tc_fence_after();
+                    if (elect_one()) {
+                        const uint64_t db = smem_desc(bstage(slot));
+#pragma unroll
+                        for (int kk = 0; kk < 4; ++kk)
+                            if (kk < kn) tc_mma_ta(tmem + DL_TM_ACC + 64 * set, tmem + DL_TM_H + 8 * kk, db + (uint64_t)(128 * kk), DL_IDESC, kk > 0 ? 1u : 0u);
+                        tc_commit(bar(DL_ACC_FULL + set));
+                        tc_commit(bar(DL_BEMPTY + slot));
+                    }
+                    __syncwarp();
+                    if (++ib == DL_NSB) { ib = 0; pb ^= 1; }
+                }
             }
-            if (n_own == 0 && elect_one()) mbar_arrive(bar(DL_SUM_FULL));
+            if (alive && elect_one()) tc_commit(bar(DL_H_FREE));      // (all products of this warp so far)
             __syncwarp();
         }
     } else {
         // ============================== worker warps ==============================
-        const int set = (warp - DL_W0) / DL_NWS;         // takes the slices s with s mod DL_NSET == set
-        const int n_own = (S - set + DL_NSET - 1) / DL_NSET;
-        const uint32_t tring = tmem + DL_TM_RING + 64 * DL_NACC * set;
+        const int set = (warp - DL_W0) / DL_NWS;         // takes the slices n with n mod 4 == set
         const int sp = warp & 3;                         // tensor-memory sub-partition: accumulator rows 32*sp .. 32*sp+31
         const int row = 32 * sp + lane;                  // this lane's token row inside the tile
-        const uint32_t tlane = (uint32_t)(32 * sp) << 16;
-        const uint32_t own_tile = (uint32_t)(row >> 6) * TILE, own_row = (uint32_t)(row & 63);
-        const uint32_t up_tile = (uint32_t)((row - 1) >> 6) * TILE, up_row = (uint32_t)((row - 1) & 63);   // (row > 0)
-        const uint32_t own_xor = (own_row & 7) << 4;
-        const uint32_t slab0 = sbase + DL_OFF_OUT + set * 2 * TILE + sp * 4096;     // pass 3: this warp's output slab, 32 rows x 128 B
-        int op_uses = 0;
-        bool alive = true;
-
-        // h = tanh(acc), acc the sum of the sets' halves, for this warp's 32 rows and its share of the 64 columns -> bf16
-        // operand rows
-        auto squash = [&]() {
-#pragma unroll
-            for (int g = 0; g < DL_NH; ++g) {
-                const int c0 = 32 * set + 16 * g;
-                float a[16], b[16];
-                tmem_ld_row16(tmem + tlane + DL_TM_SUM + c0, a);
-                if (S > 1) tmem_ld_row16(tmem + tlane + DL_TM_SUM + 64 + c0, b);
-#pragma unroll
-                for (int e = 0; e < 16; ++e) a[e] = S > 1 ? a[e] + b[e] : a[e];
-                uint32_t ow[8];
-#pragma unroll
-                for (int e = 0; e < 8; ++e) ow[e] = pack_bf16(tanh_fast(a[2 * e]), tanh_fast(a[2 * e + 1]));
-                tmem_st_row8(tmem + tlane + DL_TM_H + c0 / 2, ow);
+        const uint32_t tlane = tmem + ((uint32_t)(32 * sp) << 16);
+        const uint32_t own_off = 128 * row, own_xor = (row & 7) << 4;
+        const uint32_t up_off = row == 0 ? DL_OFF_PREV : 128 * (row - 1), up_xor = row == 0 ? 0u : ((row - 1) & 7) << 4;
+        uint32_t op_phase = 1, acc_phase = 0;            // (parity of the operand's last release; of the accumulator's next arrival)
+        int pending = -1;                                // x stage whose room holds an output slab that a store may still be reading
+        auto release_pending = [&]() {
+            if (pending >= 0) {
+                if (lane == 0) bulk_wait_read<0>();
+                __syncwarp();
+                mbar_arrive_if(bar(DL_XEMPTY + pending), lane == 0);
+                pending = -1;
             }
-            tmem_st_done();
         };
-        static_assert(DL_NSET == 2, "the sum of two halves");
-
-        int it = 0, ti = 0;
+        int ti = 0;
+        bool alive = true;
         for (long long r = r_first; r < r_end && alive; r += 128, ++ti) {
             const long long tok = r + row;
             const bool live = r + 32 * sp < r_end;       // (a tile of 64 rows: two row groups only keep the barriers company)
             const bool seq_start = (tok % p.T) == 0;     // the row above belongs to another sequence: x_prev or zero
             const bool any_start = __any_sync(0xffffffffu, seq_start);
-            const __nv_bfloat16* gp0 = (seq_start && p.x_prev && tok < p.rows) ? p.x_prev + (tok / p.T) * (long long)p.D : nullptr;
+            const __nv_bfloat16* gp = (seq_start && p.x_prev && tok < p.rows) ? p.x_prev + (tok / p.T) * (long long)p.D : nullptr;
+            int n0 = ti * 3 * S;
             // ---- passes 1 and 2: out = x + (x_above - x) * mix, mix = the pass's constants (+ l from tensor memory in pass 2).
             // The interpolation runs on packed bf16 pairs (difference, then one fused multiply-add with a single rounding):
             // its inputs and its output are bf16 anyway, and the mix is smooth in them.
-            for (int pass = 0; pass < 2 && alive; ++pass) {
-                for (int s = set; s < S; s += DL_NSET, ++it) {
-                    const int i = xslot(set, it);
-                    const uint32_t stage = sbase + i * DL_XSTAGE;
-                    if (!mbar_wait(bar(DL_XFULL + i), (it / DL_NSX) & 1, abort_flag)) { alive = false; break; }
-                    const int an = ti * 2 * n_own + s / DL_NSET, acc = an % DL_NACC;             // this slice's l: the set's an-th accumulator
+#pragma unroll 1
+            for (int pass = 0; pass < 2 && alive; ++pass, n0 += S) {
+#pragma unroll 1
+                for (int n = n0 + ((set - n0) & (DL_NSET - 1)); n < n0 + S; n += DL_NSET) {
+                    const uint32_t stage = xstage(n);
+                    if (!wait(DL_XFULL + (n & (DL_NSX - 1)), n / DL_NSX)) { alive = false; break; }
                     if (pass == 1) {
-                        if (!mbar_wait(bar(DL_ACC_FULL + DL_NACC * set + acc), (an / DL_NACC) & 1, abort_flag)) { alive = false; break; }
+                        if (!wait(DL_ACC_FULL + set, acc_phase)) { alive = false; break; }
+                        acc_phase ^= 1;
                         tc_fence_after();
                     }
-                    // this lane's row and the row above it (inside the tiles, or the extra row of the stage for the tile's
-                    // first row)
-                    const uint32_t up_base = row == 0 ? stage + DL_OFF_PREV : stage + up_tile + up_row * 128;
-                    const uint32_t up_xor = row == 0 ? 0u : (up_row & 7) << 4;
-                    const uint32_t own_base = stage + own_tile + own_row * 128;
+                    __syncwarp();
                     if (!live) {
-                        if (pass == 1) { tc_fence_before(); __syncwarp(); mbar_arrive_if(bar(DL_ACC_FREE + DL_NACC * set + acc), lane == 0); }
-                        __syncwarp();
-                        mbar_arrive_if(bar(DL_XEMPTY + i), lane == 0);
-                        if (op_uses >= 1 && !mbar_wait(bar(DL_OP_FREE + set), (op_uses - 1) & 1, abort_flag)) { alive = false; break; }
+                        if (pass == 1) { tc_fence_before(); __syncwarp(); mbar_arrive_if(bar(DL_ACC_FREE + set), lane == 0); }
+                        mbar_arrive_if(bar(DL_XEMPTY + (n & (DL_NSX - 1))), lane == 0);
+                        if (!wait(DL_OP_FREE + set, op_phase)) { alive = false; break; }
                     } else
 #pragma unroll
-                    for (int g = 0; g < DL_NH; ++g) {
-                        const int hf = g;
-                        uint32_t mixw[16];               // the mix of 32 channels as bf16 pairs
-                        if (pass == 1) {
-                            uint32_t l[32];
-                            kc::tmem_ld_row32(tring + tlane + 64 * acc + 32 * hf, l);
-                            if (g == DL_NH - 1) {        // the accumulator row has been read: hand it back
-                                tc_fence_before();
-                                __syncwarp();
-                                mbar_arrive_if(bar(DL_ACC_FREE + DL_NACC * set + acc), lane == 0);
-                            }
+                    for (int g = 0; g < 4; ++g) {        // 16 channels at a time (registers)
+                        float4 v4[4];
 #pragma unroll
-                            for (int q = 0; q < 8; ++q) {
-                                const float4 v4 = ldsf4(stage + DL_OFF_VEC + 128 * hf + 16 * q);
-                                mixw[2 * q] = pack_sum(v4.x, v4.y, l[4 * q], l[4 * q + 1]);
-                                mixw[2 * q + 1] = pack_sum(v4.z, v4.w, l[4 * q + 2], l[4 * q + 3]);
-                            }
+                        for (int q = 0; q < 4; ++q) v4[q] = ldsf4(stage + DL_OFF_VEC + 64 * g + 16 * q);
+                        uint4 a[2], b[2];
+#pragma unroll
+                        for (int q = 0; q < 2; ++q) {
+                            const uint32_t o = (uint32_t)((2 * g + q) << 4);
+                            a[q] = lds128(stage + own_off + (o ^ own_xor));
+                            b[q] = lds128(stage + up_off + (o ^ up_xor));
+                        }
+                        float l[16];
+                        if (pass == 1) {
+                            tmem_ld_row16(tlane + DL_TM_ACC + 64 * set + 16 * g, l);
                         } else {
 #pragma unroll
-                            for (int q = 0; q < 8; ++q) {
-                                const float4 v4 = ldsf4(stage + DL_OFF_VEC + 128 * hf + 16 * q);
-                                mixw[2 * q] = pack_bf16(v4.x, v4.y);
-                                mixw[2 * q + 1] = pack_bf16(v4.z, v4.w);
-                            }
+                            for (int e = 0; e < 16; ++e) l[e] = 0.f;
                         }
-                        uint4 a[4], b[4];
-#pragma unroll
-                        for (int q = 0; q < 4; ++q) {
-                            const uint32_t o = (uint32_t)((4 * hf + q) << 4);
-                            a[q] = lds128(own_base + (o ^ own_xor));
-                            b[q] = lds128(up_base + (o ^ up_xor));
-                        }
-                        if (g == DL_NH - 1) {            // all in registers: the stage is free for a later slice
+                        if (g == 3) {                    // all in registers: accumulator and stage are free for later slices
+                            if (pass == 1) tc_fence_before();
                             __syncwarp();
-                            mbar_arrive_if(bar(DL_XEMPTY + i), lane == 0);
+                            if (pass == 1) mbar_arrive_if(bar(DL_ACC_FREE + set), lane == 0);
+                            mbar_arrive_if(bar(DL_XEMPTY + (n & (DL_NSX - 1))), lane == 0);
                         }
                         if (any_start && seq_start) {
 #pragma unroll
-                            for (int q = 0; q < 4; ++q)
-                                b[q] = gp0 ? *reinterpret_cast<const uint4*>(gp0 + 64 * s + 32 * hf + 8 * q) : make_uint4(0u, 0u, 0u, 0u);
+                            for (int q = 0; q < 2; ++q)
+                                b[q] = gp ? *reinterpret_cast<const uint4*>(gp + 64 * (n - n0) + 16 * g + 8 * q) : make_uint4(0u, 0u, 0u, 0u);
                         }
-                        // the operand rows: free of the product that read them last
-                        if (g == 0 && op_uses >= 1 && !mbar_wait(bar(DL_OP_FREE + set), (op_uses - 1) & 1, abort_flag)) { alive = false; break; }
-                        uint32_t ow[16];
+                        uint32_t ow[8];
 #pragma unroll
-                        for (int q = 0; q < 4; ++q) {
+                        for (int q = 0; q < 2; ++q) {
                             const uint32_t aw[4] = {a[q].x, a[q].y, a[q].z, a[q].w}, bw[4] = {b[q].x, b[q].y, b[q].z, b[q].w};
 #pragma unroll
                             for (int e = 0; e < 4; ++e) {
+                                const float4 v = v4[2 * q + (e >> 1)];
+                                const uint32_t mix = pack_sum((e & 1) ? v.z : v.x, (e & 1) ? v.w : v.y, __float_as_uint(l[8 * q + 2 * e]), __float_as_uint(l[8 * q + 2 * e + 1]));
                                 uint32_t delta;
                                 asm("sub.rn.bf16x2 %0, %1, %2;" : "=r"(delta) : "r"(bw[e]), "r"(aw[e]));
-                                asm("fma.rn.bf16x2 %0, %1, %2, %3;" : "=r"(ow[4 * q + e]) : "r"(delta), "r"(mixw[4 * q + e]), "r"(aw[e]));
+                                asm("fma.rn.bf16x2 %0, %1, %2, %3;" : "=r"(ow[4 * q + e]) : "r"(delta), "r"(mix), "r"(aw[e]));
                             }
                         }
-                        if (g == 0) tc_fence_after();
-                        __syncwarp();
-                        tmem_st_row16(tmem + tlane + DL_TM_OP + 32 * set + 16 * hf, ow);
+                        if (g == 0) {                    // the operand rows: free of the product that read them last
+                            if (!wait(DL_OP_FREE + set, op_phase)) { alive = false; break; }
+                            tc_fence_after();
+                            __syncwarp();
+                        }
+                        tmem_st_row8(tlane + DL_TM_OP + 32 * set + 8 * g, ow);
                     }
                     if (!alive) break;
-                    ++op_uses;
+                    op_phase ^= 1;
                     tmem_st_done();
                     tc_fence_before();
                     __syncwarp();
                     mbar_arrive_if(bar(DL_OP_READY + set), lane == 0);
                 }
                 if (!alive) break;
-                // the pass's low-rank sum is complete: squash it into the operand of the next product
-                if (!mbar_wait(bar(DL_SUM_FULL), pass, abort_flag)) { alive = false; break; }      // (two uses per tile)
+                // the pass's low-rank sum is complete: h = tanh(sum), 16 columns per set -> operand of the next products
+                if (!wait(DL_SUM_FULL, pass)) { alive = false; break; }      // (two uses per tile)
+                if (pass == 0 && ti > 0 && !wait(DL_H_FREE, ti - 1)) { alive = false; break; }
                 tc_fence_after();
-                if (live) squash();
+                __syncwarp();
+                if (live && set < (pass == 0 ? p.kd : p.kw)) {
+                    float a[16];
+                    tmem_ld_row16(tlane + DL_TM_SUM + 16 * set, a);
+                    uint32_t ow[8];
+#pragma unroll
+                    for (int e = 0; e < 8; ++e) ow[e] = pack_bf16(tanh_fast(a[2 * e]), tanh_fast(a[2 * e + 1]));
+                    tmem_st_row8(tlane + DL_TM_H + 8 * set, ow);
+                    tmem_st_done();
+                }
                 tc_fence_before();
                 __syncwarp();
                 mbar_arrive_if(bar(DL_H_READY), lane == 0);
             }
             if (!alive) break;
-            // ---- pass 3: d slice -> bf16 slab -> TMA store
-            for (int s = set; s < S; s += DL_NSET, ++it) {
-                const int i = xslot(set, it);
-                const uint32_t stage = sbase + i * DL_XSTAGE;
-                if (!mbar_wait(bar(DL_XFULL + i), (it / DL_NSX) & 1, abort_flag)) { alive = false; break; }
-                const int an = ti * 2 * n_own + n_own + s / DL_NSET, acc = an % DL_NACC;         // this slice's d
-                if (!mbar_wait(bar(DL_ACC_FULL + DL_NACC * set + acc), (an / DL_NACC) & 1, abort_flag)) { alive = false; break; }
+            // ---- pass 3: d slice -> bf16, in the room of the x stage -> TMA store
+#pragma unroll 1
+            for (int n = n0 + ((set - n0) & (DL_NSET - 1)); n < n0 + S; n += DL_NSET) {
+                const uint32_t stage = xstage(n), vec = stage + DL_OFF_VEC, slab = stage + sp * 4096;
+                release_pending();
+                if (!wait(DL_XFULL + (n & (DL_NSX - 1)), n / DL_NSX) || !wait(DL_ACC_FULL + set, acc_phase)) { alive = false; break; }
+                acc_phase ^= 1;
                 tc_fence_after();
+                __syncwarp();
                 if (!live) {
                     tc_fence_before();
                     __syncwarp();
-                    mbar_arrive_if(bar(DL_ACC_FREE + DL_NACC * set + acc), lane == 0);
-                    mbar_arrive_if(bar(DL_XEMPTY + i), lane == 0);
+                    mbar_arrive_if(bar(DL_ACC_FREE + set), lane == 0);
+                    mbar_arrive_if(bar(DL_XEMPTY + (n & (DL_NSX - 1))), lane == 0);
                     continue;
                 }
-                if (lane == 0) bulk_wait_read<0>();      // this warp's previous stores have finished reading the slabs
-                __syncwarp();
 #pragma unroll
-                for (int g = 0; g < DL_NH; ++g) {
-                    const int hf = g;
-                    uint32_t v[32];
-                    kc::tmem_ld_row32(tring + tlane + 64 * acc + 32 * hf, v);
-                    if (g == DL_NH - 1) {
+                for (int g = 0; g < 4; ++g) {
+                    float4 v4[4];
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) v4[q] = ldsf4(vec + 64 * g + 16 * q);
+                    float v[16];
+                    tmem_ld_row16(tlane + DL_TM_ACC + 64 * set + 16 * g, v);
+                    if (g == 3) {
                         tc_fence_before();
                         __syncwarp();
-                        mbar_arrive_if(bar(DL_ACC_FREE + DL_NACC * set + acc), lane == 0);
+                        mbar_arrive_if(bar(DL_ACC_FREE + set), lane == 0);
                     }
+                    uint32_t o[8];
 #pragma unroll
                     for (int q = 0; q < 4; ++q) {
-                        const float4 la = ldsf4(stage + DL_OFF_VEC + 128 * hf + 32 * q), lb = ldsf4(stage + DL_OFF_VEC + 128 * hf + 32 * q + 16);
-                        sts128(slab0 + swz(lane, (4 * hf + q) << 4),
-                               make_uint4(pack_sum(la.x, la.y, v[8 * q], v[8 * q + 1]), pack_sum(la.z, la.w, v[8 * q + 2], v[8 * q + 3]),
-                                          pack_sum(lb.x, lb.y, v[8 * q + 4], v[8 * q + 5]), pack_sum(lb.z, lb.w, v[8 * q + 6], v[8 * q + 7])));
+                        o[2 * q] = pack_sum(v4[q].x, v4[q].y, __float_as_uint(v[4 * q]), __float_as_uint(v[4 * q + 1]));
+                        o[2 * q + 1] = pack_sum(v4[q].z, v4[q].w, __float_as_uint(v[4 * q + 2]), __float_as_uint(v[4 * q + 3]));
                     }
+#pragma unroll
+                    for (int q = 0; q < 2; ++q)
+                        sts128(slab + swz(lane, (2 * g + q) << 4), make_uint4(o[4 * q], o[4 * q + 1], o[4 * q + 2], o[4 * q + 3]));
                 }
-                __syncwarp();
-                mbar_arrive_if(bar(DL_XEMPTY + i), lane == 0);
                 fence_proxy_async();
                 __syncwarp();
                 const long long grow = r + 32 * sp;
                 if (lane == 0 && grow < p.rows) {
-                    tma_store_2d(&tm_d32, 64 * s, (int)grow, slab0);
+                    tma_store_2d(&tm_d32, 64 * (n - n0), (int)grow, slab);
                     bulk_commit();
                 }
+                pending = n & (DL_NSX - 1);
             }
-            if (!alive) break;
+            release_pending();
         }
         if (lane == 0) bulk_wait<0>();
     }
 
     tc_fence_before();
     __syncthreads();
-    if (warp == 1) {
+    if (warp == 2) {
         tc_fence_after();
         tmem_dealloc(tmem, 512);
     }

@@ -56,6 +56,25 @@ def test_shares_of_rows_and_slices(rows, D):
     _run(1, rows, D, 32, 64, seed=rows + D)
 
 
+@pytest.mark.parametrize("D,Rd,Rw", [(64, 64, 16), (128, 16, 64), (320, 64, 48), (448, 32, 64)])
+def test_sets_issuers_and_rings_over_several_tiles(D, Rd, Rw):
+    """Fewer slices than worker sets or none for one of the two issuers of h B, counts that are no multiple of either, and rings
+    (3, 5, 8 stages) that wrap at every offset: three tiles and a half per CTA, sequences that start inside them.  A slice, row or
+    tile that went wrong is an error of the order of d itself, in its token's norm 1 / sqrt(D / 64) or more (0.37 here): bounded by
+    the token's and the tensor's norms as above, not element by element (of 4 to 30 million elements a few lie past that bound,
+    which is five standard deviations of the roundings)."""
+    B, T = 7, (64 * 148 * 7 - 131) // 7
+    x, xp = synth.make_block_input(B, T, D, seed=D)
+    w = synth.make_decay_lora(D, Rd, Rw, seed=D + 1)
+    dev = {k: v.to(DEV) for k, v in w.items()}
+    d = gf.decay_logit(x.to(DEV), dev["mu_x"], dev["A_d"], dev["B_d"], dev["lambda_d"], dev["A_w"], dev["B_w"], dev["lambda_w"], x_prev=xp.to(DEV))
+    gf.last_device_status()
+    ref = orc.decay_logit(x, w["mu_x"], w["A_d"], w["B_d"], w["lambda_d"], w["A_w"], w["B_w"], w["lambda_w"], xp)
+    err = d.float().cpu().numpy() - ref
+    assert np.sqrt((err ** 2).sum() / (ref ** 2).sum()) <= 5e-3
+    assert np.sqrt((err ** 2).sum(-1) / (ref ** 2).sum(-1)).max() <= 1e-2
+
+
 def test_repeats_bit_for_bit():
     """Two worker sets with rings of their own: no set may pass on a phase of the other's."""
     x, xp = synth.make_block_input(4, 16384, 1024, seed=31, device=DEV)
