@@ -40,8 +40,12 @@
 // Each group has its own input stage (x, v, dy and r, k by TMA, each part re-filled as soon as its tiles fall free),
 // operand tiles, tensor-memory columns (three accumulators that the second group of products reuses once the first
 // group's have been read) and barriers; the four staging tiles of the gradients lie over operand tiles that are dead
-// by the time they are written.  One lane of a group issues its copies, two others (in other warps) its two groups of
-// products, so that no warp carries all the issuing.  Sums along the tokens (the
+// by the time they are written.  One warp of a group issues its copies, two others its two groups of
+// products, one its prefetches, so that no warp carries all the issuing; each through an elected lane of the converged warp: a thread in a
+// divergent branch takes about 100 cycles per product or copy to pass its operands through uniform registers, 36 products and
+// 16 copies a chunk (8 x 2048 x 32 heads Finch-C2 217.6 -> 194.7 us for the products, classic 4 x 4096 206 -> 199 for the copies; the next
+// chunk's prefetches behind the hand-over of the adjoint instead of at the top, where they delay the first chunks' copies: 188.6 and 193;
+// 1 x 16384 Finch-C2 287 -> 254 in all).  dV's products in a warp of their own: not better (198).  Sums along the tokens (the
 // cumulative decay; the suffix sums of the decay gradient) cross the two column slabs through shared memory.  Waits are per thread and bounded; their outcome is made uniform over the group at its next
 // barrier, and the hand-over waits watch the CTA's abort word, so after a wait that ran out both groups leave.
 // A chunk in which a channel decays by more than 2^-96 runs token by token in fp32 on its group's warps (its 64
@@ -471,20 +475,29 @@ wkv6_backward_chunked_kernel(const __grid_constant__ CUtensorMap tm_x, const __g
     const uint32_t o_dr = t_sb, o_dk = t_dpp, o_dv = t_pp, o_dx = t_gb;
     // The input copies of a chunk come in two parts, each issued as soon as its tiles are free: x, v, dy once the
     // chunk before (of this group) has finished its products, r, k once its epilogue has read them.
-    int last_a = -1, last_b = -1, last_s = -1;       // (thread 0 of the group) the last iterations whose copies were issued
-    auto issue_loads_a = [&](int it) {               // thread 0 of the group
+    // (the group's first warp issues its copies, through an elected lane: the same one every time, so that the stores it has
+    // committed are its own to wait for)
+    const int gwarp = warp & (G_GT / 32 - 1);        // warp of the group
+    int last_a = -1, last_b = -1, last_s = -1;       // (first warp of the group) the last iterations whose copies were issued
+    auto issue_loads_a = [&](int it) {               // first warp of the group
         const int row = row_at(it), col = col_at(it);
-        mbar_expect_tx(gb(GB_INA), 3 * TILE);
-        tma_load_2d(tx, &tm_x, col, row, gb(GB_INA));
-        tma_load_2d(tv, &tm_v, col, row, gb(GB_INA));
-        tma_load_2d(tdy, &tm_dy, col, row, gb(GB_INA));
+        if (elect_one()) {
+            mbar_expect_tx(gb(GB_INA), 3 * TILE);
+            tma_load_2d(tx, &tm_x, col, row, gb(GB_INA));
+            tma_load_2d(tv, &tm_v, col, row, gb(GB_INA));
+            tma_load_2d(tdy, &tm_dy, col, row, gb(GB_INA));
+        }
+        __syncwarp();
         last_a = it;
     };
     auto issue_loads_b = [&](int it) {
         const int row = row_at(it), col = col_at(it);
-        mbar_expect_tx(gb(GB_INB), 2 * TILE);
-        tma_load_2d(tr, &tm_r, col, row, gb(GB_INB));
-        tma_load_2d(tk, &tm_k, col, row, gb(GB_INB));
+        if (elect_one()) {
+            mbar_expect_tx(gb(GB_INB), 2 * TILE);
+            tma_load_2d(tr, &tm_r, col, row, gb(GB_INB));
+            tma_load_2d(tk, &tm_k, col, row, gb(GB_INB));
+        }
+        __syncwarp();
         last_b = it;
     };
     auto load_f32_block = [&](const float* src, float (&v)[G_NB][4]) {      // [64][64] fp32 block, the lane's cells
@@ -510,9 +523,14 @@ wkv6_backward_chunked_kernel(const __grid_constant__ CUtensorMap tm_x, const __g
     };
     // the chunk-start state is a bf16 [64][64] tile in memory: it lands in its operand tile by TMA (rows of the
     // checkpoint array seen as [slots * 64][64])
-    auto issue_load_s = [&](int it) {                // thread 0 of the group
-        mbar_expect_tx(gb(GB_S0), TILE);
-        tma_load_2d(t_sb, &tm_ck, 0, (int)(slot_at(it) * 64), gb(GB_S0));
+    auto issue_load_s = [&](int it) {                // first warp of the group
+        const int row = (int)(slot_at(it) * 64);
+        if (elect_one()) {
+            if (it > 1) bulk_wait_read<0>();         // the previous chunk's staging tiles have been read by the TMA unit
+            mbar_expect_tx(gb(GB_S0), TILE);
+            tma_load_2d(t_sb, &tm_ck, 0, row, gb(GB_S0));
+        }
+        __syncwarp();
         last_s = it;
     };
     auto load_bf16_block = [&](const __nv_bfloat16* src, float (&v)[G_NB][4]) {     // a checkpoint, the lane's cells
@@ -543,8 +561,20 @@ wkv6_backward_chunked_kernel(const __grid_constant__ CUtensorMap tm_x, const __g
         }
         du_acc[0] = du_acc[1] = 0.f;
     };
+    // this group's next chunk: its start state and its input tiles into L2 now, so that the copies issued later find them there
+    auto prefetch_next = [&](int it) {
+        if (it + 2 < nit && gwarp == 4) {
+            const int row = row_at(it + 2), col = col_at(it + 2), row_s = GSUM ? 0 : (int)(slot_at(it + 2) * 64);
+            if (elect_one()) {
+                tma_prefetch_2d(&tm_x, col, row); tma_prefetch_2d(&tm_r, col, row); tma_prefetch_2d(&tm_k, col, row);
+                tma_prefetch_2d(&tm_v, col, row); tma_prefetch_2d(&tm_dy, col, row);
+                if (!GSUM) tma_prefetch_2d(&tm_ck, 0, row_s);
+            }
+            __syncwarp();
+        }
+    };
     if (BAL) pc = 0;
-    if (gt == 0 && grp < nit) { issue_loads_a(grp); issue_loads_b(grp); }
+    if (gwarp == 0 && grp < nit) { issue_loads_a(grp); issue_loads_b(grp); }
     if (BAL) pc = -1;
     int mph = 0;                                     // phase bit of this group's two product barriers
     float dprod_lo = 1.f, dprod_hi = 1.f;            // summary variant: product of this group's chunk decays (rows R0, R1)
@@ -561,20 +591,10 @@ wkv6_backward_chunked_kernel(const __grid_constant__ CUtensorMap tm_x, const __g
         const int c = BAL ? pt(pc, 5) - it : chunk_of(it), valid = min(L, T - c * L);
         const bool first = BAL ? it == pt(pc, 7) : it == 0, last = BAL ? it + 1 == pt(pc, 0) : it + 1 == nit;      // of the piece
         const int use = it >> 1;                     // how often this group's input stage has been filled before
-        if (it + 2 < nit && gt == 128) {
-            // this group's next chunk: its start state and its input tiles into L2 now, so that the copies issued
-            // later find them there
-            const int row = row_at(it + 2), col = col_at(it + 2);
-            tma_prefetch_2d(&tm_x, col, row); tma_prefetch_2d(&tm_r, col, row); tma_prefetch_2d(&tm_k, col, row);
-            tma_prefetch_2d(&tm_v, col, row); tma_prefetch_2d(&tm_dy, col, row);
-            if (!GSUM) tma_prefetch_2d(&tm_ck, 0, (int)(slot_at(it + 2) * 64));
-        }
+        if (GSUM) prefetch_next(it);
         // ---- decay: log2-domain magnitudes, cumulative sums over the tokens
         bool ok = mbar_wait(gb(GB_INA), use & 1, abort_flag);
-        if (gt == 0) {
-            if (it > 1) bulk_wait_read<0>();         // the previous chunk's staging tiles have been read by the TMA unit
-            if (!GSUM) issue_load_s(it);             // (the start state's tile doubles as the staging tile of dr)
-        }
+        if (!GSUM && gwarp == 0) issue_load_s(it);   // (the start state's tile doubles as the staging tile of dr)
         float a[G_NB][4], lw2[G_NB][4];
         {
             float xv[G_NB][4];
@@ -654,19 +674,22 @@ wkv6_backward_chunked_kernel(const __grid_constant__ CUtensorMap tm_x, const __g
         fence_proxy_async();
         tc_fence_before();
         const bool unsafe = !gbar_and(grp, safe);    // (every channel is some lane's row)
-        if (!unsafe && gt == 64) {
+        if (!unsafe && gwarp == 2) {
             // the products that need nothing but the inputs; the adjoint is not needed for R^^T dY either
             tc_fence_after();
-            const uint64_t dR = smem_desc(t_rh), dK = smem_desc(t_kh), dV = smem_desc(tv), dY = smem_desc(tdy);
+            if (elect_one()) {
+                const uint64_t dR = smem_desc(t_rh), dK = smem_desc(t_kh), dV = smem_desc(tv), dY = smem_desc(tdy);
 #pragma unroll
-            for (int kk = 0; kk < 4; ++kk) {
-                const uint64_t ks = 2 * kk, ms = 128 * kk;       // K-major / MN-major step of 16 contraction indices
-                tc_mma(tmem + GT_DG, dR + ms, dY + ms, IDESC_MN_MN, kk > 0);       // dG[c][j] = R^^T dY
-                if (GSUM) continue;
-                tc_mma(tmem + GT_P, dR + ks, dK + ks, IDESC_K_K, kk > 0);          // P[t][i]  = R^ K^^T
-                tc_mma(tmem + GT_DP, dY + ks, dV + ks, IDESC_K_K, kk > 0);         // dP[t][i] = dY V^T
+                for (int kk = 0; kk < 4; ++kk) {
+                    const uint64_t ks = 2 * kk, ms = 128 * kk;       // K-major / MN-major step of 16 contraction indices
+                    tc_mma(tmem + GT_DG, dR + ms, dY + ms, IDESC_MN_MN, kk > 0);       // dG[c][j] = R^^T dY
+                    if (GSUM) continue;
+                    tc_mma(tmem + GT_P, dR + ks, dK + ks, IDESC_K_K, kk > 0);          // P[t][i]  = R^ K^^T
+                    tc_mma(tmem + GT_DP, dY + ks, dV + ks, IDESC_K_K, kk > 0);         // dP[t][i] = dY V^T
+                }
+                tc_commit(gb(GB_MA));
             }
-            tc_commit(gb(GB_MA));
+            __syncwarp();
         }
         // ---- the adjoint at the chunk's end, from the other group (the call's dstate_out for the last chunk)
         float G[G_NB][4];
@@ -923,9 +946,10 @@ wkv6_backward_chunked_kernel(const __grid_constant__ CUtensorMap tm_x, const __g
                 mph ^= 1;
                 tc_fence_before();
                 if (!gbar_and(grp, ok)) { alive = false; break; }
-                if (gt == 0 && it + 2 < nit) { issue_loads_a(it + 2); issue_loads_b(it + 2); }
+                if (gwarp == 0 && it + 2 < nit) { issue_loads_a(it + 2); issue_loads_b(it + 2); }
                 continue;
             }
+            prefetch_next(it);
             // ---- masked scores and their adjoint as operands
 #pragma unroll
             for (int h2 = 0; h2 < G_H2; ++h2) {
@@ -966,36 +990,39 @@ wkv6_backward_chunked_kernel(const __grid_constant__ CUtensorMap tm_x, const __g
             fence_proxy_async();
             tc_fence_before();
             if (!gbar_and(grp, ok)) { alive = false; break; }
-            if (gt == 160) {
+            if (gwarp == 5) {
                 tc_fence_after();
-                const uint64_t dR = smem_desc(t_rh), dK = smem_desc(t_kh), dV = smem_desc(tv), dY = smem_desc(tdy);
-                const uint64_t dS = smem_desc(t_sb), dG = smem_desc(t_gb), dP = smem_desc(t_pp), dD = smem_desc(t_dpp);
-                // dR^ and dK^ first (interleaved: products on one accumulator wait for each other), with a commit of
-                // their own: the epilogue starts on them while dV is still being formed
+                if (elect_one()) {
+                    const uint64_t dR = smem_desc(t_rh), dK = smem_desc(t_kh), dV = smem_desc(tv), dY = smem_desc(tdy);
+                    const uint64_t dS = smem_desc(t_sb), dG = smem_desc(t_gb), dP = smem_desc(t_pp), dD = smem_desc(t_dpp);
+                    // dR^ and dK^ first (interleaved: products on one accumulator wait for each other), with a commit of
+                    // their own: the epilogue starts on them while dV is still being formed
 #pragma unroll
-                for (int kk = 0; kk < 4; ++kk) {
-                    const uint64_t ks = 2 * kk;
-                    tc_mma(tmem + GT_DR, dS + ks, dY + ks, IDESC_K_K, kk > 0);         // dR^T[c][t] = S_0 dY^T
-                    tc_mma(tmem + GT_DK, dG + ks, dV + ks, IDESC_K_K, kk > 0);         // dK^T[c][i] = G^ V^T
-                }
+                    for (int kk = 0; kk < 4; ++kk) {
+                        const uint64_t ks = 2 * kk;
+                        tc_mma(tmem + GT_DR, dS + ks, dY + ks, IDESC_K_K, kk > 0);         // dR^T[c][t] = S_0 dY^T
+                        tc_mma(tmem + GT_DK, dG + ks, dV + ks, IDESC_K_K, kk > 0);         // dK^T[c][i] = G^ V^T
+                    }
 #pragma unroll
-                for (int kk = 0; kk < 4; ++kk) {
-                    const uint64_t ks = 2 * kk, ms = 128 * kk;
-                    tc_mma(tmem + GT_DR, dK + ms, dD + ks, IDESC_MN_K, 1);             // dR^T += K^^T dP'^T
-                    tc_mma(tmem + GT_DK, dR + ms, dD + ms, IDESC_MN_MN, 1);            // dK^T += R^^T dP'
-                }
-                tc_commit(gb(GB_MRK));
+                    for (int kk = 0; kk < 4; ++kk) {
+                        const uint64_t ks = 2 * kk, ms = 128 * kk;
+                        tc_mma(tmem + GT_DR, dK + ms, dD + ks, IDESC_MN_K, 1);             // dR^T += K^^T dP'^T
+                        tc_mma(tmem + GT_DK, dR + ms, dD + ms, IDESC_MN_MN, 1);            // dK^T += R^^T dP'
+                    }
+                    tc_commit(gb(GB_MRK));
 #pragma unroll
-                for (int kk = 0; kk < 4; ++kk) {
-                    const uint64_t ks = 2 * kk, ms = 128 * kk;
-                    tc_mma(tmem + GT_DV, dK + ks, dG + ms, IDESC_K_MN, kk > 0);        // dV[i][j] = K^ G^
-                }
+                    for (int kk = 0; kk < 4; ++kk) {
+                        const uint64_t ks = 2 * kk, ms = 128 * kk;
+                        tc_mma(tmem + GT_DV, dK + ks, dG + ms, IDESC_K_MN, kk > 0);        // dV[i][j] = K^ G^
+                    }
 #pragma unroll
-                for (int kk = 0; kk < 4; ++kk) {
-                    const uint64_t ms = 128 * kk;
-                    tc_mma(tmem + GT_DV, dP + ms, dY + ms, IDESC_MN_MN, 1);            // dV += P'^T dY
+                    for (int kk = 0; kk < 4; ++kk) {
+                        const uint64_t ms = 128 * kk;
+                        tc_mma(tmem + GT_DV, dP + ms, dY + ms, IDESC_MN_MN, 1);            // dV += P'^T dY
+                    }
+                    tc_commit(gb(GB_MV));
                 }
-                tc_commit(gb(GB_MV));
+                __syncwarp();
             }
             ok = mbar_wait(gb(GB_MRK), mph, abort_flag);
             tc_fence_after();
@@ -1066,7 +1093,7 @@ wkv6_backward_chunked_kernel(const __grid_constant__ CUtensorMap tm_x, const __g
             if (!mbar_wait(gb(GB_MV), mph, abort_flag)) ok = false;
             mph ^= 1;
             tc_fence_after();
-            if (gt == 0 && it + 2 < nit) issue_loads_a(it + 2);
+            if (gwarp == 0 && it + 2 < nit) issue_loads_a(it + 2);
             {
                 float acc[G_NB][4];
 #pragma unroll
@@ -1077,7 +1104,7 @@ wkv6_backward_chunked_kernel(const __grid_constant__ CUtensorMap tm_x, const __g
             tc_fence_before();
             ok = scan_tokens<true>(z, gbase + GO_TOT, grp, cx, R0, lane, ok);
             if (!ok) { alive = false; break; }
-            if (gt == 0 && it + 2 < nit) issue_loads_b(it + 2);      // (r, k were last read before the barrier of the sums)
+            if (gwarp == 0 && it + 2 < nit) issue_loads_b(it + 2);      // (r, k were last read before the barrier of the sums)
             float E[2] = {0.f, 0.f};
 #pragma unroll
             for (int o = 0; o < G_NSLAB; ++o) { E[0] += gld(GO_EP + 4 * (o * 64 + R0)); E[1] += gld(GO_EP + 4 * (o * 64 + R1)); }
@@ -1107,18 +1134,21 @@ wkv6_backward_chunked_kernel(const __grid_constant__ CUtensorMap tm_x, const __g
             // the top of the group's next iteration, issued by one thread that would otherwise not wait for the others
             gbar(grp);
         }
-        if (gt == 0) {
+        if (gwarp == 0) {
             if (valid == L) {
                 const int row = row_at(it), col = col_at(it);
-                tma_store_2d(&tm_dr, col, row, o_dr);
-                tma_store_2d(&tm_dk, col, row, o_dk);
-                tma_store_2d(&tm_dv, col, row, o_dv);
-                tma_store_2d(&tm_dx, col, row, o_dx);
-                bulk_commit();
+                if (elect_one()) {
+                    tma_store_2d(&tm_dr, col, row, o_dr);
+                    tma_store_2d(&tm_dk, col, row, o_dk);
+                    tma_store_2d(&tm_dv, col, row, o_dv);
+                    tma_store_2d(&tm_dx, col, row, o_dx);
+                    bulk_commit();
+                }
+                __syncwarp();
             }
             if (unsafe && it + 2 < nit) { issue_loads_a(it + 2); issue_loads_b(it + 2); }      // (the other path has issued them)
             if constexpr (BAL) {
-                if (last && pt(pc, 6) == 1) {
+                if (last && lane == 0 && pt(pc, 6) == 1) {
                     __threadfence();                 // (the group's barrier above: every lane's part of the adjoint is written)
                     asm volatile("st.release.gpu.global.u64 [%0], %1;" ::"l"(p.words + blockIdx.x - 1), "l"(1ull) : "memory");
                 }
@@ -1155,8 +1185,9 @@ wkv6_backward_chunked_kernel(const __grid_constant__ CUtensorMap tm_x, const __g
             for (int h = 0; h < 2; ++h) du_acc[h] += __shfl_xor_sync(0xffffffffu, du_acc[h], d);
         if (q == 0) { gsm(GO_REDV)[cx * 64 + R0] = du_acc[0]; gsm(GO_REDV)[cx * 64 + R1] = du_acc[1]; }
     }
-    if (gt == 0) {
-        bulk_wait<0>();                              // the gradient tiles have reached memory
+    if (gwarp == 0) {
+        if (elect_one()) bulk_wait<0>();             // the gradient tiles have reached memory
+        __syncwarp();
         // no copy into shared memory may stay in flight
         if (last_a >= 0) mbar_wait(gb(GB_INA), (last_a >> 1) & 1, abort_flag, false);
         if (last_b >= 0) mbar_wait(gb(GB_INB), (last_b >> 1) & 1, abort_flag, false);
