@@ -1243,14 +1243,17 @@ inline int backward_split(long long units, int T, int n_sm, int* seg_chunks)
 
 // Workspace of the chunked gradient: checkpoints, bonus gradients per unit and segment, the adjoint's segment
 // summaries, the token-by-token path's scratch (one slot of 64 states per SM and group of warps).
-// Whether a dense gradient call of more units than SMs cuts units between CTAs (BParamsBal); the same rule as the forward
-// pass's (balance_pays), here too because a chunk takes longer the more SMs are at work.  Measured (us, one CTA per unit ->
-// balanced): 160 units of 32 chunks 222 -> 145, of 128 chunks 913 -> 595; not taken: 256 of 32 chunks 223 -> 231.
-inline bool backward_balance_pays(long long units, int n_chunks, int n_sm)
+// Whether a dense gradient call of more units than SMs cuts units between CTAs (BParamsBal): a CTA's range costs two pipeline fills and
+// the hand-over, so where whole units leave more than a fifth of the last round idle, and from an eighth on where the units are long.
+// Measured (us, one CTA per unit -> balanced): 160 units of 32 chunks 189 -> 122; Finch-C2 256 of 32 189.2 -> 184.0, of 64 361.6 -> 347.9,
+// 240 of 32 187.2 -> 173.7, 256 of 16 the same, 384 of 8 88.4 -> 90.3; classic 256 of 32 191.9 -> 193.7, of 64 364.6 -> 363.8, of 94
+// 531.4 -> 522.0.  (The workspace has room for either form.)
+inline bool backward_balance_pays(long long units, int n_chunks, int n_sm, bool c2 = true)
 {
     if (units <= n_sm || units / n_sm - 1 > bc::BAL_MAX_ROUNDS) return false;
     const long long rounds = (units + n_sm - 1) / n_sm, idle = rounds * n_sm - units;
-    return idle * n_chunks > 4LL * n_sm && idle * 5 > rounds * n_sm && 2LL * n_sm * n_sm * n_chunks < (1LL << 32);
+    const int share = n_chunks >= (c2 ? 16 : 64) ? 8 : 5;
+    return idle * n_chunks > 4LL * n_sm && idle * share > rounds * n_sm && 2LL * n_sm * n_sm * n_chunks < (1LL << 32);
 }
 // Floats of the bonus partial sums of a dense call, and of a balanced launch's hand-over blocks and words behind them.
 inline size_t backward_du_floats(long long units, int nseg, bool balanced) { return (size_t)units * (balanced ? bc::BAL_DU_SLOTS : nseg) * 64; }
@@ -1346,10 +1349,11 @@ inline gf_status_t chunked_backward(const __nv_bfloat16* r, const __nv_bfloat16*
     const size_t n_ckpt = cu ? (size_t)H * ckpt_slots : (size_t)units * nck;       // checkpoints: bf16 [64][64] tiles
     if (n_ckpt * 64 >= (1ull << 31)) return GF_ERR_UNSUPPORTED;                    // (32-bit TMA row coordinates)
     float* du_part = ckpt + n_ckpt * bc::CKPT_FLOATS;
-    bool bal = !cu && backward_balance_pays(units, (int)nck - 1, n_sm);
-    float* gsum = du_part + (cu ? (size_t)units * nalloc * 64 : backward_du_floats(units, nseg, bal));
+    const bool room = !cu && backward_balance_pays(units, (int)nck - 1, n_sm);      // (the workspace's layout does not depend on the form)
+    bool bal = room && backward_balance_pays(units, (int)nck - 1, n_sm, c2);
+    float* gsum = du_part + (cu ? (size_t)units * nalloc * 64 : backward_du_floats(units, nseg, room));
     float* hand = gsum + (size_t)units * (nalloc - 1) * bc::GSUM_FLOATS;
-    float* fb = hand + (cu ? 0 : backward_hand_floats(n_sm, bal));
+    float* fb = hand + (cu ? 0 : backward_hand_floats(n_sm, room));
     const int32_t* order = nullptr;
     if (cu) {
         // packed: the sequences longest first (the order array lies between the bonus partial sums and the scratch slots)

@@ -182,3 +182,10 @@ def test_gradient_units_cut_between_ctas(B, T, H, c2, x_hi, with_dstate):
     if not c2:
         assert float((full[4].double() - du).norm() / du.norm()) < 1e-5
     gf.last_device_status()
+
+
+@pytest.mark.parametrize("T,c2", [(1025, True), (1025, False), (4100, False)])
+def test_gradient_where_an_eighth_of_the_last_round_is_idle(T, c2):
+    # 240 units on 148 SMs: long units are cut there (Finch-C2 from 16 chunks on, classic from 64), short ones are not, in a workspace
+    # laid out for either; a sequence alone has more units than half the SMs, one CTA each
+    test_gradient_units_cut_between_ctas(3, T, 80, c2, -1.0, True)

@@ -106,3 +106,12 @@ def test_nothing_is_thrown_for_want_of_random_numbers(host_library):
     assert s == 0 and len(log) == 1 and " cooperative " in log[0]
     # and where such a launch does not fit (cudaErrorCooperativeLaunchTooLarge) the call runs whole units
     assert s1 == 0 and len(log1) == 2 and "refused" in log1[0] and "cooperative" not in log1[1]
+
+
+@pytest.mark.parametrize("status", [9, 701, 912])
+def test_fp32_prefill_without_clusters(host_library, status):
+    # few units: blocks of tokens over the CTAs of a cluster; where none can be placed, the same grid of columns one CTA each
+    call = ["gf_wkv6_prefill_f32", ["p"] * 8 + [1, 256, 4, 64, None]]
+    (s, log), (s1, log1) = calls(host_library, call + [[status, 0]], call + [[0, 0]])
+    assert s1 == 0 and len(log1) == 1 and log1[0].startswith("grid 128 cluster 4 ")
+    assert s == 0 and len(log) == 2 and "refused" in log[0] and log[1].startswith("grid 32 cluster 1 ")
