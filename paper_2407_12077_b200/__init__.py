@@ -9,6 +9,8 @@ from __future__ import annotations
 
 import ctypes
 import functools
+import importlib.machinery
+import importlib.util
 import os
 
 import torch
@@ -26,6 +28,10 @@ KERNEL_AUTO, KERNEL_EXACT, KERNEL_CHUNKED = 0, 1, 2
 GF_OK = 0
 
 _lib = None
+_native = None               # the binding's C++ part (csrc/binding.cpp), once the library is loaded and if it could be built
+_NATIVE_FNS = ("gf_wkv6_prefill", "gf_wkv6_prefill_f32", "gf_wkv6_prefill_c2", "gf_wkv6_prefill_varlen", "gf_wkv6_prefill_varlen_f32",
+               "gf_wkv6_prefill_varlen_c2", "gf_wkv6_step", "gf_wkv6_step_f32", "gf_wkv6_step_c2", "gf_c2_layernorm", "gf_c2_layernorm_f32",
+               "gf_gold_key_compress", "gf_wkv6_workspace_bytes")
 _vp, _i, _sz = ctypes.c_void_p, ctypes.c_int, ctypes.c_size_t
 
 # name -> (restype, argtypes); the single place the ABI is mirrored in Python
@@ -95,7 +101,7 @@ def load_library(build_if_missing: bool = True):
     if _lib is not None:
         return _lib
     path = _build.LIB_PATH
-    if build_if_missing and _build.is_stale():
+    if build_if_missing and (_build.is_stale() or _build.binding_is_stale()):
         _build.build()
     if not os.path.exists(path):
         raise RuntimeError(f"{path} is missing: build it with `python -m paper_2407_12077_b200._build`; "
@@ -104,8 +110,25 @@ def load_library(build_if_missing: bool = True):
     for name, (res, args) in _SIGNATURES.items():
         fn = getattr(lib, name)            # AttributeError here = header / library mismatch
         fn.restype, fn.argtypes = res, args
+    _load_native(lib)
     _lib = lib
     return lib
+
+
+def _load_native(lib) -> None:
+    """The C++ part of the binding: the short way of the calls below that a program makes many times."""
+    global _native
+    path = _build.BINDING_PATH
+    if not os.path.exists(path):
+        return
+    loader = importlib.machinery.ExtensionFileLoader(__name__ + "._binding", path)
+    module = importlib.util.module_from_spec(importlib.util.spec_from_loader(loader.name, loader))
+    try:
+        loader.exec_module(module)
+    except ImportError:                          # (a torch it was not built for: the Python code does all it does)
+        return
+    module.bind(*(ctypes.cast(getattr(lib, name), ctypes.c_void_p).value for name in _NATIVE_FNS))
+    _native = module
 
 
 def status_string(status: int) -> str:
@@ -207,9 +230,14 @@ def set_workspace(buf: torch.Tensor | None) -> None:
     global _workspace
     lib = load_library()
     if buf is None:
+        if _native is not None:
+            _native.set_workspace(0, 0)
         _check(lib.gf_wkv6_set_workspace(None, 0), "gf_wkv6_set_workspace")
     else:
-        _check(lib.gf_wkv6_set_workspace(_dev(buf, "workspace"), buf.numel() * buf.element_size()), "gf_wkv6_set_workspace")
+        nbytes = buf.numel() * buf.element_size()
+        _check(lib.gf_wkv6_set_workspace(_dev(buf, "workspace"), nbytes), "gf_wkv6_set_workspace")
+        if _native is not None:                  # (as _ensure_workspace sees it)
+            _native.set_workspace(buf.get_device(), buf.numel())
     _workspace = buf
 
 
@@ -247,7 +275,13 @@ def prefill(r, k, v, x, u, state_in=None, state_out=None, y=None, stream=None, w
     u: [H,N] fp32; state_in: [B,H,N,N] fp32 or None (zero).  Returns (y, state_out);
     both are allocated here unless passed in (state_out may be state_in).  split=False unregisters
     the scratch workspace first, so that a call with few (b,h) units runs as a single launch."""
-    lib = load_library()
+    lib = _lib or load_library()
+    if _native is not None and stream is None and split and want_state and y is None and state_out is None:
+        out = _native.prefill(r, k, v, x, u, state_in, False)
+        if out is not None:
+            if type(out) is int:                 # (the status of a call that failed)
+                _check(out, "gf_wkv6_prefill" + _suffix(r.dtype))
+            return out
     shape = r.shape
     B, T, H, N = shape
     dt = r.dtype
@@ -418,7 +452,13 @@ def backward_varlen_workspace_bytes(S, total_T, H, N):
 def prefill_c2(r, k, v, x, u2=None, state_in=None, state_out=None, y=None, stream=None, want_state=True, split=True):
     """gf_wkv6_prefill_c2: the Finch-C2 form.  r,k,v,x (and u2, the per-token second-value vector, or
     None): [B,T,H,N] bf16 CUDA tensors; k is the key before the (1 - w) factor.  Returns (y, state_out)."""
-    lib = load_library()
+    lib = _lib or load_library()
+    if _native is not None and stream is None and split and want_state and y is None and state_out is None:
+        out = _native.prefill(r, k, v, x, u2, state_in, True)
+        if out is not None:
+            if type(out) is int:                 # (the status of a call that failed)
+                _check(out, "gf_wkv6_prefill_c2")
+            return out
     shape = r.shape
     B, T, H, N = shape
     bf = torch.bfloat16
@@ -447,7 +487,13 @@ def prefill_c2(r, k, v, x, u2=None, state_in=None, state_out=None, y=None, strea
 def prefill_varlen_c2(r, k, v, x, u2, cu_seqlens, max_seqlen, state_in=None, state_out=None, y=None,
                       stream=None, want_state=True, split=True):
     """gf_wkv6_prefill_varlen_c2: packed Finch-C2 prefill.  r,k,v,x,u2 (u2 may be None): [total_T,H,N] bf16."""
-    lib = load_library()
+    lib = _lib or load_library()
+    if _native is not None and stream is None and split and want_state and y is None and state_out is None:
+        out = _native.prefill_varlen(r, k, v, x, u2, cu_seqlens, max_seqlen, state_in, True)
+        if out is not None:
+            if type(out) is int:                 # (the status of a call that failed)
+                _check(out, "gf_wkv6_prefill_varlen_c2")
+            return out
     shape = r.shape
     total_T, H, N = shape
     S = cu_seqlens.numel() - 1
@@ -479,7 +525,7 @@ def prefill_varlen_c2(r, k, v, x, u2, cu_seqlens, max_seqlen, state_in=None, sta
 def step_c2(r, k, v, x, u2, state_in, state_out=None, y=None, stream=None):
     """gf_wkv6_step_c2: one Finch-C2 decode token per sequence.  r,k,v,x,u2 (u2 may be None): [B,H,N] bf16;
     state_out defaults to state_in (in-place update)."""
-    lib = load_library()
+    lib = _lib or load_library()
     shape = r.shape
     B, H, N = shape
     bf = torch.bfloat16
@@ -487,6 +533,11 @@ def step_c2(r, k, v, x, u2, state_in, state_out=None, y=None, stream=None):
         y = torch.empty_like(r)
     if state_out is None:
         state_out = state_in if state_in is not None else _new_states(B, H, N, r.device)
+    if _native is not None and stream is None:
+        status = _native.step(r, k, v, x, u2, state_in, state_out, y, True)
+        if status is not None:
+            _check(status, "gf_wkv6_step_c2")
+            return y, state_out
     args = [_dev(r, "r", bf), _dev(k, "k", bf, shape), _dev(v, "v", bf, shape), _dev(x, "x", bf, shape),
             _dev(u2, "u2", bf, shape), _dev(state_in, "state_in", torch.float32, (B, H, N, N)),
             _dev(state_out, "state_out", torch.float32, (B, H, N, N)), _dev(y, "y", bf, shape)]
@@ -531,7 +582,13 @@ def layernorm_heads(y, gamma=None, beta=None, eps=1e-5, out=None, stream=None):
     """gf_c2_layernorm(_f32): LayerNorm over all H*N channels of every token.  y: [..., H, N] CUDA tensor
     (bf16 or fp32, contiguous); gamma, beta: fp32 [H*N] (or [H, N]) or None.  out defaults to a new tensor
     (pass out=y for in place).  Returns out."""
-    lib = load_library()
+    lib = _lib or load_library()
+    if _native is not None and stream is None and out is None:
+        res = _native.layernorm(y, gamma, beta, eps)
+        if res is not None:
+            if type(res) is int:
+                _check(res, "gf_c2_layernorm" + _suffix(y.dtype))
+            return res
     H, N = y.shape[-2:]
     rows = y.numel() // (H * N) if H * N else 0
     sfx = _suffix(y.dtype)
@@ -551,7 +608,13 @@ def layernorm_heads(y, gamma=None, beta=None, eps=1e-5, out=None, stream=None):
 def key_compress(x, w_kd, out=None, stream=None):
     """gf_gold_key_compress: c = x @ w_kd.  x: [..., D] bf16 CUDA tensor (contiguous), w_kd: [D, Dc] bf16.
     Returns c [..., Dc] bf16 (allocated here unless passed as out)."""
-    lib = load_library()
+    lib = _lib or load_library()
+    if _native is not None and stream is None and out is None:
+        res = _native.key_compress(x, w_kd)
+        if res is not None:
+            if type(res) is int:
+                _check(res, "gf_gold_key_compress")
+            return res
     D, Dc = w_kd.shape
     c_shape = x.shape
     assert c_shape[-1] == D
@@ -610,7 +673,13 @@ def prefill_varlen(r, k, v, x, u, cu_seqlens, max_seqlen, state_in=None, state_o
                    stream=None, want_state=True, split=True):
     """gf_wkv6_prefill_varlen(_f32).  r,k,v,x: [total_T,H,N]; cu_seqlens: int32 CUDA [S+1];
     states [S,H,N,N].  Returns (y, state_out).  split as for prefill (cut by max_seqlen)."""
-    lib = load_library()
+    lib = _lib or load_library()
+    if _native is not None and stream is None and split and want_state and y is None and state_out is None:
+        out = _native.prefill_varlen(r, k, v, x, u, cu_seqlens, max_seqlen, state_in, False)
+        if out is not None:
+            if type(out) is int:                 # (the status of a call that failed)
+                _check(out, "gf_wkv6_prefill_varlen" + _suffix(r.dtype))
+            return out
     shape = r.shape
     total_T, H, N = shape
     S = cu_seqlens.numel() - 1
@@ -644,7 +713,7 @@ def prefill_varlen(r, k, v, x, u, cu_seqlens, max_seqlen, state_in=None, state_o
 def step(r, k, v, x, u, state_in, state_out=None, y=None, stream=None):
     """gf_wkv6_step(_f32): one decode token per sequence.  r,k,v,x: [B,H,N]; state [B,H,N,N].
     state_out defaults to state_in (in-place update).  Returns (y, state_out)."""
-    lib = load_library()
+    lib = _lib or load_library()
     shape = r.shape
     B, H, N = shape
     dt = r.dtype
@@ -653,6 +722,11 @@ def step(r, k, v, x, u, state_in, state_out=None, y=None, stream=None):
         y = torch.empty_like(r)
     if state_out is None:
         state_out = state_in if state_in is not None else _new_states(B, H, N, r.device)
+    if _native is not None and stream is None:
+        status = _native.step(r, k, v, x, u, state_in, state_out, y, False)
+        if status is not None:
+            _check(status, "gf_wkv6_step" + sfx)
+            return y, state_out
     args = [_dev(r, "r"), _dev(k, "k", dt, shape), _dev(v, "v", dt, shape),
             _dev(x, "x", dt, shape), _dev(u, "u", torch.float32, (H, N)),
             _dev(state_in, "state_in", torch.float32, (B, H, N, N)),

@@ -1,10 +1,13 @@
-"""Builds libgfwkv6.so (the C-ABI CUDA library) in-tree with nvcc for sm_100a."""
+"""Builds libgfwkv6.so (the C-ABI CUDA library) in-tree with nvcc for sm_100a, and the binding's C++ part with g++."""
 from __future__ import annotations
 
 import glob
 import os
 import shutil
 import subprocess
+import sysconfig
+
+import torch
 
 _PKG = os.path.dirname(os.path.abspath(__file__))
 _ROOT = os.path.dirname(_PKG)
@@ -16,6 +19,10 @@ NVCC_FLAGS = [
     "-shared", "-Xcompiler", "-fPIC", "-Xcompiler", "-fvisibility=hidden",
     "--expt-relaxed-constexpr",
 ]
+
+# Python and torch headers are not a stable interface: the file carries their versions
+BINDING_SRC = os.path.join(CSRC, "binding.cpp")
+BINDING_PATH = os.path.join(_PKG, f"_binding-{sysconfig.get_config_var('SOABI')}-torch{torch.__version__}.so")
 
 
 def _nvcc() -> str:
@@ -33,12 +40,37 @@ def is_stale() -> bool:
     if not os.path.exists(LIB_PATH):
         return True
     t = os.path.getmtime(LIB_PATH)
-    deps = glob.glob(os.path.join(CSRC, "*")) + glob.glob(os.path.join(_ROOT, "include", "*.h"))
+    deps = glob.glob(os.path.join(CSRC, "*.cu*")) + glob.glob(os.path.join(_ROOT, "include", "*.h"))
     return any(os.path.getmtime(d) > t for d in deps)
 
 
+def binding_is_stale() -> bool:
+    return not os.path.exists(BINDING_PATH) or os.path.getmtime(BINDING_SRC) > os.path.getmtime(BINDING_PATH)
+
+
+def build_binding(force: bool = False) -> str | None:
+    """Compile the binding's C++ part (None where there is no compiler or header for it: the Python code does without)."""
+    if not force and not binding_is_stale():
+        return BINDING_PATH
+    gxx, py = shutil.which("g++"), sysconfig.get_paths()["include"]
+    inc = os.path.join(os.path.dirname(torch.__file__), "include")
+    cuda = os.path.dirname(os.path.dirname(shutil.which("nvcc") or "/usr/local/cuda/bin/nvcc"))
+    if gxx is None or not os.path.exists(os.path.join(py, "Python.h")) or not os.path.exists(inc):
+        return None
+    tmp = f"{BINDING_PATH}.{os.getpid()}"
+    cmd = [gxx, "-O2", "-std=c++17", "-shared", "-fPIC", "-fvisibility=hidden", f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}",
+           "-I", py, "-I", inc, "-I", os.path.join(inc, "torch", "csrc", "api", "include"), "-I", os.path.join(cuda, "include"), "-o", tmp, BINDING_SRC,
+           "-L", os.path.join(os.path.dirname(torch.__file__), "lib"), "-ltorch_python", "-ltorch_cpu", "-lc10", "-lc10_cuda"]
+    res = subprocess.run(cmd, capture_output=True, text=True)
+    if res.returncode != 0:
+        raise RuntimeError("g++ failed:\n" + res.stdout + res.stderr)
+    os.replace(tmp, BINDING_PATH)
+    return BINDING_PATH
+
+
 def build(force: bool = False, verbose: bool = False) -> str:
-    """Compile every CUDA source into libgfwkv6.so.  Cross-compiles without a GPU."""
+    """Compile every CUDA source into libgfwkv6.so, and the binding's C++ part.  Cross-compiles without a GPU."""
+    build_binding(force)
     if not force and not is_stale():
         return LIB_PATH
     cmd = [_nvcc(), *NVCC_FLAGS, "-I", os.path.join(_ROOT, "include"), "-I", CSRC,
