@@ -268,6 +268,7 @@ wkv6_exact_kernel(const IO* __restrict__ r, const IO* __restrict__ k, const IO* 
             }
             return ck::fma2(D, X, dS);
         };
+        __syncwarp();
         if (G > 1) cluster_wait();               // (the mbarriers of the cluster's CTAs are there)
         __syncthreads();
         uint32_t folds = 0;                      // rounds with a small D
@@ -465,6 +466,7 @@ wkv6_exact_kernel(const IO* __restrict__ r, const IO* __restrict__ k, const IO* 
         };
         fetch(0);
         fetch(1);
+        __syncwarp();
         if (G > 1) cluster_wait();
         if (n_blocks > 0) {
             if (ASYNC) asm volatile("cp.async.wait_group 1;" ::: "memory");
