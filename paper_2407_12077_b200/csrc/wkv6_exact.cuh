@@ -52,7 +52,7 @@ __device__ __forceinline__ void cp_async16(uint32_t dst, const void* src)
 
 // Shared memory of a CTA, in floats: two block buffers {r, k, w [TB][64], v [TB][NC], coefficient [TB]}; per run dS (in the lanes'
 // layout of a compute warp; later the run's start state) and D; the same of the whole block, by parity of the round; the next round's
-// start state, by parity; whether the block's D is small, by parity; abort word; two mbarriers.
+// start state, by parity; whether the block's D is small, by parity; abort word and wait limit; two mbarriers.
 template <int CW, int NT, int TB> struct ExLayout {
     static constexpr int NC = 8 * CW;
     static constexpr int R = 0, K = TB * EX_N, W = 2 * TB * EX_N, V = 3 * TB * EX_N, COEF = V + TB * NC, BUF = COEF + TB;
@@ -100,7 +100,7 @@ __device__ __noinline__ void cluster_mbar_wait(uint32_t bar, uint32_t parity, ui
         if (ck::lds32(abort_flag)) return;
         const unsigned long long now = ck::globaltimer();
         if (t0 == 0) t0 = now;
-        if (now - t0 > 1000ull * ck::WAIT_LIMIT_US) break;
+        if (now - t0 > 1000ull * ck::lds32(abort_flag + 4)) break;
         __nanosleep(64);
     }
     ck::sts32(abort_flag, 1u);
@@ -110,13 +110,13 @@ __device__ __noinline__ void cluster_mbar_wait(uint32_t bar, uint32_t parity, ui
 // Dense: cu_seqlens == nullptr, unit = b * H + h, rows b*T .. b*T+T-1.
 // Packed: unit = s * H + h, rows cu_seqlens[s] .. cu_seqlens[s+1]-1.
 // Grid: units * (8 / CW) * G, clusters of G; CTA: the compute warps, then the staging warps.  tb: tokens per block, a multiple
-// of 4 NT up to TB.
+// of 4 NT up to TB; limit_us: of a wait for the cluster (0: the default).
 template <typename IO, int CW, int NT, int TB>
 __global__ void __launch_bounds__(32 * (EX_NCW + EX_NSW), 1)
 wkv6_exact_kernel(const IO* __restrict__ r, const IO* __restrict__ k, const IO* __restrict__ v,
                   const IO* __restrict__ x, const float* __restrict__ u,
                   const float* state_in, float* state_out, IO* __restrict__ y,
-                  const int32_t* __restrict__ cu_seqlens, int T, int H, int tb, int G)
+                  const int32_t* __restrict__ cu_seqlens, int T, int H, int tb, int G, uint32_t limit_us)
 {
     using Lay = ExLayout<CW, NT, TB>;
     constexpr int NC = Lay::NC, NSLAB = EX_N / NC;
@@ -131,6 +131,7 @@ wkv6_exact_kernel(const IO* __restrict__ r, const IO* __restrict__ k, const IO* 
         ck::mbar_init(bar_pub, G);               // every CTA's block has been published
         ck::mbar_init(bar_fold, G);              // (rounds with a small D) ... and folded by every CTA
         ck::sts32(abort_flag, 0u);
+        ck::sts32(abort_flag + 4, limit_us ? limit_us : ck::WAIT_LIMIT_US);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (G > 1) { __syncwarp(); cluster_arrive(); }
@@ -499,7 +500,7 @@ inline cudaError_t launch_exact_as(long long units, int G, int tb, cudaStream_t 
         attr_set.set(dev);
     }
     return launch_pdl_cluster(wkv6_exact_kernel<IO, CW, NT, TB>, (unsigned)(units * (8 / CW) * G), 32 * (EX_NCW + EX_NSW), ExLayout<CW, NT, TB>::BYTES, G, st,
-                              r, k, v, x, u, state_in, state_out, y, cu, T, H, tb, G);
+                              r, k, v, x, u, state_in, state_out, y, cu, T, H, tb, G, wait_limit_us().load(std::memory_order_relaxed));
 }
 
 // Launches the kernel over `units` (sequence, head) units.  What bounds it is the fp32 pipe of the SMs that take part (a two-lane
