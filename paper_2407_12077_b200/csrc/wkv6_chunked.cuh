@@ -891,6 +891,7 @@ wkv6_chunked_kernel(const __grid_constant__ CUtensorMap tm_r, const __grid_const
     static_assert(!(CKPT && SUMMARY), "the summary pass keeps its checkpoints by Params::ckpt");
     static_assert(!(TRAIL && (PERSIST || SUMMARY)), "the main launch of a split call");
     constexpr bool BAL = PERSIST == 2;
+    constexpr bool PAIR = C2 && !SUMMARY && (BAL || (CKPT && !PERSIST));          // two second-value slabs per output warp (see there)
 
     // One chunk of this CTA's work.  Single-unit launches derive it from the chunk index; persistent launches
     // read the descriptor the producer warp left for the chunk, which is visible to any warp that has waited
@@ -939,7 +940,7 @@ wkv6_chunked_kernel(const __grid_constant__ CUtensorMap tm_r, const __grid_const
         mbar_init(bar(BAR_SPRE), N_GW);
         mbar_init(bar(BAR_FB_READY), N_GW);
         mbar_init(bar(BAR_FB_DONE), N_GW);
-        for (int i = 0; i < (C2 && BAL ? 2 : 1) * N_GW; ++i) mbar_init(bar(BAR_U2 + i), 1);
+        for (int i = 0; i < (PAIR ? 2 : 1) * N_GW; ++i) mbar_init(bar(BAR_U2 + i), 1);
         if (C2 && BAL)
             for (int i = 0; i < NSIDE; ++i) sts32(sbase + OFF_DESC + 16 * i + 4, DESC_TAG);        // (of the turn before the first)
         sts32(abort_flag, 0u);
@@ -1542,11 +1543,13 @@ wkv6_chunked_kernel(const __grid_constant__ CUtensorMap tm_r, const __grid_const
             u2_parity = u2_loads & 1;
             ++u2_loads;
         };
-        if (!PERSIST && has_u2 && nchunks > 0) load_u2((int)row0, col0, nchunks - 1);
-        // Balanced launches keep every SM streaming, so a chunk's time does not hide that load: two slabs per warp (by chunk
-        // parity), second-value rows in and y rows out in their place, the load a chunk ahead and across units.  (5 x 2011
-        // tokens x 32 heads: 69.6 us with one slab, 62.3 with the pair.  With fewer SMs streaming it loses 3-5 %.)
-        constexpr bool PAIR = C2 && BAL;
+        if (!PERSIST && !PAIR && has_u2 && nchunks > 0) load_u2((int)row0, col0, nchunks - 1);
+        // Where a chunk's time does not hide that load (PAIR), two slabs per warp (by chunk parity), second-value rows in and y
+        // rows out in their place, the load a chunk ahead and, in a stream, across units.  Balanced launches keep every SM
+        // streaming (5 x 2011 tokens x 32 heads: 69.6 us with one slab, 62.3 with the pair); a training forward writes 16 KB
+        // of state per chunk beside its y (4 x 16384 x 32 315.7 -> 295.6, 4 x 4096 93.3 -> 88.0, 8 x 2048 97.4 -> 93.6, 65536 x 32
+        // in segments 381.9 -> 365.3, 8 x 1100 x 12 31.0 -> 30.9).  The plain prefill keeps one: with two, 8 x 4096 x 12
+        // 80.0 -> 82.4, 8 x 1100 x 12 25.5 -> 27.0, 4 x 4096 x 32 85.2 -> 86.0, 4 x 16384 x 32 326.5 -> 324.8.
         int u2_issued = 0, u2_used = 0;          // one load per chunk: the i-th completes phase i / 2 of the barrier of slab i % 2
         auto u2_bar = [&](int i) { return bar(BAR_U2 + N_GW * (i & 1) + sp); };
         auto slab_of = [&](int i) { return (i & 1) ? u2slab : slab; };
@@ -1569,7 +1572,8 @@ wkv6_chunked_kernel(const __grid_constant__ CUtensorMap tm_r, const __grid_const
             return true;
         };
         bool go = true;
-        if (PAIR && has_u2) go = load_pair_unit(0);
+        if (PAIR && PERSIST && has_u2) go = load_pair_unit(0);
+        if (PAIR && !PERSIST && has_u2 && nchunks > 0) load_pair((int)row0, col0, nchunks - 1);
         for (int c = 0; (!PAIR || go) && (PERSIST || c < (SUMMARY ? 0 : nchunks)); ++c) {
             const int tb = c & 1;
             if (!mbar_wait(bar(BAR_B_DONE + tb), (c >> 1) & 1, abort_flag)) break;
@@ -1583,7 +1587,7 @@ wkv6_chunked_kernel(const __grid_constant__ CUtensorMap tm_r, const __grid_const
             __syncwarp();
             if (PAIR && has_u2) {                 // ... which (chunk c - 1's) takes the rows of chunk c + 1
                 if (!ck.last) load_pair(ck.row + L, ccol, ck.rem - 1);
-                else if (!load_pair_unit(c + 1)) break;
+                else if (PERSIST && !load_pair_unit(c + 1)) break;
             }
             const uint32_t out = PAIR ? slab_of(c) : slab;
             if (!safe) {

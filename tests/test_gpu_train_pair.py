@@ -145,3 +145,24 @@ def test_pair_at_the_benchmarked_size(c2):
     gf.last_device_status()
     assert torch.equal(y, y0) and torch.equal(s, s0)
     assert all(torch.equal(p, q) for p, q in zip(ga, gb))
+
+
+@pytest.mark.parametrize("B,T,H", [(1, 1, 1), (2, 16, 3), (3, 64, 2), (2, 65, 3), (2, 129, 5), (3, 700, 4), (1, 2048, 2)])   # (the last: in segments)
+@pytest.mark.parametrize("fast", [False, True])
+def test_training_forward_with_a_second_value_at_chunk_edges(B, T, H, fast):
+    """The training forward holds the second value's rows in two slabs per warp, the plain prefill in one: one chunk, two, the
+    odd and the even slab last, ragged last rows, and (fast) chunks that take the token-by-token path and use no slab."""
+    inp = synth.make_dense(B, T, H, 64, "bf16", seed=600 + T, state_std=0.2).to(DEV)
+    if fast:
+        for c in range(0, (T + 63) // 64, 3):                      # every third chunk: both slabs are passed over
+            inp.x[:, min(64 * c + 5, T - 1), :, 7] = 4.0
+    u2 = torch.randn(inp.r.shape, generator=torch.Generator(device=DEV).manual_seed(T), device=DEV).bfloat16()
+    ws = torch.empty(gf.backward_workspace_bytes(B, T, H, 64), dtype=torch.uint8, device=DEV)
+    y, s = gf.prefill_train(inp.r, inp.k, inp.v, inp.x, inp.u, ws, inp.state_in, c2=True, u2=u2)
+    y0, s0 = gf.prefill_c2(inp.r, inp.k, inp.v, inp.x, u2, inp.state_in)
+    gf.last_device_status()
+    assert torch.equal(y, y0) and torch.equal(s, s0)
+    c = inp.to("cpu")
+    y_ref, s_ref = orc.prefill_c2(c.r, c.k, c.v, c.x, u2.cpu(), c.state_in)
+    # two bf16 operands and y, rounded to 2^-9 / sqrt 3 in the Euclidean norm each: 3.4e-3 if none cancelled; the parity tests' 5e-3
+    assert orc.rel_l2(y.float().cpu().numpy(), y_ref) <= 5e-3 and orc.rel_l2(s.cpu().numpy(), s_ref) <= 5e-3
