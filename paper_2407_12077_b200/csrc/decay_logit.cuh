@@ -15,7 +15,7 @@
 //   pass 1: z slice -> operand rows -> acc1 += z A_d[slice]                then h1 = tanh(acc1) -> operand
 //   pass 2: l = h1 B_d[:, slice] -> m slice -> operand rows -> acc3 += m A_w[slice]      then h2 = tanh(acc3) -> operand
 //   pass 3: d slice = lambda_w + h2 B_w[:, slice] -> bf16 -> TMA store
-// Four sets of four worker warps take the slices in turn, each with a tensor-memory operand and accumulator of its own:
+// Four sets of four worker warps take the slices in turn, each with a tensor-memory operand of its own:
 //   warp 0       TMA producer of the x ring (8 stages, two per set): per slice the x rows of the tile (plus the one row above
 //                it) and the 64 per-channel constants of the pass; a stage is free as soon as its rows are in registers (pass 3: its
 //                room takes the output rows, and it is free when the store has read them)
@@ -24,15 +24,22 @@
 //                bf16 -> fp32; tensor-memory allocation)
 //   warps 3, 21  an elected lane issues h1 B_d and h2 B_w of the even, the odd slices
 //   warps 4-19   the four sets; a lane owns one token row (the accumulator row of its tensor-memory sub-partition): reads its
-//                row and the row above from the swizzled x tiles, forms z / m / d for the 64 channels of the slice, 16 at a
-//                time, and writes the bf16 operand row or the output slab
+//                row and the row above from the swizzled x tiles, forms z / m / d for the 64 channels of the slice, 32 at a
+//                time (mix first, so that an accumulator is soon free), and writes the bf16 operand row or the output slab
 // z, m, h1 and h2 are A operands in tensor memory (a lane's row, two channels per column): through shared memory they were
 // a third of its traffic (16 KB written and 16 KB read per slice).
 // What bounds a slice is the chain load -> registers -> operand -> product, through warps that each spend 300-400 cycles per slice on
 // their part: 870 cycles a slice and pass with every set in flight, and 780 with one tile on an idle SM.  us per call, two sets of four warps on
-// rings of two weight stages each -> four sets -> a weight ring per issuer -> a producer and an issuer more (the present form):
+// rings of two weight stages each -> four sets -> a weight ring per issuer -> a producer and an issuer more:
 //   65536 tokens x 2048 channels 191 -> 196 -> 179 -> 175;  1000 x 2048 46.4 -> 43.5 -> 41.4 -> 40.0;  32 x 271 x 2048 50.5 -> 46.3 -> 45.7 -> 43.6;
 //   8680 x 768 20.1 -> 20.5 -> 19.6 -> 19.3.
+// That form had one chain of sums for all slices and an accumulator per set.  With the sums of the even and the odd slices apart, as two
+// sets had them, three accumulators are what tensor memory has room for.  us per call in a graph, two sets -> one chain -> present form:
+//   65536 x 2048 189.7 -> 173.9 -> 173.0;  19500 x 2048 90.1 -> 82.0 -> 83.2;  9400 x 2048 41.5 -> 36.3 -> 37.9;
+//   65536 x 1280 120.6 -> 116.0 -> 115.7;  18000 x 1280 30.2 -> 30.7 -> 30.2;  40 x 1280 26.9 -> 23.6 -> 25.2;
+//   65536 x 768 78.7 -> 78.6 -> 79.2;  18000 x 768 20.0 -> 20.7 -> 20.3;  40 x 768 17.8 -> 16.2 -> 17.4;  18000 x 256 10.7 -> 12.1 -> 12.3.
+// (l read in quarters of a slice, so that an accumulator is held for most of it: 40 x 768 17.8, 65536 x 2048 177; read as a whole first
+// 17.5 and 173.7, with two accumulators 17.6 and 175; slices 2 and 3 of a pass in the idle halves of the sum 17.8 and 178.)
 // (With one ring for both kinds of weights a slice's B_d, which its l needs early, waited for the slot of an A_w whose product comes a worker's
 // time later.)  Not better: the sum of pass 1 in an accumulator per set (175.6), rings of 5 + 6 stages with one producer (181), asking for the
 // operand rows after more of the slice (174 to 205: registers), an extra commit saved per slice at rings of 4 (192).  The three passes
@@ -75,17 +82,20 @@ enum {
     DL_OP_FREE = DL_OP_READY + DL_NSET,    // per set: the product that read them is done
     DL_ACC_FULL = DL_OP_FREE + DL_NSET,    // per set: l (pass 2) or d (pass 3) of a slice is in tensor memory
     DL_ACC_FREE = DL_ACC_FULL + DL_NSET,   // ... and read back by the warps of the set
-    DL_SUM_FULL = DL_ACC_FREE + DL_NSET,   // the sum of a pass complete
+    DL_TURN = DL_ACC_FREE + DL_NSET,       // per issuer of h B: the accumulator of its slice was free
+    DL_SUM_FULL = DL_TURN + 2,             // the sum of a pass complete
     DL_H_READY = DL_SUM_FULL + 1,      // h1 / h2 operand written by all worker warps
     DL_H_FREE = DL_H_READY + 1,        // the last product of a tile that reads h2 is done
     DL_BAR_COUNT = DL_H_FREE + 1
 };
 static_assert(16 + 8 * DL_BAR_COUNT <= 512, "barrier block");
 static_assert(DL_SMEM <= 232448, "shared memory budget of one sm_100 CTA");
-// the sum of a pass (acc1, then acc3: every warp has read acc1 before a product of pass 2's is issued, and acc3 before one of
-// the next tile's); per set l (pass 2) / d (pass 3); the A operands (lane = row, a 32-bit column = two neighbouring channels
-// in bf16): z / m of a set, h1 / h2
-constexpr int DL_TM_SUM = 0, DL_TM_ACC = 64, DL_TM_OP = DL_TM_ACC + 64 * DL_NSET, DL_TM_H = DL_TM_OP + 32 * DL_NSET;
+// the sum of a pass in two halves, its even and its odd slices, which keeps the chains of additions short (acc1, then acc3: every
+// warp has read acc1 before a product of pass 2's is issued, and acc3 before one of the next tile's); a ring of accumulators for l
+// (pass 2) / d (pass 3) in the order of the slices; the A operands (lane = row, a 32-bit column = two neighbouring channels in
+// bf16): z / m of a set, h1 / h2
+constexpr int DL_NACC = 3;
+constexpr int DL_TM_SUM = 0, DL_TM_ACC = 2 * 64, DL_TM_OP = DL_TM_ACC + 64 * DL_NACC, DL_TM_H = DL_TM_OP + 32 * DL_NSET;
 static_assert(DL_TM_H + 32 <= 512, "tensor memory columns");
 // fp32 accumulator, bf16 A (K-major) and B (MN-major), M = 128, N = 64
 constexpr uint32_t DL_IDESC = (1u << 4) | (1u << 7) | (1u << 10) | (1u << 16) | ((64u >> 3) << 17) | ((128u >> 4) << 24);
@@ -193,8 +203,10 @@ decay_logit_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_consta
             mbar_init(bar(DL_OP_READY + i), DL_NWS);
             mbar_init(bar(DL_OP_FREE + i), 1);
             mbar_init(bar(DL_ACC_FULL + i), 1);
-            mbar_init(bar(DL_ACC_FREE + i), DL_NWS);
         }
+        for (int i = 0; i < DL_NSET; ++i) mbar_init(bar(DL_ACC_FREE + i), DL_NWS);
+        mbar_init(bar(DL_TURN), 1);
+        mbar_init(bar(DL_TURN + 1), 1);
         mbar_init(bar(DL_SUM_FULL), 1);
         mbar_init(bar(DL_H_READY), DL_NWS * DL_NSET);
         mbar_init(bar(DL_H_FREE), 2);
@@ -302,7 +314,7 @@ decay_logit_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_consta
                         const uint32_t ta = tmem + DL_TM_OP + 32 * set;
 #pragma unroll
                         for (int kk = 0; kk < 4; ++kk)
-                            tc_mma_ta(tmem + DL_TM_SUM, ta + 8 * kk, db + (uint64_t)(128 * kk), DL_IDESC, (s > 0 || kk > 0) ? 1u : 0u);
+                            tc_mma_ta(tmem + DL_TM_SUM + 64 * (s & 1), ta + 8 * kk, db + (uint64_t)(128 * kk), DL_IDESC, (s > 1 || kk > 0) ? 1u : 0u);
                         tc_commit(bar(DL_OP_FREE + set));
                         tc_commit(bar(DL_AEMPTY + ia));
                         if (s == S - 1) tc_commit(bar(DL_SUM_FULL));
@@ -316,29 +328,41 @@ decay_logit_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_consta
         // ============================== MMA issuers: l = h1 B_d (pass 2), d = h2 B_w (pass 3) of the even / odd slices ==============================
         const int odd = warp > DL_WB;
         int n0 = 0, ib = 0, pb = 0;                          // (B ring position and its phase)
-        uint32_t phases = (1u << DL_NSET) - 1;               // bit: parity of the set's accumulator's last release
+        uint32_t phases = 0;                                 // bit: parity of the set's next accumulator
+        int turn = 0;                                        // slices of the other issuer so far
+        int acc = 0;                                         // accumulator of slice n: a ring that both issuers' slices take in turn
         bool alive = true;
         for (long long r = r_first; r < r_end && alive; r += 128) {
             n0 += S;
+            const int n_tile = n0;
             for (int pass = 1; pass < 3 && alive; ++pass, n0 += S) {
                 if (!wait_warp(DL_H_READY, pass - 1)) { alive = false; break; }      // (two uses per tile: parities 0, 1)
                 const int kn = pass == 1 ? p.kd : p.kw;
-                for (int n = n0 + ((n0 ^ odd) & 1); n < n0 + S; n += 2) {
-                    const int set = n & (DL_NSET - 1), slot = odd * DL_NSB + ib;
-                    // (before its first use an accumulator is free: the phase before the barrier's first)
-                    if (!wait_warp(DL_BFULL + slot, pb) || !wait_warp(DL_ACC_FREE + set, phases >> set)) { alive = false; break; }
-                    phases ^= 1u << set;
-                    tc_fence_after();
-                    if (elect_one()) {
-                        const uint64_t db = smem_desc(bstage(slot));
+                for (int n = n0; n < n0 + S; ++n) {
+                    const int set = n & (DL_NSET - 1), before = (n - DL_NACC) & (DL_NSET - 1);
+                    if ((n & 1) == odd) {
+                        const int slot = odd * DL_NSB + ib;
+                        // Slice n - 3 had the accumulator (the tile before had read all of its when h1 was ready).  Its set's slice before
+                        // that is n - 7, which this issuer has waited for, and the one after it is n + 1, whose product waits for DL_TURN.
+                        if (!wait_warp(DL_BFULL + slot, pb) || (n - DL_NACC >= n_tile && !wait_warp(DL_ACC_FREE + before, (phases >> before) + 1))) { alive = false; break; }
+                        if (n > n_tile && !wait_warp(DL_TURN + 1 - odd, turn + 1)) { alive = false; break; }
+                        mbar_arrive_if(bar(DL_TURN + odd), lane == 0);
+                        tc_fence_after();
+                        if (elect_one()) {
+                            const uint64_t db = smem_desc(bstage(slot));
 #pragma unroll
-                        for (int kk = 0; kk < 4; ++kk)
-                            if (kk < kn) tc_mma_ta(tmem + DL_TM_ACC + 64 * set, tmem + DL_TM_H + 8 * kk, db + (uint64_t)(128 * kk), DL_IDESC, kk > 0 ? 1u : 0u);
-                        tc_commit(bar(DL_ACC_FULL + set));
-                        tc_commit(bar(DL_BEMPTY + slot));
+                            for (int kk = 0; kk < 4; ++kk)
+                                if (kk < kn) tc_mma_ta(tmem + DL_TM_ACC + 64 * acc, tmem + DL_TM_H + 8 * kk, db + (uint64_t)(128 * kk), DL_IDESC, kk > 0 ? 1u : 0u);
+                            tc_commit(bar(DL_ACC_FULL + set));
+                            tc_commit(bar(DL_BEMPTY + slot));
+                        }
+                        __syncwarp();
+                        if (++ib == DL_NSB) { ib = 0; pb ^= 1; }
+                    } else {
+                        ++turn;
                     }
-                    __syncwarp();
-                    if (++ib == DL_NSB) { ib = 0; pb ^= 1; }
+                    phases ^= 1u << set;
+                    if (++acc == DL_NACC) acc = 0;
                 }
             }
             if (alive && elect_one()) tc_commit(bar(DL_H_FREE));      // (all products of this warp so far)
@@ -371,6 +395,7 @@ decay_logit_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_consta
             const bool any_start = __any_sync(0xffffffffu, seq_start);
             const __nv_bfloat16* gp = (seq_start && p.x_prev && tok < p.rows) ? p.x_prev + (tok / p.T) * (long long)p.D : nullptr;
             int n0 = ti * 3 * S;
+            auto acc_of = [&](int n) { return tlane + DL_TM_ACC + 64 * ((unsigned)(n - (ti + 1) * S) % DL_NACC); };     // (slices of pass 1 have none)
             // ---- passes 1 and 2: out = x + (x_above - x) * mix, mix = the pass's constants (+ l from tensor memory in pass 2).
             // The interpolation runs on packed bf16 pairs (difference, then one fused multiply-add with a single rounding):
             // its inputs and its output are bf16 anyway, and the mix is smooth in them.
@@ -392,54 +417,65 @@ decay_logit_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_consta
                         if (!wait(DL_OP_FREE + set, op_phase)) { alive = false; break; }
                     } else
 #pragma unroll
-                    for (int g = 0; g < 4; ++g) {        // 16 channels at a time (registers)
-                        float4 v4[4];
+                    for (int hf = 0; hf < 2 && alive; ++hf) {        // 32 channels at a time (registers)
+                        uint32_t mix[16];                // their mix as bf16 pairs
 #pragma unroll
-                        for (int q = 0; q < 4; ++q) v4[q] = ldsf4(stage + DL_OFF_VEC + 64 * g + 16 * q);
-                        uint4 a[2], b[2];
+                        for (int g = 0; g < 2; ++g) {
+                            float l[16];
+                            if (pass == 1) {
+                                tmem_ld_row16(acc_of(n) + 32 * hf + 16 * g, l);
+                            } else {
 #pragma unroll
-                        for (int q = 0; q < 2; ++q) {
-                            const uint32_t o = (uint32_t)((2 * g + q) << 4);
-                            a[q] = lds128(stage + own_off + (o ^ own_xor));
-                            b[q] = lds128(stage + up_off + (o ^ up_xor));
-                        }
-                        float l[16];
-                        if (pass == 1) {
-                            tmem_ld_row16(tlane + DL_TM_ACC + 64 * set + 16 * g, l);
-                        } else {
+                                for (int e = 0; e < 16; ++e) l[e] = 0.f;
+                            }
 #pragma unroll
-                            for (int e = 0; e < 16; ++e) l[e] = 0.f;
-                        }
-                        if (g == 3) {                    // all in registers: accumulator and stage are free for later slices
-                            if (pass == 1) tc_fence_before();
-                            __syncwarp();
-                            if (pass == 1) mbar_arrive_if(bar(DL_ACC_FREE + set), lane == 0);
-                            mbar_arrive_if(bar(DL_XEMPTY + (n & (DL_NSX - 1))), lane == 0);
-                        }
-                        if (any_start && seq_start) {
-#pragma unroll
-                            for (int q = 0; q < 2; ++q)
-                                b[q] = gp ? *reinterpret_cast<const uint4*>(gp + 64 * (n - n0) + 16 * g + 8 * q) : make_uint4(0u, 0u, 0u, 0u);
-                        }
-                        uint32_t ow[8];
-#pragma unroll
-                        for (int q = 0; q < 2; ++q) {
-                            const uint32_t aw[4] = {a[q].x, a[q].y, a[q].z, a[q].w}, bw[4] = {b[q].x, b[q].y, b[q].z, b[q].w};
-#pragma unroll
-                            for (int e = 0; e < 4; ++e) {
-                                const float4 v = v4[2 * q + (e >> 1)];
-                                const uint32_t mix = pack_sum((e & 1) ? v.z : v.x, (e & 1) ? v.w : v.y, __float_as_uint(l[8 * q + 2 * e]), __float_as_uint(l[8 * q + 2 * e + 1]));
-                                uint32_t delta;
-                                asm("sub.rn.bf16x2 %0, %1, %2;" : "=r"(delta) : "r"(bw[e]), "r"(aw[e]));
-                                asm("fma.rn.bf16x2 %0, %1, %2, %3;" : "=r"(ow[4 * q + e]) : "r"(delta), "r"(mix), "r"(aw[e]));
+                            for (int q = 0; q < 4; ++q) {
+                                const float4 v = ldsf4(stage + DL_OFF_VEC + 128 * hf + 64 * g + 16 * q);
+                                mix[8 * g + 2 * q] = pack_sum(v.x, v.y, __float_as_uint(l[4 * q]), __float_as_uint(l[4 * q + 1]));
+                                mix[8 * g + 2 * q + 1] = pack_sum(v.z, v.w, __float_as_uint(l[4 * q + 2]), __float_as_uint(l[4 * q + 3]));
                             }
                         }
-                        if (g == 0) {                    // the operand rows: free of the product that read them last
-                            if (!wait(DL_OP_FREE + set, op_phase)) { alive = false; break; }
-                            tc_fence_after();
+                        if (pass == 1 && hf == 1) {      // l has been read: its accumulator is free for a later slice
+                            tc_fence_before();
                             __syncwarp();
+                            mbar_arrive_if(bar(DL_ACC_FREE + set), lane == 0);
                         }
-                        tmem_st_row8(tlane + DL_TM_OP + 32 * set + 8 * g, ow);
+#pragma unroll
+                        for (int g = 2 * hf; g < 2 * hf + 2; ++g) {
+                            uint4 a[2], b[2];
+#pragma unroll
+                            for (int q = 0; q < 2; ++q) {
+                                const uint32_t o = (uint32_t)((2 * g + q) << 4);
+                                a[q] = lds128(stage + own_off + (o ^ own_xor));
+                                b[q] = lds128(stage + up_off + (o ^ up_xor));
+                            }
+                            if (g == 3) {                // all in registers: the stage is free for a later slice
+                                __syncwarp();
+                                mbar_arrive_if(bar(DL_XEMPTY + (n & (DL_NSX - 1))), lane == 0);
+                            }
+                            if (any_start && seq_start) {
+#pragma unroll
+                                for (int q = 0; q < 2; ++q)
+                                    b[q] = gp ? *reinterpret_cast<const uint4*>(gp + 64 * (n - n0) + 16 * g + 8 * q) : make_uint4(0u, 0u, 0u, 0u);
+                            }
+                            uint32_t ow[8];
+#pragma unroll
+                            for (int q = 0; q < 2; ++q) {
+                                const uint32_t aw[4] = {a[q].x, a[q].y, a[q].z, a[q].w}, bw[4] = {b[q].x, b[q].y, b[q].z, b[q].w};
+#pragma unroll
+                                for (int e = 0; e < 4; ++e) {
+                                    uint32_t delta;
+                                    asm("sub.rn.bf16x2 %0, %1, %2;" : "=r"(delta) : "r"(bw[e]), "r"(aw[e]));
+                                    asm("fma.rn.bf16x2 %0, %1, %2, %3;" : "=r"(ow[4 * q + e]) : "r"(delta), "r"(mix[8 * (g & 1) + 4 * q + e]), "r"(aw[e]));
+                                }
+                            }
+                            if (g == 0) {                // the operand rows: free of the product that read them last
+                                if (!wait(DL_OP_FREE + set, op_phase)) { alive = false; break; }
+                                tc_fence_after();
+                                __syncwarp();
+                            }
+                            tmem_st_row8(tlane + DL_TM_OP + 32 * set + 8 * g, ow);
+                        }
                     }
                     if (!alive) break;
                     op_phase ^= 1;
@@ -455,8 +491,13 @@ decay_logit_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_consta
                 tc_fence_after();
                 __syncwarp();
                 if (live && set < (pass == 0 ? p.kd : p.kw)) {
-                    float a[16];
+                    float a[16], b[16];
                     tmem_ld_row16(tlane + DL_TM_SUM + 16 * set, a);
+                    if (S > 1) {
+                        tmem_ld_row16(tlane + DL_TM_SUM + 64 + 16 * set, b);
+#pragma unroll
+                        for (int e = 0; e < 16; ++e) a[e] += b[e];
+                    }
                     uint32_t ow[8];
 #pragma unroll
                     for (int e = 0; e < 8; ++e) ow[e] = pack_bf16(tanh_fast(a[2 * e]), tanh_fast(a[2 * e + 1]));
@@ -490,7 +531,7 @@ decay_logit_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_consta
 #pragma unroll
                     for (int q = 0; q < 4; ++q) v4[q] = ldsf4(vec + 64 * g + 16 * q);
                     float v[16];
-                    tmem_ld_row16(tlane + DL_TM_ACC + 64 * set + 16 * g, v);
+                    tmem_ld_row16(acc_of(n) + 16 * g, v);
                     if (g == 3) {
                         tc_fence_before();
                         __syncwarp();

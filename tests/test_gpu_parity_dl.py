@@ -75,6 +75,28 @@ def test_sets_issuers_and_rings_over_several_tiles(D, Rd, Rw):
     assert np.sqrt((err ** 2).sum(-1) / (ref ** 2).sum(-1)).max() <= 1e-2
 
 
+def test_even_and_odd_slices_are_summed_apart():
+    """Sums z A_d and m A_w whose even slices are 2^25 and -2^25 and whose odd ones are of the order of one: exact where the even and
+    the odd slices are summed by themselves, while one chain of sums forgets the first odd slice (0.76 for both, 0.96 and 0.23 for
+    one of them, instead of 0.85)."""
+    x = torch.zeros(64, 1, 256)
+    x[..., 0] = x[..., 128] = 2.0 ** 12
+    x[..., 64] = x[..., 192] = 1.0
+    a = torch.zeros(256, 16)
+    a[0], a[128], a[64] = 2.0 ** 13, -2.0 ** 13, 1.0         # z A_d = 2^25 + 1 - 2^25: h1 = tanh 1
+    a_w = a.clone()
+    a_w[192] = 1.0                                           # m = x but in channel 192 (1 - h1): h2 = tanh(1 + 1 - h1)
+    b = torch.zeros(16, 256)
+    b[0, 192] = 1.0
+    b_w = torch.zeros(16, 256)
+    b_w[0] = 1.0
+    bf, zero = (lambda t: t.bfloat16().to(DEV)), torch.zeros(256, device=DEV)
+    d = gf.decay_logit(bf(x), zero, bf(a), bf(b), zero, bf(a_w), bf(b_w), zero)
+    gf.last_device_status()
+    want = np.tanh(2 - np.tanh(1.0))                         # (tanh.approx to 2^-11, h1 and m, h2 and d to bf16's 2^-9)
+    assert np.abs(d.float().cpu().numpy() - want).max() <= 4 * 2.0 ** -9 + 2 * 2.0 ** -11
+
+
 def test_repeats_bit_for_bit():
     """Two worker sets with rings of their own: no set may pass on a phase of the other's."""
     x, xp = synth.make_block_input(4, 16384, 1024, seed=31, device=DEV)
