@@ -84,16 +84,17 @@ enum {
     DL_ACC_FREE = DL_ACC_FULL + DL_NSET,   // ... and read back by the warps of the set
     DL_TURN = DL_ACC_FREE + DL_NSET,       // per issuer of h B: the accumulator of its slice was free
     DL_SUM_FULL = DL_TURN + 2,             // the sum of a pass complete
-    DL_H_READY = DL_SUM_FULL + 1,      // h1 / h2 operand written by all worker warps
-    DL_H_FREE = DL_H_READY + 1,        // the last product of a tile that reads h2 is done
+    DL_H1_READY = DL_SUM_FULL + 1,     // h1 operand written by all worker warps: one phase per tile
+    DL_H2_READY = DL_H1_READY + 1,     // h2 operand: the same (and every warp has read acc3)
+    DL_H_FREE = DL_H2_READY + 1,       // the last product of a tile that reads h2 is done
     DL_BAR_COUNT = DL_H_FREE + 1
 };
 static_assert(16 + 8 * DL_BAR_COUNT <= 512, "barrier block");
 static_assert(DL_SMEM <= 232448, "shared memory budget of one sm_100 CTA");
 // the sum of a pass in two halves, its even and its odd slices, which keeps the chains of additions short (acc1, then acc3: every
-// warp has read acc1 before a product of pass 2's is issued, and acc3 before one of the next tile's); a ring of accumulators for l
-// (pass 2) / d (pass 3) in the order of the slices; the A operands (lane = row, a 32-bit column = two neighbouring channels in
-// bf16): z / m of a set, h1 / h2
+// warp has read acc1 before a product of pass 2's is issued, and acc3 before one of the next tile's: DL_H1_READY, DL_H2_READY); a
+// ring of accumulators for l (pass 2) / d (pass 3) in the order of the slices; the A operands (lane = row, a 32-bit column = two
+// neighbouring channels in bf16): z / m of a set, h1 / h2
 constexpr int DL_NACC = 3;
 constexpr int DL_TM_SUM = 0, DL_TM_ACC = 2 * 64, DL_TM_OP = DL_TM_ACC + 64 * DL_NACC, DL_TM_H = DL_TM_OP + 32 * DL_NSET;
 static_assert(DL_TM_H + 32 <= 512, "tensor memory columns");
@@ -208,7 +209,8 @@ decay_logit_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_consta
         mbar_init(bar(DL_TURN), 1);
         mbar_init(bar(DL_TURN + 1), 1);
         mbar_init(bar(DL_SUM_FULL), 1);
-        mbar_init(bar(DL_H_READY), DL_NWS * DL_NSET);
+        mbar_init(bar(DL_H1_READY), DL_NWS * DL_NSET);
+        mbar_init(bar(DL_H2_READY), DL_NWS * DL_NSET);
         mbar_init(bar(DL_H_FREE), 2);
         sts32(abort_flag, 0u);
         sts32(abort_flag + 4, WAIT_LIMIT_US);
@@ -301,7 +303,10 @@ decay_logit_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_consta
         int n = 0, ia = 0, pa = 0;                           // (A ring position and its phase)
         uint32_t phases = 0;                                 // bit: parity of the set's next operand
         bool alive = true;
-        for (long long r = r_first; r < r_end && alive; r += 128) {
+        int ti = 0;
+        for (long long r = r_first; r < r_end && alive; r += 128, ++ti) {
+            // Every warp has read the sum of the tile before.  (Where a set has no slice in pass 3, its next operand does not say so.)
+            if (ti > 0 && !wait_warp(DL_H2_READY, ti - 1)) break;
             for (int pass = 0; pass < 2 && alive; ++pass)
                 for (int s = 0; s < S; ++s, ++n) {
                     const int set = n & (DL_NSET - 1);
@@ -332,11 +337,12 @@ decay_logit_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_consta
         int turn = 0;                                        // slices of the other issuer so far
         int acc = 0;                                         // accumulator of slice n: a ring that both issuers' slices take in turn
         bool alive = true;
-        for (long long r = r_first; r < r_end && alive; r += 128) {
+        int ti = 0;
+        for (long long r = r_first; r < r_end && alive; r += 128, ++ti) {
             n0 += S;
             const int n_tile = n0;
             for (int pass = 1; pass < 3 && alive; ++pass, n0 += S) {
-                if (!wait_warp(DL_H_READY, pass - 1)) { alive = false; break; }      // (two uses per tile: parities 0, 1)
+                if (!wait_warp(pass == 1 ? DL_H1_READY : DL_H2_READY, ti)) { alive = false; break; }
                 const int kn = pass == 1 ? p.kd : p.kw;
                 for (int n = n0; n < n0 + S; ++n) {
                     const int set = n & (DL_NSET - 1), before = (n - DL_NACC) & (DL_NSET - 1);
@@ -506,7 +512,7 @@ decay_logit_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_consta
                 }
                 tc_fence_before();
                 __syncwarp();
-                mbar_arrive_if(bar(DL_H_READY), lane == 0);
+                mbar_arrive_if(bar(pass == 0 ? DL_H1_READY : DL_H2_READY), lane == 0);
             }
             if (!alive) break;
             // ---- pass 3: d slice -> bf16, in the room of the x stage -> TMA store
