@@ -107,6 +107,21 @@ __device__ __noinline__ void cluster_mbar_wait(uint32_t bar, uint32_t parity, ui
     atomicExch(&g_dev_status, 1);
 }
 
+// Meeting points of the compute warps.  They follow code in which lanes may part (a fold goes token by token where a lane's own D
+// is small, a wait ends for each lane by itself), and an aligned barrier wants the whole warp at once: so the warp meets first.
+__device__ __forceinline__ void ex_bar_sync()
+{
+    __syncwarp();
+    asm volatile("bar.sync 1, %0;" ::"n"(32 * EX_NCW) : "memory");
+}
+__device__ __forceinline__ int ex_bar_or(int any)
+{
+    __syncwarp();
+    asm volatile("{\n\t.reg .pred p, q;\n\tsetp.ne.u32 p, %0, 0;\n\tbarrier.cta.red.or.aligned.pred q, 1, %1, p;\n\tselp.u32 %0, 1, 0, q;\n\t}"
+                 : "+r"(any) : "n"(32 * EX_NCW) : "memory");
+    return any;
+}
+
 // Dense: cu_seqlens == nullptr, unit = b * H + h, rows b*T .. b*T+T-1.
 // Packed: unit = s * H + h, rows cu_seqlens[s] .. cu_seqlens[s+1]-1.
 // Grid: units * (8 / CW) * G, clusters of G; CTA: the compute warps, then the staging warps.  tb: tokens per block, a multiple
@@ -303,7 +318,7 @@ wkv6_exact_kernel(const IO* __restrict__ r, const IO* __restrict__ k, const IO* 
                         *reinterpret_cast<float4*>(dp + 32) = make_float4(D[2].x, D[2].y, D[3].x, D[3].y);
                     }
                 }
-                asm volatile("bar.sync 1, %0;" ::"n"(32 * EX_NCW) : "memory");
+                ex_bar_sync();
                 if (G > 1) {
                     int small = 0;
                     if (publish) {                       // what the block as a whole does to a state
@@ -322,14 +337,14 @@ wkv6_exact_kernel(const IO* __restrict__ r, const IO* __restrict__ k, const IO* 
                         *reinterpret_cast<float2*>(exs + Lay::PUB_D + 64 * (b & 1) + erow) = Dt;      // (every row by several threads)
                         small = Dt.x < EX_D_MIN || Dt.y < EX_D_MIN;
                     }
-                    asm volatile("{\n\t.reg .pred p, q;\n\tsetp.ne.u32 p, %0, 0;\n\tbarrier.cta.red.or.aligned.pred q, 1, %1, p;\n\tselp.u32 %0, 1, 0, q;\n\t}"
-                                 : "+r"(small) : "n"(32 * EX_NCW) : "memory");
+                    small = ex_bar_or(small);
                     if (warp == 0) {
                         if (lane == 0) ck::sts32(sb + 4 * (Lay::SMALL + (b & 1)), small);
                         __syncwarp();
                         if (lane < G) cluster_mbar_arrive(cluster_addr(bar_pub, lane));
                     }
                     cluster_mbar_wait(bar_pub, b & 1, abort_flag);
+                    __syncwarp();
                 }
                 float2 X[CW];                            // the round's start state, kept by the CTA with the last block of the round before
                 {
@@ -356,9 +371,10 @@ wkv6_exact_kernel(const IO* __restrict__ r, const IO* __restrict__ k, const IO* 
                     if (lane < G - 1)
                         asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(small) : "r"(cluster_addr(sb + 4 * (Lay::SMALL + (b & 1)), lane)) : "memory");
                     if (__any_sync(0xffffffffu, small != 0)) {
-                        asm volatile("bar.sync 1, %0;" ::"n"(32 * EX_NCW) : "memory");
+                        ex_bar_sync();
                         if (warp == 0 && lane < G) cluster_mbar_arrive(cluster_addr(bar_fold, lane));
                         cluster_mbar_wait(bar_fold, folds & 1, abort_flag);
+                        __syncwarp();
                         ++folds;
                     }
                 }
@@ -371,7 +387,7 @@ wkv6_exact_kernel(const IO* __restrict__ r, const IO* __restrict__ k, const IO* 
                         *ds = X[c];
                         if (q < NT - 1) X[c] = apply(X[c], *reinterpret_cast<const float2*>(exs + Lay::D + 64 * q + erow), f, w_own + 4 * q * run * EX_N, run);
                     }
-                asm volatile("bar.sync 1, %0;" ::"n"(32 * EX_NCW) : "memory");
+                ex_bar_sync();
                 load_lane(exs + Lay::DS + 512 * warp);
             }
             walk(buf, ts * run, n4, tok);
