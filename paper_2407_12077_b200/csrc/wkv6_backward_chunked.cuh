@@ -1244,15 +1244,22 @@ inline int backward_split(long long units, int T, int n_sm, int* seg_chunks)
 // Workspace of the chunked gradient: checkpoints, bonus gradients per unit and segment, the adjoint's segment
 // summaries, the token-by-token path's scratch (one slot of 64 states per SM and group of warps).
 // Whether a dense gradient call of more units than SMs cuts units between CTAs (BParamsBal): a CTA's range costs two pipeline fills and
-// the hand-over, so where whole units leave more than a fifth of the last round idle, and from an eighth on where the units are long.
-// Measured (us, one CTA per unit -> balanced): 160 units of 32 chunks 189 -> 122; Finch-C2 256 of 32 189.2 -> 184.0, of 64 361.6 -> 347.9,
-// 240 of 32 187.2 -> 173.7, 256 of 16 the same, 384 of 8 88.4 -> 90.3; classic 256 of 32 191.9 -> 193.7, of 64 364.6 -> 363.8, of 94
-// 531.4 -> 522.0.  (The workspace has room for either form.)
+// the hand-over, and a chunk takes longer the more SMs are at work, so it depends on the idle part of the last round of whole units and
+// on the units' length.  Measured (us with cut units / with whole ones, in turn, two runs on different GPUs where two figures stand):
+//   a fifth and more idle (160, 200, 344 units): 0.63-0.90, with 8 chunks 0.80-0.95;
+//   0.19 idle (240, 360, 480 units, two to four rounds): 16 chunks 0.92-0.96 Finch-C2, 0.95-0.98 classic; 32 0.90-0.93, 0.94-0.96; 64
+//     0.91, 0.94-0.99; but 8 chunks 0.93-1.00;
+//   0.16 idle (248 units): 16 chunks 0.99, 1.02; 32 0.95 0.98, 0.98 1.01; 64 0.94 0.96, 0.96 0.97;
+//   0.135 idle (256, 384, 512, 640, 768 units, two to six rounds): 16 chunks 0.98-1.04, 1.00-1.06; 32 0.94-1.03 (mean 0.98), 0.99-1.06;
+//     64 0.96-1.01 (0.98), 0.99-1.04 (1.01); 94 0.96-1.01, 0.98-1.04; 128 0.94-1.01, 0.94-1.03;
+//   0.10 idle (264, 400, 536 units): 16 chunks 1.02-1.06, 1.02-1.08; 32 1.00-1.03, 1.01-1.06; 64 0.97-1.02, 1.00-1.05.
+// The workspace has room for either form (c2 cuts wherever classic does; what classic asks for in vain is 2 KB a unit and 2.4 MB, beside
+// 8 KB of checkpoints per chunk).
 inline bool backward_balance_pays(long long units, int n_chunks, int n_sm, bool c2 = true)
 {
     if (units <= n_sm || units / n_sm - 1 > bc::BAL_MAX_ROUNDS) return false;
     const long long rounds = (units + n_sm - 1) / n_sm, idle = rounds * n_sm - units;
-    const int share = n_chunks >= (c2 ? 16 : 64) ? 8 : 5;
+    const int share = n_chunks < 16 ? 5 : c2 ? (n_chunks < 32 ? 6 : 8) : (n_chunks < 64 ? 6 : 7);
     return idle * n_chunks > 4LL * n_sm && idle * share > rounds * n_sm && 2LL * n_sm * n_sm * n_chunks < (1LL << 32);
 }
 // Floats of the bonus partial sums of a dense call, and of a balanced launch's hand-over blocks and words behind them.

@@ -186,6 +186,6 @@ def test_gradient_units_cut_between_ctas(B, T, H, c2, x_hi, with_dstate):
 
 @pytest.mark.parametrize("T,c2", [(1025, True), (1025, False), (4100, False)])
 def test_gradient_where_an_eighth_of_the_last_round_is_idle(T, c2):
-    # 240 units on 148 SMs: long units are cut there (Finch-C2 from 16 chunks on, classic from 64), short ones are not, in a workspace
-    # laid out for either; a sequence alone has more units than half the SMs, one CTA each
+    # 240 units on 148 SMs, 0.19 of the last round idle: units of 17 and 65 chunks are cut there; a sequence alone has more units than
+    # half the SMs, one CTA each
     test_gradient_units_cut_between_ctas(3, T, 80, c2, -1.0, True)

@@ -115,3 +115,12 @@ def test_fp32_prefill_without_clusters(host_library, status):
     (s, log), (s1, log1) = calls(host_library, call + [[status, 0]], call + [[0, 0]])
     assert s1 == 0 and len(log1) == 1 and log1[0].startswith("grid 128 cluster 4 ")
     assert s == 0 and len(log) == 2 and "refused" in log[0] and log[1].startswith("grid 32 cluster 1 ")
+
+
+@pytest.mark.parametrize("chunks,c2,classic", [(8, 216, 216), (16, 240, 240), (31, 240, 240), (32, 256, 240), (63, 256, 240), (64, 256, 248), (128, 256, 248)])
+def test_gradient_units_are_cut_where_that_was_measured_to_pay(host_library, chunks, c2, classic):
+    # two rounds of 148 SMs, 0.27 to 0.05 of the second idle: the most units that are cut
+    units = (216, 232, 240, 248, 256, 264, 280)
+    logs = calls(host_library, *[backward(f, u // 8, 64 * chunks, 8, 1 << 40) + [[0, 0]] for f in (True, False) for u in units])
+    cut = [any(" cooperative " in line for line in log) for s, log in logs]
+    assert cut == [u <= most for most in (c2, classic) for u in units], cut
