@@ -525,6 +525,11 @@ inline cudaError_t launch_exact_as(long long units, int G, int tb, cudaStream_t 
 // B200, fp32, us per call in a graph, before (one walk per column slab, 4 or 8 slabs up to 74 units) -> now:
 //   4 units of 40 tokens 4.8 -> 4.2, 256 15.5 -> 6.7, 1024 55.9 -> 18.9;  8 of 256 15.8 -> 8.2;  12 of 256 15.8 -> 12.3, 1024 56.2 -> 36.6;
 //   20 of 256 17.6 -> 17.5, 1024 62.6 -> 47.6;  40 of 1024 98.4 -> 76.4;  60 of 400 40.3 -> 38.0;  80 of 1024 139 -> 109;  128 of 512 71.4 -> 57.5.
+// One unit per CTA and column slabs alone, before -> now: 148 of 256 38.1 -> 29.7;  256 of 256 75.8 -> 59.6, 1024 277 -> 222;
+//   512 of 256 151 -> 121;  1024 of 1 38.3 -> 19.6, 256 263 -> 212;  2048 of 256 523 -> 415, in bf16 646 -> 470.  (A CTA of this form leaves the
+//   split's buffers unused and has an SM to itself all the same.)
+// Up to 4 tokens one walk over all columns, split / not: 1 unit of 1 token 3.01 / 2.81 (2.63 before), 4 3.02 / 2.93 (2.87), 60 3.06 / 2.95 (4.20);  of 5
+//   tokens 4 units 3.02 / 3.24.
 // The lines between the forms, us (slabs alone / cluster): 8 units of 70 tokens 6.3 / 6.1, 150 8.6 / 7.4;  16 of 256 12.2 / 13, 400 17.9 / 18.1,
 // 1024 42 / 36.6;  20 of 400 25.5 / 25.3, 700 43.3 / 32.6;  40 of 70 9.5 / 10.8, 130 14.9 / 12.8.
 template <typename IO>
@@ -539,6 +544,7 @@ inline cudaError_t launch_exact(long long units, int n_sm, cudaStream_t st, cons
     else if (units * 8 <= places && T > 384) nt = 2, G = 4;
     else if (units * 4 <= places && T > 384) nt = 1, G = (int)(places / units < 6 ? places / units : 6);
     else if (units * 3 <= places && units * 4 > n_sm && T >= 128) nt = 1, G = 3;
+    if (T <= 4) nt = 1;                            // (one group of tokens: nothing to split)
     if (G > (T + 63) / 64) G = (T + 63) / 64;
     if (G < 1) G = 1;
     // tokens per block: the sequence in as few rounds of blocks of up to 64 as it takes, in equal blocks

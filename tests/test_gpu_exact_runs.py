@@ -21,7 +21,7 @@ def _status():
 
 
 # heads on both sides of each rule of launch_exact (148 SMs), lengths around the blocks and rounds of the form taken
-@pytest.mark.parametrize("H,T", [(4, 1), (4, 64), (4, 65), (4, 255), (4, 257), (4, 300), (8, 96), (8, 97), (8, 513), (12, 384), (12, 385),
+@pytest.mark.parametrize("H,T", [(4, 1), (4, 4), (4, 5), (60, 3), (4, 64), (4, 65), (4, 255), (4, 257), (4, 300), (8, 96), (8, 97), (8, 513), (12, 384), (12, 385),
                                  (20, 385), (32, 390), (36, 130), (40, 127), (40, 128), (40, 193), (60, 65), (80, 130)])
 def test_launch_forms(H, T):
     inp = synth.make_dense(1, T, H, 64, "f32", seed=1000 * H + T, state_std=0.1)

@@ -117,6 +117,12 @@ def test_fp32_prefill_without_clusters(host_library, status):
     assert s == 0 and len(log) == 2 and "refused" in log[0] and log[1].startswith("grid 32 cluster 1 ")
 
 
+@pytest.mark.parametrize("T,grid", [(1, 4), (4, 4), (5, 32)])
+def test_fp32_prefill_of_a_few_tokens_is_not_split(host_library, T, grid):
+    (s, log), = calls(host_library, ["gf_wkv6_prefill_f32", ["p"] * 8 + [1, T, 4, 64, None], [0, 0]])
+    assert s == 0 and len(log) == 1 and log[0].startswith("grid %d cluster 1 " % grid), log
+
+
 @pytest.mark.parametrize("chunks,c2,classic", [(8, 216, 216), (16, 240, 240), (31, 240, 240), (32, 256, 240), (63, 256, 240), (64, 256, 248), (128, 256, 248)])
 def test_gradient_units_are_cut_where_that_was_measured_to_pay(host_library, chunks, c2, classic):
     # two rounds of 148 SMs, 0.27 to 0.05 of the second idle: the most units that are cut
