@@ -122,8 +122,8 @@ def _load_native(lib) -> None:
     if not os.path.exists(path):
         return
     loader = importlib.machinery.ExtensionFileLoader(__name__ + "._binding", path)
-    module = importlib.util.module_from_spec(importlib.util.spec_from_loader(loader.name, loader))
     try:
+        module = importlib.util.module_from_spec(importlib.util.spec_from_loader(loader.name, loader))      # (opens the file)
         loader.exec_module(module)
     except ImportError:                          # (a torch it was not built for: the Python code does all it does)
         return
