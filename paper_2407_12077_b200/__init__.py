@@ -110,7 +110,8 @@ def load_library(build_if_missing: bool = True):
     for name, (res, args) in _SIGNATURES.items():
         fn = getattr(lib, name)            # AttributeError here = header / library mismatch
         fn.restype, fn.argtypes = res, args
-    _load_native(lib)
+    if not (build_if_missing and _build.binding_is_stale()):      # (still: it could not be built, and a file of older source is not used)
+        _load_native(lib)
     _lib = lib
     return lib
 

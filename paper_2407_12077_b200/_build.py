@@ -6,6 +6,7 @@ import os
 import shutil
 import subprocess
 import sysconfig
+import warnings
 
 import torch
 
@@ -49,30 +50,43 @@ def binding_is_stale() -> bool:
 
 
 def build_binding(force: bool = False) -> str | None:
-    """Compile the binding's C++ part (None where there is no compiler or header for it: the Python code does without)."""
+    """Compile the binding's C++ part (None where that cannot be done: no compiler or header for it, a compiler that fails, a
+    directory that cannot be written.  The Python code does without)."""
     if not force and not binding_is_stale():
         return BINDING_PATH
     gxx, py = shutil.which("g++"), sysconfig.get_paths()["include"]
     inc = os.path.join(os.path.dirname(torch.__file__), "include")
     cuda = os.path.dirname(os.path.dirname(shutil.which("nvcc") or "/usr/local/cuda/bin/nvcc"))
-    if gxx is None or not os.path.exists(os.path.join(py, "Python.h")) or not os.path.exists(inc):
+    if gxx is None or not os.path.exists(os.path.join(py, "Python.h")) or not os.path.exists(inc) or not os.access(_PKG, os.W_OK):
         return None
     tmp = f"{BINDING_PATH}.{os.getpid()}"
     cmd = [gxx, "-O2", "-std=c++17", "-shared", "-fPIC", "-fvisibility=hidden", f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}",
            "-I", py, "-I", inc, "-I", os.path.join(inc, "torch", "csrc", "api", "include"), "-I", os.path.join(cuda, "include"), "-o", tmp, BINDING_SRC,
            "-L", os.path.join(os.path.dirname(torch.__file__), "lib"), "-ltorch_python", "-ltorch_cpu", "-lc10", "-lc10_cuda"]
-    res = subprocess.run(cmd, capture_output=True, text=True)
-    if res.returncode != 0:
-        raise RuntimeError("g++ failed:\n" + res.stdout + res.stderr)
-    os.replace(tmp, BINDING_PATH)
-    return BINDING_PATH
+    try:
+        res = subprocess.run(cmd, capture_output=True, text=True)
+        if res.returncode == 0:
+            os.replace(tmp, BINDING_PATH)
+            return BINDING_PATH
+        why = res.stdout + res.stderr
+    except OSError as e:
+        why = str(e)
+    if os.path.exists(tmp):
+        os.remove(tmp)
+    warnings.warn("the binding's C++ part could not be built (calls go through Python, a few microseconds slower):\n" + why[-2000:], RuntimeWarning)
+    return None
 
 
 def build(force: bool = False, verbose: bool = False) -> str:
     """Compile every CUDA source into libgfwkv6.so, and the binding's C++ part.  Cross-compiles without a GPU."""
+    if force or is_stale():
+        build_library(verbose)
     build_binding(force)
-    if not force and not is_stale():
-        return LIB_PATH
+    return LIB_PATH
+
+
+def build_library(verbose: bool = False) -> str:
+    """Compile every CUDA source into libgfwkv6.so."""
     cmd = [_nvcc(), *NVCC_FLAGS, "-I", os.path.join(_ROOT, "include"), "-I", CSRC,
            "-o", LIB_PATH, *sources()]
     if verbose:
