@@ -51,8 +51,8 @@ def test_shapes_tails_and_ranks(B, T, D, Rd, Rw):
 @pytest.mark.parametrize("rows,D", [(63, 64), (64, 64), (65, 64), (129, 64), (127, 192), (64 * 148, 192), (64 * 149 + 1, 192),
                                     (64 * 300 - 1, 192)])
 def test_shares_of_rows_and_slices(rows, D):
-    """A CTA's share in units of 64 rows (half tiles, one CTA more or less than SMs), one slice (the second worker set has
-    none) and three (two and one)."""
+    """A CTA's share in units of 64 rows (half tiles, one CTA more or less than SMs), one slice (a pass has work for one of the four
+    worker sets, another one each pass) and three (for three of them)."""
     _run(1, rows, D, 32, 64, seed=rows + D)
 
 
@@ -98,7 +98,7 @@ def test_even_and_odd_slices_are_summed_apart():
 
 
 def test_repeats_bit_for_bit():
-    """Two worker sets with rings of their own: no set may pass on a phase of the other's."""
+    """Four worker sets and three accumulators, stages that always serve one set: no set may pass on a phase of another's."""
     x, xp = synth.make_block_input(4, 16384, 1024, seed=31, device=DEV)
     w = synth.make_decay_lora(1024, 32, 64, seed=32, device=DEV)
     run = lambda: gf.decay_logit(x, w["mu_x"], w["A_d"], w["B_d"], w["lambda_d"], w["A_w"], w["B_w"], w["lambda_w"], x_prev=xp)
